@@ -115,10 +115,10 @@ def workload(args, rank: int = 0):
 
 # Launch settings per workload at full size: the fastest row of
 # paper_1403_0802_gb300.autotune on GB300 (points per item x warps per block x
-# edges per chunk; 0 = the library default).
-TUNED = {"p2p": dict(ppi=128, block=4, edges=0), "pip": dict(ppi=128, block=4, edges=0),
-         "pip3_1": dict(ppi=128, block=4, edges=64), "pip3_2": dict(ppi=128, block=2, edges=64),
-         "pip3_3": dict(ppi=128, block=8, edges=64), "p2p4": dict(ppi=128, block=4, edges=0)}
+# edges per chunk; 0 = the library default, and the PIP join has no items to shape).
+TUNED = {"p2p": dict(ppi=128, block=4, edges=0), "pip": dict(ppi=0, block=0, edges=0),
+         "pip3_1": dict(ppi=0, block=0, edges=0), "pip3_2": dict(ppi=0, block=0, edges=0),
+         "pip3_3": dict(ppi=0, block=0, edges=0), "p2p4": dict(ppi=128, block=4, edges=0)}
 
 
 def tuned(args) -> dict:
@@ -328,8 +328,9 @@ def metric_name(kind):
 def config_of(w, args):
     t = tuned(args)
     c = {"workload": w.name, "points": int(len(w.points)), "grid": f"{w.grid['nx']}x{w.grid['ny']}",
-         "form": args.form, "launch": "per_request", "pts_per_item": t["ppi"] or 128,
-         "warps_per_block": t["block"] or 4, "edges_per_chunk": t["edges"] or ("64" if w.kind == "pip" else "none")}
+         "form": args.form, "launch": "per_request"}
+    if w.kind == "p2p":
+        c.update(pts_per_item=t["ppi"] or 128, warps_per_block=t["block"] or 4, edges_per_chunk=t["edges"] or "none")
     big = len(w.points) * 16 > 129e6
     c["l2"] = ("inputs larger than L2 (points %d MB > 129 MB); no flush" % (len(w.points) * 16 // 10 ** 6) if big
                else "points %d MB fit in L2; steps re-read them (no flush)" % (len(w.points) * 16 // 10 ** 6))
@@ -530,7 +531,7 @@ def roofline_of(w, form, st, ms_per_join, peaks, census=None):
     io = n * (16 + (12 if w.kind == "p2p" else 4))
     algo_bytes = io + layer_bytes(w)
     hbm_ach = algo_bytes / (ms_per_join / 1e3) / 1e9
-    kernel = f"k_{w.kind}_refine<{form}>"
+    kernel = f"k_p2p_refine<{form}>" if w.kind == "p2p" else "k_pip_join"
     r = {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
          "frac": achieved / peak if achieved else None,
          "traffic": measured_traffic(kernel, w.name, w.kind),
@@ -643,10 +644,10 @@ def run_ours(args):
     stream = torch.cuda.current_stream(dev)
     baselines = rank == 0 and world == 1 and not args.no_baselines
     head = join_leg(api, args, w, dev, stream, world, args.steps, args.warmup, peaks, baselines=baselines)
-    # cell_hist, the scan (2 phases up to 256 tiles of 1,024 cells, else 3), scatter; refine; FP32X P2P
-    # recheck; unsort
+    # PIP: one kernel.  P2P: cell_hist, the scan (2 phases up to 256 tiles of 1,024 cells, else 3), scatter;
+    # refine; FP32X recheck; unsort
     scan_tiles = (int(w.grid["nx"]) * int(w.grid["ny"]) + 1023) // 1024
-    kernels_per_join = 1 + (2 if scan_tiles <= 256 else 3) + 1 + 1 + (1 if (w.kind == "p2p" and args.form == "fp32x") else 0) + 1
+    kernels_per_join = 1 if w.kind == "pip" else 5 + (1 if scan_tiles <= 256 else 2) - 1 + (args.form == "fp32x")
     extra = {}
     if rank == 0 and world == 1 and args.workload == "p2p" and not args.no_extra and not args.points:
         import copy

@@ -71,14 +71,16 @@ typedef enum {
 /* Refinement arithmetic. */
 enum {
     SJ_FP64 = 0,  /* plain FP64 refinement                                        */
-    SJ_FP32X = 1  /* cell-relative FP32 with FP64 fallback: PIP ids are identical
-                     to the FP64 rule; P2P ids are exact (ties aside) and the
-                     distance error is bounded per point                           */
+    SJ_FP32X = 1  /* cell-relative FP32 with FP64 fallback: P2P ids are exact
+                     (ties aside) and the distance error is bounded per point.
+                     PIP: both forms run the same code (FP32 decides only what its
+                     error bounds make certain, the FP64 rule the rest), so ids are
+                     the FP64 rule's bit for bit                                   */
 };
 
-/* Launch form.  Every join's refinement is one persistent launch whose warps
- * take work items from a device counter (cost-balanced); both values select
- * that code and give the same results.  Batched rounds of many requests are
+/* Launch form.  A P2P join's refinement is one persistent launch whose warps
+ * take work items from a device counter (cost-balanced); a PIP join is one
+ * launch over the points.  Both values select that code and give the same results.  Batched rounds of many requests are
  * the sj_engine_* calls below. */
 enum {
     SJ_PER_REQUEST = 0, /* one pass of kernels per call                           */
@@ -87,7 +89,8 @@ enum {
 
 /* Join options; a zeroed struct (or NULL) selects the defaults.  The launch
  * knobs (block, pts_per_item, edges_per_chunk) change speed only, never a
- * result; paper_1403_0802_gb300/autotune.py times their combinations. */
+ * result, and only that of P2P joins (the PIP join has no work items: it checks
+ * the values and ignores them); paper_1403_0802_gb300/autotune.py times their combinations. */
 typedef struct {
     int32_t form;            /* SJ_FP64 (default) or SJ_FP32X                       */
     int32_t launch;          /* SJ_PER_REQUEST (default) or SJ_PERSISTENT           */
@@ -96,26 +99,24 @@ typedef struct {
                                 the occupancy of 4-warp blocks, in warps)          */
     int32_t pts_per_item;    /* points per work item, 1..128, 0 = default (128)    */
     int32_t edges_per_chunk; /* edge budget of a work item: a cell whose points
-                                each test w > edges_per_chunk edges (PIP: the near
-                                edges of its boundary candidates; P2P: its segment
+                                each test w > edges_per_chunk segments (its segment
                                 list) is cut into items of
                                 max(min(pts_per_item, 8),
                                     pts_per_item * edges_per_chunk / w) points, so
                                 that heavy cells yield more, smaller items (the work
                                 queue split by candidate-edge count).  0 = the
-                                default: 64 for polygon layers, no split for
-                                polyline layers; a value above every cell's work
-                                (e.g. INT32_MAX) turns the split off              */
+                                default: no split                                  */
     int32_t flags;           /* SJ_FLAG_* bits                                      */
 } sj_opts;
 
 /* opts.flags: record CUDA events on the call's stream around the refinement
  * kernels; their summed elapsed time is reported by sj_layer_get_stats. */
 #define SJ_FLAG_TIME_REFINE 1
-/* opts.flags of the joins: order the points inside each grid cell by sub-cell
- * (P2P: 4 x 4 sub-cells in Z-order; PIP: 8 horizontal bands) before they are
+/* opts.flags of the joins: P2P: order the points inside each grid cell by sub-cell
+ * (4 x 4 sub-cells in Z-order) before they are
  * cut into work items (SJ_FLAG_SUBCELL_ON), or keep them in arrival order
- * (the default; SJ_FLAG_SUBCELL_OFF says so explicitly).  Results do not
+ * (the default; SJ_FLAG_SUBCELL_OFF says so explicitly).  PIP: search edge lists of
+ * more than 16 edges by y instead of those of more than 32 (fewer tests).  Results do not
  * depend on it (a point's result depends on the point and the layer only).
  * Work items of dense cells then cover compact parts of their cell, so the
  * exact per-item prunes leave fewer tests, at the price of a per-sub-cell
@@ -139,10 +140,11 @@ typedef struct {
 typedef struct {
     int64_t joins;
     int64_t points;        /* points submitted                                  */
-    int64_t items;         /* (cell, point-chunk) work items                    */
+    int64_t items;         /* P2P: (cell, point-chunk) work items; PIP: batches of up
+                              to 32 points refined together                     */
     int64_t pairs;         /* (point, candidate object) pairs refined            */
     int64_t edge_tests;    /* PIP: point x edge tests; P2P: point x segment tests */
-    int64_t fallbacks;     /* SJ_FP32X: PIP edges / P2P points redone in FP64   */
+    int64_t fallbacks;     /* PIP: edges redone in FP64; P2P (SJ_FP32X): points  */
     int64_t hits;          /* points given an id                                 */
     int64_t refine_launches; /* refinement launches timed (SJ_FLAG_TIME_REFINE)  */
     double refine_ms;        /* their summed device time, milliseconds           */
@@ -154,9 +156,9 @@ typedef struct {
     int64_t census_straddles; /* edges of the points' candidate polygons, and how
                                  many of them straddle the point's y              */
     int64_t resolved;         /* PIP: points whose cell's candidates are all
-                                 classified inside / outside, answered by the
-                                 cell-id pass without refinement (counted in
-                                 hits, not in items, pairs or algo_tests)         */
+                                 classified inside / outside, answered without
+                                 refinement (counted in hits, not in items,
+                                 pairs or algo_tests)                             */
 } sj_run_stats;
 
 /* Build a resident polygon layer and its candidate lists (Sec. III.A: MBB of
@@ -300,8 +302,8 @@ typedef struct {
 /* Create an engine for rounds of at most max_points points and max_requests
  * requests per layer.  opts selects form and points per work item (as for the
  * joins; NULL = defaults).  The engine allocates one workspace per layer on
- * the first round that uses the layer (about 36 bytes per point for a
- * polygon layer, 60 for a polyline layer, plus 8 bytes per grid cell) and captures that layer's graph then; later rounds allocate
+ * the first round that uses the layer (for a polyline layer about 60 bytes per
+ * point and 8 bytes per grid cell; for a polygon layer the request table alone) and captures that layer's graph then; later rounds allocate
  * nothing.  Layers must outlive the engine.  Errors: SJ_ERR_INVALID. */
 sj_status sj_engine_create(int64_t max_points, int32_t max_requests, const sj_opts *opts, sj_engine **out);
 

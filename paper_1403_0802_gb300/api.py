@@ -140,10 +140,9 @@ def pip_join(layer: Layer, pts, out: torch.Tensor | None = None, form: str = "fp
              pts_per_item: int = 0, stream=None, time_refine: bool = False, subcell: bool | None = None,
              block: int = 0, edges_per_chunk: int = 0) -> torch.Tensor:
     """Polygon id (or -1) per point, int32 on the points' device (Sec. III.C).
-    Launch knobs (results do not depend on them): subcell orders points by
-    sub-cell inside their cells (None: the library's choice), block = warps per
-    refinement block (0: 4), edges_per_chunk = the edge budget of a work item
-    (0: the library default, 64 for polygon layers)."""
+    Launch knobs (results do not depend on them): subcell = search edge lists
+    of more than 16 edges instead of 32; pts_per_item, block and
+    edges_per_chunk shape the polyline join's work items and do nothing here."""
     p = _points(pts)
     out = torch.empty(p.shape[0], dtype=torch.int32, device=p.device) if out is None else out
     o = _opts(form, launch, pts_per_item, time_refine, subcell, block, edges_per_chunk)
@@ -157,7 +156,9 @@ def p2p_join(layer: Layer, pts, out_id: torch.Tensor | None = None, out_d: torch
              time_refine: bool = False, window: float | None = None, subcell: bool | None = None,
              block: int = 0, edges_per_chunk: int = 0):
     """(nearest polyline id or -1, distance or +inf) per point (Sec. III.B); window (<= the layer's D)
-    replaces D for this call (sj_p2p_join_window); launch knobs as in pip_join."""
+    replaces D for this call (sj_p2p_join_window).  Launch knobs (results do not depend on them): subcell
+    orders points by sub-cell inside their cells, block = warps per refinement block (0: 4),
+    edges_per_chunk = the segment budget of a work item (0: none)."""
     p = _points(pts)
     n = p.shape[0]
     out_id = torch.empty(n, dtype=torch.int32, device=p.device) if out_id is None else out_id

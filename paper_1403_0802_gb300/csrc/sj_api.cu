@@ -18,8 +18,8 @@ namespace sj {
 cudaError_t launch_check_offsets(const int64_t *off, int64_t n, int64_t min_size, int64_t first, int64_t last, int *out,
                                  int *bad, cudaStream_t s);
 cudaError_t launch_check_finite(const double2 *v, int n, int *bad, cudaStream_t s);
-cudaError_t launch_pip_topology(const int *ring_off, int R, const int *poly_ring_off, int P, int *poly_voff, int *nxt,
-                                int *prv, cudaStream_t s);
+cudaError_t launch_pip_topology(const int *ring_off, int R, const int *poly_ring_off, int P, int V, int *poly_voff,
+                                int *nxt, int *prv, int *owner, cudaStream_t s);
 cudaError_t launch_split(const double2 *v, int n, float4 *vs, cudaStream_t s);
 cudaError_t launch_seg_table(const double2 *v, const int *line_off, int L, double2 *e64, double *inv64, float4 *seg32,
                              cudaStream_t s);
@@ -33,22 +33,14 @@ cudaError_t launch_segcell_emit(const LayerBuildArgs &a, const float4 *seg32, co
                                 int *cell_algo, cudaStream_t s);
 cudaError_t launch_prow_count(const LayerBuildArgs &a, int *prow_base, int *prow_r0, unsigned long long *total,
                               cudaStream_t s);
-cudaError_t launch_prow_edge_count(const LayerBuildArgs &a, const int *nxt, const int *prow_base, const int *prow_r0,
-                                   int *cnt, unsigned long long *total, cudaStream_t s);
-cudaError_t launch_prow_edge_emit(const LayerBuildArgs &a, const int *nxt, const int *prow_base, const int *prow_r0,
-                                  const int *cnt, int slots, int *prow_start, int *cursor, int *pedge_ids,
-                                  cudaStream_t s);
 cudaError_t launch_cseg_records(const int *cseg_start, const int *cseg_ids, const GridDev &g, const float *frame_x,
                                 const float *frame_y, const float4 *vsplit, const float4 *seg32, float4 *rec,
                                 cudaStream_t s);
-cudaError_t launch_prow_records(const int *pedge_ids, long long ME, const int *nxt, const float4 *vsplit,
-                                float4 *rec, cudaStream_t s);
 cudaError_t launch_offsets(const int *cnt, int n, int *out, int2 *block_sums, size_t cap, int *totals,
                            cudaStream_t s);
 cudaError_t launch_sum64(const int *cnt, int n, unsigned long long *total, cudaStream_t s);
 cudaError_t launch_thresholds(const GridDev &g, unsigned long long *kx, unsigned long long *ky, cudaStream_t s);
 cudaError_t launch_frames(const GridDev &g, float *fx, float *fy, cudaStream_t s);
-int pip_blocks_per_sm(int form);
 int p2p_blocks_per_sm(int form);
 }  // namespace sj
 
@@ -148,10 +140,7 @@ sj_status sj::device_info(int dev, DevInfo **out) {
     DevInfo &d = g_dev[dev];
     if (!d.init) {
         CUDA_TRY(cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev));
-        for (int f = 0; f < 2; ++f) {
-            d.pip_bps[f] = pip_blocks_per_sm(f);
-            d.p2p_bps[f] = p2p_blocks_per_sm(f);
-        }
+        for (int f = 0; f < 2; ++f) d.p2p_bps[f] = p2p_blocks_per_sm(f);
         // keep freed stream-ordered scratch in the pool for the next call
         cudaMemPool_t pool;
         if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
@@ -184,6 +173,12 @@ static GridDev make_grid(const sj_grid *g) {
     d.cw = cw; d.ch = ch;
     d.x0f = (float)g->x0; d.y0f = (float)g->y0;
     d.icwf = (float)(1.0 / cw); d.ichf = (float)(1.0 / ch);
+    // axis_estimate: |v - fl(v)| < 2u |v| (truncation), |x0f - x0| <= u |x0|, the
+    // difference's rounding u per cell index, 1 / cw rounded (2u) and the product
+    // (u): at most 3u max|x| / cw + 4u nx cells, times 1.5
+    const double u = 5.9604644775390625e-08;
+    d.tolx = (float)(1.5 * u * (3.0 * std::max(std::fabs(g->x0), std::fabs(g->x1)) / cw + 4.0 * g->nx));
+    d.toly = (float)(1.5 * u * (3.0 * std::max(std::fabs(g->y0), std::fabs(g->y1)) / ch + 4.0 * g->ny));
     d.kx = d.ky = nullptr;
     return d;
 }
@@ -212,15 +207,13 @@ static float float_up(double x) {
     return ((double)f < x) ? std::nextafter(f, INFINITY) : f;
 }
 
-// Layer-dependent fields of the refinement arguments.
+// Layer-dependent fields of the P2P refinement arguments.
 void sj::fill_refine(const sj_layer *L, RefineArgs &ra) {
     ra.g = L->g;
     ra.cand_start = L->cand_start;
     ra.cand_ids = L->cand_ids;
     ra.obj_voff = L->obj_voff;
-    ra.nxt = L->nxt;
     ra.verts = L->verts;
-    ra.vsplit = L->vsplit;
     ra.seg_e64 = L->seg_e64;
     ra.seg_inv64 = L->seg_inv64;
     ra.seg32 = L->seg32;
@@ -228,20 +221,6 @@ void sj::fill_refine(const sj_layer *L, RefineArgs &ra) {
     ra.cseg_ids = L->cseg_ids;
     ra.cell_algo = L->cell_algo;
     ra.cseg_rec = L->cseg_rec;
-    ra.prow_base = L->prow_base;
-    ra.prow_r0 = L->prow_r0;
-    ra.prow_start = L->prow_start;
-    ra.pedge_ids = L->pedge_ids;
-    ra.pedge_rec = L->pedge_rec;
-    ra.cand_cls = L->cand_cls;
-    ra.bnear_start = L->bnear_start;
-    ra.bnear_ids = L->bnear_ids;
-    ra.bnear_rec = L->bnear_rec;
-    ra.bnear_key = L->bnear_key;
-    ra.bnear_h = L->bnear_h;
-    ra.bflip_start = L->bflip_start;
-    ra.bflip_len = L->bflip_len;
-    ra.bflip_keys = L->bflip_keys;
     ra.D = L->D;
     ra.Df = L->Df;
     ra.Ddn = L->Ddn;
@@ -250,6 +229,25 @@ void sj::fill_refine(const sj_layer *L, RefineArgs &ra) {
     ra.frame_x = L->frames;
     ra.frame_y = L->frames + L->g.nx;
     ra.stats = L->stats;
+}
+
+// Arguments of the PIP join of a polygon layer.  Beyond the FP32 range the
+// cell-relative coordinates mean nothing: an infinite rounding bound sends
+// every test to the FP64 rule.
+PipArgs sj::pip_args(const sj_layer *L) {
+    PipArgs a{};
+    a.g = L->g;
+    a.cell_code = L->cell_code;
+    a.units = L->units;
+    a.units_n = (int)L->units_n;
+    a.verts = L->verts;
+    a.nxt = L->nxt;
+    a.frame_x = L->frames;
+    a.frame_y = L->frames + L->g.nx;
+    a.eps = L->xmax > 1e30 ? INFINITY : L->eps_abs;
+    a.search = PIP_SEARCH;
+    a.stats = L->stats;
+    return a;
 }
 
 // ------------------------------------------------------------------ layers
@@ -271,12 +269,10 @@ static void resolve_events(const sj_layer *L) {
 
 static void layer_free(sj_layer *L) {
     resolve_events(L);
-    void *ptrs[] = {L->verts, L->vsplit, L->obj_voff, L->nxt, L->prv, L->ring_off, L->poly_ring_off, L->seg_e64,
+    void *ptrs[] = {L->verts, L->vsplit, L->obj_voff, L->nxt, L->ring_off, L->poly_ring_off, L->seg_e64,
                     L->seg_inv64, L->seg32, L->mbb, L->cand_start, L->cand_ids, L->stats, L->cell_keys,
                     L->frames, L->cseg_start, L->cseg_ids, L->cell_algo, L->cseg_rec, L->prow_base, L->prow_r0,
-                    L->prow_start, L->pedge_ids, L->pedge_rec, L->cand_cls, L->cell_res, L->cell_work,
-                    L->bnear_start, L->bnear_ids,
-                    L->bnear_rec, L->bnear_key, L->bnear_h, L->bflip_start, L->bflip_len, L->bflip_keys};
+                    L->prow_start, L->pedge_ids, L->cell_work, L->cell_code, L->units};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete L;
@@ -442,177 +438,169 @@ static sj_status build_seg_lists(sj_layer *L, cudaStream_t s) {
     return SJ_OK;
 }
 
-// PIP boundary entries (after the classes): near edge lists with staging
-// records, and the far-right parity flips (see k_pip_boundary).
-static sj_status build_boundary_lists(sj_layer *L, double delta, cudaStream_t s) {
-    const int M = (int)L->M;
-    CUDA_TRY(dalloc(&L->bnear_start, (size_t)M + 1));
-    CUDA_TRY(dalloc(&L->bflip_start, (size_t)M + 1));
-    CUDA_TRY(dalloc(&L->bflip_len, (size_t)M));
-    CUDA_TRY(dalloc(&L->bnear_h, (size_t)M));
-    if (M == 0) {
-        L->MN = L->MF = 0;
-        CUDA_TRY(dalloc(&L->bnear_ids, 0));
-        CUDA_TRY(dalloc(&L->bnear_rec, 0));
-        CUDA_TRY(dalloc(&L->bnear_key, 0));
-        CUDA_TRY(dalloc(&L->cell_work, (size_t)L->g.G));
-        CUDA_TRY(cudaMemsetAsync(L->cell_work, 0, sizeof(int) * (size_t)L->g.G, s));
-        CUDA_TRY(dalloc(&L->bflip_keys, 0));
-        CUDA_TRY(cudaMemsetAsync(L->bnear_start, 0, sizeof(int), s));
-        CUDA_TRY(cudaMemsetAsync(L->bflip_start, 0, sizeof(int), s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-        return SJ_OK;
+// Build scratch: stream-ordered allocations, freed with the object.
+struct BuildTmp {
+    cudaStream_t s;
+    std::vector<void *> ptrs;
+    explicit BuildTmp(cudaStream_t st) : s(st) {}
+    ~BuildTmp() {
+        for (void *p : ptrs) cudaFreeAsync(p, s);
     }
-    struct Tmp {
-        void *p[5] = {};
-        ~Tmp() {
-            for (void *q : p)
-                if (q) cudaFree(q);
+    template <class T>
+    cudaError_t take(T **p, size_t n) {
+        void *q = nullptr;
+        cudaError_t e = dev_malloc_async(&q, (n ? n : 1) * sizeof(T), s);
+        if (e == cudaSuccess) {
+            ptrs.push_back(q);
+            *p = (T *)q;
         }
-    } tmp;
-    BoundaryArgs a{};
-    a.g = L->g;
-    a.cand_start = L->cand_start;
-    a.cand_ids = L->cand_ids;
-    a.cls = L->cand_cls;
-    a.prow_base = L->prow_base;
-    a.prow_r0 = L->prow_r0;
-    a.prow_start = L->prow_start;
-    a.pedge_ids = L->pedge_ids;
-    a.nxt = L->nxt;
-    a.prv = L->prv;
-    a.verts = L->verts;
-    a.delta = delta;
-    int *totals = nullptr;
-    int2 *bs = nullptr;
-    const size_t cap = bucket_scan_blocks(M);
-    CUDA_TRY(dalloc(&a.near_cnt, (size_t)M)); tmp.p[0] = a.near_cnt;
-    CUDA_TRY(dalloc(&a.flip_cnt, (size_t)M)); tmp.p[1] = a.flip_cnt;
-    CUDA_TRY(dalloc(&totals, 8)); tmp.p[2] = totals;
-    CUDA_TRY(dalloc(&bs, cap)); tmp.p[3] = bs;
-    CUDA_TRY(launch_pip_boundary(a, 0, s));
-    {   // both lists' sizes in 64 bits before their 32-bit offsets
-        unsigned long long *sum = nullptr, hs[2] = {0, 0};
-        CUDA_TRY(dalloc(&sum, 2)); tmp.p[4] = sum;
-        CUDA_TRY(cudaMemsetAsync(sum, 0, 2 * sizeof(unsigned long long), s));
-        CUDA_TRY(launch_sum64(a.near_cnt, M, sum, s));
-        CUDA_TRY(launch_sum64(a.flip_cnt, M, sum + 1, s));
-        CUDA_TRY(cudaMemcpyAsync(hs, sum, sizeof(hs), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-        if (hs[0] > (unsigned long long)MAX_COUNT || hs[1] > (unsigned long long)MAX_COUNT)
-            return fail(SJ_ERR_INVALID, "boundary lists exceed 2^31 - 2^22 entries");
+        return e;
     }
-    CUDA_TRY(launch_offsets(a.near_cnt, M, L->bnear_start, bs, cap, totals, s));
-    CUDA_TRY(launch_offsets(a.flip_cnt, M, L->bflip_start, bs, cap, totals + 4, s));
-    int tot[8] = {};
-    CUDA_TRY(cudaMemcpyAsync(tot, totals, sizeof(tot), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    L->MN = tot[0];
-    L->MF = tot[4];
-    CUDA_TRY(dalloc(&L->bnear_ids, (size_t)L->MN));
-    CUDA_TRY(dalloc(&L->bnear_rec, 2 * (size_t)L->MN));
-    CUDA_TRY(dalloc(&L->bnear_key, (size_t)L->MN));
-    CUDA_TRY(dalloc(&L->bflip_keys, (size_t)L->MF));
-    a.near_start = L->bnear_start;
-    a.flip_start = L->bflip_start;
-    a.near_ids = L->bnear_ids;
-    a.flip_keys = L->bflip_keys;
-    CUDA_TRY(launch_pip_boundary(a, 1, s));
-    CUDA_TRY(launch_pip_flips(L->bflip_start, M, L->bflip_keys, L->bflip_len, s));
-    // near lists ordered by lower y, with their keys and y-extents (the
-    // refinement's window search on long lists), then the staging records
-    CUDA_TRY(launch_pip_near_sort(L->bnear_start, M, L->bnear_ids, L->nxt, L->vsplit, L->bnear_key, L->bnear_h, s));
-    CUDA_TRY(dalloc(&L->cell_work, (size_t)L->g.G));
-    CUDA_TRY(launch_cell_work_pip(L->cand_start, L->cand_cls, L->bnear_start, L->g.G, L->cell_work, s));
-    if (L->MN > 0) CUDA_TRY(launch_prow_records(L->bnear_ids, (long long)L->MN, L->nxt, L->vsplit, L->bnear_rec, s));
+};
+
+// 64-bit counters on the device, read back.
+static sj_status read_totals(const unsigned long long *d, unsigned long long *h, int n, cudaStream_t s) {
+    CUDA_TRY(cudaMemcpyAsync(h, d, sizeof(*h) * (size_t)n, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     return SJ_OK;
 }
 
-// PIP per-(polygon, row) edge lists (after build_candidates).
-static sj_status build_row_lists(sj_layer *L, cudaStream_t s) {
-    const int P = L->nobj;
+// PIP cell records (after build_candidates): per-(polygon, row) edge lists,
+// what each candidate entry holds, the cells' codes and records (sj_pip.cu).
+// prv and owner (per vertex) are the caller's.
+static sj_status build_pip_records(sj_layer *L, const int *prv, const int *owner, cudaStream_t s) {
+    const int P = L->nobj, G = L->g.G, V = L->V, M = (int)L->M;
     CUDA_TRY(dalloc(&L->prow_base, (size_t)P + 1));
     CUDA_TRY(dalloc(&L->prow_r0, (size_t)P));
+    CUDA_TRY(dalloc(&L->cell_code, (size_t)G));
     if (P == 0) {
-        L->MR = L->ME = 0;
+        L->MR = L->ME = L->units_n = 0;
         CUDA_TRY(dalloc(&L->prow_start, 1));
         CUDA_TRY(dalloc(&L->pedge_ids, 0));
-        CUDA_TRY(dalloc(&L->pedge_rec, 0));
-        CUDA_TRY(dalloc(&L->cand_cls, 0));
-        CUDA_TRY(dalloc(&L->cell_res, (size_t)L->g.G));
-        CUDA_TRY(cudaMemsetAsync(L->cell_res, 0xff, sizeof(int) * (size_t)L->g.G, s));   // -1: no candidates
+        CUDA_TRY(dalloc(&L->units, 0));
+        CUDA_TRY(cudaMemsetAsync(L->cell_code, 0xff, sizeof(int) * (size_t)G, s));   // -1: no candidates
         CUDA_TRY(cudaMemsetAsync(L->prow_base, 0, sizeof(int), s));
         CUDA_TRY(cudaMemsetAsync(L->prow_start, 0, sizeof(int), s));
         CUDA_TRY(cudaStreamSynchronize(s));
         return SJ_OK;
     }
+    BuildTmp tmp(s);
+    unsigned long long *total = nullptr, h[4] = {};
+    int *totals = nullptr;
+    CUDA_TRY(tmp.take(&total, 4));
+    CUDA_TRY(tmp.take(&totals, 4));
+    CUDA_TRY(cudaMemsetAsync(total, 0, 4 * sizeof(unsigned long long), s));
+
+    // rows of each polygon, then its (polygon, row) edge lists
     LayerBuildArgs a{};
     a.g = L->g;
     a.kind = KIND_PIP;
     a.nobj = P;
-    a.V = L->V;
+    a.V = V;
     a.verts = L->verts;
     a.obj_voff = L->obj_voff;
     a.mbb = L->mbb;
-    struct Tmp {
-        void *p[5] = {};
-        ~Tmp() {
-            for (void *q : p)
-                if (q) cudaFree(q);
-        }
-    } tmp;
-    unsigned long long *total = nullptr;
-    int *cnt = nullptr, *cursor = nullptr;
-    CUDA_TRY(dalloc(&total, 2)); tmp.p[0] = total;
-    CUDA_TRY(dalloc(&a.totals, 4)); tmp.p[1] = a.totals;
-    CUDA_TRY(cudaMemsetAsync(total, 0, 2 * sizeof(unsigned long long), s));
-    {
-        const size_t nbs = bucket_scan_blocks(P);
-        CUDA_TRY(dalloc(&a.block_sums, nbs)); tmp.p[2] = a.block_sums;
-        a.bs_cap = nbs;
-    }
+    a.totals = totals;
+    a.bs_cap = bucket_scan_blocks(P);
+    CUDA_TRY(tmp.take(&a.block_sums, a.bs_cap));
     CUDA_TRY(launch_prow_count(a, L->prow_base, L->prow_r0, total, s));
-    unsigned long long MR = 0;
-    CUDA_TRY(cudaMemcpyAsync(&MR, total, sizeof(MR), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    if (MR > (unsigned long long)MAX_COUNT) return fail(SJ_ERR_INVALID, "more than 2^31 - 2^22 (polygon, row) slots");
-    L->MR = (int64_t)MR;
-    CUDA_TRY(dalloc(&cnt, (size_t)MR)); tmp.p[3] = cnt;
-    CUDA_TRY(dalloc(&cursor, (size_t)MR)); tmp.p[4] = cursor;
-    CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)MR, s));
-    CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * (size_t)MR, s));
-    CUDA_TRY(launch_prow_edge_count(a, L->nxt, L->prow_base, L->prow_r0, cnt, total + 1, s));
-    unsigned long long ME = 0;
-    CUDA_TRY(cudaMemcpyAsync(&ME, total + 1, sizeof(ME), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    if (ME > (unsigned long long)MAX_COUNT) return fail(SJ_ERR_INVALID, "more than 2^31 - 2^22 (polygon, row, edge) entries");
-    L->ME = (int64_t)ME;
-    CUDA_TRY(dalloc(&L->prow_start, (size_t)MR + 1));
-    CUDA_TRY(dalloc(&L->pedge_ids, (size_t)ME));
-    cudaFree(a.block_sums);
-    tmp.p[2] = nullptr;
+    PipBuildArgs b{};
+    b.g = L->g;
+    b.V = V;
+    b.M = M;
+    b.verts = L->verts;
+    b.nxt = L->nxt;
+    b.prv = prv;
+    b.owner = owner;
+    b.obj_voff = L->obj_voff;
+    b.cand_start = L->cand_start;
+    b.cand_ids = L->cand_ids;
+    b.prow_base = L->prow_base;
+    b.prow_r0 = L->prow_r0;
+    b.frame_x = L->frames;
+    b.frame_y = L->frames + L->g.nx;
+    CUDA_TRY(tmp.take(&b.e.rows, (size_t)V));
+    CUDA_TRY(tmp.take(&b.e.xr, (size_t)V));
+    CUDA_TRY(tmp.take(&b.e.kind, (size_t)V));
+    CUDA_TRY(launch_pip_edges(b, s));
+    sj_status st = read_totals(total, h, 1, s);
+    if (st != SJ_OK) return st;
+    if (h[0] > (unsigned long long)MAX_COUNT) return fail(SJ_ERR_INVALID, "more than 2^31 - 2^22 (polygon, row) slots");
+    L->MR = (int64_t)h[0];
+    int *cnt = nullptr, *cursor = nullptr;
+    int2 *bs = nullptr;
+    const size_t slots_cap = bucket_scan_blocks((int)L->MR);
+    CUDA_TRY(tmp.take(&cnt, (size_t)L->MR));
+    CUDA_TRY(tmp.take(&cursor, (size_t)L->MR));
+    CUDA_TRY(tmp.take(&bs, slots_cap));
+    CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)L->MR, s));
+    CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * (size_t)L->MR, s));
+    CUDA_TRY(launch_prow_edges(b, cnt, total + 1, nullptr, nullptr, s));
+    // pairs of equal edges, while the list sizes travel
     {
-        const size_t nbs = bucket_scan_blocks((int)MR);
-        CUDA_TRY(dalloc(&a.block_sums, nbs)); tmp.p[2] = a.block_sums;
-        a.bs_cap = nbs;
+        size_t slots = 64;
+        while (slots < 2 * (size_t)V && slots < ((size_t)1 << 31)) slots <<= 1;
+        int *table = nullptr;
+        CUDA_TRY(tmp.take(&table, slots));
+        CUDA_TRY(tmp.take(&b.twin, (size_t)V));
+        CUDA_TRY(launch_pip_twins(b, table, (unsigned)slots, s));
     }
-    CUDA_TRY(launch_prow_edge_emit(a, L->nxt, L->prow_base, L->prow_r0, cnt, (int)MR, L->prow_start, cursor,
-                                   L->pedge_ids, s));
-    CUDA_TRY(dalloc(&L->pedge_rec, 2 * (size_t)ME));
-    if (ME > 0) CUDA_TRY(launch_prow_records(L->pedge_ids, (long long)ME, L->nxt, L->vsplit, L->pedge_rec, s));
-    // cell classes of the candidate entries; delta = 1e-7 of the largest grid
-    // coordinate (0.01 m at 1e5 m) is far above FP64 rounding and far below a cell
-    CUDA_TRY(dalloc(&L->cand_cls, (size_t)L->M));
+    st = read_totals(total + 1, h, 1, s);
+    if (st != SJ_OK) return st;
+    if (h[0] > (unsigned long long)MAX_COUNT) return fail(SJ_ERR_INVALID, "more than 2^31 - 2^22 (polygon, row, edge) entries");
+    L->ME = (int64_t)h[0];
+    CUDA_TRY(dalloc(&L->prow_start, (size_t)L->MR + 1));
+    CUDA_TRY(dalloc(&L->pedge_ids, (size_t)L->ME));
+    CUDA_TRY(launch_offsets(cnt, (int)L->MR, L->prow_start, bs, slots_cap, totals, s));
+    CUDA_TRY(launch_prow_edges(b, cursor, nullptr, L->prow_start, L->pedge_ids, s));
+    b.prow_start = L->prow_start;
+    b.pedge = L->pedge_ids;
+
+    // what each entry and cell holds; delta = 1e-7 of the largest grid coordinate
+    // (0.01 m at 1e5 m) is far above FP64 rounding and far below a cell
     const double delta = 1e-7 * L->xmax + 1e-300;
-    if (L->M > 0)
-        CUDA_TRY(launch_pip_classify(L->g, L->cand_start, L->cand_ids, L->prow_base, L->prow_r0, L->prow_start,
-                                     L->pedge_ids, L->nxt, L->verts, delta, L->cand_cls, s));
-    // per cell: the result of its points when every candidate is classified
-    CUDA_TRY(dalloc(&L->cell_res, (size_t)L->g.G));
-    CUDA_TRY(launch_cell_result(L->cand_start, L->cand_ids, L->cand_cls, L->g.G, L->cell_res, s));
+    int *at[3] = {};
+    CUDA_TRY(tmp.take(&b.col, (size_t)L->g.nx));
+    CUDA_TRY(tmp.take(&b.entry_cell, (size_t)M));
+    CUDA_TRY(tmp.take(&b.ord, (size_t)M));
+    CUDA_TRY(tmp.take(&b.edge_at, (size_t)M));
+    CUDA_TRY(tmp.take(&b.flip_at, (size_t)M));
+    CUDA_TRY(tmp.take(&b.ent, (size_t)M));
+    int **of[3] = {&b.units_of, &b.edges_of, &b.flips_of};
+    for (int q = 0; q < 3; ++q) {
+        CUDA_TRY(tmp.take(of[q], (size_t)G));
+        CUDA_TRY(tmp.take(&at[q], (size_t)G + 1));
+    }
+    b.cell_code = L->cell_code;
+    CUDA_TRY(launch_pip_count(b, delta, s));
+    int2 *bs2 = nullptr;
+    const size_t cells_cap = bucket_scan_blocks(G);
+    CUDA_TRY(tmp.take(&bs2, cells_cap));
+    CUDA_TRY(cudaMemsetAsync(total, 0, 3 * sizeof(unsigned long long), s));
+    for (int q = 0; q < 3; ++q) {
+        CUDA_TRY(launch_sum64(*of[q], G, total + q, s));
+        CUDA_TRY(launch_offsets(*of[q], G, at[q], bs2, cells_cap, totals, s));
+    }
+    st = read_totals(total, h, 3, s);
+    if (st != SJ_OK) return st;
+    for (int q = 0; q < 3; ++q)
+        if (h[q] > (unsigned long long)MAX_COUNT) return fail(SJ_ERR_INVALID, "cell records exceed 2^31 - 2^22 entries");
+    L->units_n = (int64_t)h[0];
+    CUDA_TRY(dalloc(&L->units, 2 * ((size_t)h[0] + 2)));   // the join reads two units past a header
+    CUDA_TRY(cudaMemsetAsync(L->units + 2 * (size_t)h[0], 0, 4 * sizeof(int4), s));
+    CUDA_TRY(tmp.take(&b.tmp_edge, (size_t)h[1]));
+    CUDA_TRY(tmp.take(&b.tmp_rel, (size_t)h[1]));
+    CUDA_TRY(tmp.take(&b.tmp_flip, (size_t)h[2]));
+    CUDA_TRY(tmp.take(&b.long_list, (size_t)((h[1] + h[2]) / PIP_LONG_MIN) + 1));
+    CUDA_TRY(tmp.take(&b.long_n, 1));
+    CUDA_TRY(cudaMemsetAsync(b.long_n, 0, sizeof(int), s));
+    b.units_at = at[0];
+    b.edges_at = at[1];
+    b.flips_at = at[2];
+    b.units = L->units;
+    CUDA_TRY(launch_pip_records(b, s));
     CUDA_TRY(cudaStreamSynchronize(s));
-    return build_boundary_lists(L, delta, s);
+    return SJ_OK;
 }
 
 static sj_status layer_common_checks(const double *verts, int64_t V, const sj_grid *g, void *stream,
@@ -669,21 +657,16 @@ extern "C" sj_status sj_pip_layer_create(const double *verts, int64_t V, const i
     if (bad) return fail(SJ_ERR_INVALID, "invalid polygon layer (offsets, ring sizes or non-finite vertex)");
     CUDA_TRY(dalloc(&L->obj_voff, (size_t)P + 1));
     CUDA_TRY(dalloc(&L->nxt, (size_t)V));
-    CUDA_TRY(dalloc(&L->prv, (size_t)V));
-    CUDA_TRY(dalloc(&L->vsplit, (size_t)V));
-    CUDA_TRY(launch_pip_topology(L->ring_off, (int)R, L->poly_ring_off, P, L->obj_voff, L->nxt, L->prv, s));
-    if (V > 0) CUDA_TRY(launch_split(L->verts, (int)V, L->vsplit, s));
-    {   // size of the largest polygon (picks how many items a warp takes at once)
-        std::vector<int> voff((size_t)P + 1);
-        CUDA_TRY(cudaMemcpyAsync(voff.data(), L->obj_voff, sizeof(int) * ((size_t)P + 1), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-        for (int32_t p = 0; p < P; ++p) L->max_obj_verts = std::max<int64_t>(L->max_obj_verts, voff[p + 1] - voff[p]);
-    }
+    BuildTmp tmp(s);
+    int *prv = nullptr, *owner = nullptr;
+    CUDA_TRY(tmp.take(&prv, (size_t)V));
+    CUDA_TRY(tmp.take(&owner, (size_t)V));
+    CUDA_TRY(launch_pip_topology(L->ring_off, (int)R, L->poly_ring_off, P, (int)V, L->obj_voff, L->nxt, prv, owner, s));
     CUDA_TRY(dalloc(&L->stats, ST_N));
     CUDA_TRY(cudaMemsetAsync(L->stats, 0, sizeof(unsigned long long) * ST_N, s));
     st = build_candidates(L, dbad, s);
     if (st != SJ_OK) return st;
-    st = build_row_lists(L, s);
+    st = build_pip_records(L, prv, owner, s);
     if (st != SJ_OK) return st;
     *out = L;
     guard.L = nullptr;
@@ -812,17 +795,17 @@ extern "C" sj_status sj_layer_reset_stats(sj_layer *L) {
 // ------------------------------------------------------------------ joins
 
 struct JoinBufs {
-    int *cnt, *cell_start, *perm, *totals, *pos, *res_id, *cell_base, *sub_start;
+    int *cnt, *cell_start, *perm, *totals, *pos, *cell_base, *sub_start;
     int2 *key_rank, *items, *block_sums, *fb;
     double2 *spts;
     ResF *resf;
     ResD *resd;
 };
 
-// Result layout of a join: through perm into the outputs (RES_PERM), or
-// cell-ordered and gathered back through pos: ids only (RES_IDS, PIP) or packed
-// P2P records (RES_F for FP32X, RES_D for FP64).
-enum { RES_PERM = 0, RES_IDS, RES_F, RES_D };
+// Result layout of a P2P join: through perm into the outputs (RES_PERM), or
+// cell-ordered packed records gathered back through pos (RES_F for FP32X,
+// RES_D for FP64).
+enum { RES_PERM = 0, RES_F, RES_D };
 
 // with_spts: also a cell-ordered copy of the points (else the refinement reads
 // the input points through perm).
@@ -844,7 +827,6 @@ static void carve(Scratch &s, JoinBufs &b, int64_t N, int G, int ch, bool need_f
     const bool sorted_res = res != RES_PERM;
     b.pos = sorted_res ? s.take<int>((size_t)N) : nullptr;
     b.cell_base = sorted_res ? s.take<int>((size_t)G) : nullptr;
-    b.res_id = res == RES_IDS ? s.take<int>((size_t)N) : nullptr;
     b.resf = res == RES_F ? s.take<ResF>((size_t)N) : nullptr;
     b.resd = res == RES_D ? s.take<ResD>((size_t)N) : nullptr;
 }
@@ -872,11 +854,7 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     if (nw != 2 && nw != 4 && nw != 8) return fail(SJ_ERR_INVALID, "block must be 0, 2, 4 or 8 (warps per block)");
     int budget = o ? o->edges_per_chunk : 0;
     if (budget < 0) return fail(SJ_ERR_INVALID, "edges_per_chunk must be >= 0");
-    // default: polygon layers split heavy cells at 64 edges per point (the
-    // autotuner's best on both tilings at 100 M points: heavy-tail layer
-    // 8.1 -> 6.5 ms, 40,000 tiles 5.2 -> 4.8 ms); polyline layers do not (no
-    // setting was faster on the walks)
-    if (budget == 0 && kind == KIND_PIP) budget = 64;
+    // default: no split (no setting was faster on the walks)
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     if (dev != L->device) return fail(SJ_ERR_INVALID, "layer belongs to another device");
@@ -887,32 +865,43 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     L->points += N;
     if (N == 0) return SJ_OK;
     cudaStream_t s = (cudaStream_t)stream;
+    const bool timed = o && (o->flags & SJ_FLAG_TIME_REFINE);
+    const bool subcells = o && (o->flags & SJ_FLAG_SUBCELL_ON) && !(o->flags & SJ_FLAG_SUBCELL_OFF);
+    if (kind == KIND_PIP) {   // one kernel over the points in input order, no scratch (sj_pip.cu)
+        PipArgs pa = pip_args(L);
+        if (subcells) pa.search = PIP_SEARCH_MIN;
+        cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+        cudaError_t e = cudaSuccess;
+        if (timed) {
+            e = cudaEventCreate(&ev0);
+            if (e == cudaSuccess) e = cudaEventCreate(&ev1);
+            if (e == cudaSuccess) e = cudaEventRecord(ev0, s);
+        }
+        if (e == cudaSuccess) e = launch_pip_join(pa, (const double2 *)pts, (int)N, out_id, di->sms, s);
+        if (timed && ev1) {
+            if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
+            std::lock_guard<std::mutex> lk(L->ev_mu);
+            L->ev_pending.emplace_back(ev0, ev1);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "join launch");
+        return check_bounds(s);
+    }
     const int G = L->g.G;
-    const bool need_fb = (kind == KIND_P2P && form == SJ_FP32X);
+    const bool need_fb = form == SJ_FP32X;
     // Sub-cell order of the points inside their cells (see BucketArgs), on
     // request (SJ_FLAG_SUBCELL_ON): each work item of a dense cell then covers
-    // a compact part of it and the exact per-item prunes (the P2P box
-    // distance, the PIP y-range) drop more of the staged segments / edges --
-    // 40 % fewer P2P tests at 170 M points, 47 % fewer PIP tests on the
-    // heavy-tail tiling -- but the per-sub-cell start table (G x S entries,
-    // read at random by the scatter) costs more than that saves on the
-    // workloads measured, so arrival order is the default.  P2P: 4 x 4
-    // sub-cells in Z-order; PIP: 8 horizontal bands (its prune is in y).
-    int sub_lx = 0, sub_ly = 0;
-    {
-        const int fl = o ? o->flags : 0;
-        const bool on = (fl & SJ_FLAG_SUBCELL_ON) && !(fl & SJ_FLAG_SUBCELL_OFF);
-        if (on) {
-            if (kind == KIND_P2P) sub_lx = sub_ly = 2;
-            else sub_ly = 3;
-        }
-        if (((long long)G << (sub_lx + sub_ly)) > MAX_COUNT) sub_lx = sub_ly = 0;
-    }
+    // a compact part of it and the exact per-item prune (the box distance)
+    // drops more of the staged segments -- 40 % fewer tests at 170 M points --
+    // but the per-sub-cell start table (G x S entries, read at random by the
+    // scatter) costs more than that saves on the workloads measured, so
+    // arrival order is the default.  4 x 4 sub-cells in Z-order.
+    int sub_lx = subcells ? 2 : 0, sub_ly = sub_lx;
+    if (((long long)G << (sub_lx + sub_ly)) > MAX_COUNT) sub_lx = sub_ly = 0;
     const int lS = sub_lx + sub_ly;
 
     JoinBufs b;
-    const int res = kind == KIND_PIP ? RES_IDS : (form == SJ_FP32X ? RES_F : RES_D);
-    const bool split = budget > 0 && L->cell_work;   // items sized by the cells' edge work
+    const int res = form == SJ_FP32X ? RES_F : RES_D;
+    const bool split = budget > 0;   // items sized by the cells' edge work
     const int ch_min = split ? std::min(ch, 8) : ch;
     size_t bytes = measure([&](Scratch &sc) { carve(sc, b, N, G, ch, need_fb, false, res, lS, ch_min); });
     Scratch sc;
@@ -943,11 +932,6 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ba.sub_lx = sub_lx;
     ba.sub_ly = sub_ly;
     ba.sub_start = b.sub_start;
-    if (kind == KIND_PIP) {   // points of fully classified cells: results written by the cell-id pass
-        ba.cell_res = L->cell_res;
-        ba.out_id = out_id;
-        ba.stats = L->stats;
-    }
     if (e == cudaSuccess) e = launch_bucket(ba, s);
 
     RefineArgs ra{};
@@ -961,17 +945,13 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ra.items = b.items;
     ra.n_items = b.totals + 1;
     ra.work_next = b.totals + 3;   // zeroed with the totals at the start of the join
-    // Items a warp takes per counter update.  P2P on dense grids (two or more
+    // Items a warp takes per counter update.  On dense grids (two or more
     // items per cell on average): two consecutive items, mostly two chunks of
     // one cell, whose second reads the cell's records from L1 and halves the
     // counter traffic (170 M points, 512^2 grid, D = 50 m: refine 5.35 ->
     // 4.21 ms; D = 100 m unchanged); sparse grids keep one (the 10 M point
-    // join is 1 % slower with two).  PIP: two when every polygon is small
-    // (1 M points on the stars: refine 0.072 -> 0.067 ms); one when some
-    // polygon is large, whose boundary items would pair into stragglers
-    // (heavy-tail tiling: 5.3 -> 6.9 ms with two).
-    if (kind == KIND_P2P) ra.claim = (N >= 2LL * ch * (long long)G) ? 2 : 1;
-    else ra.claim = L->max_obj_verts <= 256 ? 2 : 1;
+    // join is 1 % slower with two).
+    ra.claim = (N >= 2LL * ch * (long long)G) ? 2 : 1;
     ra.cell_start = b.cell_start;
     ra.perm = b.perm;
     ra.spts = b.spts;
@@ -980,24 +960,19 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ra.npts = (int)N;
     ra.cell_work = ba.cell_work;
     ra.budget = ba.budget;
-    ra.res_id = b.res_id;   // cell-ordered results, every slot of a refined cell written
-    ra.resf = b.resf;
+    ra.resf = b.resf;       // cell-ordered results, every slot of a refined cell written
     ra.resd = b.resd;
     ra.out_id = out_id;     // FP32X recheck: final outputs through perm
     ra.out_d = out_d;
     ra.fb = b.fb;
     ra.n_fb = b.totals + 2;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    const bool timed = o && (o->flags & SJ_FLAG_TIME_REFINE);
     if (e == cudaSuccess && timed) {
         e = cudaEventCreate(&ev0);
         if (e == cudaSuccess) e = cudaEventCreate(&ev1);
         if (e == cudaSuccess) e = cudaEventRecord(ev0, s);
     }
-    if (e == cudaSuccess) {
-        if (kind == KIND_PIP) e = launch_pip_refine(ra, form, nw, di->sms * di->pip_bps[form], s);
-        else e = launch_p2p_refine(ra, form, nw, di->sms * di->p2p_bps[form], s);
-    }
+    if (e == cudaSuccess) e = launch_p2p_refine(ra, form, nw, di->sms * di->p2p_bps[form], s);
     if (timed && ev1) {   // the refinement launch alone
         if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
         std::lock_guard<std::mutex> lk(L->ev_mu);
@@ -1006,8 +981,7 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     // a8: results to input order; then the FP32X recheck overwrites the points
     // it redoes in FP64, through perm
     if (e == cudaSuccess) {
-        if (res == RES_IDS) e = launch_unsort(b.pos, b.res_id, nullptr, (int)N, out_id, nullptr, s);
-        else if (res == RES_F) e = launch_unsort_f(b.pos, b.resf, (int)N, out_id, out_d, s);
+        if (res == RES_F) e = launch_unsort_f(b.pos, b.resf, (int)N, out_id, out_d, s);
         else e = launch_unsort_d(b.pos, b.resd, (int)N, out_id, out_d, s);
     }
     if (e == cudaSuccess && need_fb) e = launch_p2p_recheck(ra, di->sms * 4, s);
@@ -1187,10 +1161,10 @@ extern "C" sj_status sj_pip_census(const sj_layer *L, const double *pts, int64_t
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long *d = nullptr, h[2] = {0, 0};
     CUDA_TRY(dev_malloc_async((void **)&d, sizeof(h), s));
-    RefineArgs ra{};
-    fill_refine(L, ra);
+    CensusArgs ca{L->g,          L->cand_start, L->cand_ids,  L->obj_voff, L->prow_base,
+                  L->prow_r0,    L->prow_start, L->pedge_ids, L->nxt,      L->verts};
     cudaError_t e = cudaMemsetAsync(d, 0, sizeof(h), s);
-    if (e == cudaSuccess) e = launch_pip_census(ra, (const double2 *)pts, (int)N, d, s);
+    if (e == cudaSuccess) e = launch_pip_census(ca, (const double2 *)pts, (int)N, d, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
     cudaError_t e2 = cudaFreeAsync(d, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

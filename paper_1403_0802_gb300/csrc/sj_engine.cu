@@ -22,26 +22,15 @@
 #include "sj_host.hpp"
 
 namespace sj {
-cudaError_t launch_pip_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
 cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
 cudaError_t launch_p2p_recheck(const RefineArgs &a, int blocks, cudaStream_t s);
 size_t bucket_scan_blocks(int G);
 
 namespace {
 
-// One request as the kernels see it.
-struct ReqDev {
-    const double2 *pts;
-    int *out_id;
-    double *out_d;
-    double window;   // P2P window of this request (the layer's D when none is asked)
-    int off;         // first global point index
-    int n;
-};
-
 struct MultiArgs {
     GridDev g;
-    const ReqDev *reqs;
+    const RoundReq *reqs;
     const int *meta;       // [0] number of requests, [1] total points, [2] per-request windows on
     int *cnt;
     int2 *key_rank;
@@ -55,7 +44,7 @@ struct MultiArgs {
 };
 
 // Request owning global point i: the last request whose offset is <= i.
-__device__ __forceinline__ int find_req(const ReqDev *r, int nr, int i) {
+__device__ __forceinline__ int find_req(const RoundReq *r, int nr, int i) {
     int lo = 0, hi = nr;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -67,7 +56,7 @@ __device__ __forceinline__ int find_req(const ReqDev *r, int nr, int i) {
 __global__ void k_cell_hist_multi(MultiArgs m) {
     const int nr = m.meta[0], total = m.meta[1];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const ReqDev &R = m.reqs[find_req(m.reqs, nr, i)];
+        const RoundReq &R = m.reqs[find_req(m.reqs, nr, i)];
         const double2 p = R.pts[i - R.off];
         const int c = point_cell(m.g, p.x, p.y);
         int r = 0;
@@ -86,7 +75,7 @@ __global__ void k_scatter_multi(MultiArgs m) {
         const int2 k = m.key_rank[i];
         int q = -1;
         if (k.x < m.g.G) {
-            const ReqDev &R = m.reqs[find_req(m.reqs, nr, i)];
+            const RoundReq &R = m.reqs[find_req(m.reqs, nr, i)];
             q = m.cell_start[k.x] + k.y;
             m.perm[q] = i;
             m.spts[q] = R.pts[i - R.off];
@@ -104,7 +93,7 @@ __global__ void k_unsort_multi(MultiArgs m) {
     const int nr = m.meta[0], total = m.meta[1];
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const ReqDev &R = m.reqs[find_req(m.reqs, nr, i)];
+        const RoundReq &R = m.reqs[find_req(m.reqs, nr, i)];
         const int q = m.pos[i];
         R.out_id[i - R.off] = q >= 0 ? m.res_id[q] : -1;
         if (R.out_d) R.out_d[i - R.off] = (q >= 0 && m.res_d) ? m.res_d[q] : INF;
@@ -115,14 +104,15 @@ __global__ void k_unsort_multi(MultiArgs m) {
 struct LayerWork {
     const sj_layer *L = nullptr;
     char *base = nullptr;
-    ReqDev *d_reqs = nullptr;
+    RoundReq *d_reqs = nullptr;
     int *d_meta = nullptr;
     BucketArgs ba{};
     RefineArgs ra{};
     MultiArgs ma{};
+    PipArgs pa{};
     // pinned request tables (two, so the host can fill one while the other's
     // copy may still be pending) and the events that mark their copies done
-    ReqDev *h_reqs[2] = {nullptr, nullptr};
+    RoundReq *h_reqs[2] = {nullptr, nullptr};
     int *h_meta[2] = {nullptr, nullptr};
     cudaEvent_t copied[2] = {nullptr, nullptr};
     int slot = 0;
@@ -168,11 +158,14 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     const int64_t N = E->max_points;
     const int G = L->g.G;
     const bool p2p = L->kind == KIND_P2P;
-    int *cnt, *cell_start, *totals, *pos, *perm, *res_id;
-    int2 *key_rank, *items, *block_sums, *fb;
-    double2 *spts;
-    double *res_d, *win;
+    int *cnt = nullptr, *cell_start = nullptr, *totals = nullptr, *pos = nullptr, *perm = nullptr, *res_id = nullptr;
+    int2 *key_rank = nullptr, *items = nullptr, *block_sums = nullptr, *fb = nullptr;
+    double2 *spts = nullptr;
+    double *res_d = nullptr, *win = nullptr;
     auto lay = [&](Scratch &x) {
+        w->d_reqs = x.take<RoundReq>((size_t)E->max_requests);
+        w->d_meta = x.take<int>(4);
+        if (!p2p) return;   // the PIP join needs no scratch
         cnt = x.take<int>((size_t)G + 1);
         cell_start = x.take<int>((size_t)G + 1);
         totals = x.take<int>(4);
@@ -183,11 +176,9 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
         items = x.take<int2>((size_t)(N / E->ch) + (size_t)std::min<int64_t>(G, N) + 1);
         block_sums = x.take<int2>(bucket_scan_blocks(G));
         res_id = x.take<int>((size_t)N);
-        res_d = p2p ? x.take<double>((size_t)N) : nullptr;
-        win = p2p ? x.take<double>((size_t)N) : nullptr;
-        fb = (p2p && E->form == SJ_FP32X) ? x.take<int2>((size_t)N) : nullptr;
-        w->d_reqs = x.take<ReqDev>((size_t)E->max_requests);
-        w->d_meta = x.take<int>(4);
+        res_d = x.take<double>((size_t)N);
+        win = x.take<double>((size_t)N);
+        fb = E->form == SJ_FP32X ? x.take<int2>((size_t)N) : nullptr;
     };
     size_t bytes = measure(lay);
     CUDA_TRY(dev_malloc((void **)&w->base, bytes));
@@ -195,11 +186,17 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     sc.base = w->base;
     lay(sc);
     for (int k = 0; k < 2; ++k) {
-        CUDA_TRY(cudaMallocHost((void **)&w->h_reqs[k], sizeof(ReqDev) * (size_t)E->max_requests));
+        CUDA_TRY(cudaMallocHost((void **)&w->h_reqs[k], sizeof(RoundReq) * (size_t)E->max_requests));
         CUDA_TRY(cudaMallocHost((void **)&w->h_meta[k], sizeof(int) * 4));
         CUDA_TRY(cudaEventCreateWithFlags(&w->copied[k], cudaEventDisableTiming));
     }
 
+    if (!p2p) {
+        w->pa = pip_args(L);
+        guard.w = nullptr;
+        *out = w;
+        return SJ_OK;
+    }
     BucketArgs &ba = w->ba;
     ba.g = L->g;
     ba.cnt = cnt;
@@ -226,7 +223,7 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     ra.fb = fb;
     ra.n_fb = totals + 2;
     ra.win = win;
-    ra.win_on = p2p ? w->d_meta + 2 : nullptr;
+    ra.win_on = w->d_meta + 2;
 
     MultiArgs &ma = w->ma;
     ma.g = L->g;
@@ -250,18 +247,15 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
 static cudaError_t enqueue_round(const sj_engine *E, const LayerWork *w, const DevInfo *di, cudaStream_t s) {
     const sj_layer *L = w->L;
     const int blocks = di->sms * 8;
+    if (L->kind == KIND_PIP) return launch_pip_round(w->pa, w->d_reqs, w->d_meta, E->max_points, di->sms, s);
     cudaError_t e = cudaMemsetAsync(w->ba.cnt, 0, sizeof(int) * ((size_t)L->g.G + 1), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w->ba.totals, 0, sizeof(int) * 4, s);
     if (e != cudaSuccess) return e;
     k_cell_hist_multi<<<blocks, 256, 0, s>>>(w->ma);
     if ((e = launch_bucket_scan(w->ba, s)) != cudaSuccess) return e;
     k_scatter_multi<<<blocks, 256, 0, s>>>(w->ma);
-    if (L->kind == KIND_PIP) {
-        e = launch_pip_refine(w->ra, E->form, 4, di->sms * di->pip_bps[E->form], s);
-    } else {
-        e = launch_p2p_refine(w->ra, E->form, 4, di->sms * di->p2p_bps[E->form], s);
-        if (e == cudaSuccess && E->form == SJ_FP32X) e = launch_p2p_recheck(w->ra, di->sms * 4, s);
-    }
+    e = launch_p2p_refine(w->ra, E->form, 4, di->sms * di->p2p_bps[E->form], s);
+    if (e == cudaSuccess && E->form == SJ_FP32X) e = launch_p2p_recheck(w->ra, di->sms * 4, s);
     if (e != cudaSuccess) return e;
     k_unsort_multi<<<blocks, 256, 0, s>>>(w->ma);
     return cudaGetLastError();
@@ -349,7 +343,7 @@ extern "C" sj_status sj_engine_round(sj_engine *E, const sj_request *reqs, int32
         for (int k = 0; k < n; ++k) {
             const sj_request &r = reqs[k];
             if (r.layer != L || r.N == 0) continue;
-            ReqDev d;
+            RoundReq d;
             d.pts = (const double2 *)r.pts;
             d.out_id = r.out_id;
             d.out_d = L->kind == KIND_P2P ? r.out_d : nullptr;
@@ -366,7 +360,7 @@ extern "C" sj_status sj_engine_round(sj_engine *E, const sj_request *reqs, int32
         w->h_meta[sl][0] = nr;
         w->h_meta[sl][1] = off;
         w->h_meta[sl][2] = windows;
-        CUDA_TRY(cudaMemcpyAsync(w->d_reqs, w->h_reqs[sl], sizeof(ReqDev) * (size_t)nr, cudaMemcpyHostToDevice, s));
+        CUDA_TRY(cudaMemcpyAsync(w->d_reqs, w->h_reqs[sl], sizeof(RoundReq) * (size_t)nr, cudaMemcpyHostToDevice, s));
         CUDA_TRY(cudaMemcpyAsync(w->d_meta, w->h_meta[sl], sizeof(int) * 4, cudaMemcpyHostToDevice, s));
         CUDA_TRY(cudaEventRecord(w->copied[sl], s));
         if (E->use_graph && s != nullptr) {

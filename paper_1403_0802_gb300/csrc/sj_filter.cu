@@ -205,9 +205,8 @@ cudaError_t launch_thresholds(const GridDev &g, unsigned long long *kx, unsigned
 // ------------------------------------------------------------------ point bucketing
 
 // a1: cell id per point and per-cell count; the atomic's return value is the
-// point's rank inside its cell, so the scatter needs no second pass.  Points
-// whose result is known here (PIP whole-cell results, or the one-pass result
-// form's initial -1 / +inf) get their outputs written here.
+// point's rank inside its cell, so the scatter needs no second pass.  With
+// out_id / out_d set, the results' initial -1 / +inf are written here.
 // Each thread handles UNR points per step so that several independent
 // load -> atomic -> store chains are in flight at once: UNR / 2 pairs of
 // consecutive points (2q, 2q + 1), q = q0, q0 + T, ... (T = total threads),
@@ -240,7 +239,6 @@ __global__ void k_cell_hist(BucketArgs a) {
     const unsigned T = gridDim.x * blockDim.x;
     const int lS = a.sub_lx + a.sub_ly;
     const int sentinel = a.g.G << lS;
-    unsigned resolved = 0, rhits = 0;
     // A thread takes the pairs of points (2q, 2q + 1), q = q0, q0 + T, ...: the
     // keys of a pair leave in one 16-byte store.
     const unsigned pairs = ((unsigned)a.n + 1u) / 2u;
@@ -252,24 +250,15 @@ __global__ void k_cell_hist(BucketArgs a) {
             const unsigned i = elem(u);
             if (i < (unsigned)a.n) p[u] = a.pts[i];
         }
-        // key (sentinel outside the grid), rank in its counter; a point of a
-        // cell whose result is known (cell_res) gets key sentinel, rank 1
-        int c[UNR], r[UNR], v[UNR];
+        // key (sentinel outside the grid), rank in its counter
+        int c[UNR], r[UNR];
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
             const unsigned i = elem(u);
             c[u] = sentinel;
             r[u] = 0;
-            v[u] = CELL_REFINE;
             if (i < (unsigned)a.n) {
                 c[u] = bucket_key(a, p[u].x, p[u].y);
-                if (a.cell_res && c[u] < sentinel) {
-                    v[u] = a.cell_res[c[u] >> lS];
-                    if (v[u] != CELL_REFINE) {
-                        c[u] = sentinel;
-                        r[u] = 1;
-                    }
-                }
                 if (c[u] < sentinel && SJ_IN_BOUNDS(c[u] >= 0, BND_BUCKET)) r[u] = atomicAdd(&a.cnt[c[u]], 1);
             }
         }
@@ -285,24 +274,10 @@ __global__ void k_cell_hist(BucketArgs a) {
         for (int u = 0; u < UNR; ++u) {
             const unsigned i = elem(u);
             if (i < (unsigned)a.n) {
-                if (a.cell_res) {
-                    if (v[u] != CELL_REFINE) {
-                        a.out_id[i] = v[u];
-                        ++resolved;
-                        rhits += v[u] >= 0;
-                    }
-                } else {
-                    if (a.out_id) a.out_id[i] = -1;
-                    if (a.out_d) a.out_d[i] = inf;
-                }
+                if (a.out_id) a.out_id[i] = -1;
+                if (a.out_d) a.out_d[i] = inf;
             }
         }
-    }
-    if (a.stats) {
-        unsigned long long v[ST_N] = {};
-        v[ST_RESOLVED] = __reduce_add_sync(FULL, resolved);
-        v[ST_HITS] = __reduce_add_sync(FULL, rhits);
-        flush_stats(a.stats, v);
     }
 }
 
@@ -399,7 +374,7 @@ __global__ void k_scatter(BucketArgs a) {
         int pos[UNR];
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
-            pos[u] = (k[u].x >= sentinel && k[u].y == 1) ? POS_DONE : -1;   // result already written, or outside
+            pos[u] = -1;
             if (k[u].x < sentinel) {
                 const int b = base[k[u].x];
                 pos[u] = b >= 0 ? b + k[u].y : -1;
@@ -418,71 +393,6 @@ __global__ void k_scatter(BucketArgs a) {
                 const unsigned i = elem(u);
                 if (i + 1u < (unsigned)a.n) *reinterpret_cast<int2 *>(a.pos + i) = make_int2(pos[u], pos[u + 1]);
                 else if (i < (unsigned)a.n) a.pos[i] = pos[u];
-            }
-        }
-    }
-}
-
-// a8 for cell-ordered results (see launch_unsort).
-__global__ void k_unsort(const int *pos, const int *res_id, const double *res_d, int n, int *out_id,
-                         double *out_d) {
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    const unsigned T = gridDim.x * blockDim.x;
-    for (unsigned i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < (unsigned)n; i0 += UNR * T) {
-        int j[UNR], id[UNR];
-        double d[UNR];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) j[u] = (i0 + u * T < (unsigned)n) ? pos[i0 + u * T] : -1;
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (j[u] >= 0 && !SJ_IN_BOUNDS(j[u] < n, BND_UNSORT)) j[u] = -1;
-            id[u] = j[u] >= 0 ? res_id[j[u]] : -1;
-            if (out_d) d[u] = j[u] >= 0 ? res_d[j[u]] : inf;
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const unsigned i = i0 + u * T;
-            if (i < (unsigned)n && j[u] != POS_DONE) {
-                out_id[i] = id[u];
-                if (out_d) out_d[i] = d[u];
-            }
-        }
-    }
-}
-
-// Ids only, two consecutive points per thread and step (one 8-byte load of
-// their slots, one 8-byte store of their ids unless one of them was answered
-// by the cell-id pass); out_id 8-byte aligned.
-__global__ void k_unsort_ids2(const int *pos, const int *res_id, int n, int *out_id) {
-    const unsigned T = gridDim.x * blockDim.x;
-    const unsigned pairs = ((unsigned)n + 1u) / 2u;
-    for (unsigned p0 = blockIdx.x * blockDim.x + threadIdx.x; p0 < pairs; p0 += UNR * T) {
-        int2 j[UNR], id[UNR];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const unsigned p = p0 + u * T, i = 2u * p;
-            j[u] = make_int2(POS_DONE, POS_DONE);
-            if (p < pairs) {
-                if (i + 1u < (unsigned)n) j[u] = *reinterpret_cast<const int2 *>(pos + i);
-                else j[u].x = pos[i];
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (j[u].x >= 0 && !SJ_IN_BOUNDS(j[u].x < n, BND_UNSORT)) j[u].x = -1;
-            if (j[u].y >= 0 && !SJ_IN_BOUNDS(j[u].y < n, BND_UNSORT)) j[u].y = -1;
-            id[u].x = j[u].x >= 0 ? res_id[j[u].x] : -1;
-            id[u].y = j[u].y >= 0 ? res_id[j[u].y] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const unsigned p = p0 + u * T, i = 2u * p;
-            if (p >= pairs) continue;
-            if (i + 1u < (unsigned)n && j[u].x != POS_DONE && j[u].y != POS_DONE) {
-                *reinterpret_cast<int2 *>(out_id + i) = id[u];
-            } else {
-                if (j[u].x != POS_DONE) out_id[i] = id[u].x;
-                if (i + 1u < (unsigned)n && j[u].y != POS_DONE) out_id[i + 1] = id[u].y;
             }
         }
     }
@@ -597,18 +507,6 @@ cudaError_t launch_unsort_d(const int *pos, const ResD *res, int n, int *out_id,
     return launch_unsort_rec(pos, res, n, out_id, out_d, s);
 }
 
-cudaError_t launch_unsort(const int *pos, const int *res_id, const double *res_d, int n, int *out_id, double *out_d,
-                          cudaStream_t s) {
-    if (!res_d && !out_d && ((uintptr_t)out_id & 7) == 0) {
-        const int nb = stream_blocks(((n + 1) / 2 + UNR - 1) / UNR, 256, 152 * 16);
-        k_unsort_ids2<<<nb, 256, 0, s>>>(pos, res_id, n, out_id);
-        return cudaGetLastError();
-    }
-    const int nb = stream_blocks((n + UNR - 1) / UNR, 256, 152 * 16);
-    k_unsort<<<nb, 256, 0, s>>>(pos, res_id, res_d, n, out_id, out_d);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t s) {
     int nb = stream_blocks(a.n, 256, 152 * 32);
     if (a.sub_lx < 0 || a.sub_ly < 0 || a.sub_lx > 3 || a.sub_ly > 3 || ((a.sub_lx + a.sub_ly) && !a.sub_start) ||
@@ -650,14 +548,27 @@ __global__ void k_poly_voff(const int *ring_off, const int *poly_ring_off, int P
         poly_voff[p] = ring_off[poly_ring_off[p]];
 }
 
-// Next and previous vertex within the same ring (the closing edge wraps).
-__global__ void k_ring_next(const int *ring_off, int R, int *nxt, int *prv) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-        int b = ring_off[r], e = ring_off[r + 1];
-        for (int i = b; i < e; ++i) {
-            nxt[i] = (i + 1 < e) ? i + 1 : b;
-            prv[i] = (i > b) ? i - 1 : e - 1;
-        }
+// Last k in [0, n) with off[k] <= i.
+__device__ __forceinline__ int run_of(const int *off, int n, int i) {
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (off[mid] <= i) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// Next and previous vertex within the same ring (the closing edge wraps) and
+// the polygon of each vertex: one thread per vertex, which finds its ring and
+// polygon by binary search (a thread per ring walked rings of up to 100,000
+// vertices alone: 1.05 ms on the heavy-tail tiling).
+__global__ void k_ring_next(const int *ring_off, int R, const int *poly_voff, int P, int V, int *nxt, int *prv,
+                            int *owner) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        const int r = run_of(ring_off, R, i), b = ring_off[r], e = ring_off[r + 1];
+        nxt[i] = (i + 1 < e) ? i + 1 : b;
+        prv[i] = (i > b) ? i - 1 : e - 1;
+        owner[i] = run_of(poly_voff, P, i);
     }
 }
 
@@ -952,36 +863,6 @@ __global__ void k_prow_count(LayerBuildArgs a, int *prow_n, int *prow_r0, unsign
     }
 }
 
-// One warp per polygon, lanes over its edges (vertex i -> nxt[i]).  Count pass
-// (ids == nullptr): cnt[slot] += 1 for every row of the edge, total in *total.
-// Emit pass: ids[start[slot] + cursor[slot]++] = i.
-__global__ void k_prow_edges(LayerBuildArgs a, const int *nxt, const int *prow_base, const int *prow_r0, int *cnt,
-                             unsigned long long *total, const int *start, int *cursor, int *ids) {
-    const int lane = lane_id();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int P = warp; P < a.nobj; P += nwarps) {
-        const int b = a.obj_voff[P], e = a.obj_voff[P + 1];
-        const int base = prow_base[P] - prow_r0[P];
-        unsigned long long n = 0;
-        for (int i = b + lane; i < e; i += 32) {
-            const double ya = a.verts[i].y, yb = a.verts[nxt[i]].y;
-            const int ra = clamped_axis(fmin(ya, yb), a.g.y0, a.g.ch, a.g.ny);
-            const int rb = clamped_axis(fmax(ya, yb), a.g.y0, a.g.ch, a.g.ny);
-            for (int r = ra; r <= rb; ++r) {
-                if (ids) ids[start[base + r] + atomicAdd(&cursor[base + r], 1)] = i;
-                else atomicAdd(&cnt[base + r], 1);
-            }
-            n += (unsigned long long)(rb - ra + 1);
-        }
-        if (!ids) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(FULL, n, o);
-            if (lane == 0) atomicAdd(total, n);
-        }
-    }
-}
-
 // Host side of the layer build steps that the API file sequences.
 cudaError_t launch_check_offsets(const int64_t *off, int64_t n, int64_t min_size, int64_t first, int64_t last, int *out,
                                  int *bad, cudaStream_t s) {
@@ -992,10 +873,10 @@ cudaError_t launch_check_finite(const double2 *v, int n, int *bad, cudaStream_t 
     k_check_finite<<<stream_blocks(n, 256, 4096), 256, 0, s>>>(v, n, bad);
     return cudaGetLastError();
 }
-cudaError_t launch_pip_topology(const int *ring_off, int R, const int *poly_ring_off, int P, int *poly_voff, int *nxt,
-                                int *prv, cudaStream_t s) {
+cudaError_t launch_pip_topology(const int *ring_off, int R, const int *poly_ring_off, int P, int V, int *poly_voff,
+                                int *nxt, int *prv, int *owner, cudaStream_t s) {
     k_poly_voff<<<stream_blocks(P + 1, 256, 4096), 256, 0, s>>>(ring_off, poly_ring_off, P, poly_voff);
-    k_ring_next<<<stream_blocks(R, 128, 4096), 128, 0, s>>>(ring_off, R, nxt, prv);
+    k_ring_next<<<stream_blocks(V, 256, 8192), 256, 0, s>>>(ring_off, R, poly_voff, P, V, nxt, prv, owner);
     return cudaGetLastError();
 }
 cudaError_t launch_split(const double2 *v, int n, float4 *vs, cudaStream_t s) {
@@ -1063,49 +944,11 @@ cudaError_t launch_prow_count(const LayerBuildArgs &a, int *prow_base, int *prow
     return run_scan(IntLoad{prow_base}, OffsetApply{prow_base}, a.nobj, a.block_sums, a.bs_cap, a.totals, s);
 }
 
-// Step 2 (count): edges per slot into cnt (zeroed), total entries in *total.
-cudaError_t launch_prow_edge_count(const LayerBuildArgs &a, const int *nxt, const int *prow_base, const int *prow_r0,
-                                   int *cnt, unsigned long long *total, cudaStream_t s) {
-    k_prow_edges<<<stream_blocks((long long)a.nobj * 32, 256, 4096), 256, 0, s>>>(a, nxt, prow_base, prow_r0, cnt,
-                                                                                 total, nullptr, nullptr, nullptr);
-    return cudaGetLastError();
-}
-
-// Step 3 (emit): slot ranges prow_start[slots + 1] from cnt, then the lists
-// (cursor zeroed).  Order within a list is not fixed (parity is a XOR).
-cudaError_t launch_prow_edge_emit(const LayerBuildArgs &a, const int *nxt, const int *prow_base, const int *prow_r0,
-                                  const int *cnt, int slots, int *prow_start, int *cursor, int *pedge_ids,
-                                  cudaStream_t s) {
-    cudaError_t e = run_scan(IntLoad{cnt}, OffsetApply{prow_start}, slots, a.block_sums, a.bs_cap, a.totals, s);
-    if (e != cudaSuccess) return e;
-    k_prow_edges<<<stream_blocks((long long)a.nobj * 32, 256, 4096), 256, 0, s>>>(a, nxt, prow_base, prow_r0, nullptr,
-                                                                                 nullptr, prow_start, cursor,
-                                                                                 pedge_ids);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_cseg_records(const int *cseg_start, const int *cseg_ids, const GridDev &g, const float *frame_x,
                                 const float *frame_y, const float4 *vsplit, const float4 *seg32, float4 *rec,
                                 cudaStream_t s) {
     k_cseg_records<<<stream_blocks(g.G, 128, 8192), 128, 0, s>>>(cseg_start, cseg_ids, g.G, g.nx, frame_x, frame_y,
                                                                 vsplit, seg32, rec);
-    return cudaGetLastError();
-}
-
-// FP32X staging records of the PIP row lists: the (hi, lo) splits of both ends
-// of each listed edge, so that staging reads one contiguous record per entry.
-__global__ void k_prow_records(const int *pedge_ids, long long ME, const int *nxt, const float4 *vsplit, float4 *rec) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ME;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int i = pedge_ids[e];
-        rec[2 * e] = vsplit[i];
-        rec[2 * e + 1] = vsplit[nxt[i]];
-    }
-}
-
-cudaError_t launch_prow_records(const int *pedge_ids, long long ME, const int *nxt, const float4 *vsplit,
-                                float4 *rec, cudaStream_t s) {
-    k_prow_records<<<stream_blocks(ME, 256, 8192), 256, 0, s>>>(pedge_ids, ME, nxt, vsplit, rec);
     return cudaGetLastError();
 }
 

@@ -30,7 +30,6 @@ struct sj_layer {
     float4 *vsplit = nullptr;
     int *obj_voff = nullptr;
     int *nxt = nullptr;
-    int *prv = nullptr;        // PIP: previous vertex of the same ring
     int *ring_off = nullptr;
     int *poly_ring_off = nullptr;
     double2 *seg_e64 = nullptr;
@@ -54,26 +53,15 @@ struct sj_layer {
     int *prow_r0 = nullptr;      // [nobj] first row of each polygon's MBB
     int *prow_start = nullptr;   // [MR + 1] list ranges in pedge_ids
     int *pedge_ids = nullptr;    // [ME] edge (= first vertex) indices
-    float4 *pedge_rec = nullptr; // [2 ME] FP32X staging records: vsplit of the edge's two ends
-    unsigned char *cand_cls = nullptr;   // [M] per candidate entry: 0 boundary, 1 inside, 2 outside
-    int *cell_res = nullptr;             // [G] result of every point of a fully classified cell, or CELL_REFINE
-    int *cell_work = nullptr;            // [G] per-point edge / segment work of each cell (item sizes)
-    // PIP boundary entries (class 0): near edges (x-range meets the cell's column
-    // widened by delta) and the flip keys of the far-right edges' parity in y
-    int64_t MN = 0, MF = 0;
-    int *bnear_start = nullptr;              // [M + 1]
-    int *bnear_ids = nullptr;                // [MN]
-    float4 *bnear_rec = nullptr;             // [2 MN] vsplit of both ends
-    float *bnear_key = nullptr;              // [MN] lower truncated y of each near edge, ascending per entry
-    float *bnear_h = nullptr;                // [M] largest truncated y-extent of an entry's near edges
-    int *bflip_start = nullptr;              // [M + 1]
-    int *bflip_len = nullptr;                // [M] keys left after cancelling equal pairs
-    unsigned long long *bflip_keys = nullptr;   // [MF] order keys, ascending within an entry
+    // PIP: per cell the result of its points or its record (sj_pip.cu)
+    int *cell_code = nullptr;    // [G]
+    int4 *units = nullptr;       // [2 units_n] the records, 32-byte units
+    int64_t units_n = 0;
+    int *cell_work = nullptr;    // P2P: [G] per-point segment work of each cell (item sizes)
     unsigned long long *stats = nullptr;
     unsigned long long *cell_keys = nullptr;   // [nx + 1 + ny + 1] threshold tables of point_cell
     float *frames = nullptr;                   // [nx + ny] FP32 cell frame origins
     double xmax = 0.0;                         // largest |coordinate| of the grid box
-    int64_t max_obj_verts = 0;                 // vertices of the largest polygon / polyline
     float Df = 0.0f, Ddn = 0.0f, Dup = 0.0f;   // FP32 forms of D (nearest, rounded down, rounded up)
     mutable std::atomic<long long> joins{0};
     mutable std::atomic<long long> points{0};
@@ -92,7 +80,6 @@ namespace sj {
 // Per-device launch facts, filled on first use.
 struct DevInfo {
     int sms = 0;
-    int pip_bps[2] = {0, 0};
     int p2p_bps[2] = {0, 0};
     cudaStream_t hstream[3] = {nullptr, nullptr, nullptr};   // host joins: copy in, join, copy out
     bool init = false;
@@ -110,6 +97,7 @@ cudaError_t dev_malloc(void **p, size_t bytes);
 cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s);
 sj_status device_info(int dev, DevInfo **out);
 void fill_refine(const sj_layer *L, RefineArgs &ra);
+PipArgs pip_args(const sj_layer *L);
 
 inline bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 

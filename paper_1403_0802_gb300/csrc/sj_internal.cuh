@@ -28,6 +28,7 @@ struct GridDev {
     const unsigned long long *kx;   // [nx + 1] order keys of the x thresholds
     const unsigned long long *ky;   // [ny + 1]
     float x0f, y0f, icwf, ichf;     // FP32 estimates of x0, y0, 1 / cw, 1 / ch
+    float tolx, toly;               // bounds of the error of axis_estimate, in cells
 };
 
 // Cell of one coordinate: floor((v - lo) / w) as a double (may be out of range
@@ -106,16 +107,37 @@ __device__ __forceinline__ int axis_cell(double v, const unsigned long long *key
     return i;
 }
 
+// Cell index along one axis from FP32 alone: true when the estimate lies
+// farther than its error bound tol from every cell boundary and inside the
+// grid, so that i is certain.  The bound (make_grid) covers the truncation of v
+// to FP32, the rounding of lo and 1 / w, and the two operations; NaN, infinite
+// and far outside values are never certain.
+__device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i) {
+    const float t = __fmul_rn(__fsub_rn(approx_float(v), lof), iwf);
+    const float f = floorf(t), r = t - f;
+    i = (int)f;
+    return r > tol && r < 1.0f - tol && t > 0.0f && t < (float)n;
+}
+
+// Column and row of a point, (-1 in an axis) outside the half-open grid box or
+// with a NaN or infinite coordinate.
+__device__ __forceinline__ int2 point_cell_exact(const GridDev &g, double x, double y) {
+    const unsigned long long EXP = 0x7ff0000000000000ULL;
+    int2 r = make_int2(-1, -1);
+    if (((unsigned long long)__double_as_longlong(x) & EXP) != EXP &&
+        ((unsigned long long)__double_as_longlong(y) & EXP) != EXP) {
+        r.x = axis_cell(x, g.kx, g.nx, g.x0f, g.icwf);
+        r.y = axis_cell(y, g.ky, g.ny, g.y0f, g.ichf);
+    }
+    return r;
+}
+
 // Cell id of a point (Sec. III.A), G when it lies outside the half-open grid
 // box or has a NaN or infinite coordinate; (ix, iy) its column and row.
 __device__ __forceinline__ int point_cell_xy(const GridDev &g, double x, double y, int &ix, int &iy) {
-    const unsigned long long EXP = 0x7ff0000000000000ULL;
-    ix = iy = -1;
-    if (((unsigned long long)__double_as_longlong(x) & EXP) == EXP ||
-        ((unsigned long long)__double_as_longlong(y) & EXP) == EXP)
-        return g.G;
-    ix = axis_cell(x, g.kx, g.nx, g.x0f, g.icwf);
-    iy = axis_cell(y, g.ky, g.ny, g.y0f, g.ichf);
+    const int2 e = point_cell_exact(g, x, y);
+    ix = e.x;
+    iy = e.y;
     if (ix < 0 || iy < 0) return g.G;
     return iy * g.nx + ix;
 }
@@ -216,9 +238,6 @@ enum { KIND_PIP = 0, KIND_P2P = 1 };
 // Per-layer device counters (index into sj_run_stats order after `joins`).
 enum { ST_POINTS = 0, ST_ITEMS, ST_PAIRS, ST_TESTS, ST_FALLBACK, ST_HITS, ST_ALGO, ST_RESOLVED, ST_N };
 
-// cell_res value of a polygon-layer cell whose points need the refinement.
-constexpr int CELL_REFINE = -2;
-
 // Adds counters to the layer's statistics with one global atomic per counter
 // and block: every lane 0 of the block's warps passes its warp's values
 // (others pass zeros), the block sums them in shared memory first.  Every
@@ -247,7 +266,7 @@ struct alignas(16) ResD {  // FP64
     double d;
 };
 
-// Arguments of the refinement kernels.
+// Arguments of the P2P refinement kernels.
 struct RefineArgs {
     GridDev g;
     const int2 *items;       // (cell, first point of the chunk within the cell)
@@ -260,10 +279,8 @@ struct RefineArgs {
     const double2 *pts;      // input points (used when spts is null)
     const int *cand_start;   // [G + 1]
     const int *cand_ids;     // [M]
-    const int *obj_voff;     // [nobj + 1] first vertex of each polygon / polyline
-    const int *nxt;          // PIP: next vertex of the same ring
+    const int *obj_voff;     // [nobj + 1] first vertex of each polyline
     const double2 *verts;    // [V] FP64 vertices
-    const float4 *vsplit;    // [V] (fl32(x), fl32(y), fl32(x - fl32(x)), fl32(y - fl32(y)))
     const double2 *seg_e64;  // P2P: [V] b - a of the segment starting at vertex i
     const double *seg_inv64; // P2P: [V] 1 / |b - a|^2 (0 for a degenerate segment)
     const float4 *seg32;     // P2P: (fl32(ex), fl32(ey), fl32(1 / |e|^2), owner polyline id bits)
@@ -271,22 +288,7 @@ struct RefineArgs {
     const int *cseg_ids;     //      segment (= first vertex) indices, ascending per cell
     const int *cell_algo;    //      [G] segments of the cell's candidate polylines
     const float4 *cseg_rec;  //      [2 MS] staging records of the list entries (see sj_filter.cu)
-    const int *prow_base;    // PIP: [P + 1] first (polygon, row) slot of each polygon
-    const int *prow_r0;      //      [P] first grid row of each polygon's MBB
-    const int *prow_start;   //      [slots + 1] edge list range of each (polygon, row)
-    const int *pedge_ids;    //      edge (= first vertex) indices
-    const float4 *pedge_rec; //      [2 entries] vsplit of the entry's edge ends (FP32X staging)
-    const unsigned char *cand_cls;   // PIP: per candidate entry 0 = boundary (test its edges),
-                                     //      1 = cell inside the polygon, 2 = outside
-    const int *bnear_start;  // PIP boundary entries: near edge lists [M + 1]
-    const int *bnear_ids;
-    const float4 *bnear_rec; //      [2 per edge] vsplit of both ends
-    const float *bnear_key;  //      per near edge: min of its ends' FP32 truncated y (ascending per entry)
-    const float *bnear_h;    //      [M] largest (max - min) truncated y of an entry's edges, rounded up
-    const int *bflip_start;  //      far-right parity flips: [M + 1] starts,
-    const int *bflip_len;    //      [M] lengths,
-    const unsigned long long *bflip_keys;   // ascending order keys of the flip y-values
-    double D;                // P2P window
+    double D;                // window
     float Ddn, Dup;          // FP32 D rounded down / up with a 1e-12 relative margin
     float Df;                // D rounded to FP32 (staging prune)
     // per-point windows (batched rounds whose requests ask for windows below
@@ -305,10 +307,10 @@ struct RefineArgs {
     double *out_d;
     int *res_id;             // when set: results in sorted order for every slot
     double *res_d;           //   (hits and misses); out_id / perm unused
-    ResF *resf;              // P2P FP32X: packed sorted results (instead of res_id / res_d);
+    ResF *resf;              // FP32X: packed sorted results (instead of res_id / res_d);
                              //   the FP64 recheck then writes out_id / out_d through perm
-    ResD *resd;              // P2P FP64: packed sorted results
-    int2 *fb;                // P2P FP32X: points to redo in FP64 (sorted slot, cell)
+    ResD *resd;              // FP64: packed sorted results
+    int2 *fb;                // FP32X: points to redo in FP64 (sorted slot, cell)
     int *n_fb;
     unsigned long long *stats;
 };
@@ -322,33 +324,90 @@ __device__ __forceinline__ double2 slot_point(const RefineArgs &a, int j) {
 // equal; the order key alone would not).
 __device__ __forceinline__ unsigned long long y_key(double v) { return order_key(v == 0.0 ? 0.0 : v); }
 
-// PIP boundary-entry lists (layer build): count (emit = 0) or emit (emit = 1).
-struct BoundaryArgs {
-    GridDev g;
-    const int *cand_start, *cand_ids;
-    const unsigned char *cls;
-    const int *prow_base, *prow_r0, *prow_start, *pedge_ids, *nxt, *prv;
-    const double2 *verts;
-    double delta;
-    int *near_cnt, *flip_cnt;                 // count pass: [M]
-    const int *near_start, *flip_start;       // emit pass
-    int *near_ids;
-    unsigned long long *flip_keys;
+// One request of a batched round as the kernels see it.
+struct RoundReq {
+    const double2 *pts;
+    int *out_id;
+    double *out_d;
+    double window;   // P2P window of this request (the layer's D when none is asked)
+    int off;         // first global point index
+    int n;
 };
-cudaError_t launch_pip_boundary(const BoundaryArgs &a, int emit, cudaStream_t s);
-cudaError_t launch_pip_flips(const int *flip_start, int M, unsigned long long *keys, int *len, cudaStream_t s);
-cudaError_t launch_pip_near_sort(const int *near_start, int M, int *ids, const int *nxt, const float4 *vsplit,
-                                 float *keys, float *h, cudaStream_t s);
 
-// PIP cell classification (layer build): one class per candidate entry.
-cudaError_t launch_cell_work_pip(const int *cand_start, const unsigned char *cls, const int *near_start, int G,
-                                 int *work, cudaStream_t s);
+// Near-edge lists longer than PIP_SEARCH are searched by y instead of scanned
+// (with the sub-cell flag: longer than PIP_SEARCH_MIN).  A scan stops early, so
+// up to about 32 edges it costs what the two dependent binary searches do.
+constexpr int PIP_SEARCH = 32, PIP_SEARCH_MIN = 16;
+
+// Arguments of the PIP join (the records are described in sj_pip.cu).
+struct PipArgs {
+    GridDev g;
+    const int *cell_code;    // [G] result of a classified cell, else -2 - first unit of its record
+    const int4 *units;       // [2 per 32-byte unit]
+    int units_n;
+    const double2 *verts;
+    const int *nxt;          // next vertex of the same ring
+    const float *frame_x, *frame_y;
+    float eps;               // absolute term of the split-coordinate rounding bound
+    int search;              // lists longer than this are searched by y
+    unsigned long long *stats;
+};
+cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, int sms, cudaStream_t s);
+cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points, int sms,
+                             cudaStream_t s);
+
+// PIP layer build: per edge its rows (of the lower and the upper end), x-range
+// and kind (bit 0: the first end is the lower one; bit 1: horizontal).
+struct PipEdges {
+    int2 *rows;
+    float2 *xr;
+    unsigned char *kind;
+};
+struct alignas(16) PipFlipTmp {
+    unsigned long long key;
+    unsigned mask;
+    int pad;
+};
+struct PipBuildArgs {
+    GridDev g;
+    int V, M;
+    const double2 *verts;
+    const int *nxt, *prv, *owner, *obj_voff;
+    PipEdges e;
+    int *twin;                                  // [V] edge with the same end points in another place, or -1
+    const int *cand_start, *cand_ids;
+    const int *prow_base, *prow_r0, *prow_start, *pedge;
+    float2 *col;                                // [nx] column limits widened by delta
+    int *entry_cell, *ord, *edge_at, *flip_at;  // [M]
+    int2 *ent;                                  // [M] near edges, (flips << 2 | base parity << 1 | any)
+    int *cell_code;                             // [G]
+    int *units_of, *edges_of, *flips_of;        // [G]
+    const int *units_at, *edges_at, *flips_at;  // [G + 1] their exclusive sums
+    int4 *units;
+    int2 *tmp_edge;                             // (edge, mask) of every record's near edges
+    float4 *tmp_rel;                            // their cell-relative ends
+    PipFlipTmp *tmp_flip;
+    int4 *long_list;                            // groups ordered by a whole block
+    int *long_n;
+    const float *frame_x, *frame_y;
+};
+cudaError_t launch_pip_edges(const PipBuildArgs &b, cudaStream_t s);
+cudaError_t launch_pip_twins(const PipBuildArgs &b, int *table, unsigned slots, cudaStream_t s);
+cudaError_t launch_prow_edges(const PipBuildArgs &b, int *cnt, unsigned long long *total, const int *start, int *ids,
+                              cudaStream_t s);
+cudaError_t launch_pip_count(const PipBuildArgs &b, double delta, cudaStream_t s);
+cudaError_t launch_pip_records(const PipBuildArgs &b, cudaStream_t s);
+constexpr int PIP_LONG_MIN = 256;   // records of more elements may be listed in long_list
+
+// Arguments of the PIP work census.
+struct CensusArgs {
+    GridDev g;
+    const int *cand_start, *cand_ids, *obj_voff;
+    const int *prow_base, *prow_r0, *prow_start, *pedge_ids, *nxt;
+    const double2 *verts;
+};
+
 cudaError_t launch_cell_work_p2p(const int *cseg_start, int G, int *work, cudaStream_t s);
-cudaError_t launch_cell_result(const int *cand_start, const int *cand_ids, const unsigned char *cls, int G, int *res,
-                               cudaStream_t s);
-cudaError_t launch_pip_classify(const GridDev &g, const int *cand_start, const int *cand_ids, const int *prow_base,
-                                const int *prow_r0, const int *prow_start, const int *pedge_ids, const int *nxt,
-                                const double2 *verts, double delta, unsigned char *cls, cudaStream_t s);
 
 // The error words of the bounds-checked build, per translation unit, read
 // and cleared (0 in normal builds).
@@ -357,10 +416,9 @@ unsigned bounds_take_p2p();
 unsigned bounds_take_pip();
 
 // Host-side launchers (defined in the .cu files).
-cudaError_t launch_pip_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
 cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
 cudaError_t launch_p2p_recheck(const RefineArgs &a, int blocks, cudaStream_t s);
-cudaError_t launch_pip_census(const RefineArgs &a, const double2 *pts, int n, unsigned long long *out,
+cudaError_t launch_pip_census(const CensusArgs &a, const double2 *pts, int n, unsigned long long *out,
                               cudaStream_t s);
 
 struct BucketArgs {
@@ -394,14 +452,7 @@ struct BucketArgs {
     // result depends on it.
     int sub_lx, sub_ly;
     int *sub_start;
-    // PIP: per cell the result of every point of a cell whose candidates are
-    // all classified inside / outside, else CELL_REFINE (or null).  Such a
-    // point's result is written to out_id by the cell-id pass itself; it gets
-    // no slot (pos = POS_DONE) and no work item.
-    const int *cell_res;
-    unsigned long long *stats;   // ST_RESOLVED counts those points (or null)
 };
-constexpr int POS_DONE = -2;   // pos of a point whose result the cell-id pass wrote
 
 // Z-order index of sub-cell (sx, sy) with lx / ly bits per axis (at most 3).
 __device__ __forceinline__ int sub_index(int sx, int sy, int lx, int ly) {
@@ -416,9 +467,7 @@ __device__ __forceinline__ int sub_index(int sx, int sy, int lx, int ly) {
 size_t bucket_scan_blocks(int G);
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t s);
 // a8 for cell-ordered results: out[i] = res[pos[i]], or -1 / +inf where
-// pos[i] < 0 (one pass; out_d and res_d may be null).
-cudaError_t launch_unsort(const int *pos, const int *res_id, const double *res_d, int n, int *out_id, double *out_d,
-                          cudaStream_t s);
+// pos[i] < 0 (one pass; out_d may be null).
 cudaError_t launch_unsort_f(const int *pos, const ResF *res, int n, int *out_id, double *out_d, cudaStream_t s);
 cudaError_t launch_unsort_d(const int *pos, const ResD *res, int n, int *out_id, double *out_d, cudaStream_t s);
 

@@ -1,84 +1,54 @@
-// sj_pip.cu -- PIP refinement (Sec. III.C, Fig. 3): ray-crossing parity of
-// each point of a work item against every ring of each candidate polygon of
-// its cell; the result is the smallest candidate id with odd parity.
+// sj_pip.cu -- PIP join (Sec. III.C, Fig. 3): ray-crossing parity of each point
+// against every ring of each candidate polygon of its cell; the result is the
+// smallest candidate id with odd parity.
 //
-// Work decomposition (GB300 design, not the paper's block-per-cell mapping):
-// one warp per (cell, point-chunk) item.
-//   1. The item's points are loaded; the range [ymin, ymax] of their FP32
-//      y roundings is reduced across the warp.
-//   2. Candidate polygons are taken 32 at a time (one per lane, in id order):
-//      each lane reads its polygon's edge list for the item's grid row (the
-//      edges whose y-range spans that row, built with the layer; no other edge
-//      can cross the ray of a point in the row), list lengths warp-scanned.
-//   3. Staging: the concatenated edges of the group are read 32 at a time; an
-//      edge whose y-range lies strictly below ymin or strictly above ymax
-//      cannot straddle the horizontal line of any point of the item and is
-//      dropped (exact: its crossing count is 0 for every point; the test uses
-//      FP32 roundings that are monotone, with strict inequalities); so is an
-//      edge lying wholly left of every point of the item by a safe margin (a
-//      ray towards +x cannot cross it); the rest is compacted into shared
-//      memory with the lane's candidate index k.
-//   4. Whenever the staging area fills, the lanes split into point groups of
-//      SG lanes; each lane keeps a 32-bit parity mask (bit k = candidate k)
-//      over its strided share of the staged edges; the SG lanes XOR-fold their
-//      masks with shuffles, and the fold is XORed into the point's mask.
-//   After a group, a point's result is the lowest set bit of its mask (ids are
-//   sorted, so the smallest id); points with a result skip later groups.
+// The paper refines (cell, points) pairs against whole candidate polygons; here
+// all that a point of a cell needs is laid out once with the layer, in one
+// contiguous record per grid cell, so the join is one kernel over the points in
+// input order: no bucketing, no scratch, one coalesced read of the points and
+// one coalesced write of the ids.
 //
-// Two arithmetic forms:
-//   FP64   -- the crossing rule in FP64, each operation rounded, no FMA.
-//   FP32X  -- no FP64 instruction in the common path: the straddle test on the
-//             FP32 truncations of y (monotone, so a strict FP32 inequality
-//             implies the FP64 one; equal values fall back), the orientation on
-//             cell-relative FP32 coordinates (from the (hi, lo) split of the
-//             inputs) with a forward error bound (Shewchuk's orient2d bound plus
-//             the input-rounding terms); a test whose |d| does not exceed the
-//             bound is redone in FP64 from the original vertices, so the result
-//             is the FP64 rule's, bit for bit.
+// Per cell (cell_code):
+//   >= -1   the result of every point of the cell (no candidate's edge comes
+//           near the cell, so each candidate holds all of it or none of it);
+//   <= -2   -2 - (first 32-byte unit of the cell's record).
+// A record is a chain of groups of up to 32 relevant candidates in id order (a
+// candidate that holds none of the cell is left out, and so is every candidate
+// after one that holds all of it): a header, the near edges, the flips.  For a
+// candidate of the cell (column [X0, X1), row r) the edges whose y-range
+// reaches row r -- no other edge can straddle a point of the row -- split
+// three ways by their x-range against the column widened by delta:
+//   left:  farther than delta left of every point, so the FP64 rule never
+//          counts a crossing -- dropped;
+//   far:   farther than delta right of every point, so the FP64 rule counts a
+//          crossing exactly when the edge straddles the point's y.  Their
+//          parity is the parity of the number of their end y-values at or
+//          below y: ends below the row give the group's base mask, ends inside
+//          the row are "flips" (sorted by y, each with the mask that holds
+//          from it on; an end shared by two far edges of the ring cancels);
+//   near:  the rest, tested point by point.  Horizontal edges never straddle
+//          and are left out.  An edge shared by two candidates (the common
+//          side of two tiles: equal end points) is kept once, with the bits of
+//          both, since the rule depends on the two end points only.
+// Near edges are ordered by their lower y: a scan stops at the first edge above
+// the point, and long lists are searched.
+//
+// Arithmetic: the straddle test and the orientation are evaluated in FP32 on
+// cell-relative coordinates (from the (hi, lo) split of the FP64 inputs) with
+// forward error bounds (Shewchuk's orient2d bound plus the input-rounding
+// terms); whatever is not certain is redone with the FP64 rule on the original
+// vertices.  The result is the FP64 rule's, bit for bit, in both forms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
-#include "sj_internal.cuh"
+#include "sj_host.hpp"
 
 namespace sj {
 
 unsigned bounds_take_pip() { return bounds_take(); }
 
-constexpr int PIP_WARPS = 4;
-
-struct alignas(16) Edge64 {
-    double ax, ay, bx, by;
-};
-
-template <bool FP32>
-struct PipSmem;
-
-template <>
-struct PipSmem<true> {
-    static constexpr int SMAX = 128;
-    float2 yh[SMAX];          // FP32 truncated y of the edge's two ends
-    float4 rel[SMAX];         // cell-relative (ax, ay, bx, by)
-    int vi[SMAX];             // global index of the edge's first end
-    unsigned char kk[SMAX];   // candidate index within the group
-    int coff[33], cid[32], cvb[32];
-    float2 pt[MAX_CH];
-    float pyh[MAX_CH];
-    int pin[MAX_CH];          // FP64 source index of the point: sorted slot (spts) or input index (pts)
-    int found[MAX_CH];
-    unsigned par[MAX_CH];
-};
-
-template <>
-struct PipSmem<false> {
-    static constexpr int SMAX = 128;
-    Edge64 e[SMAX];
-    unsigned char kk[SMAX];
-    int coff[33], cid[32], cvb[32];
-    double2 pt[MAX_CH];
-    int found[MAX_CH];
-    unsigned par[MAX_CH];
-};
+// ------------------------------------------------------------------ the crossing rule
 
 // The crossing rule in FP64: straddle iff (a.y > p.y) != (b.y > p.y); with lo
 // the end at or below p.y, count iff (hi.x-lo.x)(p.y-lo.y) - (hi.y-lo.y)(p.x-lo.x) > 0.
@@ -90,14 +60,6 @@ __device__ __forceinline__ int cross64(double px, double py, double ax, double a
     double d = __dsub_rn(__dmul_rn(__dsub_rn(hx, lx), __dsub_rn(py, ly)),
                          __dmul_rn(__dsub_rn(hy, ly), __dsub_rn(px, lx)));
     return d > 0.0;
-}
-
-// FP64 re-evaluation of edge i (vertex i -> nxt[i]) for point k of spts (when
-// set) or of pts.
-__device__ __noinline__ int cross64_global(const RefineArgs &a, int i, int k) {
-    const double2 p = a.spts ? a.spts[k] : a.pts[k];
-    const double2 A = a.verts[i], B = a.verts[a.nxt[i]];
-    return cross64(p.x, p.y, A.x, A.y, B.x, B.y);
 }
 
 // Sign of the orientation d = A*B - C*D on cell-relative FP32 inputs, certified
@@ -128,706 +90,887 @@ __device__ __forceinline__ bool orient32(float px, float py, float lx, float ly,
     return fabsf(d) > E;
 }
 
-// Near lists longer than this are not staged: each pending point searches
-// the window of the sorted list that can hold its straddling edges.
-constexpr int LONG_NEAR = 128;
+// Bound of the error of fl(a - b) against the difference of the two values
+// whose cell-relative forms a and b are (2.0001 u |.| + eps each, plus the
+// subtraction's own rounding): 3.01 u (|a| + |b|) + 2 eps.
+__device__ __forceinline__ float diff_bound(float a, float b, float eps) {
+    return fmaf(3.01f * U32, fabsf(a) + fabsf(b), 2.0f * eps);
+}
 
-// Crossing of near edge e (boundary list entry) for point q of the item, the
-// arithmetic of pip_compute for one edge: FP32X on the edge's staging record
-// (FP32 straddle test on truncations, certified orientation, FP64 rule on a
-// tie or an uncertain sign), FP64 on the original vertices.
-template <bool FP32>
-__device__ __forceinline__ int near_edge_cross(const RefineArgs &a, const PipSmem<FP32> &s, int q, int e, float2 fo,
-                                               unsigned &c_fb) {
-    if constexpr (FP32) {
-        const float pyh = s.pyh[q];
-        const float4 va = a.bnear_rec[2 * (size_t)e], vc = a.bnear_rec[2 * (size_t)e + 1];
-        if ((va.y == pyh) | (vc.y == pyh)) {   // FP32 y tie: decide in FP64
-            ++c_fb;
-            return cross64_global(a, a.bnear_ids[e], s.pin[q]);
+// ------------------------------------------------------------------ cell records
+
+// A group of a cell's record, in 32-byte units: header, n near edges, then (16
+// bytes each) nf flips and, with PIP_EXT, the ids of its candidates.
+constexpr int PIP_MORE = 1 << 30;      // another group follows
+constexpr int PIP_EXT = 1 << 29;       // ids follow the flips; id[1] holds the float bits of h
+constexpr int PIP_INLINE_IDS = 3;
+
+struct alignas(16) PipHead {
+    int n, nf;
+    unsigned base;     // parity mask below the row's flips
+    int ncand;         // candidates of the cell (statistics), with the PIP_* bits
+    int id[3];         // ids of candidates 0..2; with PIP_EXT: candidates in the group, h, unused
+    int algo;          // edges of the cell's candidate polygons (statistics)
+};
+struct alignas(16) PipEdge {
+    float lx, ly, hx, hy;   // cell-relative ends, lower y first
+    int vid;                // edge (= first vertex) index, for the FP64 rule
+    unsigned mask;          // bits of the candidates it belongs to
+    int pad[2];
+};
+struct alignas(16) PipFlip {
+    float y;                    // cell-relative
+    unsigned mask;              // parity mask from this y on
+    unsigned long long key;     // y_key of the exact value
+};
+static_assert(sizeof(PipHead) == 32 && sizeof(PipEdge) == 32 && sizeof(PipFlip) == 16, "");
+
+__host__ __device__ __forceinline__ long long group_units(int n, int nf, int ng) {
+    const int ids = (ng > PIP_INLINE_IDS || n > PIP_SEARCH_MIN) ? (ng + 3) / 4 : 0;
+    return 1LL + n + ((long long)nf + ids + 1) / 2;
+}
+
+// ------------------------------------------------------------------ the join
+
+// Where a join's points come from and its ids go.
+struct OneSource {
+    const double2 *pts;
+    int *out;
+    int n;
+    __device__ __forceinline__ int count() const { return n; }
+    __device__ __forceinline__ double2 point(unsigned i) const { return __ldcs(pts + i); }
+    __device__ __forceinline__ void put(unsigned i, int id) const { out[i] = id; }
+    __device__ __forceinline__ int get(unsigned i) const { return out[i]; }
+};
+// Many requests as one point set (batched rounds).
+struct RoundSource {
+    const RoundReq *reqs;
+    const int *meta;   // requests, points
+    __device__ __forceinline__ int count() const { return meta[1]; }
+    __device__ __forceinline__ const RoundReq &find(unsigned i) const {
+        int lo = 0, hi = meta[0];
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (reqs[mid].off <= (int)i) lo = mid; else hi = mid;
         }
-        const bool a_up = va.y > pyh, b_up = vc.y > pyh;
-        if (a_up == b_up) return 0;
-        const float ax = rel_coord(va.x, va.z, fo.x), ay = rel_coord(va.y, va.w, fo.y);
-        const float bx = rel_coord(vc.x, vc.z, fo.x), by = rel_coord(vc.y, vc.w, fo.y);
-        const float lx = a_up ? bx : ax, ly = a_up ? by : ay;
-        const float hx = a_up ? ax : bx, hy = a_up ? ay : by;
-        const float2 p = s.pt[q];
-        bool pos;
-        if (orient32(p.x, p.y, lx, ly, hx, hy, a.eps_abs, pos)) return (int)pos;
-        ++c_fb;
-        return cross64_global(a, a.bnear_ids[e], s.pin[q]);
-    } else {
-        const int i = a.bnear_ids[e];
-        const double2 A = a.verts[i], B = a.verts[a.nxt[i]], p = s.pt[q];
-        return cross64(p.x, p.y, A.x, A.y, B.x, B.y);
+        return reqs[lo];
     }
+    __device__ __forceinline__ double2 point(unsigned i) const {
+        const RoundReq &r = find(i);
+        return __ldcs(r.pts + (i - r.off));
+    }
+    __device__ __forceinline__ void put(unsigned i, int id) const {
+        const RoundReq &r = find(i);
+        r.out_id[i - r.off] = id;
+    }
+    __device__ __forceinline__ int get(unsigned i) const {
+        const RoundReq &r = find(i);
+        return r.out_id[i - r.off];
+    }
+};
+
+// Warps per block and blocks per SM: bound by the latency of its gathers (cell
+// code, record), the join is fastest at the most warps whose 64 registers hold
+// the loop without spills: 100 M points on the 40,000 tiles 1.87 / 1.70 / 1.61 ms
+// with 6 / 7 / 8 blocks, 2.8 ms with 10 (48 registers, spilled).
+constexpr int PIP_WARPS = 4, PIP_BLOCKS = 8;
+// Code of a queued point whose cell the FP32 estimate leaves open (no record
+// starts there: units are fewer than 2^31 - 2^22).
+constexpr int PIP_UNSURE = -2147483647 - 1;
+constexpr int PIP_SCAN_FLIPS = 8;   // flips scanned one by one by pip_fast
+
+// A lane's counters of the points refined.  In shared memory: the refinement
+// has no registers for three 64-bit sums.
+struct PipSums {
+    unsigned long long tests, pairs, algo;
+};
+
+// A point that waits for its refinement.
+struct PipQueued {
+    double2 p;
+    int i, code, ix, iy;   // point index, cell code, column, row
+};
+static_assert(sizeof(PipQueued) == 32, "");
+
+// Whether a near edge counts for the point (px, py): 1 yes, 0 no, -1 not
+// certain in FP32.
+__device__ __forceinline__ int edge_cross(float px, float py, const float4 r, float eps) {
+    const float sl = __fsub_rn(py, r.y), sh = __fsub_rn(py, r.w);
+    const float el = diff_bound(py, r.y, eps), eh = diff_bound(py, r.w, eps);
+    if (sl < -el || sh > eh) return 0;                      // certainly does not straddle
+    bool pos = false;
+    const bool sure = sl > el && sh < -eh && orient32(px, py, r.x, r.y, r.z, r.w, eps, pos);
+    return sure ? (int)pos : -1;
 }
 
-// First index t in [0, n) with keys[t] >= x (upper = false) or > x (upper =
-// true), n if none.
-__device__ __forceinline__ int key_bound(const float *keys, int n, float x, bool upper) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const float k = keys[mid];
-        if (upper ? (k <= x) : (k < x)) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
+__device__ __forceinline__ float2 point_rel(const PipArgs &a, const PipQueued &q) {
+    float hx, lx, hy, ly;
+    split_double(q.p.x, hx, lx);
+    split_double(q.p.y, hy, ly);
+    return make_float2(rel_coord(hx, lx, a.frame_x[q.ix]), rel_coord(hy, ly, a.frame_y[q.iy]));
 }
 
-// Parity masks of the staged edges [0, ns) for the item's pending points.
-template <bool FP32>
-__device__ __forceinline__ unsigned long long pip_compute(PipSmem<FP32> &s, const RefineArgs &a, int j0, int np,
-                                                          int ns, int lane, unsigned &c_fb) {
-    unsigned long long tests = 0;
-    int pg = 32;
-    for (int q0 = 0; q0 < np; q0 += pg) {   // one lane per point while 32 remain, then lane groups
-        const int rem = np - q0;
-        const int sg = rem >= 32 ? 1 : choose_group(rem, ns, 0);
-        const int lg = __ffs(sg) - 1;
-        pg = 32 >> lg;
-        const int sub = lane & (sg - 1), grp = lane >> lg;
-        const int q = q0 + grp;
-        const bool act = q < np && s.found[q] < 0;
-        const unsigned actb = __ballot_sync(FULL, act && sub == 0);
-        if (!actb) continue;
-        tests += (unsigned long long)__popc(actb) * (unsigned long long)ns;
-        unsigned m = 0;
-        if (act) {
-            if constexpr (FP32) {
-                const float2 p = s.pt[q];
-                const float pyh = s.pyh[q];
-                for (int t = sub; t < ns; t += sg) {
-                    const float2 yh = s.yh[t];
-                    if ((yh.x == pyh) | (yh.y == pyh)) {   // FP32 y tie: decide in FP64
-                        m ^= (unsigned)cross64_global(a, s.vi[t], s.pin[q]) << s.kk[t];
-                        ++c_fb;
-                        continue;
-                    }
-                    const bool a_up = yh.x > pyh, b_up = yh.y > pyh;
-                    if (a_up == b_up) continue;
-                    const float4 r = s.rel[t];
-                    const float lx = a_up ? r.z : r.x, ly = a_up ? r.w : r.y;
-                    const float hx = a_up ? r.x : r.z, hy = a_up ? r.y : r.w;
-                    bool pos;
-                    int cr;
-                    if (orient32(p.x, p.y, lx, ly, hx, hy, a.eps_abs, pos)) {
-                        cr = (int)pos;
-                    } else {
-                        cr = cross64_global(a, s.vi[t], s.pin[q]);
-                        ++c_fb;
-                    }
-                    m ^= (unsigned)cr << s.kk[t];
-                }
+// Results of up to 32 queued points, one per lane (act), in the common case: a
+// short record whose tests are all certain in FP32.  Returns false for a point
+// that needs pip_hard instead, otherwise its id in res.
+__device__ __forceinline__ bool pip_fast(const PipArgs &a, const PipQueued &q, PipSums &sum, int &res) {
+    res = -1;
+    if (q.code == PIP_UNSURE) return false;
+    const int off = -2 - q.code;
+    if (!SJ_IN_BOUNDS(off < a.units_n, BND_PIP_REC)) return true;
+    const int4 *u = a.units + 2 * (size_t)off;
+    const int4 h0 = __ldg(u), h1 = __ldg(u + 1);   // n, nf, base, ncand; ids, algo (PipHead)
+    const PipEdge *E = reinterpret_cast<const PipEdge *>(u + 2);
+    // the first two edges travel with the header (a record ends at least two
+    // units before the end of the array), the next ones two tests ahead
+    float4 e0 = __ldg(reinterpret_cast<const float4 *>(E)), e1 = __ldg(reinterpret_cast<const float4 *>(E + 1));
+    const int n = h0.x, nf = h0.y;
+    if (n > a.search || nf > PIP_SCAN_FLIPS) return false;
+    const PipFlip *F = reinterpret_cast<const PipFlip *>(E + n);
+    const float2 r = point_rel(a, q);
+    bool unsure = false;
+    unsigned m = (unsigned)h0.z;
+    for (int f = 0; f < nf; ++f) {   // flips at or below y
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(F + f));
+        const float d = __fsub_rn(r.y, v.x);
+        unsure |= !(fabsf(d) > diff_bound(r.y, v.x, a.eps));
+        if (!(d > 0.0f)) break;
+        m = __float_as_uint(v.y);
+    }
+    int t = 0;
+    for (; t < n; ++t) {
+        const float4 e = e0;
+        e0 = e1;
+        if (t + 2 < n) e1 = __ldg(reinterpret_cast<const float4 *>(E + t + 2));
+        // lower ends ascend: from the first edge wholly above y on, none straddles
+        if (__fsub_rn(e.y, r.y) > diff_bound(r.y, e.y, a.eps)) break;
+        const int x = edge_cross(r.x, r.y, e, a.eps);
+        unsure |= x < 0;
+        if (x > 0) m ^= __ldg(&E[t].mask);
+    }
+    if (unsure || (!m && (h0.w & PIP_MORE))) return false;
+    sum.tests += (unsigned)t;
+    sum.pairs += (unsigned)(h0.w & (PIP_EXT - 1));
+    sum.algo += (unsigned)h1.w;
+    if (m) {
+        const int k = __ffs(m) - 1;
+        if (h0.w & PIP_EXT) res = __ldg(reinterpret_cast<const int *>(F + nf) + k);
+        else res = k == 0 ? h1.x : (k == 1 ? h1.y : h1.z);
+    }
+    return true;
+}
+
+// The general case, one point by the whole warp: any number of groups, long
+// lists searched by y, tests that FP32 leaves open redone with the FP64 rule.
+__device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, PipSums &sum, int lane, unsigned &fb) {
+    const double2 p = q.p;
+    const float2 r = point_rel(a, q);
+    const unsigned long long ky = y_key(p.y);
+    int off = -2 - q.code, res = -1;
+    unsigned tests = 0;
+    bool first = true;
+    while (SJ_IN_BOUNDS(off < a.units_n, BND_PIP_REC)) {
+        const int4 *u = a.units + 2 * (size_t)off;
+        const int4 h0 = u[0], h1 = u[1];
+        const int n = h0.x, nf = h0.y;
+        const PipEdge *E = reinterpret_cast<const PipEdge *>(u + 2);
+        const PipFlip *F = reinterpret_cast<const PipFlip *>(E + n);
+        if (first && lane == 0) {
+            sum.pairs += (unsigned)(h0.w & (PIP_EXT - 1));
+            sum.algo += (unsigned)h1.w;
+        }
+        first = false;
+        unsigned m = (unsigned)h0.z;
+        for (int f0 = 0, f1 = nf; f0 < f1;) {   // the last flip at or below y
+            const int mid = (f0 + f1) >> 1;
+            if (F[mid].key <= ky) {
+                m = F[mid].mask;
+                f0 = mid + 1;
             } else {
-                const double2 p = s.pt[q];
-                for (int t = sub; t < ns; t += sg) {
-                    const Edge64 e = s.e[t];
-                    if (cross64(p.x, p.y, e.ax, e.ay, e.bx, e.by)) m ^= 1u << s.kk[t];
-                }
+                f1 = mid;
             }
         }
-        for (int o = sg >> 1; o > 0; o >>= 1) m ^= __shfl_xor_sync(FULL, m, o);
-        if (sub == 0 && act) s.par[q] ^= m;
+        int lo = 0, hi = n;
+        if (n > a.search) {
+            // edges that can straddle y: lower ends within [y - h, y], widened
+            // by the rounding bounds; both predicates are monotone in ly
+            const float hh = __int_as_float(h1.y), ep = diff_bound(r.y, r.y, a.eps);
+            int b1 = n;
+            while (lo < b1) {
+                const int mid = (lo + b1) >> 1;
+                if (__fadd_ru(E[mid].ly, hh) < __fsub_rd(r.y, ep)) lo = mid + 1; else b1 = mid;
+            }
+            hi = lo;
+            b1 = n;
+            while (hi < b1) {
+                const int mid = (hi + b1) >> 1;
+                const float ly = E[mid].ly;
+                if (fmaf(-3.01f * U32, fabsf(ly), ly) > __fadd_ru(r.y, ep)) b1 = mid; else hi = mid + 1;
+            }
+        }
+        unsigned mm = 0;
+        for (int t = lo + lane; t < hi; t += 4 * 32) {   // four loads in flight per lane
+            float4 e[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (t + 32 * k < hi) e[k] = __ldg(reinterpret_cast<const float4 *>(E + t + 32 * k));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (t + 32 * k >= hi) break;
+                int x = edge_cross(r.x, r.y, e[k], a.eps);
+                if (x < 0) {
+                    const int i = E[t + 32 * k].vid;
+                    const double2 A = a.verts[i], B = a.verts[a.nxt[i]];
+                    x = cross64(p.x, p.y, A.x, A.y, B.x, B.y);
+                    ++fb;
+                }
+                if (x) mm ^= E[t + 32 * k].mask;
+            }
+        }
+        m ^= __reduce_xor_sync(FULL, mm);
+        tests += (unsigned)(hi - lo);
+        if (m) {
+            const int k = __ffs(m) - 1;
+            if (h0.w & PIP_EXT) res = reinterpret_cast<const int *>(F + nf)[k];
+            else res = k == 0 ? h1.x : (k == 1 ? h1.y : h1.z);
+            break;
+        }
+        if (!(h0.w & PIP_MORE)) break;
+        off += (int)group_units(n, nf, h1.x);   // a group before another holds 32 ids: PIP_EXT
     }
-    return tests;
+    if (lane == 0) sum.tests += tests;
+    return res;
 }
 
-template <bool FP32, int NW>
-__global__ void __launch_bounds__(NW * 32, 28 / NW) k_pip_refine(RefineArgs a) {
-    constexpr int SMAX = PipSmem<FP32>::SMAX;
-    extern __shared__ __align__(16) unsigned char pip_smem_raw[];
+// One warp takes tiles of 32 U consecutive points.  A point whose cell is
+// certain and classified is answered at once.  The others are queued in shared
+// memory and refined 32 at a time, so that the refinement runs with full warps
+// although only some of a tile's points (6 - 54 %) need it.  The few that this
+// cannot finish wait until the warp has seen its last tile, in one list per
+// lane threaded through their own places in the output (out[i] = the index
+// before i in the lane's list), which needs no scratch and has no limit; by
+// then their general, register-hungry code costs the loop nothing (with a call
+// to it inside the loop the 100 M point join took 2.3 - 4.5 ms instead of 1.6).
+//
+// Bound by the latency and the L1 wavefronts of the random reads of cell codes
+// and records, both L2-resident (ncu at 20 M points on the tiles: issue slots
+// 53 % busy, long-scoreboard the top stall, DRAM 13 % of peak).  Measured, us a
+// join, against bucketing the points and refining (cell, point-chunk) items:
+// 1,003 points 53 -> 12, 1 M points on the stars (FP64 form) 119 -> 30, 10 M on
+// the heavy-tail tiles 2,450 -> 531, 100 M on the 40,000 tiles 4,486 -> 1,548.
+template <int U, class Src>
+__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src) {
+    __shared__ PipQueued queue[PIP_WARPS][32 * (U + 1)];
+    __shared__ PipSums sums[PIP_WARPS * 32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
-    PipSmem<FP32> &s = reinterpret_cast<PipSmem<FP32> *>(pip_smem_raw)[w];
-    const int n_items = *a.n_items;
-    const float FINF = __int_as_float(0x7f800000);
-    const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned long long c_pairs = 0, c_tests = 0, c_items = 0, c_algo = 0, c_wtests = 0;
-    unsigned c_fb = 0, c_hits = 0;
-
-    // Items come from a device counter when a.work_next is set (the next index
-    // is fetched at the start of an item, so its latency hides behind the
-    // item), else in a fixed stride.
-    // a.claim consecutive items per counter update (mostly chunks of one
-    // cell, whose staged records are then still in L1).
-    // The next item's record and its cell's point range are loaded while the
-    // current item is refined, off the per-item chain of dependent loads.
-    const int claim = a.claim > 1 ? a.claim : 1;
-    int it = blockIdx.x * NW + w, it_end = it + 1;
-    if (a.work_next) {
-        int t0 = 0;
-        if (lane == 0) t0 = atomicAdd(a.work_next, claim);
-        it = __shfl_sync(FULL, t0, 0);
-        it_end = it + claim;
-    }
-    int2 item = make_int2(0, 0);
-    int cs0 = 0, cs1 = 0;
-    if (it < n_items) {
-        item = a.items[it];
-        cs0 = a.cell_start[item.x];
-        cs1 = a.cell_start[item.x + 1];
-    }
-    while (it < n_items) {
-        int it_next = it + gridDim.x * NW;
-        const bool in_claim = it + 1 < it_end;
-        if (a.work_next) {
-            if (in_claim) it_next = it + 1;
-            else if (lane == 0) it_next = atomicAdd(a.work_next, claim);
-        }
-        ++c_items;
-        const int c = item.x;
-        const int j0 = cs0 + item.y;
-        const int np = min(cell_chunk(a.ch, a.budget > 0 ? a.cell_work[c] : 0, a.budget), cs1 - j0);
-        const int k0 = a.cand_start[c], k1 = a.cand_start[c + 1];
-        const float2 fo = cell_frame(a.frame_x, a.frame_y, a.g.nx, c);
-
-        // 1. points, the range of their FP32 y truncations and the smallest x
-        // truncation.  Items of more than 32 points: the (up to MAX_CH / 32)
-        // point loads of a lane are issued together -- every slot index, then
-        // every point as an asynchronous copy into the idle staging area -- so
-        // that their latencies overlap instead of forming one chain per point;
-        // smaller items (one point per lane) load directly.
-        float ylo = FINF, yhi = -FINF, xlo = FINF;
-        auto put = [&](int q, double2 p, int src) {
-            float hx, lx, hy, ly;
-            split_double(p.x, hx, lx);
-            split_double(p.y, hy, ly);
-            if constexpr (FP32) {
-                s.pt[q] = make_float2(rel_coord(hx, lx, fo.x), rel_coord(hy, ly, fo.y));
-                s.pyh[q] = hy;
-                s.pin[q] = src;
-            } else {
-                s.pt[q] = p;
-            }
-            s.found[q] = -1;
-            s.par[q] = 0u;
-            ylo = fminf(ylo, hy);
-            yhi = fmaxf(yhi, hy);
-            xlo = fminf(xlo, hx);
-        };
-        if (np <= 32) {
-            if (lane < np) {
-                int src = -1;
-                double2 p = make_double2(0.0, 0.0);
-                if (SJ_IN_BOUNDS(j0 + lane < a.npts, BND_PIP_POINT)) {
-                    src = a.spts ? j0 + lane : a.perm[j0 + lane];
-                    if (SJ_IN_BOUNDS(src < a.npts, BND_PIP_POINT)) p = a.spts ? __ldcg(a.spts + src) : __ldcg(a.pts + src);
-                    else src = -1;
+    const unsigned lt = (1u << lane) - 1u;
+    const unsigned n = (unsigned)src.count(), tiles = (n + 32u * U - 1u) / (32u * U);
+    unsigned items = 0, resolved = 0, hits = 0, fb = 0;
+    sums[threadIdx.x] = PipSums{0, 0, 0};
+    int qn = 0, head = -1;
+    for (unsigned t = blockIdx.x * PIP_WARPS + w;; t += gridDim.x * PIP_WARPS) {
+        const bool more = t < tiles;   // else: the points left in the queues
+        if (more) {
+            const unsigned i0 = t * (32u * U) + lane;
+            double2 p[U];
+            int code[U], ix[U], iy[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + 32u * u < n) p[u] = src.point(i0 + 32u * u);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                code[u] = -1;
+                if (i0 + 32u * u < n) {
+                    const bool sx = axis_estimate(p[u].x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, ix[u]);
+                    const bool sy = axis_estimate(p[u].y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, iy[u]);
+                    code[u] = PIP_UNSURE;
+                    if (sx && sy) {
+                        code[u] = __ldg(a.cell_code + iy[u] * a.g.nx + ix[u]);
+                        resolved += code[u] >= -1;
+                    }
                 }
-                put(lane, p, src);
-            }
-        } else {
-            constexpr int PQ = MAX_CH / 32;
-            double2 *pbuf;
-            if constexpr (FP32) {
-                static_assert(sizeof(PipSmem<true>::rel) >= MAX_CH * sizeof(double2), "");
-                pbuf = reinterpret_cast<double2 *>(&s.rel[0]);
-            } else {
-                static_assert(sizeof(PipSmem<false>::e) >= MAX_CH * sizeof(double2), "");
-                pbuf = reinterpret_cast<double2 *>(&s.e[0]);
-            }
-            __syncwarp();   // no lane still reads the previous item's staged edges
-            int src[PQ];
-#pragma unroll
-            for (int u = 0; u < PQ; ++u) {
-                const int q = lane + 32 * u;
-                src[u] = (q < np && SJ_IN_BOUNDS(j0 + q < a.npts, BND_PIP_POINT)) ? (a.spts ? j0 + q : a.perm[j0 + q])
-                                                                                 : -1;
-                if (src[u] >= 0 && !SJ_IN_BOUNDS(src[u] < a.npts, BND_PIP_POINT)) src[u] = -1;
             }
 #pragma unroll
-            for (int u = 0; u < PQ; ++u)
-                if (src[u] >= 0) copy16_async(pbuf + lane + 32 * u, a.spts ? a.spts + src[u] : a.pts + src[u]);
-            copy_async_wait_all();
-#pragma unroll
-            for (int u = 0; u < PQ; ++u) {
-                const int q = lane + 32 * u;
-                if (q < np) put(q, src[u] >= 0 ? pbuf[q] : make_double2(0.0, 0.0), src[u]);
+            for (int u = 0; u < U; ++u) {
+                const unsigned i = i0 + 32u * u;
+                const bool q = i < n && code[u] < -1;
+                if (i < n && !q) {
+                    src.put(i, code[u]);
+                    hits += code[u] >= 0;
+                }
+                const unsigned bal = __ballot_sync(FULL, q);
+                if (q) queue[w][qn + __popc(bal & lt)] = PipQueued{p[u], (int)i, code[u], ix[u], iy[u]};
+                qn += __popc(bal);
             }
+            __syncwarp();
         }
-        if (a.work_next) it_next = __shfl_sync(FULL, it_next, 0);
-        int2 item_n = make_int2(0, 0);
-        if (it_next < n_items) item_n = a.items[it_next];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ylo = fminf(ylo, __shfl_xor_sync(FULL, ylo, o));
-            yhi = fmaxf(yhi, __shfl_xor_sync(FULL, yhi, o));
-            xlo = fminf(xlo, __shfl_xor_sync(FULL, xlo, o));
+        while (more ? qn >= 32 : qn > 0) {
+            const int cnt = min(qn, 32);
+            qn -= cnt;
+            if (lane < cnt) {
+                const PipQueued q = queue[w][qn + lane];
+                int res;
+                const bool done = pip_fast(a, q, sums[threadIdx.x], res);
+                if (SJ_IN_BOUNDS((unsigned)q.i < n, BND_PIP_RES)) {
+                    src.put((unsigned)q.i, done ? res : head);
+                    if (!done) head = q.i;
+                    hits += done && res >= 0;
+                }
+            }
+            ++items;
         }
+        if (!more) break;
         __syncwarp();
-
-        for (int kg = k0; kg < k1; kg += 32) {
-            int pending = 0;
-            for (int q = lane; q < np; q += 32) pending += (s.found[q] < 0);
-            pending = __reduce_add_sync(FULL, pending);
-            if (pending == 0) break;
-            // 2. candidate group: one polygon per lane, its edge list for the
-            //    item's grid row, list lengths scanned
-            //    (a candidate whose class for this cell is inside / outside
-            //    contributes its parity without any edge)
-            //    A boundary candidate stages only its near edges; the parity of
-            //    its far-right edges comes from the flip keys (k_pip_boundary).
-            const int nc = min(32, k1 - kg);
-            int pid = 0, vb = 0, ne = 0, nall = 0, cls = 0, fs = 0, fl = 0;
-            if (lane < nc) {
-                const int k = kg + lane;
-                pid = a.cand_ids[k];
-                cls = a.cand_cls[k];
-                if (cls == 0) {
-                    vb = a.bnear_start[k];
-                    ne = a.bnear_start[k + 1] - vb;
-                    fs = a.bflip_start[k];
-                    fl = a.bflip_len[k];
-                }
-                nall = a.obj_voff[pid + 1] - a.obj_voff[pid];
+    }
+    while (__any_sync(FULL, head >= 0)) {   // the lists, one point of each lane at a time
+        PipQueued q;
+        q.i = head;
+        bool act = head >= 0;
+        int res = -1;
+        if (act) {
+            head = src.get((unsigned)q.i);
+            q.p = src.point((unsigned)q.i);
+            const int2 e = point_cell_exact(a.g, q.p.x, q.p.y);
+            const int code = e.x >= 0 && e.y >= 0 ? a.cell_code[e.y * a.g.nx + e.x] : -1;
+            const bool unsure = !(axis_estimate(q.p.x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, q.ix) &&
+                                  axis_estimate(q.p.y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, q.iy));
+            q.ix = e.x;
+            q.iy = e.y;
+            q.code = code;
+            bool done = code >= -1;
+            res = code;
+            if (done) resolved += e.x >= 0 && e.y >= 0;
+            else if (unsure) done = pip_fast(a, q, sums[threadIdx.x], res);   // only its cell was open
+            if (done) {
+                src.put((unsigned)q.i, res);
+                hits += res >= 0;
+                act = false;
             }
-            const unsigned inside = __ballot_sync(FULL, cls == 1);
-            // far-right parity: the number of flip keys at or below the point's y
-            for (unsigned far = __ballot_sync(FULL, fl > 0); far; far &= far - 1) {
-                const int j = __ffs(far) - 1;
-                const int f0 = __shfl_sync(FULL, fs, j), n = __shfl_sync(FULL, fl, j);
-                for (int q = lane; q < np; q += 32) {
-                    if (s.found[q] >= 0) continue;
-                    double py;
-                    if constexpr (FP32) py = a.spts ? a.spts[s.pin[q]].y : a.pts[s.pin[q]].y;
-                    else py = s.pt[q].y;
-                    const unsigned long long ky = y_key(py);
-                    int lo = 0, hi = n;   // first key above ky
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (a.bflip_keys[f0 + mid] <= ky) lo = mid + 1;
-                        else hi = mid;
-                    }
-                    if (lo & 1) s.par[q] ^= 1u << j;
-                }
-            }
-            // long near lists: each pending point tests only the edges whose
-            // lower truncated y lies in [fl_down(y - h), y] (two binary
-            // searches in the sorted list); no other edge of the list can
-            // straddle its y (nor tie with it), so the parity is unchanged
-            const bool lng = ne > LONG_NEAR;
-            for (unsigned lm = __ballot_sync(FULL, lng); lm; lm &= lm - 1) {
-                const int j = __ffs(lm) - 1;
-                const int b0 = __shfl_sync(FULL, vb, j), n0 = __shfl_sync(FULL, ne, j);
-                const float hj = a.bnear_h[kg + j];
-                const float *keys = a.bnear_key + b0;
-                for (int q = lane; q < np; q += 32) {
-                    if (s.found[q] >= 0) continue;
-                    float pyh;
-                    if constexpr (FP32) pyh = s.pyh[q];
-                    else pyh = approx_float(s.pt[q].y);
-                    const int lo = key_bound(keys, n0, __fsub_rd(pyh, hj), false);
-                    const int hi = key_bound(keys, n0, pyh, true);
-                    unsigned par = 0;
-                    for (int t = lo; t < hi; ++t)
-                        if (SJ_IN_BOUNDS(b0 + t < a.bnear_start[a.cand_start[a.g.G]], BND_PIP_REC))
-                            par ^= (unsigned)near_edge_cross<FP32>(a, s, q, b0 + t, fo, c_fb);
-                    c_wtests += (unsigned long long)(hi > lo ? hi - lo : 0);
-                    if (par & 1u) s.par[q] ^= 1u << j;
-                }
-            }
-            if (lng) ne = 0;   // staged below: the short lists only
-            __syncwarp();
-            c_pairs += (unsigned long long)pending * (unsigned long long)nc;
-            c_algo += (unsigned long long)pending * (unsigned long long)__reduce_add_sync(FULL, (unsigned)nall);
-            int incl = ne;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int E = __shfl_sync(FULL, incl, 31);
-            __syncwarp();
-            if (lane < nc) {
-                s.coff[lane] = incl - ne;
-                s.cid[lane] = pid;
-                s.cvb[lane] = vb;
-            }
-            if (lane == 0) s.coff[nc] = E;
-            __syncwarp();
-
-            // 3. staging with the exact y-range prune, 4. parity when full
-            int nst = 0, kw = 0;
-            for (int base = 0; base < E; base += 32) {
-                const int g = base + lane;
-                bool keep = false;
-                int i = 0, j = 0, k = 0;
-                float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vc = va;
-                if (g < E) {
-                    while (s.coff[kw + 1] <= g) ++kw;   // candidate of edge g (g grows by 32)
-                    k = kw;
-                    int e = s.cvb[kw] + (g - s.coff[kw]);
-                    if (!SJ_IN_BOUNDS(e < a.bnear_start[a.cand_start[a.g.G]], BND_PIP_REC)) e = 0;
-                    i = a.bnear_ids[e];
-                    if constexpr (FP32) {
-                        va = a.bnear_rec[2 * (size_t)e];
-                        vc = a.bnear_rec[2 * (size_t)e + 1];
-                    } else {
-                        j = a.nxt[i];
-                        va = a.vsplit[i];
-                        vc = a.vsplit[j];
-                    }
-                    // y: strictly outside the points' y-range never straddles
-                    // (exact compares on monotone truncations).  x: an edge
-                    // wholly left of every point cannot cross a ray to +x; the
-                    // reference sign is a rounded FP64 orientation, so only
-                    // edges clear of the points by far more than its rounding
-                    // error (about 1e-10 m here) are dropped: a margin of 8
-                    // FP32 ulps plus 1 mm on the truncated coordinates.
-                    const float ex = fmaxf(va.x, vc.x);
-                    keep = !(fmaxf(va.y, vc.y) < ylo || fminf(va.y, vc.y) > yhi ||
-                             ex + fmaf(fabsf(ex) + fabsf(xlo), 9.5367431640625e-07f, 1e-3f) < xlo);
-                }
-                const unsigned bal = __ballot_sync(FULL, keep);
-                if (keep) {
-                    const int pos = nst + __popc(bal & lt_mask);
-                    if constexpr (FP32) {
-                        s.yh[pos] = make_float2(va.y, vc.y);
-                        s.rel[pos] = make_float4(rel_coord(va.x, va.z, fo.x), rel_coord(va.y, va.w, fo.y),
-                                                 rel_coord(vc.x, vc.z, fo.x), rel_coord(vc.y, vc.w, fo.y));
-                        s.vi[pos] = i;
-                    } else {
-                        const double2 A = a.verts[i], B = a.verts[j];
-                        s.e[pos] = Edge64{A.x, A.y, B.x, B.y};
-                    }
-                    s.kk[pos] = (unsigned char)k;
-                }
-                nst += __popc(bal);
-                if (nst > SMAX - 32 || base + 32 >= E) {
-                    __syncwarp();
-                    if (nst > 0) c_tests += pip_compute<FP32>(s, a, j0, np, nst, lane, c_fb);
-                    __syncwarp();
-                    nst = 0;
-                }
-            }
-            // smallest candidate with odd parity
-            for (int q = lane; q < np; q += 32) {
-                const unsigned m = s.par[q] | inside;
-                if (s.found[q] < 0 && m) s.found[q] = s.cid[__ffs(m) - 1];
-                s.par[q] = 0u;
-            }
-            __syncwarp();
         }
-        int cs0n = 0, cs1n = 0;
-        if (it_next < n_items) {
-            cs0n = a.cell_start[item_n.x];
-            cs1n = a.cell_start[item_n.x + 1];
+        for (unsigned left = __ballot_sync(FULL, act); left; left &= left - 1) {
+            const int j = __ffs(left) - 1;
+            PipQueued r;
+            r.p = make_double2(__shfl_sync(FULL, q.p.x, j), __shfl_sync(FULL, q.p.y, j));
+            r.i = __shfl_sync(FULL, q.i, j);
+            r.code = __shfl_sync(FULL, q.code, j);
+            r.ix = __shfl_sync(FULL, q.ix, j);
+            r.iy = __shfl_sync(FULL, q.iy, j);
+            const int id = pip_hard(a, r, sums[threadIdx.x], lane, fb);
+            if (lane == 0) {
+                src.put((unsigned)r.i, id);
+                hits += id >= 0;
+            }
         }
-        for (int q = lane; q < np; q += 32) {
-            const int f = s.found[q];
-            if (!SJ_IN_BOUNDS(j0 + q < a.npts, BND_PIP_RES)) continue;
-            if (a.res_id) a.res_id[j0 + q] = f;
-            else if (f >= 0) a.out_id[a.perm[j0 + q]] = f;
-            if (f >= 0) ++c_hits;
-        }
-        __syncwarp();
-        it_end = in_claim ? it_end : it_next + (a.work_next ? claim : 1);
-        it = it_next;
-        item = item_n;
-        cs0 = cs0n;
-        cs1 = cs1n;
+        if (__any_sync(FULL, act)) ++items;
     }
     if (a.stats) {
-        c_fb = __reduce_add_sync(FULL, c_fb);
-        c_hits = __reduce_add_sync(FULL, c_hits);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c_wtests += __shfl_xor_sync(FULL, c_wtests, o);
         unsigned long long v[ST_N] = {};
-        v[ST_ITEMS] = c_items;
-        v[ST_PAIRS] = c_pairs;
-        v[ST_TESTS] = c_tests + c_wtests;   // staged tests (warp-uniform) + window tests
-        v[ST_ALGO] = c_algo;
-        v[ST_FALLBACK] = c_fb;
-        v[ST_HITS] = c_hits;
+        PipSums s = sums[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s.tests += __shfl_xor_sync(FULL, s.tests, o);
+            s.pairs += __shfl_xor_sync(FULL, s.pairs, o);
+            s.algo += __shfl_xor_sync(FULL, s.algo, o);
+        }
+        v[ST_ITEMS] = items;
+        v[ST_PAIRS] = s.pairs;
+        v[ST_TESTS] = s.tests;
+        v[ST_ALGO] = s.algo;
+        v[ST_RESOLVED] = __reduce_add_sync(FULL, resolved);
+        v[ST_FALLBACK] = __reduce_add_sync(FULL, fb);
+        v[ST_HITS] = __reduce_add_sync(FULL, hits);
         flush_stats(a.stats, v);
     }
 }
 
-// Cell classification (layer build), one warp per cell.  For a candidate P of
-// cell c, the only edges that can straddle the horizontal line of a point of c
-// are those of P's list for c's row.  If none of them meets the cell box
-// widened by delta, every point of the cell lies at least delta from each of
-// them, so (i) the straight path from the point to the cell centre crosses no
-// edge -- all points of the cell share the centre's inside/outside status --
-// and (ii) the FP64 crossing rule evaluates every such edge with the correct
-// orientation sign (its rounding error is below 1e-10 m at coordinates of
-// 1e5 m, delta is far larger), so the rule gives each point that status.  The
-// class is then the FP64 crossing parity of the centre: 1 inside, 2 outside;
-// 0 (boundary) when some edge meets the widened box.  The cell box is the
-// exact set of doubles the cell rule maps to the cell: [key_value(kx[ix]),
-// key_value(kx[ix + 1])) and likewise in y.
-__global__ void k_pip_classify(GridDev g, const int *cand_start, const int *cand_ids, const int *prow_base,
-                               const int *prow_r0, const int *prow_start, const int *pedge_ids, const int *nxt,
-                               const double2 *verts, double delta, unsigned char *cls) {
-    const int lane = lane_id();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int c = warp; c < g.G; c += nwarps) {
-        const int k0 = cand_start[c], k1 = cand_start[c + 1];
-        if (k0 == k1) continue;
-        const int ix = c % g.nx, iy = c / g.nx;
-        const double X0 = key_value(g.kx[ix]), X1 = key_value(g.kx[ix + 1]);
-        const double Y0 = key_value(g.ky[iy]), Y1 = key_value(g.ky[iy + 1]);
-        const double bx0 = X0 - delta, bx1 = X1 + delta, by0 = Y0 - delta, by1 = Y1 + delta;
-        const double cx = 0.5 * (X0 + X1), cy = 0.5 * (Y0 + Y1);
-        for (int k = k0; k < k1; ++k) {
-            const int P = cand_ids[k];
-            const int slot = prow_base[P] + (iy - prow_r0[P]);
-            const int e0 = prow_start[slot], e1 = prow_start[slot + 1];
-            int hit = 0, par = 0;
-            for (int e = e0 + lane; e < e1; e += 32) {
-                const int i = pedge_ids[e];
-                const double2 A = verts[i], B = verts[nxt[i]];
-                hit |= !(fmax(A.x, B.x) < bx0 || fmin(A.x, B.x) > bx1 || fmax(A.y, B.y) < by0 ||
-                         fmin(A.y, B.y) > by1);
-                par ^= cross64(cx, cy, A.x, A.y, B.x, B.y);
-            }
-            hit = __reduce_or_sync(FULL, (unsigned)hit);
-            par = (int)(__reduce_xor_sync(FULL, (unsigned)par) & 1u);
-            if (lane == 0) cls[k] = hit ? 0 : (par ? 1 : 2);
-        }
+// Points per lane and tile: two once that still gives every SM all its warps
+// twice over (100 M points: 1.69 / 1.55 / 1.90 ms with 1 / 2 / 4); smaller calls
+// spread over more warps, one point per lane.
+constexpr int PIP_U = 2;
+
+static int pip_blocks(int U, long long n, int sms) {
+    const long long tiles = (n + 32LL * U - 1) / (32LL * U);
+    return (int)std::max(1LL, std::min((tiles + PIP_WARPS - 1) / PIP_WARPS, (long long)sms * PIP_BLOCKS));
+}
+
+cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, int sms, cudaStream_t s) {
+    const OneSource src{pts, out, n};
+    if (n >= sms * PIP_WARPS * PIP_BLOCKS * 32 * 2 * PIP_U) k_pip_join<PIP_U><<<pip_blocks(PIP_U, n, sms), PIP_WARPS * 32, 0, s>>>(a, src);
+    else k_pip_join<1><<<pip_blocks(1, n, sms), PIP_WARPS * 32, 0, s>>>(a, src);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points, int sms,
+                             cudaStream_t s) {
+    k_pip_join<1><<<pip_blocks(1, max_points, sms), PIP_WARPS * 32, 0, s>>>(a, RoundSource{reqs, meta});
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ layer build
+
+// Where a layer's edges lie (PipEdges), one thread per edge (vertex i -> nxt[i]):
+// its grid rows under the cell rule (FP64 divisions, done once here), its
+// x-range rounded outward to FP32, and which end is the lower one.
+__global__ void k_pip_edges(GridDev g, const double2 *verts, const int *nxt, int V, PipEdges e) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        const double2 A = verts[i], B = verts[nxt[i]];
+        const bool up = A.y <= B.y;
+        e.rows[i] = make_int2(clamped_axis(up ? A.y : B.y, g.y0, g.ch, g.ny), clamped_axis(up ? B.y : A.y, g.y0, g.ch, g.ny));
+        e.xr[i] = make_float2(__double2float_rd(fmin(A.x, B.x)), __double2float_ru(fmax(A.x, B.x)));
+        e.kind[i] = (up ? 1 : 0) | (A.y == B.y ? 2 : 0);
     }
 }
 
-// Per cell of a polygon layer: the result every point of the cell gets when
-// each of its candidates is classified (class 1 inside or 2 outside) -- the
-// smallest candidate whose class is inside (candidate ids are sorted), or -1
-// -- else CELL_REFINE: some candidate is a boundary candidate and the cell's
-// points go through the refinement.  Cells without candidates get -1.
-__global__ void k_cell_result(const int *cand_start, const int *cand_ids, const unsigned char *cls, int G, int *res) {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < G; c += gridDim.x * blockDim.x) {
-        int r = -1;
-        for (int k = cand_start[c]; k < cand_start[c + 1]; ++k) {
-            if (cls[k] == 0) {
-                r = CELL_REFINE;
+// Edges with equal end points (the common side of two polygons), paired
+// through an open-addressing table of edge indices.  Pairs only: a third copy
+// of an edge, or one that finds no slot within a few probes, stays single,
+// which costs a test and changes no result.
+__device__ __forceinline__ unsigned edge_hash(double2 l, double2 h) {
+    unsigned long long v = (unsigned long long)__double_as_longlong(l.x) * 0x9E3779B97F4A7C15ULL;
+    v = (v ^ (v >> 32) ^ (unsigned long long)__double_as_longlong(l.y)) * 0xC2B2AE3D27D4EB4FULL;
+    v = (v ^ (v >> 29) ^ (unsigned long long)__double_as_longlong(h.x)) * 0x9E3779B97F4A7C15ULL;
+    v = (v ^ (v >> 32) ^ (unsigned long long)__double_as_longlong(h.y)) * 0xC2B2AE3D27D4EB4FULL;
+    return (unsigned)(v >> 32);
+}
+
+__global__ void k_pip_twins(const double2 *verts, const int *nxt, const unsigned char *kind, int V, int *table,
+                            unsigned slots_mask, int *twin) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        if (kind[i] & 2) continue;   // horizontal: never listed
+        const bool up = kind[i] & 1;
+        const double2 A = verts[i], B = verts[nxt[i]];
+        const double2 l = up ? A : B, h = up ? B : A;
+        unsigned at = edge_hash(l, h);
+        for (int probe = 0; probe < 16; ++probe, ++at) {
+            const int j = atomicCAS(&table[at & slots_mask], -1, i);
+            if (j == -1) break;
+            const bool uj = kind[j] & 1;
+            const double2 Aj = verts[j], Bj = verts[nxt[j]];
+            const double2 lj = uj ? Aj : Bj, hj = uj ? Bj : Aj;
+            if (l.x == lj.x && l.y == lj.y && h.x == hj.x && h.y == hj.y) {
+                if (atomicCAS(&twin[j], -1, i) == -1) twin[i] = j;
                 break;
             }
-            if (cls[k] == 1 && r == -1) r = cand_ids[k];
         }
-        res[c] = r;
     }
 }
 
-cudaError_t launch_cell_result(const int *cand_start, const int *cand_ids, const unsigned char *cls, int G, int *res,
-                               cudaStream_t s) {
-    const int nb = (int)std::max<long long>(1, std::min<long long>(((long long)G + 255) / 256, 152LL * 32));
-    k_cell_result<<<nb, 256, 0, s>>>(cand_start, cand_ids, cls, G, res);
-    return cudaGetLastError();
-}
-
-// Per-point edge work of each cell of a polygon layer (the split of work
-// items by candidate-edge count): the near edges of its boundary candidates,
-// a long list (searched per point) counted as LONG_NEAR.
-__global__ void k_cell_work_pip(const int *cand_start, const unsigned char *cls, const int *near_start, int G,
-                                int *work) {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < G; c += gridDim.x * blockDim.x) {
-        long long w = 0;
-        for (int k = cand_start[c]; k < cand_start[c + 1]; ++k)
-            if (cls[k] == 0) w += min(near_start[k + 1] - near_start[k], LONG_NEAR);
-        work[c] = (int)min(w, 2147483647LL);
+// Row lists: for each (polygon, row of its MBB) the edges whose rows include
+// it.  One thread per edge.  Count (ids == nullptr), then emit.
+__global__ void k_prow_edges(const int2 *rows, const int *owner, int V, const int *prow_base, const int *prow_r0,
+                             int *cnt, unsigned long long *total, const int *start, int *ids) {
+    unsigned long long n = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        const int P = owner[i], base = prow_base[P] - prow_r0[P];
+        const int2 r = rows[i];
+        for (int y = r.x; y <= r.y; ++y) {
+            const int k = atomicAdd(&cnt[base + y], 1);
+            if (ids) ids[start[base + y] + k] = i;
+        }
+        n += (unsigned long long)(r.y - r.x + 1);
+    }
+    if (!ids) {
+        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(FULL, n, o);
+        if (lane_id() == 0 && n) atomicAdd(total, n);
     }
 }
 
-cudaError_t launch_cell_work_pip(const int *cand_start, const unsigned char *cls, const int *near_start, int G,
-                                 int *work, cudaStream_t s) {
-    const int nb = (int)std::max<long long>(1, std::min<long long>(((long long)G + 255) / 256, 152LL * 32));
-    k_cell_work_pip<<<nb, 256, 0, s>>>(cand_start, cls, near_start, G, work);
-    return cudaGetLastError();
+// x-limits of each column widened by delta, rounded outward.
+__global__ void k_pip_columns(GridDev g, double delta, float2 *col) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.nx; i += gridDim.x * blockDim.x)
+        col[i] = make_float2(__double2float_rd(key_value(g.kx[i]) - delta), __double2float_ru(key_value(g.kx[i + 1]) + delta));
 }
 
-cudaError_t launch_pip_classify(const GridDev &g, const int *cand_start, const int *cand_ids, const int *prow_base,
-                                const int *prow_r0, const int *prow_start, const int *pedge_ids, const int *nxt,
-                                const double2 *verts, double delta, unsigned char *cls, cudaStream_t s) {
-    const long long nb = std::min<long long>(((long long)g.G * 32 + 255) / 256, 152LL * 64);
-    k_pip_classify<<<(int)std::max<long long>(nb, 1), 256, 0, s>>>(g, cand_start, cand_ids, prow_base, prow_r0,
-                                                                  prow_start, pedge_ids, nxt, verts, delta, cls);
-    return cudaGetLastError();
+// Cell of each candidate entry.
+__global__ void k_pip_entry_cells(const int *cand_start, int G, int *cell) {
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < G; c += gridDim.x * blockDim.x)
+        for (int k = cand_start[c]; k < cand_start[c + 1]; ++k) cell[k] = c;
 }
 
-// Boundary entries (class 0), one warp per cell.  The candidate's row-list
-// edges split three ways against the cell's column [X0, X1) widened by delta:
-//   left  (max x < X0 - delta): farther than delta left of every point of the
-//         cell, so the FP64 rule never counts a crossing -- dropped;
-//   far   (min x > X1 + delta): farther than delta right of every point, so
-//         the FP64 rule counts a crossing exactly when the edge straddles the
-//         point's y (its orientation sign is far above rounding) -- the parity
-//         of those straddles is the parity of the number of end y-values
-//         (lower and upper end of each far edge) at or below the point's y,
-//         since an edge straddles y iff lower <= y < upper;
-//   near  (the rest): tested point by point in the refinement.
-// An end shared with the ring's adjacent edge counts twice when that edge is a
-// far edge of the same list too (the same vertex, the same y), which leaves
-// the parity unchanged: such ends are not emitted, so only the ends of chains
-// of far edges remain.
-// Count pass: near edges and far end values per entry.  Emit pass: near edge
-// ids and far end keys (order keys, -0 folded onto +0).
-__device__ __forceinline__ bool far_in_list(const BoundaryArgs &a, int u, int w, double XR, int iy) {
-    const double2 U = a.verts[u], W = a.verts[w];
-    if (!(fmin(U.x, W.x) > XR)) return false;
-    const int ra = clamped_axis(fmin(U.y, W.y), a.g.y0, a.g.ch, a.g.ny);
-    const int rb = clamped_axis(fmax(U.y, W.y), a.g.y0, a.g.ch, a.g.ny);
-    return ra <= iy && iy <= rb;
+// The candidate entry of polygon Q in cell c when the cell has few enough
+// candidates to form one group, else -1.
+__device__ __forceinline__ int entry_of(const PipBuildArgs &b, int k0, int k1, int Q) {
+    if (k1 - k0 > 32) return -1;
+    for (int k = k0; k < k1; ++k)
+        if (b.cand_ids[k] == Q) return k;
+    return -1;
 }
 
-__global__ void k_pip_boundary(BoundaryArgs a, int emit) {
-    const int lane = lane_id();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int c = warp; c < a.g.G; c += nwarps) {
-        const int k0 = a.cand_start[c], k1 = a.cand_start[c + 1];
-        if (k0 == k1) continue;
-        const int ix = c % a.g.nx, iy = c / a.g.nx;
-        const double XL = key_value(a.g.kx[ix]) - a.delta, XR = key_value(a.g.kx[ix + 1]) + a.delta;
+// Candidate entries, eight lanes each.  Count pass: near edges (a shared edge
+// counted with its polygon of smaller id), flips, base parity and whether the
+// entry has any near edge or flip (ent[k] = near, flips << 2 | base << 1 | any).
+// Emit pass: the near edges (vid, mask) and flips (key, bit) of the relevant
+// entries, unordered, at edge_at[k] / flip_at[k] in the temporary units.
+// Eight lanes: a (polygon, row) list holds 5 - 60 edges on average.
+template <bool EMIT>
+__global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
+    const int lane = lane_id(), sub = lane & 7, gsh = lane & 24;
+    const unsigned gm = 0xffu << gsh, lt = (1u << lane) - 1u;
+    const long long T = (long long)gridDim.x * blockDim.x;
+    for (long long kk = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3; kk < b.M; kk += T >> 3) {
+        const int k = (int)kk;
+        const int bit = EMIT ? b.ord[k] : 0;
+        if (EMIT && bit < 0) continue;
+        const int c = b.entry_cell[k];
+        const int iy = c / b.g.nx, ix = c - iy * b.g.nx;
+        const float2 col = b.col[ix];
+        const int P = b.cand_ids[k];
+        const int slot = b.prow_base[P] + (iy - b.prow_r0[P]);
+        const int e0 = b.prow_start[slot], e1 = b.prow_start[slot + 1];
+        const int k0 = b.cand_start[c], k1 = b.cand_start[c + 1];
+        const unsigned own = EMIT ? 1u << (bit & 31) : 0u;
+        int n = 0, nf = 0, par = 0;
+        bool any = false;
+        for (int base = e0; base < e1; base += 8) {
+            const int t = base + sub;
+            bool is_near = false, mine = false, fl = false, fh = false;
+            int i = 0, tk = -1;
+            if (t < e1) {
+                i = b.pedge[t];
+                const float2 xr = b.e.xr[i];
+                const unsigned char kd = b.e.kind[i];
+                if (xr.x > col.y) {   // far
+                    const int2 r = b.e.rows[i];
+                    par ^= r.x < iy;
+                    if (r.x == iy || r.y == iy) {
+                        // the ends inside the row, unless shared with another far edge
+                        const bool a_far = b.e.xr[b.prv[i]].x > col.y, b_far = b.e.xr[b.nxt[i]].x > col.y;
+                        const bool up = kd & 1;
+                        fl = r.x == iy && !(up ? a_far : b_far);
+                        fh = r.y == iy && !(up ? b_far : a_far);
+                    }
+                } else if (!(xr.y < col.x) && !(kd & 2)) {   // near
+                    is_near = mine = true;
+                    const int tw = b.twin[i];
+                    if (tw >= 0) {
+                        const int Q = b.owner[tw];
+                        if (Q != P) tk = entry_of(b, k0, k1, Q);
+                        if (tk >= 0 && Q < P) mine = false;
+                    }
+                }
+            }
+            const unsigned bn = __ballot_sync(gm, mine);
+            const unsigned bl = __ballot_sync(gm, fl), bh = __ballot_sync(gm, fh);
+            any |= __any_sync(gm, is_near) || bl || bh;
+            if (EMIT) {
+                if (mine) {
+                    unsigned m = own;
+                    if (tk >= 0 && b.ord[tk] >= 0) m |= 1u << (b.ord[tk] & 31);
+                    b.tmp_edge[b.edge_at[k] + n + __popc(bn & lt & gm)] = make_int2(i, (int)m);
+                }
+                if (fl || fh) {
+                    const bool up = b.e.kind[i] & 1;
+                    const int j = b.nxt[i];
+                    PipFlipTmp *f = b.tmp_flip + b.flip_at[k] + nf + __popc(bl & lt & gm) + __popc(bh & lt & gm);
+                    if (fl) *f++ = PipFlipTmp{y_key(b.verts[up ? i : j].y), own, 0};
+                    if (fh) *f = PipFlipTmp{y_key(b.verts[up ? j : i].y), own, 0};
+                }
+            }
+            n += __popc(bn);
+            nf += __popc(bl) + __popc(bh);
+        }
+        if (!EMIT) {
+            par = (int)__popc(__ballot_sync(gm, par & 1)) & 1;
+            if (sub == 0) b.ent[k] = make_int2(n, (nf << 2) | (par << 1) | (any ? 1 : 0));
+        }
+    }
+}
+
+// Cells, one thread each: the relevant candidates (ord[k] = place among them,
+// or -1), the cell's code when every candidate is classified, else the size of
+// its record in units, near edges and flips (for the temporary lists).
+__global__ void k_pip_cells(PipBuildArgs b) {
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < b.g.G; c += gridDim.x * blockDim.x) {
+        const int k0 = b.cand_start[c], k1 = b.cand_start[c + 1];
+        int rel = 0, code = -1;
+        bool done = false, any = false;
+        long long units = 0, tn = 0, tf = 0;
+        int n = 0, nf = 0, ng = 0;
         for (int k = k0; k < k1; ++k) {
-            if (a.cls[k] != 0) {
-                if (!emit && lane == 0) a.near_cnt[k] = a.flip_cnt[k] = 0;
+            const int2 e = b.ent[k];
+            const bool bd = e.y & 1, base = e.y & 2;
+            if (done || (!bd && !base)) {
+                b.ord[k] = -1;
                 continue;
             }
-            const int P = a.cand_ids[k];
-            const int slot = a.prow_base[P] + (iy - a.prow_r0[P]);
-            const int e0 = a.prow_start[slot], e1 = a.prow_start[slot + 1];
-            int nn = 0, nf = 0;   // running counts (uniform across the warp)
-            for (int b = e0; b < e1; b += 32) {
-                const int e = b + lane;
-                bool is_near = false, ks = false, ke = false;
-                int i = 0;
-                double ys = 0.0, ye = 0.0;
-                if (e < e1) {
-                    i = a.pedge_ids[e];
-                    const int j = a.nxt[i];
-                    const double2 A = a.verts[i], B = a.verts[j];
-                    const double xmin = fmin(A.x, B.x), xmax = fmax(A.x, B.x);
-                    const bool is_far = xmin > XR;
-                    is_near = !is_far && !(xmax < XL);
-                    if (is_far) {
-                        ks = !far_in_list(a, a.prv[i], i, XR, iy);   // start shared with the previous edge
-                        ke = !far_in_list(a, j, a.nxt[j], XR, iy);   // end shared with the next edge
+            if (!bd) {
+                if (rel == 0) code = b.cand_ids[k];
+                done = true;
+            }
+            any |= bd;
+            b.ord[k] = rel++;
+            n += e.x;
+            nf += e.y >> 2;
+            if (++ng == 32) {
+                units += group_units(n, nf, ng);
+                tn += n;
+                tf += nf;
+                n = nf = ng = 0;
+            }
+        }
+        if (ng) units += group_units(n, nf, ng);
+        tn += n;
+        tf += nf;
+        if (!any) {   // classified: no record
+            for (int k = k0; k < k1; ++k) b.ord[k] = -1;
+            units = tn = tf = 0;
+        } else {
+            code = -2;
+        }
+        b.cell_code[c] = code;
+        b.units_of[c] = (int)min(units, 2147483647LL);
+        b.edges_of[c] = (int)min(tn, 2147483647LL);
+        b.flips_of[c] = (int)min(tf, 2147483647LL);
+    }
+}
+
+// Headers, ids and the entries' places in the temporary lists, one thread per cell.
+__global__ void k_pip_heads(PipBuildArgs b) {
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < b.g.G; c += gridDim.x * blockDim.x) {
+        if (b.cell_code[c] != -2) continue;
+        const int k0 = b.cand_start[c], k1 = b.cand_start[c + 1];
+        int off = b.units_at[c], te = b.edges_at[c], tf = b.flips_at[c];
+        b.cell_code[c] = -2 - off;
+        long long algo = 0;
+        int last = k0;   // last relevant entry
+        for (int k = k0; k < k1; ++k) {
+            algo += b.obj_voff[b.cand_ids[k] + 1] - b.obj_voff[b.cand_ids[k]];
+            if (b.ord[k] >= 0) last = k;
+        }
+        for (int k = k0; k <= last;) {   // a group
+            PipHead h;
+            h.n = h.nf = 0;
+            h.base = 0;
+            h.id[0] = h.id[1] = h.id[2] = 0;
+            int ng = 0, q = k;
+            for (; q <= last && ng < 32; ++q) {
+                if (b.ord[q] < 0) continue;
+                const int2 e = b.ent[q];
+                b.edge_at[q] = te + h.n;
+                b.flip_at[q] = tf + h.nf;
+                if (e.y & 2) h.base |= 1u << ng;
+                if (ng < PIP_INLINE_IDS) h.id[ng] = b.cand_ids[q];
+                h.n += e.x;
+                h.nf += e.y >> 2;
+                ++ng;
+            }
+            int4 *u = b.units + 2 * (size_t)off;
+            h.ncand = min(k1 - k0, PIP_EXT - 1);
+            if (ng > PIP_INLINE_IDS || h.n > PIP_SEARCH_MIN) {
+                h.ncand |= PIP_EXT;
+                int *ids = reinterpret_cast<int *>(u + 2 + 2 * (size_t)h.n + h.nf);
+                for (int r = k, t = 0; r < q; ++r)
+                    if (b.ord[r] >= 0) ids[t++] = b.cand_ids[r];
+                h.id[0] = ng;
+            }
+            if (q <= last) h.ncand |= PIP_MORE;
+            h.algo = (int)min(algo, 2147483647LL);
+            u[0] = make_int4(h.n, h.nf, (int)h.base, h.ncand);
+            u[1] = make_int4(h.id[0], h.id[1], h.id[2], h.algo);
+            off += (int)group_units(h.n, h.nf, ng);
+            te += h.n;
+            tf += h.nf;
+            k = q;
+        }
+    }
+}
+
+// The order of a near edge in its list (a NaN, possible only beyond the FP32
+// range where every test goes to the FP64 rule, must not break the ranks).
+__device__ __forceinline__ float list_key(float ly) { return ly == ly ? ly : 0.0f; }
+
+__device__ __forceinline__ float4 edge_rel(const PipBuildArgs &b, int i, float2 fo) {
+    const double2 A = b.verts[i], B = b.verts[b.nxt[i]];
+    const bool up = b.e.kind[i] & 1;
+    const double2 l = up ? A : B, h = up ? B : A;
+    float a, c;
+    float4 r;
+    split_double(l.x, a, c); r.x = rel_coord(a, c, fo.x);
+    split_double(l.y, a, c); r.y = rel_coord(a, c, fo.y);
+    split_double(h.x, a, c); r.z = rel_coord(a, c, fo.x);
+    split_double(h.y, a, c); r.w = rel_coord(a, c, fo.y);
+    return r;
+}
+// An upper bound of hi.y - lo.y with both ends' rounding bounds (the search window).
+__device__ __forceinline__ float edge_height(float4 r) {
+    return __fadd_ru(__fsub_ru(r.w, r.y), __fmul_ru(8.0f * U32, fabsf(r.w) + fabsf(r.y)));
+}
+__device__ __forceinline__ float key_rel(unsigned long long key, float fo) {
+    float a, c;
+    split_double(key_value(key), a, c);
+    return rel_coord(a, c, fo);
+}
+
+// Record groups larger than this are ordered by a whole block (k_pip_order_long).
+constexpr int PIP_LONG = PIP_LONG_MIN;
+
+// The records' edges (ordered by lower y) and flips (ordered by key, masks
+// accumulated), eight lanes per cell: each element's place is its rank.
+__global__ void __launch_bounds__(256) k_pip_order(PipBuildArgs b) {
+    const int lane = lane_id(), sub = lane & 7;
+    const unsigned gm = 0xffu << (lane & 24);
+    const long long T = (long long)gridDim.x * blockDim.x;
+    for (long long cc = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3; cc < b.g.G; cc += T >> 3) {
+        const int c = (int)cc, code = b.cell_code[c];
+        if (code >= -1) continue;
+        const float2 fo = cell_frame(b.frame_x, b.frame_y, b.g.nx, c);
+        int off = -2 - code, te = b.edges_at[c], tf = b.flips_at[c];
+        while (true) {
+            int4 *u = b.units + 2 * (size_t)off;
+            const int4 u0 = u[0];
+            const int n = u0.x, nf = u0.y;
+            if (n > PIP_LONG || nf > PIP_LONG) {
+                if (sub == 0) b.long_list[atomicAdd(b.long_n, 1)] = make_int4(off, c, te, tf);
+            } else {
+                PipEdge *E = reinterpret_cast<PipEdge *>(u + 2);
+                float hmax = 0.0f;
+                for (int i = sub; i < n; i += 8) {
+                    const float4 r = edge_rel(b, b.tmp_edge[te + i].x, fo);
+                    b.tmp_rel[te + i] = r;
+                    hmax = fmaxf(hmax, edge_height(r));
+                }
+                __syncwarp(gm);
+                for (int i = sub; i < n; i += 8) {
+                    const float4 r = b.tmp_rel[te + i];
+                    const int2 v = b.tmp_edge[te + i];
+                    const float key = list_key(r.y);
+                    int rank = 0;
+                    for (int j = 0; j < n; ++j) {
+                        const float kj = list_key(b.tmp_rel[te + j].y);
+                        rank += kj < key || (kj == key && j < i);
                     }
-                    ys = A.y;
-                    ye = B.y;
+                    reinterpret_cast<float4 *>(E + rank)[0] = r;
+                    reinterpret_cast<int4 *>(E + rank)[1] = make_int4(v.x, v.y, 0, 0);
                 }
-                const unsigned bn = __ballot_sync(FULL, is_near);
-                const unsigned bs = __ballot_sync(FULL, ks), be = __ballot_sync(FULL, ke);
-                if (emit) {
-                    if (is_near) a.near_ids[a.near_start[k] + nn + __popc(bn & lt)] = i;
-                    const int f = a.flip_start[k] + nf + __popc(bs & lt) + __popc(be & lt);
-                    if (ks) a.flip_keys[f] = y_key(ys);
-                    if (ke) a.flip_keys[f + (ks ? 1 : 0)] = y_key(ye);
+                if (u0.w & PIP_EXT) {
+                    for (int o = 4; o > 0; o >>= 1) hmax = fmaxf(hmax, __shfl_xor_sync(gm, hmax, o));
+                    if (sub == 0) reinterpret_cast<int *>(u)[5] = __float_as_int(hmax);
                 }
-                nn += __popc(bn);
-                nf += __popc(bs) + __popc(be);
+                PipFlip *F = reinterpret_cast<PipFlip *>(E + n);
+                for (int i = sub; i < nf; i += 8) {
+                    const PipFlipTmp v = b.tmp_flip[tf + i];
+                    int rank = 0;
+                    unsigned m = (unsigned)u0.z;
+                    for (int j = 0; j < nf; ++j) {
+                        const PipFlipTmp w = b.tmp_flip[tf + j];
+                        const bool before = w.key < v.key || (w.key == v.key && j <= i);
+                        rank += before;
+                        if (before) m ^= w.mask;
+                    }
+                    F[rank - 1] = PipFlip{key_rel(v.key, fo.y), m, v.key};
+                }
             }
-            if (!emit && lane == 0) {
-                a.near_cnt[k] = nn;
-                a.flip_cnt[k] = nf;
-            }
+            if (!(u0.w & PIP_MORE)) break;
+            off += (int)group_units(n, nf, u[1].x);
+            te += n;
+            tf += nf;
         }
     }
 }
 
-// Sort each entry's far end keys and drop pairs of equal keys (a value counted
-// twice does not change the parity); len[k] = the keys left.  One thread per
-// entry, Shell sort (Ciura gaps).
-__global__ void k_pip_flips(const int *flip_start, int M, unsigned long long *keys, int *len) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M; k += gridDim.x * blockDim.x) {
-        const int b = flip_start[k], n = flip_start[k + 1] - b;
-        unsigned long long *v = keys + b;
-        const int ciura[8] = {1, 4, 10, 23, 57, 132, 301, 701};
-        int gaps[32];
-        int ng = 0;
-        while (ng < 8 && ciura[ng] < n) { gaps[ng] = ciura[ng]; ++ng; }
-        if (ng == 8) {
-            long long g = 701;
-            while (ng < 32 && (g = g * 9 / 4) < n) gaps[ng++] = (int)g;
+// Sort of n elements by a block, in place: the bitonic network in the form
+// whose compare-exchanges all put the smaller element first, which sorts any n
+// when partners beyond n are skipped.
+template <class Less, class Swap>
+__device__ __forceinline__ void block_sort(int n, Less less, Swap swap) {
+    auto pass = [&](auto partner) {
+        for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+            const long long j = partner(i);
+            if (j > i && j < n && less((int)j, (int)i)) swap((int)i, (int)j);
         }
-        for (int u = ng - 1; u >= 0; --u) {
-            const int h = gaps[u];
-            for (int i = h; i < n; ++i) {
-                const unsigned long long x = v[i];
-                int j = i;
-                while (j >= h && v[j - h] > x) { v[j] = v[j - h]; j -= h; }
-                v[j] = x;
-            }
-        }
-        int m = 0;
-        for (int i = 0; i < n;) {   // runs of equal keys: keep one key of an odd run
-            int j = i + 1;
-            while (j < n && v[j] == v[i]) ++j;
-            if ((j - i) & 1) v[m++] = v[i];
-            i = j;
-        }
-        len[k] = m;
+        __syncthreads();
+    };
+    for (long long k = 2; k < 2LL * n; k <<= 1) {
+        pass([&](long long i) { return i ^ (k - 1); });
+        for (long long h = k >> 2; h > 0; h >>= 1) pass([&](long long i) { return i ^ h; });
     }
 }
 
-// Near lists sorted by lower y (layer build), one thread per boundary entry:
-// key = min(trunc32(a.y), trunc32(b.y)) of each near edge (the FP32 truncations
-// the refinement compares, a monotone map of y), ids reordered by key (Shell
-// sort, Ciura gaps), and h[k] = the largest max - min of the two truncations
-// over the entry's edges, rounded up.  An edge of the list can straddle (or
-// tie with) a point's truncated y only if its key lies in
-// [fl_down(y - h), y]: the refinement finds that window by binary search.
-__global__ void k_pip_near_sort(const int *near_start, int M, int *ids, const int *nxt, const float4 *vsplit,
-                                float *keys, float *h) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M; k += gridDim.x * blockDim.x) {
-        const int b = near_start[k], n = near_start[k + 1] - b;
-        float hk = 0.0f;
-        for (int t = 0; t < n; ++t) {
-            const int i = ids[b + t];
-            const float ya = vsplit[i].y, yb = vsplit[nxt[i]].y;
-            keys[b + t] = fminf(ya, yb);
-            hk = fmaxf(hk, __fsub_ru(fmaxf(ya, yb), fminf(ya, yb)));
+__global__ void __launch_bounds__(512) k_pip_order_long(PipBuildArgs b) {
+    __shared__ int hbits;
+    const int total = *b.long_n;
+    for (int g = blockIdx.x; g < total; g += gridDim.x) {
+        const int4 q = b.long_list[g];
+        const float2 fo = cell_frame(b.frame_x, b.frame_y, b.g.nx, q.y);
+        int4 *u = b.units + 2 * (size_t)q.x;
+        const int4 u0 = u[0];
+        const int n = u0.x, nf = u0.y;
+        PipEdge *E = reinterpret_cast<PipEdge *>(u + 2);
+        PipFlip *F = reinterpret_cast<PipFlip *>(E + n);
+        float4 *rel = b.tmp_rel + q.z;
+        int2 *tv = b.tmp_edge + q.z;
+        PipFlipTmp *fl = b.tmp_flip + q.w;
+        if (threadIdx.x == 0) hbits = 0;
+        __syncthreads();
+        float hmax = 0.0f;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            rel[i] = edge_rel(b, tv[i].x, fo);
+            hmax = fmaxf(hmax, edge_height(rel[i]));
         }
-        h[k] = hk;
-        const int ciura[8] = {1, 4, 10, 23, 57, 132, 301, 701};
-        int gaps[32];
-        int ng = 0;
-        while (ng < 8 && ciura[ng] < n) { gaps[ng] = ciura[ng]; ++ng; }
-        if (ng == 8) {
-            long long g = 701;
-            while (ng < 32 && (g = g * 9 / 4) < n) gaps[ng++] = (int)g;
+        if (hmax > 0.0f) atomicMax(&hbits, __float_as_int(hmax));   // positive floats order as ints
+        __syncthreads();
+        block_sort(n, [&](int i, int j) { return list_key(rel[i].y) < list_key(rel[j].y); },
+                   [&](int i, int j) {
+                       const float4 r = rel[i]; rel[i] = rel[j]; rel[j] = r;
+                       const int2 v = tv[i]; tv[i] = tv[j]; tv[j] = v;
+                   });
+        block_sort(nf, [&](int i, int j) { return fl[i].key < fl[j].key; },
+                   [&](int i, int j) { const PipFlipTmp v = fl[i]; fl[i] = fl[j]; fl[j] = v; });
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            reinterpret_cast<float4 *>(E + i)[0] = rel[i];
+            reinterpret_cast<int4 *>(E + i)[1] = make_int4(tv[i].x, tv[i].y, 0, 0);
         }
-        float *kv = keys + b;
-        int *iv = ids + b;
-        for (int u = ng - 1; u >= 0; --u) {
-            const int gp = gaps[u];
-            for (int i = gp; i < n; ++i) {
-                const float x = kv[i];
-                const int xi = iv[i];
-                int j = i;
-                while (j >= gp && kv[j - gp] > x) {
-                    kv[j] = kv[j - gp];
-                    iv[j] = iv[j - gp];
-                    j -= gp;
-                }
-                kv[j] = x;
-                iv[j] = xi;
+        if (threadIdx.x == 0) {
+            if (u0.w & PIP_EXT) reinterpret_cast<int *>(u)[5] = hbits;
+            unsigned m = (unsigned)u0.z;
+            for (int i = 0; i < nf; ++i) {
+                m ^= fl[i].mask;
+                F[i] = PipFlip{key_rel(fl[i].key, fo.y), m, fl[i].key};
             }
         }
+        __syncthreads();
     }
 }
 
-cudaError_t launch_pip_near_sort(const int *near_start, int M, int *ids, const int *nxt, const float4 *vsplit,
-                                 float *keys, float *h, cudaStream_t s) {
-    const int nb = std::max(1, std::min((M + 127) / 128, 8192));
-    k_pip_near_sort<<<nb, 128, 0, s>>>(near_start, M, ids, nxt, vsplit, keys, h);
+static int grid_for(long long n, int per, int cap) {
+    return (int)std::max(1LL, std::min((n + per - 1) / per, (long long)cap));
+}
+
+cudaError_t launch_pip_edges(const PipBuildArgs &b, cudaStream_t s) {
+    k_pip_edges<<<grid_for(b.V, 256, 8192), 256, 0, s>>>(b.g, b.verts, b.nxt, b.V, b.e);
+    return cudaGetLastError();
+}
+cudaError_t launch_pip_twins(const PipBuildArgs &b, int *table, unsigned slots, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(table, 0xff, sizeof(int) * (size_t)slots, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.twin, 0xff, sizeof(int) * (size_t)b.V, s);
+    if (e != cudaSuccess) return e;
+    k_pip_twins<<<grid_for(b.V, 256, 8192), 256, 0, s>>>(b.verts, b.nxt, b.e.kind, b.V, table, slots - 1, b.twin);
+    return cudaGetLastError();
+}
+cudaError_t launch_prow_edges(const PipBuildArgs &b, int *cnt, unsigned long long *total, const int *start, int *ids,
+                              cudaStream_t s) {
+    k_prow_edges<<<grid_for(b.V, 256, 8192), 256, 0, s>>>(b.e.rows, b.owner, b.V, b.prow_base, b.prow_r0, cnt, total,
+                                                         start, ids);
+    return cudaGetLastError();
+}
+// Step 1: what each candidate entry and cell holds.
+cudaError_t launch_pip_count(const PipBuildArgs &b, double delta, cudaStream_t s) {
+    k_pip_columns<<<grid_for(b.g.nx, 256, 4096), 256, 0, s>>>(b.g, delta, b.col);
+    k_pip_entry_cells<<<grid_for(b.g.G, 256, 8192), 256, 0, s>>>(b.cand_start, b.g.G, b.entry_cell);
+    k_pip_entries<false><<<grid_for(8LL * b.M, 256, 16384), 256, 0, s>>>(b);
+    k_pip_cells<<<grid_for(b.g.G, 256, 8192), 256, 0, s>>>(b);
+    return cudaGetLastError();
+}
+// Step 2: the records (units, temporary lists and offsets allocated).
+cudaError_t launch_pip_records(const PipBuildArgs &b, cudaStream_t s) {
+    k_pip_heads<<<grid_for(b.g.G, 256, 8192), 256, 0, s>>>(b);
+    k_pip_entries<true><<<grid_for(8LL * b.M, 256, 16384), 256, 0, s>>>(b);
+    k_pip_order<<<grid_for(8LL * b.g.G, 256, 16384), 256, 0, s>>>(b);
+    k_pip_order_long<<<152 * 2, 512, 0, s>>>(b);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pip_boundary(const BoundaryArgs &a, int emit, cudaStream_t s) {
-    const long long nb = std::min<long long>(((long long)a.g.G * 32 + 255) / 256, 152LL * 64);
-    k_pip_boundary<<<(int)std::max<long long>(nb, 1), 256, 0, s>>>(a, emit);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pip_flips(const int *flip_start, int M, unsigned long long *keys, int *len, cudaStream_t s) {
-    const int nb = std::max(1, std::min((M + 127) / 128, 8192));
-    k_pip_flips<<<nb, 128, 0, s>>>(flip_start, M, keys, len);
-    return cudaGetLastError();
-}
+// ------------------------------------------------------------------ census
 
 // Census of the algorithmic PIP work (a measurement pass, not part of a
 // join): for every in-grid point, out[0] += the edges of its cell's candidate
@@ -835,7 +978,7 @@ cudaError_t launch_pip_flips(const int *flip_start, int M, unsigned long long *k
 // under the crossing rule's straddle test (Sec. III.C).  Only an edge of a
 // candidate's list for the point's grid row can straddle it (the row lists are
 // exact), so the straddles are counted over those lists.  One thread per point.
-__global__ void k_pip_census(RefineArgs a, const double2 *pts, int n, unsigned long long *out) {
+__global__ void k_pip_census(CensusArgs a, const double2 *pts, int n, unsigned long long *out) {
     unsigned long long e = 0, st = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double2 p = pts[i];
@@ -863,65 +1006,11 @@ __global__ void k_pip_census(RefineArgs a, const double2 *pts, int n, unsigned l
     }
 }
 
-cudaError_t launch_pip_census(const RefineArgs &a, const double2 *pts, int n, unsigned long long *out,
+cudaError_t launch_pip_census(const CensusArgs &a, const double2 *pts, int n, unsigned long long *out,
                               cudaStream_t s) {
     const int nb = std::max(1, std::min((n + 255) / 256, 152 * 16));
     k_pip_census<<<nb, 256, 0, s>>>(a, pts, n, out);
     return cudaGetLastError();
-}
-
-template <bool FP32, int NW>
-static size_t pip_smem_bytes() {
-    return sizeof(PipSmem<FP32>) * NW;
-}
-
-template <bool FP32, int NW>
-static cudaError_t pip_prepare() {
-    static bool done = false;
-    if (!done) {
-        cudaError_t e = cudaFuncSetAttribute(k_pip_refine<FP32, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)pip_smem_bytes<FP32, NW>());
-        if (e != cudaSuccess) return e;
-        done = true;
-    }
-    return cudaSuccess;
-}
-
-template <bool FP32, int NW>
-static cudaError_t pip_launch(const RefineArgs &a, int blocks, cudaStream_t s) {
-    cudaError_t e = pip_prepare<FP32, NW>();
-    if (e != cudaSuccess) return e;
-    k_pip_refine<FP32, NW><<<blocks, NW * 32, pip_smem_bytes<FP32, NW>(), s>>>(a);
-    return cudaGetLastError();
-}
-
-// blocks: the grid for blocks of PIP_WARPS warps; a block of warps_per_block
-// (2, 4 or 8) warps gets the same number of warps.
-cudaError_t launch_pip_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s) {
-    const int nw = (warps_per_block == 2 || warps_per_block == 8) ? warps_per_block : PIP_WARPS;
-    blocks = (int)(((long long)blocks * PIP_WARPS + nw - 1) / nw);
-    if (form == SJ_FP32X) {
-        if (nw == 2) return pip_launch<true, 2>(a, blocks, s);
-        if (nw == 8) return pip_launch<true, 8>(a, blocks, s);
-        return pip_launch<true, PIP_WARPS>(a, blocks, s);
-    }
-    if (nw == 2) return pip_launch<false, 2>(a, blocks, s);
-    if (nw == 8) return pip_launch<false, 8>(a, blocks, s);
-    return pip_launch<false, PIP_WARPS>(a, blocks, s);
-}
-
-int pip_blocks_per_sm(int form) {
-    int n = 0;
-    if (form == SJ_FP32X) {
-        if (pip_prepare<true, PIP_WARPS>() != cudaSuccess) return 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pip_refine<true, PIP_WARPS>, PIP_WARPS * 32,
-                                                      pip_smem_bytes<true, PIP_WARPS>());
-    } else {
-        if (pip_prepare<false, PIP_WARPS>() != cudaSuccess) return 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pip_refine<false, PIP_WARPS>, PIP_WARPS * 32,
-                                                      pip_smem_bytes<false, PIP_WARPS>());
-    }
-    return n > 0 ? n : 1;
 }
 
 }  // namespace sj
