@@ -208,15 +208,12 @@ static float float_up(double x) {
 }
 
 // Layer-dependent fields of the P2P refinement arguments.
-void sj::fill_refine(const sj_layer *L, RefineArgs &ra) {
+void sj::fill_refine(const sj_layer *L, int form, RefineArgs &ra) {
     ra.g = L->g;
     ra.cand_start = L->cand_start;
     ra.cand_ids = L->cand_ids;
     ra.obj_voff = L->obj_voff;
-    ra.verts = L->verts;
-    ra.seg_e64 = L->seg_e64;
-    ra.seg_inv64 = L->seg_inv64;
-    ra.seg32 = L->seg32;
+    ra.seg = SegArgs{L->verts, L->seg_e64, L->seg_inv64, L->seg32};
     ra.cseg_start = L->cseg_start;
     ra.cseg_ids = L->cseg_ids;
     ra.cell_algo = L->cell_algo;
@@ -226,6 +223,10 @@ void sj::fill_refine(const sj_layer *L, RefineArgs &ra) {
     ra.Ddn = L->Ddn;
     ra.Dup = L->Dup;
     ra.eps_abs = L->eps_abs;
+    // FP64 form: where the squares of coordinates or the FP32 inverse lengths
+    // could leave the FP32 range, an infinite bound sends every point to the
+    // FP64 recheck
+    if (form == SJ_FP64 && !(L->xmax <= 1e15 && L->xmax >= 1e-6)) ra.eps_abs = INFINITY;
     ra.frame_x = L->frames;
     ra.frame_y = L->frames + L->g.nx;
     ra.stats = L->stats;
@@ -797,22 +798,14 @@ extern "C" sj_status sj_layer_reset_stats(sj_layer *L) {
 struct JoinBufs {
     int *cnt, *cell_start, *perm, *totals, *pos, *cell_base, *sub_start;
     int2 *key_rank, *items, *block_sums, *fb;
-    double2 *spts;
-    ResF *resf;
-    ResD *resd;
 };
 
-// Result layout of a P2P join: through perm into the outputs (RES_PERM), or
-// cell-ordered packed records gathered back through pos (RES_F for FP32X,
-// RES_D for FP64).
-enum { RES_PERM = 0, RES_F, RES_D };
-
-// with_spts: also a cell-ordered copy of the points (else the refinement reads
-// the input points through perm).
+// Scratch of a P2P join.  The slots' result records take the place of key_rank,
+// which the scatter has used up (P2PRec has its size).  to_input: with the
+// slot of each input point (pos), for outputs written in input order.
 // ch_min: the smallest work item (cell_chunk's floor when items are split by
 // edge budget, else ch).
-static void carve(Scratch &s, JoinBufs &b, int64_t N, int G, int ch, bool need_fb, bool with_spts = true,
-                  int res = RES_PERM, int lS = 0, int ch_min = 0) {
+static void carve(Scratch &s, JoinBufs &b, int64_t N, int G, int ch, bool to_input, int lS = 0, int ch_min = 0) {
     size_t max_items = (size_t)(N / (ch_min > 0 ? ch_min : ch)) + (size_t)std::min<int64_t>(G, N) + 1;
     b.cnt = s.take<int>(((size_t)G << lS) + 1);
     b.sub_start = lS ? s.take<int>((size_t)G << lS) : nullptr;
@@ -820,16 +813,13 @@ static void carve(Scratch &s, JoinBufs &b, int64_t N, int G, int ch, bool need_f
     b.totals = s.take<int>(4);
     b.key_rank = s.take<int2>((size_t)N);
     b.perm = s.take<int>((size_t)N);
-    b.spts = with_spts ? s.take<double2>((size_t)N) : nullptr;
     b.items = s.take<int2>(max_items);
     b.block_sums = s.take<int2>(bucket_scan_blocks(G));
-    b.fb = need_fb ? s.take<int2>((size_t)N) : nullptr;
-    const bool sorted_res = res != RES_PERM;
-    b.pos = sorted_res ? s.take<int>((size_t)N) : nullptr;
-    b.cell_base = sorted_res ? s.take<int>((size_t)G) : nullptr;
-    b.resf = res == RES_F ? s.take<ResF>((size_t)N) : nullptr;
-    b.resd = res == RES_D ? s.take<ResD>((size_t)N) : nullptr;
+    b.fb = s.take<int2>((size_t)N);
+    b.pos = to_input ? s.take<int>((size_t)N) : nullptr;
+    b.cell_base = to_input ? s.take<int>((size_t)G) : nullptr;
 }
+static_assert(sizeof(P2PRec) == sizeof(int2), "");
 
 // window < 0: the layer's D; else a P2P window 0 <= window <= D for this call
 // alone (the layer's lists, built for D, hold every segment within any smaller
@@ -887,7 +877,6 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
         return check_bounds(s);
     }
     const int G = L->g.G;
-    const bool need_fb = form == SJ_FP32X;
     // Sub-cell order of the points inside their cells (see BucketArgs), on
     // request (SJ_FLAG_SUBCELL_ON): each work item of a dense cell then covers
     // a compact part of it and the exact per-item prune (the box distance)
@@ -900,13 +889,12 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     const int lS = sub_lx + sub_ly;
 
     JoinBufs b;
-    const int res = form == SJ_FP32X ? RES_F : RES_D;
     const bool split = budget > 0;   // items sized by the cells' edge work
     const int ch_min = split ? std::min(ch, 8) : ch;
-    size_t bytes = measure([&](Scratch &sc) { carve(sc, b, N, G, ch, need_fb, false, res, lS, ch_min); });
+    size_t bytes = measure([&](Scratch &sc) { carve(sc, b, N, G, ch, true, lS, ch_min); });
     Scratch sc;
     CUDA_TRY(dev_malloc_async((void **)&sc.base, bytes, s));
-    carve(sc, b, N, G, ch, need_fb, false, res, lS, ch_min);
+    carve(sc, b, N, G, ch, true, lS, ch_min);
     cudaError_t e = cudaMemsetAsync(b.cnt, 0, sizeof(int) * (((size_t)G << lS) + 1), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b.totals, 0, sizeof(int) * 4, s);
 
@@ -918,7 +906,6 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ba.key_rank = b.key_rank;
     ba.cell_start = b.cell_start;
     ba.perm = b.perm;
-    ba.spts = b.spts;
     ba.cand_start = L->cand_start;
     ba.ch = ch;
     ba.cell_work = split ? L->cell_work : nullptr;
@@ -935,7 +922,7 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     if (e == cudaSuccess) e = launch_bucket(ba, s);
 
     RefineArgs ra{};
-    fill_refine(L, ra);
+    fill_refine(L, form, ra);
     if (window >= 0.0) {
         ra.D = window;
         ra.Df = (float)window;
@@ -954,16 +941,12 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ra.claim = (N >= 2LL * ch * (long long)G) ? 2 : 1;
     ra.cell_start = b.cell_start;
     ra.perm = b.perm;
-    ra.spts = b.spts;
     ra.pts = (const double2 *)pts;
     ra.ch = ch;
     ra.npts = (int)N;
     ra.cell_work = ba.cell_work;
     ra.budget = ba.budget;
-    ra.resf = b.resf;       // cell-ordered results, every slot of a refined cell written
-    ra.resd = b.resd;
-    ra.out_id = out_id;     // FP32X recheck: final outputs through perm
-    ra.out_d = out_d;
+    ra.rec = reinterpret_cast<P2PRec *>(b.key_rank);   // every slot of a refined cell written
     ra.fb = b.fb;
     ra.n_fb = b.totals + 2;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -978,13 +961,8 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
         std::lock_guard<std::mutex> lk(L->ev_mu);
         L->ev_pending.emplace_back(ev0, ev1);
     }
-    // a8: results to input order; then the FP32X recheck overwrites the points
-    // it redoes in FP64, through perm
-    if (e == cudaSuccess) {
-        if (res == RES_F) e = launch_unsort_f(b.pos, b.resf, (int)N, out_id, out_d, s);
-        else e = launch_unsort_d(b.pos, b.resd, (int)N, out_id, out_d, s);
-    }
-    if (e == cudaSuccess && need_fb) e = launch_p2p_recheck(ra, di->sms * 4, s);
+    if (e == cudaSuccess) e = launch_p2p_recheck(ra, form, di->sms * 4, s);
+    if (e == cudaSuccess) e = launch_p2p_finish(ra, form, b.pos, (int)N, out_id, out_d, s);   // a8
     cudaError_t e2 = cudaFreeAsync(sc.base, s);
     if (e != cudaSuccess) return cuda_fail(e, "join launch");
     if (e2 != cudaSuccess) return cuda_fail(e2, "cudaFreeAsync");
@@ -1203,7 +1181,7 @@ namespace {
 constexpr int64_t NOALLOC_MAX_POINTS = SJ_NOALLOC_MAX_POINTS;
 constexpr int64_t NOALLOC_MAX_CELLS = SJ_NOALLOC_MAX_CELLS;
 constexpr int NOALLOC_CH = 64;
-constexpr size_t NOALLOC_BYTES = 32u << 20;   // holds carve() at the two limits above (about 31.6 MB)
+constexpr size_t NOALLOC_BYTES = 32u << 20;   // holds carve() at the two limits above (about 27 MB)
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
@@ -1258,13 +1236,12 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     if (N == 0) return SJ_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const int G = L->g.G;
-    const bool need_fb = form == SJ_FP32X;
     JoinBufs b;
-    size_t bytes = measure([&](Scratch &sc) { carve(sc, b, N, G, NOALLOC_CH, need_fb); });
+    size_t bytes = measure([&](Scratch &sc) { carve(sc, b, N, G, NOALLOC_CH, false); });
     if (bytes > NOALLOC_BYTES) return fail(SJ_ERR_INVALID, "sj_p2p_join_noalloc: scratch does not fit");
     Scratch sc;
     sc.base = base;
-    carve(sc, b, N, G, NOALLOC_CH, need_fb);
+    carve(sc, b, N, G, NOALLOC_CH, false);
     CUDA_TRY(cudaMemsetAsync(b.cnt, 0, sizeof(int) * ((size_t)G + 1), s));
     CUDA_TRY(cudaMemsetAsync(b.totals, 0, sizeof(int) * 4, s));
 
@@ -1276,7 +1253,6 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     ba.key_rank = b.key_rank;
     ba.cell_start = b.cell_start;
     ba.perm = b.perm;
-    ba.spts = b.spts;
     ba.cand_start = L->cand_start;
     ba.ch = NOALLOC_CH;
     ba.items = b.items;
@@ -1286,24 +1262,26 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     ba.out_id = out_id;
     ba.out_d = out_d;
     CUDA_TRY(launch_bucket(ba, s));
+    // slots of cells without candidates are not refined: no polyline
+    CUDA_TRY(cudaMemsetAsync(b.key_rank, 0xff, sizeof(int2) * (size_t)N, s));
 
     RefineArgs ra{};
-    fill_refine(L, ra);
+    fill_refine(L, form, ra);
     ra.items = b.items;
     ra.n_items = b.totals + 1;
     ra.cell_start = b.cell_start;
     ra.perm = b.perm;
-    ra.spts = b.spts;
+    ra.pts = (const double2 *)pts;
     ra.ch = NOALLOC_CH;
     ra.npts = (int)N;
-    ra.out_id = out_id;
-    ra.out_d = out_d;
+    ra.rec = reinterpret_cast<P2PRec *>(b.key_rank);
     ra.fb = b.fb;
     ra.n_fb = b.totals + 2;
     // items from the device counter, as in join_impl (totals[3], zeroed above)
     ra.work_next = b.totals + 3;
     ra.claim = (N >= 2LL * NOALLOC_CH * (long long)G) ? 2 : 1;
     CUDA_TRY(launch_p2p_refine(ra, form, 4, di->sms * di->p2p_bps[form], s));
-    if (need_fb) CUDA_TRY(launch_p2p_recheck(ra, di->sms * 4, s));
+    CUDA_TRY(launch_p2p_recheck(ra, form, di->sms * 4, s));
+    CUDA_TRY(launch_p2p_finish_slots(ra, form, b.totals, (int)N, out_id, out_d, s));
     return check_bounds(s);
 }

@@ -22,8 +22,6 @@
 #include "sj_host.hpp"
 
 namespace sj {
-cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
-cudaError_t launch_p2p_recheck(const RefineArgs &a, int blocks, cudaStream_t s);
 size_t bucket_scan_blocks(int G);
 
 namespace {
@@ -38,25 +36,14 @@ struct MultiArgs {
     const int *cell_start;
     int *perm;
     double2 *spts;
-    int *res_id;           // cell-ordered results (refinement writes the points of work items)
-    double *res_d;
+    P2PRec *rec;           // per slot (the refinement writes the points of work items)
     double *win;           // P2P: per-slot window, written when meta[2] != 0
 };
-
-// Request owning global point i: the last request whose offset is <= i.
-__device__ __forceinline__ int find_req(const RoundReq *r, int nr, int i) {
-    int lo = 0, hi = nr;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (r[mid].off <= i) lo = mid; else hi = mid;
-    }
-    return lo;
-}
 
 __global__ void k_cell_hist_multi(MultiArgs m) {
     const int nr = m.meta[0], total = m.meta[1];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const RoundReq &R = m.reqs[find_req(m.reqs, nr, i)];
+        const RoundReq &R = m.reqs[find_request(m.reqs, nr, i)];
         const double2 p = R.pts[i - R.off];
         const int c = point_cell(m.g, p.x, p.y);
         int r = 0;
@@ -65,38 +52,23 @@ __global__ void k_cell_hist_multi(MultiArgs m) {
     }
 }
 
-// Also initialises every in-grid slot's result to (-1, +inf): points of cells
-// without candidates belong to no work item and keep that result.
+// Also initialises every in-grid slot's record to "none": points of cells
+// without candidates belong to no work item and keep it.
 __global__ void k_scatter_multi(MultiArgs m) {
     const int nr = m.meta[0], total = m.meta[1];
     const bool pw = m.win && m.meta[2];
-    const double INF = __longlong_as_double(0x7ff0000000000000LL);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int2 k = m.key_rank[i];
         int q = -1;
         if (k.x < m.g.G) {
-            const RoundReq &R = m.reqs[find_req(m.reqs, nr, i)];
+            const RoundReq &R = m.reqs[find_request(m.reqs, nr, i)];
             q = m.cell_start[k.x] + k.y;
             m.perm[q] = i;
             m.spts[q] = R.pts[i - R.off];
-            m.res_id[q] = -1;
-            if (m.res_d) m.res_d[q] = INF;
+            m.rec[q] = P2PRec{-1, -1};
             if (pw) m.win[q] = R.window;
         }
         m.pos[i] = q;
-    }
-}
-
-// Every request's outputs in input order: a gather from the cell-ordered
-// results, coalesced writes.
-__global__ void k_unsort_multi(MultiArgs m) {
-    const int nr = m.meta[0], total = m.meta[1];
-    const double INF = __longlong_as_double(0x7ff0000000000000LL);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const RoundReq &R = m.reqs[find_req(m.reqs, nr, i)];
-        const int q = m.pos[i];
-        R.out_id[i - R.off] = q >= 0 ? m.res_id[q] : -1;
-        if (R.out_d) R.out_d[i - R.off] = (q >= 0 && m.res_d) ? m.res_d[q] : INF;
     }
 }
 
@@ -158,10 +130,11 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     const int64_t N = E->max_points;
     const int G = L->g.G;
     const bool p2p = L->kind == KIND_P2P;
-    int *cnt = nullptr, *cell_start = nullptr, *totals = nullptr, *pos = nullptr, *perm = nullptr, *res_id = nullptr;
+    int *cnt = nullptr, *cell_start = nullptr, *totals = nullptr, *pos = nullptr, *perm = nullptr;
     int2 *key_rank = nullptr, *items = nullptr, *block_sums = nullptr, *fb = nullptr;
     double2 *spts = nullptr;
-    double *res_d = nullptr, *win = nullptr;
+    double *win = nullptr;
+    P2PRec *rec = nullptr;
     auto lay = [&](Scratch &x) {
         w->d_reqs = x.take<RoundReq>((size_t)E->max_requests);
         w->d_meta = x.take<int>(4);
@@ -175,10 +148,9 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
         spts = x.take<double2>((size_t)N);
         items = x.take<int2>((size_t)(N / E->ch) + (size_t)std::min<int64_t>(G, N) + 1);
         block_sums = x.take<int2>(bucket_scan_blocks(G));
-        res_id = x.take<int>((size_t)N);
-        res_d = x.take<double>((size_t)N);
+        rec = x.take<P2PRec>((size_t)N);
         win = x.take<double>((size_t)N);
-        fb = E->form == SJ_FP32X ? x.take<int2>((size_t)N) : nullptr;
+        fb = x.take<int2>((size_t)N);
     };
     size_t bytes = measure(lay);
     CUDA_TRY(dev_malloc((void **)&w->base, bytes));
@@ -209,7 +181,7 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     ba.totals = totals;
 
     RefineArgs &ra = w->ra;
-    fill_refine(L, ra);
+    fill_refine(L, E->form, ra);
     ra.items = items;
     ra.n_items = totals + 1;
     ra.work_next = totals + 3;     // zeroed with the totals at the start of each round
@@ -218,8 +190,7 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     ra.spts = spts;
     ra.ch = E->ch;
     ra.npts = (int)E->max_points;   // slots and point indices of a round stay below it
-    ra.res_id = res_id;
-    ra.res_d = res_d;
+    ra.rec = rec;
     ra.fb = fb;
     ra.n_fb = totals + 2;
     ra.win = win;
@@ -235,8 +206,7 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     ma.cell_start = cell_start;
     ma.perm = perm;
     ma.spts = spts;
-    ma.res_id = res_id;
-    ma.res_d = res_d;
+    ma.rec = rec;
     ma.win = win;
     guard.w = nullptr;
     *out = w;
@@ -255,10 +225,10 @@ static cudaError_t enqueue_round(const sj_engine *E, const LayerWork *w, const D
     if ((e = launch_bucket_scan(w->ba, s)) != cudaSuccess) return e;
     k_scatter_multi<<<blocks, 256, 0, s>>>(w->ma);
     e = launch_p2p_refine(w->ra, E->form, 4, di->sms * di->p2p_bps[E->form], s);
-    if (e == cudaSuccess && E->form == SJ_FP32X) e = launch_p2p_recheck(w->ra, di->sms * 4, s);
-    if (e != cudaSuccess) return e;
-    k_unsort_multi<<<blocks, 256, 0, s>>>(w->ma);
-    return cudaGetLastError();
+    if (e == cudaSuccess) e = launch_p2p_recheck(w->ra, E->form, di->sms * 4, s);
+    if (e == cudaSuccess)
+        e = launch_p2p_finish_round(w->ra, E->form, w->d_reqs, w->d_meta, w->ma.pos, E->max_points, s);
+    return e;
 }
 
 extern "C" sj_status sj_engine_create(int64_t max_points, int32_t max_requests, const sj_opts *o, sj_engine **out) {

@@ -414,99 +414,6 @@ cudaError_t launch_bucket_scan(const BucketArgs &a, cudaStream_t s) {
                     a.g.G, a.block_sums, a.bs_cap, a.totals, s);
 }
 
-// Packed records: one gather per point.  FP32X distances widen exactly.
-template <typename R>
-__global__ void k_unsort_rec(const int *pos, const R *res, int n, int *out_id, double *out_d) {
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    const unsigned T = gridDim.x * blockDim.x;
-    for (unsigned i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < (unsigned)n; i0 += UNR * T) {
-        int j[UNR];
-        R r[UNR];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) j[u] = (i0 + u * T < (unsigned)n) ? pos[i0 + u * T] : -1;
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (j[u] >= 0 && !SJ_IN_BOUNDS(j[u] < n, BND_UNSORT)) j[u] = -1;
-            if (j[u] >= 0) r[u] = res[j[u]];
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const unsigned i = i0 + u * T;
-            if (i < (unsigned)n) {
-                out_id[i] = j[u] >= 0 ? r[u].id : -1;
-                if (out_d) out_d[i] = j[u] >= 0 ? (double)r[u].d : inf;
-            }
-        }
-    }
-}
-
-// The same with two consecutive points per thread and step: one 8-byte load of
-// their slots and 8- / 16-byte stores of their results, half the memory
-// instructions of the form above (whose load / store queue fills first).
-// out_id 8-byte and out_d 16-byte aligned.
-template <typename R>
-__global__ void k_unsort_rec2(const int *pos, const R *res, int n, int *out_id, double *out_d) {
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    const unsigned T = gridDim.x * blockDim.x;
-    const unsigned pairs = ((unsigned)n + 1u) / 2u;
-    for (unsigned p0 = blockIdx.x * blockDim.x + threadIdx.x; p0 < pairs; p0 += UNR * T) {
-        int2 j[UNR];
-        R r0[UNR], r1[UNR];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const unsigned p = p0 + u * T, i = 2u * p;
-            j[u] = make_int2(-1, -1);
-            if (p < pairs) {
-                if (i + 1u < (unsigned)n) j[u] = *reinterpret_cast<const int2 *>(pos + i);
-                else j[u].x = pos[i];
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (j[u].x >= 0 && !SJ_IN_BOUNDS(j[u].x < n, BND_UNSORT)) j[u].x = -1;
-            if (j[u].y >= 0 && !SJ_IN_BOUNDS(j[u].y < n, BND_UNSORT)) j[u].y = -1;
-            if (j[u].x >= 0) r0[u] = res[j[u].x];
-            if (j[u].y >= 0) r1[u] = res[j[u].y];
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const unsigned p = p0 + u * T, i = 2u * p;
-            if (p >= pairs) continue;
-            const int id0 = j[u].x >= 0 ? r0[u].id : -1, id1 = j[u].y >= 0 ? r1[u].id : -1;
-            const double d0 = j[u].x >= 0 ? (double)r0[u].d : inf, d1 = j[u].y >= 0 ? (double)r1[u].d : inf;
-            if (i + 1u < (unsigned)n) {
-                *reinterpret_cast<int2 *>(out_id + i) = make_int2(id0, id1);
-                if (out_d) *reinterpret_cast<double2 *>(out_d + i) = make_double2(d0, d1);
-            } else {
-                out_id[i] = id0;
-                if (out_d) out_d[i] = d0;
-            }
-        }
-    }
-}
-
-template <typename R>
-static cudaError_t launch_unsort_rec(const int *pos, const R *res, int n, int *out_id, double *out_d,
-                                     cudaStream_t s) {
-    const bool paired = ((uintptr_t)out_id & 7) == 0 && ((uintptr_t)out_d & 15) == 0;
-    if (paired) {
-        const int nb = stream_blocks(((n + 1) / 2 + UNR - 1) / UNR, 256, 152 * 16);
-        k_unsort_rec2<R><<<nb, 256, 0, s>>>(pos, res, n, out_id, out_d);
-    } else {
-        const int nb = stream_blocks((n + UNR - 1) / UNR, 256, 152 * 16);
-        k_unsort_rec<R><<<nb, 256, 0, s>>>(pos, res, n, out_id, out_d);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_unsort_f(const int *pos, const ResF *res, int n, int *out_id, double *out_d, cudaStream_t s) {
-    return launch_unsort_rec(pos, res, n, out_id, out_d, s);
-}
-
-cudaError_t launch_unsort_d(const int *pos, const ResD *res, int n, int *out_id, double *out_d, cudaStream_t s) {
-    return launch_unsort_rec(pos, res, n, out_id, out_d, s);
-}
-
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t s) {
     int nb = stream_blocks(a.n, 256, 152 * 32);
     if (a.sub_lx < 0 || a.sub_ly < 0 || a.sub_lx > 3 || a.sub_ly > 3 || ((a.sub_lx + a.sub_ly) && !a.sub_start) ||

@@ -254,16 +254,21 @@ __device__ __forceinline__ void flush_stats(unsigned long long *stats, const uns
     if (threadIdx.x < ST_N && blk[threadIdx.x]) atomicAdd(&stats[threadIdx.x], blk[threadIdx.x]);
 }
 
-// Cell-ordered P2P results of a per-request join, one record per slot so that
-// the final gather to input order reads one place per point.
-struct ResF {            // FP32X: id and the certified FP32 distance (+inf on a miss)
-    int id;
-    float d;
+// What the P2P refinement leaves in a slot, for the finishing kernels.
+//   FP32X: id >= 0: the polyline, aux = the bits of its certified FP32 distance;
+//          id < -1: the nearest segment is -2 - id (FP64 distance to be taken).
+//   FP64:  id >= 0: a segment, aux >= 0: a second one; the nearest is among them.
+//   id == -1: no polyline within the window.
+struct alignas(8) P2PRec {
+    int id, aux;
 };
-struct alignas(16) ResD {  // FP64
-    int id;
-    int pad;
-    double d;
+
+// Segment tables: the segment that starts at vertex i.
+struct SegArgs {
+    const double2 *verts;    // [V] FP64 vertices
+    const double2 *seg_e64;  // [V] b - a
+    const double *seg_inv64; // [V] 1 / |b - a|^2 (0 for a degenerate segment)
+    const float4 *seg32;     // [V] (fl32(ex), fl32(ey), fl32(1 / |e|^2), owner polyline id bits)
 };
 
 // Arguments of the P2P refinement kernels.
@@ -280,11 +285,8 @@ struct RefineArgs {
     const int *cand_start;   // [G + 1]
     const int *cand_ids;     // [M]
     const int *obj_voff;     // [nobj + 1] first vertex of each polyline
-    const double2 *verts;    // [V] FP64 vertices
-    const double2 *seg_e64;  // P2P: [V] b - a of the segment starting at vertex i
-    const double *seg_inv64; // P2P: [V] 1 / |b - a|^2 (0 for a degenerate segment)
-    const float4 *seg32;     // P2P: (fl32(ex), fl32(ey), fl32(1 / |e|^2), owner polyline id bits)
-    const int *cseg_start;   // P2P: [G + 1] per-cell segment lists
+    SegArgs seg;
+    const int *cseg_start;   // [G + 1] per-cell segment lists
     const int *cseg_ids;     //      segment (= first vertex) indices, ascending per cell
     const int *cell_algo;    //      [G] segments of the cell's candidate polylines
     const float4 *cseg_rec;  //      [2 MS] staging records of the list entries (see sj_filter.cu)
@@ -303,14 +305,8 @@ struct RefineArgs {
     int ch;                  // points per work item (at most; see cell_chunk)
     const int *cell_work;    // [G] per-point edge / segment work of each cell (or null)
     int budget;              // edge budget per point of an item (0: none)
-    int *out_id;
-    double *out_d;
-    int *res_id;             // when set: results in sorted order for every slot
-    double *res_d;           //   (hits and misses); out_id / perm unused
-    ResF *resf;              // FP32X: packed sorted results (instead of res_id / res_d);
-                             //   the FP64 recheck then writes out_id / out_d through perm
-    ResD *resd;              // FP64: packed sorted results
-    int2 *fb;                // FP32X: points to redo in FP64 (sorted slot, cell)
+    P2PRec *rec;             // [n] per slot
+    int2 *fb;                // points to redo in FP64 (sorted slot, cell)
     int *n_fb;
     unsigned long long *stats;
 };
@@ -319,10 +315,6 @@ struct RefineArgs {
 __device__ __forceinline__ double2 slot_point(const RefineArgs &a, int j) {
     return a.spts ? a.spts[j] : a.pts[a.perm[j]];
 }
-
-// Order key of a y-value with -0 folded onto +0 (IEEE compares treat them as
-// equal; the order key alone would not).
-__device__ __forceinline__ unsigned long long y_key(double v) { return order_key(v == 0.0 ? 0.0 : v); }
 
 // One request of a batched round as the kernels see it.
 struct RoundReq {
@@ -333,6 +325,20 @@ struct RoundReq {
     int off;         // first global point index
     int n;
 };
+
+// The request that holds global point i: the last one whose offset is <= i.
+__device__ __forceinline__ int find_request(const RoundReq *r, int nr, int i) {
+    int lo = 0, hi = nr;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (r[mid].off <= i) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// Order key of a y-value with -0 folded onto +0 (IEEE compares treat them as
+// equal; the order key alone would not).
+__device__ __forceinline__ unsigned long long y_key(double v) { return order_key(v == 0.0 ? 0.0 : v); }
 
 // Near-edge lists longer than PIP_SEARCH are searched by y instead of scanned
 // (with the sub-cell flag: longer than PIP_SEARCH_MIN).  A scan stops early, so
@@ -417,7 +423,13 @@ unsigned bounds_take_pip();
 
 // Host-side launchers (defined in the .cu files).
 cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
-cudaError_t launch_p2p_recheck(const RefineArgs &a, int blocks, cudaStream_t s);
+cudaError_t launch_p2p_recheck(const RefineArgs &a, int form, int blocks, cudaStream_t s);
+cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int n, int *out_id, double *out_d,
+                              cudaStream_t s);
+cudaError_t launch_p2p_finish_slots(const RefineArgs &a, int form, const int *in_grid, int n, int *out_id,
+                                    double *out_d, cudaStream_t s);
+cudaError_t launch_p2p_finish_round(const RefineArgs &a, int form, const RoundReq *reqs, const int *meta,
+                                    const int *pos, long long n_max, cudaStream_t s);
 cudaError_t launch_pip_census(const CensusArgs &a, const double2 *pts, int n, unsigned long long *out,
                               cudaStream_t s);
 
@@ -466,11 +478,6 @@ __device__ __forceinline__ int sub_index(int sx, int sy, int lx, int ly) {
 }
 size_t bucket_scan_blocks(int G);
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t s);
-// a8 for cell-ordered results: out[i] = res[pos[i]], or -1 / +inf where
-// pos[i] < 0 (one pass; out_d may be null).
-cudaError_t launch_unsort_f(const int *pos, const ResF *res, int n, int *out_id, double *out_d, cudaStream_t s);
-cudaError_t launch_unsort_d(const int *pos, const ResD *res, int n, int *out_id, double *out_d, cudaStream_t s);
-
 struct LayerBuildArgs {
     GridDev g;
     int kind;

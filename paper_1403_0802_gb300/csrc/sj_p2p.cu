@@ -13,36 +13,49 @@
 //   3. Staging: a segment whose bounding box is farther than D (plus a
 //      rounding slack) from the points' box cannot be within D of any point of
 //      the item and is dropped (exact: it cannot change any result); the others
-//      are compacted into shared memory (a, e = b - a, 1 / |e|^2, polyline id)
-//      with a ballot.
+//      are compacted into shared memory (a, e = b - a, 1 / |e|^2, a tag) with a
+//      ballot.
 //   4. Whenever the staging area fills, the warp splits its lanes into point
 //      groups of SG lanes (SG chosen so that np points x staged segments fill
-//      the warp); each lane strides over the staged segments keeping a running
-//      "top-2" -- the best (squared distance, polyline) and the best distance
-//      of any other polyline -- and the SG lanes of a group fold their top-2s
-//      with shuffles (the cross-lane min of the vertex-per-lane alternative of
-//      Sec. III.B); the fold is merged into the point's state in shared memory.
+//      the warp); each lane strides over the staged segments keeping the
+//      smallest squared distances of its point, and the SG lanes of a group fold
+//      theirs with shuffles (the cross-lane min of the vertex-per-lane
+//      alternative of Sec. III.B).  After the last segments the point's result is
+//      made from the fold at once, in registers; only a list that fills the
+//      staging area more than once keeps its points' state in shared memory in
+//      between.
 //
 // The point-to-segment distance is the two-case distance of Fig. 2 written as
 // the clamped projection: t = clamp(((p - a) . e) / |e|^2, 0, 1) and
 // d^2 = |p - a - t e|^2 (t = 0 or 1 gives the nearer end, 0 < t < 1 the
 // perpendicular foot; a zero-length segment has 1 / |e|^2 = 0, hence t = 0).
 //
-// Two arithmetic forms:
-//   FP64   -- the formula in FP64 (ties of equal squared distance go to the
-//             smaller id); agrees with the two-case FP64 evaluation to a few
-//             ulps of the coordinates' magnitude.
-//   FP32X  -- cell-relative FP32 coordinates from the (hi, lo) split of the FP64
-//             inputs; no FP64 instruction is executed.  Every (point, polyline)
-//             distance carries the bound E = 64 u M + 4 eps (u = 2^-24, M the
-//             largest |coordinate| of the point and of the item's staged
-//             segments).  A point is final only when its best polyline is ahead
-//             of the runner-up by more than 2E and its distance differs from D
-//             by more than E; otherwise it is queued and redone in FP64
-//             (k_p2p_recheck), so ids agree with FP64 up to exact ties.
+// Both forms test the segments in FP32 on cell-relative coordinates (from the
+// (hi, lo) split of the FP64 inputs): every distance carries the bound
+// E = 64 u M + 4 eps (u = 2^-24, M the largest |coordinate| of the point and of
+// the item's staged segments).
+//   FP32X  -- keeps the best polyline and the best distance of any other one
+//             (tag: polyline id).  A point is final only when its best polyline
+//             is ahead of the runner-up by more than 2E and its distance
+//             differs from D by more than E; the result is the FP32 distance.
+//   FP64   -- keeps the best two segments and the third-best distance (tag:
+//             segment).  A segment more than 2E behind the best cannot hold the
+//             smallest FP64 distance, so the FP64 formula is evaluated for the
+//             best one, for the second when it is within 2E (the two segments
+//             of a vertex), and the result is the smallest (d^2, id) of all
+//             segments in FP64 arithmetic, bit for bit.
+// A point that this does not settle (FP32X: not certified; FP64: three
+// segments within 2E) is queued and redone in FP64 over its cell's whole list
+// (k_p2p_recheck).  Either way the point's slot ends up with an 8-byte record
+// (P2PRec), from which k_p2p_finish* makes the outputs in input order.
+//
+// FP64 arithmetic runs at 1/64 of the FP32 rate (a warp instruction holds the
+// SM's FP64 pipe for 16 cycles), which is what the FP64 form is bound by: all
+// tests in FP64 took 3.33 ms for 3 M points on the 100,000 walks (106 M tests).
+// The one or two evaluations that a point needs are left to the finishing
+// kernel, whose warps are full of points: made at the end of each item, with
+// half of the lanes idle, they still took most of the refinement (0.43 ms).
 #include <cuda_runtime.h>
-
-#include <type_traits>
 
 #include "sj_internal.cuh"
 
@@ -52,45 +65,41 @@ unsigned bounds_take_p2p() { return bounds_take(); }
 
 constexpr int P2P_WARPS = 4;
 
-struct alignas(16) Seg64 {
-    double ax, ay, ex, ey;
-};
-
-template <bool FP32>
-struct P2PSmem;
-
-// FP32X staging holds segments in pairs (2k, 2k + 1), each quantity of the
+// Staging holds segments in pairs (2k, 2k + 1), each quantity of the
 // pair side by side, so that one lane evaluates both with the packed FP32
 // instructions (FADD2 / FMUL2 / FFMA2: two IEEE round-to-nearest operations
 // each, the same roundings as the scalar ones).  The stored values are
 // negated (-a, -e, -1 / |e|^2), which keeps every packed operation an add or
 // a fused multiply-add of the stored operands; the arithmetic is the clamped
 // projection below, operation for operation.
+template <bool F64>
+struct Best;
+// FP32X: smallest squared distance, its polyline, smallest of any other polyline.
 template <>
-struct P2PSmem<true> {
+struct Best<false> {
+    float b1, b2;
+    int i1;
+};
+// FP64: the two smallest with their segments, and the third.
+template <>
+struct Best<true> {
+    float b1, b2, b3;
+    int i1, i2;
+};
+
+template <bool F64>
+struct P2PSmem {
     static constexpr int SMAX = 128;   // even
     float4 sa[SMAX / 2];     // (-ax, -ax', -ay, -ay') cell-relative
     float4 se[SMAX / 2];     // (-ex, -ex', -ey, -ey')
-    float4 si[SMAX / 2];     // (-1 / |e|^2, -1 / |e'|^2, polyline id bits, id' bits)
+    float4 si[SMAX / 2];     // (-1 / |e|^2, -1 / |e'|^2, tag, tag')
     float2 pt[MAX_CH];
-    float b1[MAX_CH], b2[MAX_CH];
-    int i1[MAX_CH];
-};
-
-template <>
-struct P2PSmem<false> {
-    static constexpr int SMAX = 128;
-    Seg64 seg[SMAX];
-    double inv[SMAX];
-    int sid[SMAX];
-    double2 pt[MAX_CH];
-    double b1[MAX_CH], b2[MAX_CH];
-    int i1[MAX_CH];
+    Best<F64> st[MAX_CH];    // used between the parts of a list longer than SMAX
 };
 
 // Squared distance from p to the segment (a, a + e) by the clamped projection:
 // d = p - a, t = clamp((e . d) / |e|^2, 0, 1), |d - t e|^2, each operation
-// rounded once (FP64 here; the FP32X loop in p2p_compute evaluates the same
+// rounded once (FP64 here; the loop in p2p_compute evaluates the same
 // operations in FP32 on segment pairs).
 __device__ __forceinline__ double seg_d2(double px, double py, double ax, double ay, double ex, double ey,
                                          double inv) {
@@ -101,59 +110,75 @@ __device__ __forceinline__ double seg_d2(double px, double py, double ax, double
     return __fma_rn(qx, qx, __dmul_rn(qy, qy));
 }
 
-// Running result of one point over a set of segments: b1 = smallest squared
-// distance, i1 = its polyline, b2 = smallest squared distance of any segment of
-// another polyline (FP32X certificate; unused in FP64).
-template <typename T>
-struct Best {
-    T b1, b2;
-    int i1;
+__device__ __forceinline__ Best<false> best_none(Best<false> *) {
+    const float INF = __int_as_float(0x7f800000);
+    return Best<false>{INF, INF, -1};
+}
+__device__ __forceinline__ Best<true> best_none(Best<true> *) {
+    const float INF = __int_as_float(0x7f800000);
+    return Best<true>{INF, INF, INF, -1, -1};
+}
+
+// A further segment at squared distance d with tag l.
+__device__ __forceinline__ void consider(Best<false> &s, float d, int l) {
+    // b1 <= b2 always; the runner-up becomes max(d, b1) when l is another
+    // polyline (whichever of the old best and d is not the new best).
+    const bool lt = d < s.b1;
+    const float nb2 = (l == s.i1) ? s.b2 : fminf(s.b2, fmaxf(d, s.b1));
+    s.b1 = fminf(s.b1, d);
+    s.i1 = lt ? l : s.i1;
+    s.b2 = nb2;
+}
+__device__ __forceinline__ void consider(Best<true> &s, float d, int l) {
+    const bool lt1 = d < s.b1, lt2 = d < s.b2;
+    s.b3 = fminf(s.b3, fmaxf(d, s.b2));
+    s.b2 = fminf(s.b2, fmaxf(d, s.b1));
+    s.b1 = fminf(s.b1, d);
+    s.i2 = lt1 ? s.i1 : (lt2 ? l : s.i2);
+    s.i1 = lt1 ? l : s.i1;
+}
+
+// Result over the union of two disjoint segment sets (commutative and associative).
+__device__ __forceinline__ Best<false> merge(Best<false> A, Best<false> B) {
+    Best<false> r;
+    if (A.i1 == B.i1) {
+        r.b1 = fminf(A.b1, B.b1); r.i1 = A.i1; r.b2 = fminf(A.b2, B.b2);
+    } else if (B.b1 < A.b1 || (B.b1 == A.b1 && B.i1 < A.i1)) {
+        r.b1 = B.b1; r.i1 = B.i1; r.b2 = fminf(B.b2, A.b1);
+    } else {
+        r.b1 = A.b1; r.i1 = A.i1; r.b2 = fminf(A.b2, B.b1);
+    }
+    return r;
+}
+__device__ __forceinline__ Best<true> merge(Best<true> A, Best<true> B) {
+    consider(A, B.b1, B.i1);
+    consider(A, B.b2, B.i2);
+    A.b3 = fminf(A.b3, B.b3);
+    return A;
+}
+__device__ __forceinline__ Best<false> shfl_best(const Best<false> &s, int o) {
+    return Best<false>{__shfl_xor_sync(FULL, s.b1, o), __shfl_xor_sync(FULL, s.b2, o), __shfl_xor_sync(FULL, s.i1, o)};
+}
+__device__ __forceinline__ Best<true> shfl_best(const Best<true> &s, int o) {
+    return Best<true>{__shfl_xor_sync(FULL, s.b1, o), __shfl_xor_sync(FULL, s.b2, o), __shfl_xor_sync(FULL, s.b3, o),
+                      __shfl_xor_sync(FULL, s.i1, o), __shfl_xor_sync(FULL, s.i2, o)};
+}
+
+// FP64 result of one point over some segments: the smallest (squared distance,
+// polyline id), and a segment that has it.
+struct Best64 {
+    double d2;
+    int id, seg;
 };
-
-template <bool FP32, typename T>
-__device__ __forceinline__ void consider(Best<T> &s, T d, int l) {
-    if constexpr (FP32) {
-        // b1 <= b2 always; the runner-up becomes max(d, b1) when l is another
-        // polyline (whichever of the old best and d is not the new best).
-        const bool lt = d < s.b1;
-        const T nb2 = (l == s.i1) ? s.b2 : fminf(s.b2, fmaxf(d, s.b1));
-        s.b1 = fminf(s.b1, d);
-        s.i1 = lt ? l : s.i1;
-        s.b2 = nb2;
-    } else {
-        if (d < s.b1 || (d == s.b1 && l < s.i1)) {
-            s.b1 = d;
-            s.i1 = l;
-        }
-    }
+__device__ __forceinline__ void consider64(Best64 &s, double d2, int id, int seg) {
+    if (d2 < s.d2 || (d2 == s.d2 && id < s.id)) s = Best64{d2, id, seg};
 }
-
-// Result over the union of two segment sets (commutative and associative).
-template <bool FP32, typename T>
-__device__ __forceinline__ Best<T> merge(Best<T> A, Best<T> B) {
-    Best<T> r;
-    if constexpr (FP32) {
-        if (A.i1 == B.i1) {
-            r.b1 = fminf(A.b1, B.b1); r.i1 = A.i1; r.b2 = fminf(A.b2, B.b2);
-        } else if (B.b1 < A.b1 || (B.b1 == A.b1 && B.i1 < A.i1)) {
-            r.b1 = B.b1; r.i1 = B.i1; r.b2 = fminf(B.b2, A.b1);
-        } else {
-            r.b1 = A.b1; r.i1 = A.i1; r.b2 = fminf(A.b2, B.b1);
-        }
-    } else {
-        r = (B.b1 < A.b1 || (B.b1 == A.b1 && B.i1 < A.i1)) ? B : A;
-    }
-    return r;
+// Squared distance from p to segment i, FP64.
+__device__ __forceinline__ double seg_d2(const SegArgs &a, double2 p, int i) {
+    const double2 v = a.verts[i], e = a.seg_e64[i];
+    return seg_d2(p.x, p.y, v.x, v.y, e.x, e.y, a.seg_inv64[i]);
 }
-
-template <bool FP32, typename T>
-__device__ __forceinline__ Best<T> shfl_best(const Best<T> &s, int o) {
-    Best<T> r;
-    r.b1 = __shfl_xor_sync(FULL, s.b1, o);
-    r.i1 = __shfl_xor_sync(FULL, s.i1, o);
-    r.b2 = FP32 ? __shfl_xor_sync(FULL, s.b2, o) : s.b2;
-    return r;
-}
+__device__ __forceinline__ int seg_owner(const SegArgs &a, int i) { return __float_as_int(a.seg32[i].w); }
 
 // A window w in FP32, rounded down / up with the same 1e-12 relative margin
 // the layer's D gets on the host (explicit roundings, no contraction).
@@ -173,15 +198,58 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k ^ ((
 __device__ __forceinline__ float warp_min(float v) { return key_float(__reduce_min_sync(FULL, float_key(v))); }
 __device__ __forceinline__ float warp_max(float v) { return key_float(__reduce_max_sync(FULL, float_key(v))); }
 
-// Refine the staged segments [0, ns) for the item's np points (FP32X: ns
-// counts segment pairs).  Rounds of 32
+// What one point's result needs besides its fold.
+struct P2PItem {
+    int j0, c;      // first slot of the item, cell
+    float mag;      // largest |cell-relative coordinate| of the points and staged segments
+};
+
+// The record of slot j (point pt, cell-relative) from its complete fold; a
+// point that it does not settle is queued for the FP64 recheck.
+template <bool F64, bool PW>
+__device__ __forceinline__ void p2p_result(const RefineArgs &a, const P2PItem &it, int j, float2 pt, const Best<F64> &st,
+                                           bool pw, unsigned &c_fb, unsigned &c_hits) {
+    const float d = sqrtf(st.b1), d2 = sqrtf(st.b2);
+    const float e = fmaf(64.0f * U32, fmaxf(it.mag, fmaxf(fabsf(pt.x), fabsf(pt.y))), 4.0f * a.eps_abs) *
+                    (1.0f + 8.0f * U32);
+    const float sep = 2.0f * e * (1.0f + 4.0f * U32);
+    float Ddn = a.Ddn, Dup = a.Dup;
+    if (PW && pw) window_f32(a.win[j], Ddn, Dup);
+    P2PRec r{-1, -1};
+    bool redo = false;
+    // F64, e infinite: coordinates beyond the range of the bound (every point is redone)
+    if (F64 && !(e < __int_as_float(0x7f800000))) {
+        redo = true;
+    } else if (st.i1 >= 0 && !((d - e) * (1.0f - 4.0f * U32) > Dup)) {   // not certainly outside the window
+        const bool alone = (d2 - d) * (1.0f - 4.0f * U32) > sep;         // no other one within 2E
+        if constexpr (F64) {
+            redo = !((sqrtf(st.b3) - d) * (1.0f - 4.0f * U32) > sep);
+            r = P2PRec{st.i1, alone ? -1 : st.i2};
+        } else {
+            const bool in_window = (d + e) * (1.0f + 4.0f * U32) < Ddn;
+            redo = !(in_window && alone);
+            r = P2PRec{st.i1, __float_as_int(d)};
+        }
+    }
+    if (redo) {
+        const int slot = atomicAdd(a.n_fb, 1);
+        a.fb[slot] = make_int2(j, it.c);
+        ++c_fb;
+    } else if (SJ_IN_BOUNDS(j < a.npts, BND_P2P_RES)) {
+        a.rec[j] = r;
+        if (!F64) c_hits += r.id >= 0;
+    }
+}
+
+// Refine the staged segment pairs [0, ns) for the item's np points.  Rounds of 32
 // points take one lane per point (every lane busy, no merge); the last round,
 // of fewer than 32 points, splits each point's segments over a group of sg
 // lanes chosen by the cost model (more lanes per point, log2(sg) merges).
-template <bool FP32>
-__device__ __forceinline__ void p2p_compute(P2PSmem<FP32> &s, int np, int ns, int lane) {
-    using T = typename std::conditional<FP32, float, double>::type;
-    const T INF = (T)__longlong_as_double(0x7ff0000000000000LL);
+// first / last: the list's first / last part.
+template <bool F64, bool PW>
+__device__ __forceinline__ void p2p_compute(const RefineArgs &a, P2PSmem<F64> &s, const P2PItem &it, int np, int ns,
+                                            int lane, bool first, bool last, bool pw, unsigned &c_fb,
+                                            unsigned &c_hits) {
     int pg = 32;
     for (int q0 = 0; q0 < np; q0 += pg) {
         const int rem = np - q0;
@@ -190,45 +258,36 @@ __device__ __forceinline__ void p2p_compute(P2PSmem<FP32> &s, int np, int ns, in
         pg = 32 >> lg;
         const int sub = lane & (sg - 1), grp = lane >> lg;
         const int q = q0 + grp;
-        Best<T> st{INF, INF, -1};
+        Best<F64> st = best_none((Best<F64> *)nullptr);
+        float2 p = make_float2(0.0f, 0.0f);
         if (q < np) {
-            if constexpr (FP32) {
-                // the squared distances of the pair by the clamped projection
-                // in FP32: dx = px - ax, t = sat(fma(ex, dx, ey * dy) / |e|^2),
-                // q = fma(-t, e, d), |q|^2 = fma(qx, qx, qy * qy), written with
-                // the negated operands (p + (-a) = p - a, fma(-ex, dx, -ey * dy)
-                // * (-1 / |e|^2) = (e . d) / |e|^2, fma(t, -e, d) = d - t e:
-                // each rounding the same as the unnegated one)
-                const float2 p = s.pt[q];
-                const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y);
+            // the squared distances of the pair by the clamped projection
+            // in FP32: dx = px - ax, t = sat(fma(ex, dx, ey * dy) / |e|^2),
+            // q = fma(-t, e, d), |q|^2 = fma(qx, qx, qy * qy), written with
+            // the negated operands (p + (-a) = p - a, fma(-ex, dx, -ey * dy)
+            // * (-1 / |e|^2) = (e . d) / |e|^2, fma(t, -e, d) = d - t e:
+            // each rounding the same as the unnegated one)
+            p = s.pt[q];
+            const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y);
 #pragma unroll 1
-                for (int t = sub; t < ns; t += sg) {
-                    const float4 A = s.sa[t], E = s.se[t], I = s.si[t];
-                    const float2 nex = make_float2(E.x, E.y), ney = make_float2(E.z, E.w);
-                    const float2 dx = __fadd2_rn(px, make_float2(A.x, A.y));
-                    const float2 dy = __fadd2_rn(py, make_float2(A.z, A.w));
-                    const float2 w = __ffma2_rn(nex, dx, __fmul2_rn(ney, dy));
-                    const float2 tt = make_float2(__saturatef(__fmul_rn(w.x, I.x)), __saturatef(__fmul_rn(w.y, I.y)));
-                    const float2 qx = __ffma2_rn(tt, nex, dx), qy = __ffma2_rn(tt, ney, dy);
-                    const float2 d = __ffma2_rn(qx, qx, __fmul2_rn(qy, qy));
-                    consider<true>(st, d.x, __float_as_int(I.z));
-                    consider<true>(st, d.y, __float_as_int(I.w));
-                }
-            } else {
-                const double2 p = s.pt[q];
-                for (int t = sub; t < ns; t += sg) {
-                    const Seg64 g = s.seg[t];
-                    consider<false>(st, seg_d2(p.x, p.y, g.ax, g.ay, g.ex, g.ey, s.inv[t]), s.sid[t]);
-                }
+            for (int t = sub; t < ns; t += sg) {
+                const float4 A = s.sa[t], E = s.se[t], I = s.si[t];
+                const float2 nex = make_float2(E.x, E.y), ney = make_float2(E.z, E.w);
+                const float2 dx = __fadd2_rn(px, make_float2(A.x, A.y));
+                const float2 dy = __fadd2_rn(py, make_float2(A.z, A.w));
+                const float2 w = __ffma2_rn(nex, dx, __fmul2_rn(ney, dy));
+                const float2 tt = make_float2(__saturatef(__fmul_rn(w.x, I.x)), __saturatef(__fmul_rn(w.y, I.y)));
+                const float2 qx = __ffma2_rn(tt, nex, dx), qy = __ffma2_rn(tt, ney, dy);
+                const float2 d = __ffma2_rn(qx, qx, __fmul2_rn(qy, qy));
+                consider(st, d.x, __float_as_int(I.z));
+                consider(st, d.y, __float_as_int(I.w));
             }
         }
-        for (int o = sg >> 1; o > 0; o >>= 1) st = merge<FP32>(st, shfl_best<FP32>(st, o));
+        for (int o = sg >> 1; o > 0; o >>= 1) st = merge(st, shfl_best(st, o));
         if (sub == 0 && q < np) {
-            Best<T> cur{s.b1[q], s.b2[q], s.i1[q]};
-            cur = merge<FP32>(cur, st);
-            s.b1[q] = cur.b1;
-            s.b2[q] = cur.b2;
-            s.i1[q] = cur.i1;
+            if (!first) st = merge(s.st[q], st);
+            if (last) p2p_result<F64, PW>(a, it, it.j0 + q, p, st, pw, c_fb, c_hits);
+            else s.st[q] = st;
         }
     }
 }
@@ -237,15 +296,13 @@ __device__ __forceinline__ void p2p_compute(P2PSmem<FP32> &s, int np, int ns, in
 // PW = false, whose code has no window load at all.  Eight blocks per SM is
 // the shared-memory limit already; saying so keeps the register allocator at
 // 64 registers without spills.
-template <bool FP32, bool PW, int NW>
+template <bool F64, bool PW, int NW>
 __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
-    using T = typename std::conditional<FP32, float, double>::type;
-    constexpr int SMAX = P2PSmem<FP32>::SMAX;
+    constexpr int SMAX = P2PSmem<F64>::SMAX;
     extern __shared__ __align__(16) unsigned char p2p_smem_raw[];
     const int lane = lane_id(), w = threadIdx.x >> 5;
-    P2PSmem<FP32> &s = reinterpret_cast<P2PSmem<FP32> *>(p2p_smem_raw)[w];
+    P2PSmem<F64> &s = reinterpret_cast<P2PSmem<F64> *>(p2p_smem_raw)[w];
     const int n_items = *a.n_items;
-    const T INF = (T)__longlong_as_double(0x7ff0000000000000LL);
     const float FINF = __int_as_float(0x7f800000);
     const unsigned lt_mask = (1u << lane) - 1u;
     unsigned long long c_pairs = 0, c_tests = 0, c_items = 0, c_algo = 0;
@@ -296,14 +353,8 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         // (idle) staging area -- so that their latencies overlap instead of
         // forming one chain per point.
         constexpr int PQ = MAX_CH / 32;
-        double2 *pbuf;
-        if constexpr (FP32) {
-            static_assert(sizeof(P2PSmem<true>::sa) + sizeof(P2PSmem<true>::se) >= MAX_CH * sizeof(double2), "");
-            pbuf = reinterpret_cast<double2 *>(&s.sa[0]);   // sa and se, contiguous
-        } else {
-            static_assert(sizeof(P2PSmem<false>::seg) >= MAX_CH * sizeof(double2), "");
-            pbuf = reinterpret_cast<double2 *>(&s.seg[0]);
-        }
+        static_assert(sizeof(P2PSmem<F64>::sa) + sizeof(P2PSmem<F64>::se) >= MAX_CH * sizeof(double2), "");
+        double2 *pbuf = reinterpret_cast<double2 *>(&s.sa[0]);   // sa and se, contiguous
         {
             int src[PQ];
 #pragma unroll
@@ -324,11 +375,7 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
             split_double(p.x, hx, lx);
             split_double(p.y, hy, ly);
             const float rx = rel_coord(hx, lx, fo.x), ry = rel_coord(hy, ly, fo.y);
-            if constexpr (FP32) s.pt[q] = make_float2(rx, ry);
-            else s.pt[q] = p;
-            s.b1[q] = INF;
-            s.b2[q] = INF;
-            s.i1[q] = -1;
+            s.pt[q] = make_float2(rx, ry);
             bxlo = fminf(bxlo, rx); bxhi = fmaxf(bxhi, rx);
             bylo = fminf(bylo, ry); byhi = fmaxf(byhi, ry);
         }
@@ -341,7 +388,7 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         const int end_next = in_claim ? it_end : it_next + (a.work_next ? claim : 1);
         int2 item_n = make_int2(0, 0);
         if (it_next < n_items) item_n = a.items[it_next];
-        float mag = pmag;   // FP32X: largest |cell-relative coordinate| refined for this item
+        float mag = pmag;   // largest |cell-relative coordinate| refined for this item
         c_pairs += (unsigned long long)np * (unsigned long long)(k1 - k0);
         c_algo += (unsigned long long)np * (unsigned long long)a.cell_algo[c];
 
@@ -349,10 +396,12 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         // 3. staging with the exact distance prune, 4. refinement when full
         const int g0 = a.cseg_start[c], g1 = a.cseg_start[c + 1];
         int nst = 0;
-        for (int base = g0; base < g1; base += 32) {
+        bool first = true;
+        int base = g0;
+        do {
             const int g = base + lane;
             bool keep = false;
-            int i = 0, sid = 0;
+            int tag = 0;
             float ax = 0.0f, ay = 0.0f, ex = 0.0f, ey = 0.0f, inv = 0.0f, smag = 0.0f;
             if (g < g1 && SJ_IN_BOUNDS(g < a.cseg_start[a.g.G], BND_P2P_REC)) {
                 const float4 r0 = a.cseg_rec[2 * (size_t)g], r1 = a.cseg_rec[2 * (size_t)g + 1];
@@ -361,9 +410,8 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
                 ex = r0.z;
                 ey = r0.w;
                 inv = r1.x;
-                sid = __float_as_int(r1.y);
+                tag = __float_as_int(F64 ? r1.w : r1.y);   // segment or polyline
                 smag = r1.z;
-                i = __float_as_int(r1.w);
                 const float bx = ax + ex, by = ay + ey;
                 const float gx = fmaxf(0.0f, fmaxf(fminf(ax, bx) - bxhi, bxlo - fmaxf(ax, bx)));
                 const float gy = fmaxf(0.0f, fmaxf(fminf(ay, by) - byhi, bylo - fmaxf(ay, by)));
@@ -374,101 +422,44 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
             const unsigned bal = __ballot_sync(FULL, keep);
             if (keep) {
                 const int pos = nst + __popc(bal & lt_mask);
-                if constexpr (FP32) {
-                    const int k = pos >> 1, h = pos & 1;
-                    float *A = reinterpret_cast<float *>(&s.sa[k]);
-                    float *E = reinterpret_cast<float *>(&s.se[k]);
-                    float *I = reinterpret_cast<float *>(&s.si[k]);
-                    A[h] = -ax; A[2 + h] = -ay;
-                    E[h] = -ex; E[2 + h] = -ey;
-                    I[h] = -inv; I[2 + h] = __int_as_float(sid);
-                    mag = fmaxf(mag, smag);
-                } else {
-                    const double2 v = a.verts[i], e = a.seg_e64[i];
-                    s.seg[pos] = Seg64{v.x, v.y, e.x, e.y};
-                    s.inv[pos] = a.seg_inv64[i];
-                    s.sid[pos] = sid;
-                }
+                const int k = pos >> 1, h = pos & 1;
+                float *A = reinterpret_cast<float *>(&s.sa[k]);
+                float *E = reinterpret_cast<float *>(&s.se[k]);
+                float *I = reinterpret_cast<float *>(&s.si[k]);
+                A[h] = -ax; A[2 + h] = -ay;
+                E[h] = -ex; E[2 + h] = -ey;
+                I[h] = -inv; I[2 + h] = __int_as_float(tag);
+                mag = fmaxf(mag, smag);
             }
             nst += __popc(bal);
-            if (nst > SMAX - 32 || base + 32 >= g1) {
-                if constexpr (FP32) {
-                    // an odd count: the pair's second slot gets a segment at
-                    // infinite distance (a far point, zero length), which never
-                    // changes a point's top-2
-                    if ((nst & 1) && lane == 0) {
-                        const int k = nst >> 1;
-                        reinterpret_cast<float *>(&s.sa[k])[1] = -3.0e38f;
-                        reinterpret_cast<float *>(&s.sa[k])[3] = -3.0e38f;
-                        reinterpret_cast<float *>(&s.se[k])[1] = 0.0f;
-                        reinterpret_cast<float *>(&s.se[k])[3] = 0.0f;
-                        reinterpret_cast<float *>(&s.si[k])[1] = 0.0f;
-                        reinterpret_cast<float *>(&s.si[k])[3] = __int_as_float(-2);
-                    }
+            base += 32;
+            const bool last = base >= g1;
+            if (nst > SMAX - 32 || last) {
+                // an odd count: the pair's second slot gets a segment at
+                // infinite distance (a far point, zero length), which never
+                // changes a point's fold
+                if ((nst & 1) && lane == 0) {
+                    const int k = nst >> 1;
+                    reinterpret_cast<float *>(&s.sa[k])[1] = -3.0e38f;
+                    reinterpret_cast<float *>(&s.sa[k])[3] = -3.0e38f;
+                    reinterpret_cast<float *>(&s.se[k])[1] = 0.0f;
+                    reinterpret_cast<float *>(&s.se[k])[3] = 0.0f;
+                    reinterpret_cast<float *>(&s.si[k])[1] = 0.0f;
+                    reinterpret_cast<float *>(&s.si[k])[3] = __int_as_float(-2);
                 }
                 __syncwarp();
-                if (nst > 0) {
-                    p2p_compute<FP32>(s, np, FP32 ? (nst + 1) >> 1 : nst, lane);
-                    c_tests += (unsigned long long)np * (unsigned long long)nst;
-                }
+                mag = warp_max(mag);
+                p2p_compute<F64, PW>(a, s, P2PItem{j0, c, mag}, np, (nst + 1) >> 1, lane, first, last, pw, c_fb, c_hits);
+                c_tests += (unsigned long long)np * (unsigned long long)nst;
                 __syncwarp();
                 nst = 0;
+                first = false;
             }
-        }
+        } while (base < g1);
         int cs0n = 0, cs1n = 0;
         if (it_next < n_items) {
             cs0n = a.cell_start[item_n.x];
             cs1n = a.cell_start[item_n.x + 1];
-        }
-        if constexpr (FP32) mag = warp_max(mag);
-        for (int q = lane; q < np; q += 32) {
-            const int id = s.i1[q];
-            int out = -1;
-            double dd = __longlong_as_double(0x7ff0000000000000LL);
-            float df = FINF;
-            if (id >= 0) {
-                if constexpr (FP32) {
-                    const float d = sqrtf(s.b1[q]), d2 = sqrtf(s.b2[q]);
-                    const float2 p = s.pt[q];
-                    const float e = fmaf(64.0f * U32, fmaxf(mag, fmaxf(fabsf(p.x), fabsf(p.y))), 4.0f * a.eps_abs) *
-                                    (1.0f + 8.0f * U32);
-                    float Ddn = a.Ddn, Dup = a.Dup;
-                    if (pw) window_f32(a.win[j0 + q], Ddn, Dup);
-                    if (!((d - e) * (1.0f - 4.0f * U32) > Dup)) {                    // not certainly outside D
-                        const bool in_window = (d + e) * (1.0f + 4.0f * U32) < Ddn;
-                        const bool separated = (d2 - d) * (1.0f - 4.0f * U32) > 2.0f * e * (1.0f + 4.0f * U32);
-                        if (!(in_window && separated)) {                              // redo in FP64
-                            const int slot = atomicAdd(a.n_fb, 1);
-                            a.fb[slot] = make_int2(j0 + q, c);
-                            ++c_fb;
-                            continue;
-                        }
-                        out = id;
-                        dd = widen(d);
-                        df = d;
-                    }
-                } else {
-                    const double d = sqrt(s.b1[q]);
-                    if (d <= (pw ? a.win[j0 + q] : a.D)) {
-                        out = id;
-                        dd = d;
-                    }
-                }
-            }
-            if (!SJ_IN_BOUNDS(j0 + q < a.npts, BND_P2P_RES)) continue;
-            if (a.resf) {
-                a.resf[j0 + q] = ResF{out, df};
-            } else if (a.resd) {
-                a.resd[j0 + q] = ResD{out, 0, dd};
-            } else if (a.res_id) {
-                a.res_id[j0 + q] = out;
-                if (a.res_d) a.res_d[j0 + q] = dd;
-            } else if (out >= 0) {
-                const int i = a.perm[j0 + q];
-                a.out_id[i] = out;
-                if (a.out_d) a.out_d[i] = dd;
-            }
-            if (out >= 0) ++c_hits;
         }
         __syncwarp();
         it = it_next;
@@ -489,9 +480,11 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
     }
 }
 
-// FP64 recomputation of the points the FP32X pass could not certify: one warp
+// FP64 recomputation of the points the FP32 pass did not settle: one warp
 // per point, lanes over the cell's segment list, each lane keeping the
-// smallest (squared distance, polyline id), then a warp fold.
+// smallest (squared distance, polyline id), then a warp fold.  The record is
+// left as the segment found, for the finishing kernel.
+template <bool F64>
 __global__ void __launch_bounds__(256) k_p2p_recheck(RefineArgs a) {
     const int lane = lane_id();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -504,63 +497,312 @@ __global__ void __launch_bounds__(256) k_p2p_recheck(RefineArgs a) {
         const int2 e = a.fb[f];
         const int j = e.x, c = e.y;
         const double2 p = slot_point(a, j);
-        Best<double> st{INF, INF, -1};
+        Best64 st{INF, 0x7fffffff, -1};
         for (int g = a.cseg_start[c] + lane; g < a.cseg_start[c + 1]; g += 32) {
             const int i = a.cseg_ids[g];
-            const double2 v = a.verts[i], ev = a.seg_e64[i];
-            consider<false>(st, seg_d2(p.x, p.y, v.x, v.y, ev.x, ev.y, a.seg_inv64[i]), __float_as_int(a.seg32[i].w));
+            consider64(st, seg_d2(a.seg, p, i), seg_owner(a.seg, i), i);
         }
-        for (int o = 16; o > 0; o >>= 1) st = merge<false>(st, shfl_best<false>(st, o));
-        const double best = sqrt(st.b1);
-        const bool hit = st.i1 >= 0 && best <= (pw ? a.win[j] : a.D);
+        for (int o = 16; o > 0; o >>= 1)
+            consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
+                       __shfl_xor_sync(FULL, st.seg, o));
+        const bool hit = st.seg >= 0 && sqrt(st.d2) <= (pw ? a.win[j] : a.D);
         if (lane == 0) {
-            if (a.res_id) {
-                a.res_id[j] = hit ? st.i1 : -1;
-                if (a.res_d) a.res_d[j] = hit ? best : INF;
-            } else {   // final outputs through perm (hits and misses)
-                const int i = a.perm[j];
-                a.out_id[i] = hit ? st.i1 : -1;
-                if (a.out_d) a.out_d[i] = hit ? best : INF;
-            }
+            a.rec[j] = !hit ? P2PRec{-1, -1} : (F64 ? P2PRec{st.seg, -1} : P2PRec{-2 - st.seg, 0});
             if (hit) ++c_hits;
         }
     }
-    if (a.stats) {
+    if (!F64 && a.stats) {   // F64: the finishing kernel counts the hits
         c_hits = __reduce_add_sync(FULL, c_hits);
         if (lane == 0 && c_hits) atomicAdd(&a.stats[ST_HITS], (unsigned long long)c_hits);
     }
 }
 
-template <bool FP32, int NW>
-static size_t p2p_smem_bytes() {
-    return sizeof(P2PSmem<FP32>) * NW;
+// ------------------------------------------------------------------ outputs in input order
+
+// FP32X: out[i] from the record of i's slot (pos[i], -1: no slot): the id and
+// the FP32 distance, widened exactly, or the FP64 distance to the segment that
+// the recheck found.
+__device__ __forceinline__ void fp32x_output(const SegArgs &a, const P2PRec r, double2 p, int &id, double &d) {
+    id = r.id;
+    d = r.id >= 0 ? widen(__int_as_float(r.aux)) : __longlong_as_double(0x7ff0000000000000LL);
+    if (r.id < -1) {
+        id = seg_owner(a, -2 - r.id);
+        d = sqrt(seg_d2(a, p, -2 - r.id));
+    }
 }
 
-template <bool FP32, bool PW, int NW>
+constexpr int FIN_U = 4;
+
+// One request, two consecutive points per thread and step (one 8-byte load of
+// their slots, 8- and 16-byte stores): half the memory instructions of one
+// point at a time, whose load / store queue fills first.  out_id 8-byte and
+// out_d 16-byte aligned, n even or odd.
+__global__ void k_p2p_finish_pairs(SegArgs a, const int *pos, const P2PRec *rec, const double2 *pts, int n, int *out_id,
+                                   double *out_d) {
+    const unsigned T = gridDim.x * blockDim.x;
+    const unsigned pairs = ((unsigned)n + 1u) / 2u;
+    for (unsigned p0 = blockIdx.x * blockDim.x + threadIdx.x; p0 < pairs; p0 += FIN_U * T) {
+        int2 j[FIN_U];
+        P2PRec r0[FIN_U], r1[FIN_U];
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            const unsigned p = p0 + u * T, i = 2u * p;
+            j[u] = make_int2(-1, -1);
+            if (p < pairs) {
+                if (i + 1u < (unsigned)n) j[u] = *reinterpret_cast<const int2 *>(pos + i);
+                else j[u].x = pos[i];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            if (j[u].x >= 0 && !SJ_IN_BOUNDS(j[u].x < n, BND_UNSORT)) j[u].x = -1;
+            if (j[u].y >= 0 && !SJ_IN_BOUNDS(j[u].y < n, BND_UNSORT)) j[u].y = -1;
+            r0[u] = j[u].x >= 0 ? rec[j[u].x] : P2PRec{-1, -1};
+            r1[u] = j[u].y >= 0 ? rec[j[u].y] : P2PRec{-1, -1};
+        }
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            const unsigned p = p0 + u * T, i = 2u * p;
+            if (p >= pairs) continue;
+            const bool two = i + 1u < (unsigned)n;
+            int id0, id1;
+            double d0, d1;
+            fp32x_output(a, r0[u], r0[u].id < -1 ? pts[i] : make_double2(0.0, 0.0), id0, d0);
+            fp32x_output(a, r1[u], r1[u].id < -1 ? pts[i + 1u] : make_double2(0.0, 0.0), id1, d1);
+            if (two) {
+                *reinterpret_cast<int2 *>(out_id + i) = make_int2(id0, id1);
+                if (out_d) *reinterpret_cast<double2 *>(out_d + i) = make_double2(d0, d1);
+            } else {
+                out_id[i] = id0;
+                if (out_d) out_d[i] = d0;
+            }
+        }
+    }
+}
+
+// Where a finishing kernel's points come from: a call's points in input order,
+// a call's slots (no scratch for pos), or the requests of a batched round.
+struct FinOne {
+    const int *pos;
+    const double2 *pts;
+    int *out_id;
+    double *out_d;
+    int n;
+    double window;
+    __device__ __forceinline__ int count() const { return n; }
+    __device__ __forceinline__ int slot(int i) const { return pos[i]; }
+    __device__ __forceinline__ double2 point(int i) const { return pts[i]; }
+    __device__ __forceinline__ double win(int) const { return window; }
+    __device__ __forceinline__ void put(int i, int id, double d) const {
+        out_id[i] = id;
+        if (out_d) out_d[i] = d;
+    }
+};
+struct FinSlots {
+    const int *perm, *in_grid;   // in_grid: device count of slots
+    const double2 *pts;
+    int *out_id;
+    double *out_d;
+    double window;
+    __device__ __forceinline__ int count() const { return *in_grid; }
+    __device__ __forceinline__ int slot(int i) const { return i; }
+    __device__ __forceinline__ double2 point(int i) const { return pts[perm[i]]; }
+    __device__ __forceinline__ double win(int) const { return window; }
+    __device__ __forceinline__ void put(int i, int id, double d) const {
+        const int k = perm[i];
+        out_id[k] = id;
+        if (out_d) out_d[k] = d;
+    }
+};
+struct FinRound {
+    const RoundReq *reqs;
+    const int *meta, *pos;
+    __device__ __forceinline__ const RoundReq &find(int i) const { return reqs[find_request(reqs, meta[0], i)]; }
+    __device__ __forceinline__ int count() const { return meta[1]; }
+    __device__ __forceinline__ int slot(int i) const { return pos[i]; }
+    __device__ __forceinline__ double2 point(int i) const {
+        const RoundReq &r = find(i);
+        return r.pts[i - r.off];
+    }
+    __device__ __forceinline__ double win(int i) const { return find(i).window; }
+    __device__ __forceinline__ void put(int i, int id, double d) const {
+        const RoundReq &r = find(i);
+        r.out_id[i - r.off] = id;
+        if (r.out_d) r.out_d[i - r.off] = d;
+    }
+};
+
+template <class Src>
+__global__ void k_p2p_finish_fp32x(SegArgs a, const P2PRec *rec, Src src) {
+    const int n = src.count();
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)k, j = src.slot(i);
+        const P2PRec r = j >= 0 ? rec[j] : P2PRec{-1, -1};
+        int id;
+        double d;
+        fp32x_output(a, r, r.id < -1 ? src.point(i) : make_double2(0.0, 0.0), id, d);
+        src.put(i, id, d);
+    }
+}
+
+// FP64: the FP64 distances to the one or two segments of each point's record.
+// A warp takes FIN_U x 32 points; the second segments, which about a third of
+// the points have, are gathered in shared memory and evaluated with full warps,
+// since the FP64 pipe takes as long for one lane as for 32.  The compares of
+// the (non-negative, finite) distances and of t are made on their bit patterns,
+// off that pipe.
+__device__ __forceinline__ double clamp01(double t) {
+    const long long b = __double_as_longlong(t);   // a NaN (0 times an infinite 1 / |e|^2) gives 0, as fmax does
+    return (b <= 0 || b > 0x7ff0000000000000LL) ? 0.0 : (b > 0x3ff0000000000000LL ? 1.0 : t);
+}
+__device__ __forceinline__ double seg_d2_finite(const SegArgs &a, double2 p, int i) {
+    const double2 v = a.verts[i], e = a.seg_e64[i];
+    const double dx = __dsub_rn(p.x, v.x), dy = __dsub_rn(p.y, v.y);
+    const double t = clamp01(__dmul_rn(__fma_rn(e.x, dx, __dmul_rn(e.y, dy)), a.seg_inv64[i]));
+    const double qx = __fma_rn(-t, e.x, dx), qy = __fma_rn(-t, e.y, dy);
+    return __fma_rn(qx, qx, __dmul_rn(qy, qy));
+}
+
+constexpr int FIN_WARPS = 8;
+
+template <class Src>
+__global__ void __launch_bounds__(FIN_WARPS * 32) k_p2p_finish_fp64(SegArgs a, const P2PRec *rec, Src src,
+                                                                    unsigned long long *stats) {
+    __shared__ int2 q[FIN_WARPS][32 * FIN_U];        // (point of the tile, second segment)
+    __shared__ double d2s[FIN_WARPS][32 * FIN_U];
+    const double INF = __longlong_as_double(0x7ff0000000000000LL);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const long long n = src.count();
+    unsigned hits = 0;
+    for (long long base = (blockIdx.x * (long long)FIN_WARPS + w) * (32 * FIN_U); base < n;
+         base += (long long)gridDim.x * FIN_WARPS * (32 * FIN_U)) {
+        P2PRec r[FIN_U];
+        double d2[FIN_U];
+        int nq = 0;
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            const long long i = base + 32 * u + lane;
+            const int j = i < n ? src.slot((int)i) : -1;
+            r[u] = j >= 0 ? rec[j] : P2PRec{-1, -1};
+        }
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            const bool two = r[u].id >= 0 && r[u].aux >= 0;
+            const unsigned bal = __ballot_sync(FULL, two);
+            if (two) q[w][nq + __popc(bal & lt)] = make_int2(32 * u + lane, r[u].aux);
+            nq += __popc(bal);
+            d2[u] = r[u].id >= 0 ? seg_d2_finite(a, src.point((int)(base + 32 * u + lane)), r[u].id) : INF;
+        }
+        __syncwarp();
+        for (int k = lane; k < nq; k += 32) {
+            const int2 e = q[w][k];
+            d2s[w][e.x] = seg_d2_finite(a, src.point((int)(base + e.x)), e.y);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < FIN_U; ++u) {
+            const long long i = base + 32 * u + lane;
+            if (i >= n) continue;
+            int id = -1;
+            double d = INF;
+            if (r[u].id >= 0) {
+                int oid = seg_owner(a, r[u].id);
+                if (r[u].aux >= 0) {   // the smaller (squared distance, id)
+                    const double e2 = d2s[w][32 * u + lane];
+                    const long long x = __double_as_longlong(d2[u]), y = __double_as_longlong(e2);
+                    const int o2 = seg_owner(a, r[u].aux);
+                    if (y < x || (y == x && o2 < oid)) {
+                        d2[u] = e2;
+                        oid = o2;
+                    }
+                }
+                const double s = sqrt(d2[u]);
+                if (s <= src.win((int)i)) {
+                    id = oid;
+                    d = s;
+                }
+            }
+            src.put((int)i, id, d);
+            hits += id >= 0;
+        }
+        __syncwarp();
+    }
+    if (stats) {
+        unsigned long long v[ST_N] = {};
+        v[ST_HITS] = __reduce_add_sync(FULL, hits);
+        flush_stats(stats, v);
+    }
+}
+
+static int fin_blocks(long long n, int per_block, int cap) {
+    const long long b = (n + per_block - 1) / per_block;
+    return (int)(b < 1 ? 1 : (b > cap ? cap : b));
+}
+
+template <class Src>
+static void finish(const RefineArgs &a, int form, const Src &src, long long n_max, cudaStream_t s) {
+    if (form == SJ_FP32X)
+        k_p2p_finish_fp32x<Src><<<fin_blocks(n_max, 256, 152 * 16), 256, 0, s>>>(a.seg, a.rec, src);
+    else
+        k_p2p_finish_fp64<Src><<<fin_blocks(n_max, 32 * FIN_U * FIN_WARPS, 152 * 16), FIN_WARPS * 32, 0, s>>>(
+            a.seg, a.rec, src, a.stats);
+}
+
+// a8: outputs in input order from the slots' records (pos: slot of each input point or -1).
+cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int n, int *out_id, double *out_d,
+                              cudaStream_t s) {
+    if (form == SJ_FP32X && ((uintptr_t)out_id & 7) == 0 && ((uintptr_t)out_d & 15) == 0)
+        k_p2p_finish_pairs<<<fin_blocks(((n + 1LL) / 2 + FIN_U - 1) / FIN_U, 256, 152 * 16), 256, 0, s>>>(
+            a.seg, pos, a.rec, a.pts, n, out_id, out_d);
+    else
+        finish(a, form, FinOne{pos, a.pts, out_id, out_d, n, a.D}, n, s);
+    return cudaGetLastError();
+}
+// The same slot by slot through perm (in_grid: device count of slots).
+cudaError_t launch_p2p_finish_slots(const RefineArgs &a, int form, const int *in_grid, int n, int *out_id,
+                                    double *out_d, cudaStream_t s) {
+    finish(a, form, FinSlots{a.perm, in_grid, a.pts, out_id, out_d, a.D}, n, s);
+    return cudaGetLastError();
+}
+cudaError_t launch_p2p_finish_round(const RefineArgs &a, int form, const RoundReq *reqs, const int *meta,
+                                    const int *pos, long long n_max, cudaStream_t s) {
+    finish(a, form, FinRound{reqs, meta, pos}, n_max, s);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ launches
+
+template <bool F64, int NW>
+static size_t p2p_smem_bytes() {
+    return sizeof(P2PSmem<F64>) * NW;
+}
+
+template <bool F64, bool PW, int NW>
 static cudaError_t p2p_prepare() {
     static bool done = false;   // per process; the attribute is per function
     if (!done) {
-        cudaError_t e = cudaFuncSetAttribute(k_p2p_refine<FP32, PW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)p2p_smem_bytes<FP32, NW>());
+        cudaError_t e = cudaFuncSetAttribute(k_p2p_refine<F64, PW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)p2p_smem_bytes<F64, NW>());
         if (e != cudaSuccess) return e;
         done = true;
     }
     return cudaSuccess;
 }
 
-template <bool FP32, bool PW, int NW>
+template <bool F64, bool PW, int NW>
 static cudaError_t p2p_launch(const RefineArgs &a, int blocks, cudaStream_t s) {
-    cudaError_t e = p2p_prepare<FP32, PW, NW>();
+    cudaError_t e = p2p_prepare<F64, PW, NW>();
     if (e != cudaSuccess) return e;
-    k_p2p_refine<FP32, PW, NW><<<blocks, NW * 32, p2p_smem_bytes<FP32, NW>(), s>>>(a);
+    k_p2p_refine<F64, PW, NW><<<blocks, NW * 32, p2p_smem_bytes<F64, NW>(), s>>>(a);
     return cudaGetLastError();
 }
 
-template <bool FP32, bool PW>
+template <bool F64, bool PW>
 static cudaError_t p2p_launch_nw(const RefineArgs &a, int nw, int blocks, cudaStream_t s) {
-    if (nw == 2) return p2p_launch<FP32, PW, 2>(a, blocks, s);
-    if (nw == 8) return p2p_launch<FP32, PW, 8>(a, blocks, s);
-    return p2p_launch<FP32, PW, P2P_WARPS>(a, blocks, s);
+    if (nw == 2) return p2p_launch<F64, PW, 2>(a, blocks, s);
+    if (nw == 8) return p2p_launch<F64, PW, 8>(a, blocks, s);
+    return p2p_launch<F64, PW, P2P_WARPS>(a, blocks, s);
 }
 
 // blocks: the grid for blocks of P2P_WARPS warps (resident blocks x SMs); a
@@ -569,25 +811,26 @@ cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block
     const int nw = (warps_per_block == 2 || warps_per_block == 8) ? warps_per_block : P2P_WARPS;
     blocks = (int)(((long long)blocks * P2P_WARPS + nw - 1) / nw);
     const bool pw = a.win && a.win_on;
-    if (form == SJ_FP32X) return pw ? p2p_launch_nw<true, true>(a, nw, blocks, s) : p2p_launch_nw<true, false>(a, nw, blocks, s);
-    return pw ? p2p_launch_nw<false, true>(a, nw, blocks, s) : p2p_launch_nw<false, false>(a, nw, blocks, s);
+    if (form == SJ_FP32X) return pw ? p2p_launch_nw<false, true>(a, nw, blocks, s) : p2p_launch_nw<false, false>(a, nw, blocks, s);
+    return pw ? p2p_launch_nw<true, true>(a, nw, blocks, s) : p2p_launch_nw<true, false>(a, nw, blocks, s);
 }
 
-cudaError_t launch_p2p_recheck(const RefineArgs &a, int blocks, cudaStream_t s) {
-    k_p2p_recheck<<<blocks, 256, 0, s>>>(a);
+cudaError_t launch_p2p_recheck(const RefineArgs &a, int form, int blocks, cudaStream_t s) {
+    if (form == SJ_FP32X) k_p2p_recheck<false><<<blocks, 256, 0, s>>>(a);
+    else k_p2p_recheck<true><<<blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 int p2p_blocks_per_sm(int form) {
     int n = 0;
     if (form == SJ_FP32X) {
-        if (p2p_prepare<true, false, P2P_WARPS>() != cudaSuccess) return 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_p2p_refine<true, false, P2P_WARPS>, P2P_WARPS * 32,
-                                                      p2p_smem_bytes<true, P2P_WARPS>());
-    } else {
         if (p2p_prepare<false, false, P2P_WARPS>() != cudaSuccess) return 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_p2p_refine<false, false, P2P_WARPS>, P2P_WARPS * 32,
                                                       p2p_smem_bytes<false, P2P_WARPS>());
+    } else {
+        if (p2p_prepare<true, false, P2P_WARPS>() != cudaSuccess) return 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_p2p_refine<true, false, P2P_WARPS>, P2P_WARPS * 32,
+                                                      p2p_smem_bytes<true, P2P_WARPS>());
     }
     return n > 0 ? n : 1;
 }

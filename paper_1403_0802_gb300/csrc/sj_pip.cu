@@ -148,12 +148,7 @@ struct RoundSource {
     const int *meta;   // requests, points
     __device__ __forceinline__ int count() const { return meta[1]; }
     __device__ __forceinline__ const RoundReq &find(unsigned i) const {
-        int lo = 0, hi = meta[0];
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (reqs[mid].off <= (int)i) lo = mid; else hi = mid;
-        }
-        return reqs[lo];
+        return reqs[find_request(reqs, meta[0], (int)i)];
     }
     __device__ __forceinline__ double2 point(unsigned i) const {
         const RoundReq &r = find(i);
