@@ -144,7 +144,8 @@ typedef struct {
                               to 32 points refined together                     */
     int64_t pairs;         /* (point, candidate object) pairs refined            */
     int64_t edge_tests;    /* PIP: point x edge tests; P2P: point x segment tests */
-    int64_t fallbacks;     /* PIP: edges redone in FP64; P2P (SJ_FP32X): points  */
+    int64_t fallbacks;     /* PIP: edges redone in FP64; P2P: points refined again
+                              in FP64 over their cell's whole list              */
     int64_t hits;          /* points given an id                                 */
     int64_t refine_launches; /* refinement launches timed (SJ_FLAG_TIME_REFINE)  */
     double refine_ms;        /* their summed device time, milliseconds           */

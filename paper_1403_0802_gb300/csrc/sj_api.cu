@@ -210,13 +210,9 @@ static float float_up(double x) {
 // Layer-dependent fields of the P2P refinement arguments.
 void sj::fill_refine(const sj_layer *L, int form, RefineArgs &ra) {
     ra.g = L->g;
-    ra.cand_start = L->cand_start;
-    ra.cand_ids = L->cand_ids;
-    ra.obj_voff = L->obj_voff;
     ra.seg = SegArgs{L->verts, L->seg_e64, L->seg_inv64, L->seg32};
     ra.cseg_start = L->cseg_start;
     ra.cseg_ids = L->cseg_ids;
-    ra.cell_algo = L->cell_algo;
     ra.cseg_rec = L->cseg_rec;
     ra.D = L->D;
     ra.Df = L->Df;
@@ -907,6 +903,8 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ba.cell_start = b.cell_start;
     ba.perm = b.perm;
     ba.cand_start = L->cand_start;
+    ba.cell_algo = L->cell_algo;
+    ba.stats = L->stats;
     ba.ch = ch;
     ba.cell_work = split ? L->cell_work : nullptr;
     ba.budget = split ? budget : 0;
@@ -1254,6 +1252,8 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     ba.cell_start = b.cell_start;
     ba.perm = b.perm;
     ba.cand_start = L->cand_start;
+    ba.cell_algo = L->cell_algo;
+    ba.stats = L->stats;
     ba.ch = NOALLOC_CH;
     ba.items = b.items;
     ba.block_sums = b.block_sums;

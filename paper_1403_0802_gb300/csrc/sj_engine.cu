@@ -174,6 +174,8 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     ba.cnt = cnt;
     ba.cell_start = cell_start;
     ba.cand_start = L->cand_start;
+    ba.cell_algo = L->cell_algo;
+    ba.stats = L->stats;
     ba.ch = E->ch;
     ba.items = items;
     ba.block_sums = block_sums;

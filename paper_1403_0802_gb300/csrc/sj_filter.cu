@@ -87,10 +87,12 @@ __global__ void __launch_bounds__(1024) k_scan_top(int2 *block_sums, int nb, int
     }
 }
 
-// Phase 3: rescan each tile with its offset; ap(c, exclusive prefix, value).
+// Phase 3: rescan each tile with its offset; ap(c, exclusive prefix, value, n,
+// acc), then ap.done(acc) by every thread.
 template <class Load, class Apply>
 __global__ void __launch_bounds__(SCAN_T) k_scan_apply(Load ld, Apply ap, int n, const int2 *block_sums) {
     int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
+    typename Apply::Acc acc{};
     int2 v[SCAN_V];
     int2 tsum = make_int2(0, 0);
 #pragma unroll
@@ -105,9 +107,10 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply(Load ld, Apply ap, int n,
 #pragma unroll
     for (int j = 0; j < SCAN_V; ++j) {
         int c = base + j;
-        if (c < n) ap(c, ex, v[j], n);
+        if (c < n) ap(c, ex, v[j], n, acc);
         ex = add2(ex, v[j]);
     }
+    ap.done(acc);
 }
 
 // Phases 2 and 3 in one launch for at most SCAN_FUSE tiles: each block sums
@@ -123,6 +126,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply_fused(Load ld, Apply ap, 
     int2 offset;
     block_incl_scan<SCAN_T>(pre, offset);   // its total: the tile's exclusive prefix
     int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
+    typename Apply::Acc acc{};
     int2 v[SCAN_V];
     int2 tsum = make_int2(0, 0);
 #pragma unroll
@@ -137,9 +141,10 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply_fused(Load ld, Apply ap, 
 #pragma unroll
     for (int j = 0; j < SCAN_V; ++j) {
         int c = base + j;
-        if (c < n) ap(c, ex, v[j], n);
+        if (c < n) ap(c, ex, v[j], n, acc);
         ex = add2(ex, v[j]);
     }
+    ap.done(acc);
     if ((int)blockIdx.x == nb - 1 && threadIdx.x == 0) {
         const int2 grand = add2(offset, total);
         block_sums[nb] = grand;
@@ -172,8 +177,10 @@ struct IntLoad {
     __device__ int2 operator()(int c) const { return make_int2(a[c], 0); }
 };
 struct OffsetApply {
+    struct Acc {};
     int *out;
-    __device__ void operator()(int c, int2 ex, int2 v, int n) const {
+    __device__ void done(const Acc &) const {}
+    __device__ void operator()(int c, int2 ex, int2 v, int n, Acc &) const {
         out[c] = ex.x;
         if (c == n - 1) out[n] = ex.x + v.x;
     }
@@ -307,6 +314,9 @@ struct BucketLoad {
     }
 };
 struct BucketApply {
+    struct Acc {   // points x candidates and points x their segments (statistics)
+        unsigned long long pairs, algo;
+    };
     int *cell_start;
     int2 *items;
     int ch;
@@ -316,7 +326,26 @@ struct BucketApply {
     int lS;
     const int *cell_work;
     int budget;
-    __device__ void operator()(int c, int2 ex, int2 v, int n) const {
+    const int *cand_start, *cell_algo;
+    unsigned long long *stats;
+    __device__ void done(const Acc &acc) const {
+        if (!stats) return;
+        unsigned long long p = acc.pairs, q = acc.algo;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            p += __shfl_xor_sync(FULL, p, o);
+            q += __shfl_xor_sync(FULL, q, o);
+        }
+        unsigned long long v[ST_N] = {};
+        v[ST_PAIRS] = p;
+        v[ST_ALGO] = q;
+        flush_stats(stats, v);
+    }
+    __device__ void operator()(int c, int2 ex, int2 v, int n, Acc &acc) const {
+        if (stats && v.y > 0) {
+            acc.pairs += (unsigned long long)v.x * (unsigned)(cand_start[c + 1] - cand_start[c]);
+            acc.algo += (unsigned long long)v.x * (unsigned)cell_algo[c];
+        }
         cell_start[c] = ex.x;
         if (cell_base) cell_base[c] = v.y > 0 ? ex.x : -1;
         if (c == n - 1) cell_start[n] = ex.x + v.x;
@@ -410,7 +439,8 @@ static int stream_blocks(long long n, int per_block, int cap) {
 cudaError_t launch_bucket_scan(const BucketArgs &a, cudaStream_t s) {
     const int lS = a.sub_lx + a.sub_ly;
     return run_scan(BucketLoad{a.cnt, a.cand_start, a.ch, lS, a.cell_work, a.budget},
-                    BucketApply{a.cell_start, a.items, a.ch, a.cell_base, a.cnt, a.sub_start, lS, a.cell_work, a.budget},
+                    BucketApply{a.cell_start, a.items, a.ch, a.cell_base, a.cnt, a.sub_start, lS, a.cell_work, a.budget,
+                                a.cand_start, a.cell_algo, a.stats},
                     a.g.G, a.block_sums, a.bs_cap, a.totals, s);
 }
 

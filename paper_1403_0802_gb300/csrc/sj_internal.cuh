@@ -212,21 +212,6 @@ __host__ __device__ __forceinline__ int cell_chunk(int ch, int work, int budget)
     return c < lo ? lo : (c > ch ? ch : (int)c);
 }
 
-// Lanes per point group for a chunk of `nw` work units (edges / segments) and
-// `np` points: the power of two SG in {1..32} that minimises the number of
-// warp iterations ceil(np / (32 / SG)) * (ceil(nw / SG) + reduction steps).
-__device__ __forceinline__ int choose_group(int np, int nw, int red_cost) {
-    int best_sg = 1, best = 0x7fffffff;
-#pragma unroll
-    for (int lg = 0; lg <= 5; ++lg) {
-        // powers of two: shifts, not divisions
-        const int rounds = (np + (32 >> lg) - 1) >> (5 - lg);
-        const int cost = rounds * (((nw + (1 << lg) - 1) >> lg) + lg * red_cost);
-        if (cost < best) { best = cost; best_sg = 1 << lg; }
-    }
-    return best_sg;
-}
-
 // Minimum bounding box of an object.
 struct Box {
     double xmin, ymin, xmax, ymax;
@@ -282,13 +267,9 @@ struct RefineArgs {
     const int *perm;         // sorted slot -> input index
     const double2 *spts;     // sorted points (FP64), or null: the point of slot j is pts[perm[j]]
     const double2 *pts;      // input points (used when spts is null)
-    const int *cand_start;   // [G + 1]
-    const int *cand_ids;     // [M]
-    const int *obj_voff;     // [nobj + 1] first vertex of each polyline
     SegArgs seg;
     const int *cseg_start;   // [G + 1] per-cell segment lists
     const int *cseg_ids;     //      segment (= first vertex) indices, ascending per cell
-    const int *cell_algo;    //      [G] segments of the cell's candidate polylines
     const float4 *cseg_rec;  //      [2 MS] staging records of the list entries (see sj_filter.cu)
     double D;                // window
     float Ddn, Dup;          // FP32 D rounded down / up with a 1e-12 relative margin
@@ -450,6 +431,8 @@ struct BucketArgs {
     int2 *block_sums;    // scan scratch
     size_t bs_cap;       // its capacity in int2 (launches fail when it is too small)
     int *totals;         // [2]: in-grid points, items
+    const int *cell_algo;        // with stats: [G] segments of the cell's candidate polylines
+    unsigned long long *stats;   // ST_PAIRS, ST_ALGO of the points of cells with candidates (or null)
     int *out_id;         // initialised to -1 (or null)
     double *out_d;       // initialised to +inf (or null)
     int *pos;            // [n] sorted slot of each input point, -1 when its cell has no

@@ -15,15 +15,16 @@
 //      the item and is dropped (exact: it cannot change any result); the others
 //      are compacted into shared memory (a, e = b - a, 1 / |e|^2, a tag) with a
 //      ballot.
-//   4. Whenever the staging area fills, the warp splits its lanes into point
-//      groups of SG lanes (SG chosen so that np points x staged segments fill
-//      the warp); each lane strides over the staged segments keeping the
-//      smallest squared distances of its point, and the SG lanes of a group fold
-//      theirs with shuffles (the cross-lane min of the vertex-per-lane
-//      alternative of Sec. III.B).  After the last segments the point's result is
-//      made from the fold at once, in registers; only a list that fills the
-//      staging area more than once keeps its points' state in shared memory in
-//      between.
+//   4. The warp takes the item's points in rounds.  Each splits the lanes into
+//      point groups of SG lanes (SG so that the round's points fill the warp);
+//      each lane strides over the staged segments keeping the smallest squared
+//      distances of its point, and the SG lanes of a group fold theirs with
+//      shuffles (the cross-lane min of the vertex-per-lane alternative of
+//      Sec. III.B); the point's record is made from the fold in registers.  The
+//      few lists that fill the staging area more than once are staged part by
+//      part in every round, so no state of a point lives in shared memory: what
+//      the kernel does not take there is L1, which holds the records that the
+//      items of a cell share.
 //
 // The point-to-segment distance is the two-case distance of Fig. 2 written as
 // the clamped projection: t = clamp(((p - a) . e) / |e|^2, 0, 1) and
@@ -55,6 +56,8 @@
 // The one or two evaluations that a point needs are left to the finishing
 // kernel, whose warps are full of points: made at the end of each item, with
 // half of the lanes idle, they still took most of the refinement (0.43 ms).
+// Now the FP64 form's refinement takes 0.27 ms and its finishing 0.13 ms there,
+// the join 0.50 ms instead of 3.50.
 #include <cuda_runtime.h>
 
 #include "sj_internal.cuh"
@@ -87,14 +90,12 @@ struct Best<true> {
     int i1, i2;
 };
 
-template <bool F64>
 struct P2PSmem {
     static constexpr int SMAX = 128;   // even
     float4 sa[SMAX / 2];     // (-ax, -ax', -ay, -ay') cell-relative
     float4 se[SMAX / 2];     // (-ex, -ex', -ey, -ey')
     float4 si[SMAX / 2];     // (-1 / |e|^2, -1 / |e'|^2, tag, tag')
     float2 pt[MAX_CH];
-    Best<F64> st[MAX_CH];    // used between the parts of a list longer than SMAX
 };
 
 // Squared distance from p to the segment (a, a + e) by the clamped projection:
@@ -200,8 +201,8 @@ __device__ __forceinline__ float warp_max(float v) { return key_float(__reduce_m
 
 // What one point's result needs besides its fold.
 struct P2PItem {
-    int j0, c;      // first slot of the item, cell
-    float mag;      // largest |cell-relative coordinate| of the points and staged segments
+    int c;          // cell
+    float mag;      // largest |cell-relative coordinate| of the item's points and staged segments
 };
 
 // The record of slot j (point pt, cell-relative) from its complete fold; a
@@ -241,71 +242,19 @@ __device__ __forceinline__ void p2p_result(const RefineArgs &a, const P2PItem &i
     }
 }
 
-// Refine the staged segment pairs [0, ns) for the item's np points.  Rounds of 32
-// points take one lane per point (every lane busy, no merge); the last round,
-// of fewer than 32 points, splits each point's segments over a group of sg
-// lanes chosen by the cost model (more lanes per point, log2(sg) merges).
-// first / last: the list's first / last part.
-template <bool F64, bool PW>
-__device__ __forceinline__ void p2p_compute(const RefineArgs &a, P2PSmem<F64> &s, const P2PItem &it, int np, int ns,
-                                            int lane, bool first, bool last, bool pw, unsigned &c_fb,
-                                            unsigned &c_hits) {
-    int pg = 32;
-    for (int q0 = 0; q0 < np; q0 += pg) {
-        const int rem = np - q0;
-        const int sg = rem >= 32 ? 1 : choose_group(rem, ns, 2);
-        const int lg = __ffs(sg) - 1;
-        pg = 32 >> lg;
-        const int sub = lane & (sg - 1), grp = lane >> lg;
-        const int q = q0 + grp;
-        Best<F64> st = best_none((Best<F64> *)nullptr);
-        float2 p = make_float2(0.0f, 0.0f);
-        if (q < np) {
-            // the squared distances of the pair by the clamped projection
-            // in FP32: dx = px - ax, t = sat(fma(ex, dx, ey * dy) / |e|^2),
-            // q = fma(-t, e, d), |q|^2 = fma(qx, qx, qy * qy), written with
-            // the negated operands (p + (-a) = p - a, fma(-ex, dx, -ey * dy)
-            // * (-1 / |e|^2) = (e . d) / |e|^2, fma(t, -e, d) = d - t e:
-            // each rounding the same as the unnegated one)
-            p = s.pt[q];
-            const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y);
-#pragma unroll 1
-            for (int t = sub; t < ns; t += sg) {
-                const float4 A = s.sa[t], E = s.se[t], I = s.si[t];
-                const float2 nex = make_float2(E.x, E.y), ney = make_float2(E.z, E.w);
-                const float2 dx = __fadd2_rn(px, make_float2(A.x, A.y));
-                const float2 dy = __fadd2_rn(py, make_float2(A.z, A.w));
-                const float2 w = __ffma2_rn(nex, dx, __fmul2_rn(ney, dy));
-                const float2 tt = make_float2(__saturatef(__fmul_rn(w.x, I.x)), __saturatef(__fmul_rn(w.y, I.y)));
-                const float2 qx = __ffma2_rn(tt, nex, dx), qy = __ffma2_rn(tt, ney, dy);
-                const float2 d = __ffma2_rn(qx, qx, __fmul2_rn(qy, qy));
-                consider(st, d.x, __float_as_int(I.z));
-                consider(st, d.y, __float_as_int(I.w));
-            }
-        }
-        for (int o = sg >> 1; o > 0; o >>= 1) st = merge(st, shfl_best(st, o));
-        if (sub == 0 && q < np) {
-            if (!first) st = merge(s.st[q], st);
-            if (last) p2p_result<F64, PW>(a, it, it.j0 + q, p, st, pw, c_fb, c_hits);
-            else s.st[q] = st;
-        }
-    }
-}
-
 // PW: per-point windows (a.win_on set; batched rounds).  The direct joins use
-// PW = false, whose code has no window load at all.  Eight blocks per SM is
-// the shared-memory limit already; saying so keeps the register allocator at
-// 64 registers without spills.
+// PW = false, whose code has no window load at all.  32 warps per SM: 64
+// registers without spills.
 template <bool F64, bool PW, int NW>
 __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
-    constexpr int SMAX = P2PSmem<F64>::SMAX;
+    constexpr int SMAX = P2PSmem::SMAX;
     extern __shared__ __align__(16) unsigned char p2p_smem_raw[];
     const int lane = lane_id(), w = threadIdx.x >> 5;
-    P2PSmem<F64> &s = reinterpret_cast<P2PSmem<F64> *>(p2p_smem_raw)[w];
+    P2PSmem &s = reinterpret_cast<P2PSmem *>(p2p_smem_raw)[w];
     const int n_items = *a.n_items;
     const float FINF = __int_as_float(0x7f800000);
     const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned long long c_pairs = 0, c_tests = 0, c_items = 0, c_algo = 0;
+    unsigned long long c_tests = 0, c_items = 0;
     unsigned c_fb = 0, c_hits = 0;
     const bool pw = PW && *a.win_on;   // per-point windows in this launch (uniform)
 
@@ -343,7 +292,6 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         const int c = item.x;
         const int j0 = cs0 + item.y;
         const int np = min(cell_chunk(a.ch, a.budget > 0 ? a.cell_work[c] : 0, a.budget), cs1 - j0);
-        const int k0 = a.cand_start[c], k1 = a.cand_start[c + 1];
         const float2 fo = cell_frame(a.frame_x, a.frame_y, a.g.nx, c);
 
         // 1. points: cell-relative FP32 coordinates, their box and magnitude
@@ -353,7 +301,7 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         // (idle) staging area -- so that their latencies overlap instead of
         // forming one chain per point.
         constexpr int PQ = MAX_CH / 32;
-        static_assert(sizeof(P2PSmem<F64>::sa) + sizeof(P2PSmem<F64>::se) >= MAX_CH * sizeof(double2), "");
+        static_assert(sizeof(P2PSmem::sa) + sizeof(P2PSmem::se) >= MAX_CH * sizeof(double2), "");
         double2 *pbuf = reinterpret_cast<double2 *>(&s.sa[0]);   // sa and se, contiguous
         {
             int src[PQ];
@@ -389,52 +337,53 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         int2 item_n = make_int2(0, 0);
         if (it_next < n_items) item_n = a.items[it_next];
         float mag = pmag;   // largest |cell-relative coordinate| refined for this item
-        c_pairs += (unsigned long long)np * (unsigned long long)(k1 - k0);
-        c_algo += (unsigned long long)np * (unsigned long long)a.cell_algo[c];
 
         // 2. the cell's segment list, 32 segments at a time (one per lane),
-        // 3. staging with the exact distance prune, 4. refinement when full
+        // 3. staging with the exact distance prune, 4. rounds of points
         const int g0 = a.cseg_start[c], g1 = a.cseg_start[c + 1];
-        int nst = 0;
-        bool first = true;
-        int base = g0;
-        do {
-            const int g = base + lane;
-            bool keep = false;
-            int tag = 0;
-            float ax = 0.0f, ay = 0.0f, ex = 0.0f, ey = 0.0f, inv = 0.0f, smag = 0.0f;
-            if (g < g1 && SJ_IN_BOUNDS(g < a.cseg_start[a.g.G], BND_P2P_REC)) {
-                const float4 r0 = a.cseg_rec[2 * (size_t)g], r1 = a.cseg_rec[2 * (size_t)g + 1];
-                ax = r0.x;
-                ay = r0.y;
-                ex = r0.z;
-                ey = r0.w;
-                inv = r1.x;
-                tag = __float_as_int(F64 ? r1.w : r1.y);   // segment or polyline
-                smag = r1.z;
-                const float bx = ax + ex, by = ay + ey;
-                const float gx = fmaxf(0.0f, fmaxf(fminf(ax, bx) - bxhi, bxlo - fmaxf(ax, bx)));
-                const float gy = fmaxf(0.0f, fmaxf(fminf(ay, by) - byhi, bylo - fmaxf(ay, by)));
-                // rounding slack of the relative coordinates of both boxes (far above it)
-                const float lim = a.Df * (1.0f + 1e-6f) + 8.0f * U32 * (smag + pmag) + 8.0f * a.eps_abs;
-                keep = gx * gx + gy * gy <= lim * lim * (1.0f + 8.0f * U32);
-            }
-            const unsigned bal = __ballot_sync(FULL, keep);
-            if (keep) {
-                const int pos = nst + __popc(bal & lt_mask);
-                const int k = pos >> 1, h = pos & 1;
-                float *A = reinterpret_cast<float *>(&s.sa[k]);
-                float *E = reinterpret_cast<float *>(&s.se[k]);
-                float *I = reinterpret_cast<float *>(&s.si[k]);
-                A[h] = -ax; A[2 + h] = -ay;
-                E[h] = -ex; E[2 + h] = -ey;
-                I[h] = -inv; I[2 + h] = __int_as_float(tag);
-                mag = fmaxf(mag, smag);
-            }
-            nst += __popc(bal);
-            base += 32;
-            const bool last = base >= g1;
-            if (nst > SMAX - 32 || last) {
+        int base = g0, nst = 0, q0 = 0, sg = 0;
+        bool fill = true, parts = false;
+        Best<F64> st = best_none((Best<F64> *)nullptr);
+        while (true) {
+            if (fill) {
+                __syncwarp();   // no lane still reads what the fill overwrites
+                nst = 0;
+                while (base < g1 && nst <= SMAX - 32) {
+                    const int g = base + lane;
+                    bool keep = false;
+                    int tag = 0;
+                    float ax = 0.0f, ay = 0.0f, ex = 0.0f, ey = 0.0f, inv = 0.0f, smag = 0.0f;
+                    if (g < g1 && SJ_IN_BOUNDS(g < a.cseg_start[a.g.G], BND_P2P_REC)) {
+                        const float4 r0 = a.cseg_rec[2 * (size_t)g], r1 = a.cseg_rec[2 * (size_t)g + 1];
+                        ax = r0.x;
+                        ay = r0.y;
+                        ex = r0.z;
+                        ey = r0.w;
+                        inv = r1.x;
+                        tag = __float_as_int(F64 ? r1.w : r1.y);   // segment or polyline
+                        smag = r1.z;
+                        const float bx = ax + ex, by = ay + ey;
+                        const float gx = fmaxf(0.0f, fmaxf(fminf(ax, bx) - bxhi, bxlo - fmaxf(ax, bx)));
+                        const float gy = fmaxf(0.0f, fmaxf(fminf(ay, by) - byhi, bylo - fmaxf(ay, by)));
+                        // rounding slack of the relative coordinates of both boxes (far above it)
+                        const float lim = a.Df * (1.0f + 1e-6f) + 8.0f * U32 * (smag + pmag) + 8.0f * a.eps_abs;
+                        keep = gx * gx + gy * gy <= lim * lim * (1.0f + 8.0f * U32);
+                    }
+                    const unsigned bal = __ballot_sync(FULL, keep);
+                    if (keep) {
+                        const int pos = nst + __popc(bal & lt_mask);
+                        const int k = pos >> 1, h = pos & 1;
+                        float *A = reinterpret_cast<float *>(&s.sa[k]);
+                        float *E = reinterpret_cast<float *>(&s.se[k]);
+                        float *I = reinterpret_cast<float *>(&s.si[k]);
+                        A[h] = -ax; A[2 + h] = -ay;
+                        E[h] = -ex; E[2 + h] = -ey;
+                        I[h] = -inv; I[2 + h] = __int_as_float(tag);
+                        mag = fmaxf(mag, smag);
+                    }
+                    nst += __popc(bal);
+                    base += 32;
+                }
                 // an odd count: the pair's second slot gets a segment at
                 // infinite distance (a far point, zero length), which never
                 // changes a point's fold
@@ -448,14 +397,54 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
                     reinterpret_cast<float *>(&s.si[k])[3] = __int_as_float(-2);
                 }
                 __syncwarp();
-                mag = warp_max(mag);
-                p2p_compute<F64, PW>(a, s, P2PItem{j0, c, mag}, np, (nst + 1) >> 1, lane, first, last, pw, c_fb, c_hits);
-                c_tests += (unsigned long long)np * (unsigned long long)nst;
-                __syncwarp();
-                nst = 0;
-                first = false;
+                parts |= base < g1;
             }
-        } while (base < g1);
+            const int ns = (nst + 1) >> 1, rem = np - q0;
+            if (sg == 0) {   // a round begins: one lane per point while 32 remain, then groups that fill the warp
+                sg = rem > 16 ? 1 : min(1 << (__clz(rem - 1) - 27), parts ? 32 : 1 << (32 - __clz(max(ns, 1) - 1)));
+            }
+            const int lg = __ffs(sg) - 1;
+            const int sub = lane & (sg - 1), q = q0 + (lane >> lg);
+            const float2 p = s.pt[min(q, np - 1)];
+            if (q < np) {
+                // the squared distances of the pair by the clamped projection
+                // in FP32: dx = px - ax, t = sat(fma(ex, dx, ey * dy) / |e|^2),
+                // q = fma(-t, e, d), |q|^2 = fma(qx, qx, qy * qy), written with
+                // the negated operands (p + (-a) = p - a, fma(-ex, dx, -ey * dy)
+                // * (-1 / |e|^2) = (e . d) / |e|^2, fma(t, -e, d) = d - t e:
+                // each rounding the same as the unnegated one)
+                const float2 px = make_float2(p.x, p.x), py = make_float2(p.y, p.y);
+#pragma unroll 1
+                for (int t = sub; t < ns; t += sg) {
+                    const float4 A = s.sa[t], E = s.se[t], I = s.si[t];
+                    const float2 nex = make_float2(E.x, E.y), ney = make_float2(E.z, E.w);
+                    const float2 dx = __fadd2_rn(px, make_float2(A.x, A.y));
+                    const float2 dy = __fadd2_rn(py, make_float2(A.z, A.w));
+                    const float2 w2 = __ffma2_rn(nex, dx, __fmul2_rn(ney, dy));
+                    const float2 tt =
+                        make_float2(__saturatef(__fmul_rn(w2.x, I.x)), __saturatef(__fmul_rn(w2.y, I.y)));
+                    const float2 qx = __ffma2_rn(tt, nex, dx), qy = __ffma2_rn(tt, ney, dy);
+                    const float2 d = __ffma2_rn(qx, qx, __fmul2_rn(qy, qy));
+                    consider(st, d.x, __float_as_int(I.z));
+                    consider(st, d.y, __float_as_int(I.w));
+                }
+            }
+            const int pg = 32 >> lg;
+            c_tests += (unsigned long long)min(rem, pg) * (unsigned long long)nst;
+            if (base < g1) {   // the list's next part
+                fill = true;
+                continue;
+            }
+            for (int o = sg >> 1; o > 0; o >>= 1) st = merge(st, shfl_best(st, o));
+            const float m = warp_max(mag);
+            if (sub == 0 && q < np) p2p_result<F64, PW>(a, P2PItem{c, m}, j0 + q, p, st, pw, c_fb, c_hits);
+            q0 += pg;
+            if (q0 >= np) break;
+            sg = 0;
+            st = best_none((Best<F64> *)nullptr);
+            fill = parts;
+            if (parts) base = g0;
+        }
         int cs0n = 0, cs1n = 0;
         if (it_next < n_items) {
             cs0n = a.cell_start[item_n.x];
@@ -471,9 +460,7 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
     if (a.stats) {
         unsigned long long v[ST_N] = {};
         v[ST_ITEMS] = c_items;
-        v[ST_PAIRS] = c_pairs;
         v[ST_TESTS] = c_tests;
-        v[ST_ALGO] = c_algo;
         v[ST_FALLBACK] = __reduce_add_sync(FULL, c_fb);
         v[ST_HITS] = __reduce_add_sync(FULL, c_hits);
         flush_stats(a.stats, v);
@@ -773,17 +760,12 @@ cudaError_t launch_p2p_finish_round(const RefineArgs &a, int form, const RoundRe
 
 // ------------------------------------------------------------------ launches
 
-template <bool F64, int NW>
-static size_t p2p_smem_bytes() {
-    return sizeof(P2PSmem<F64>) * NW;
-}
-
 template <bool F64, bool PW, int NW>
 static cudaError_t p2p_prepare() {
     static bool done = false;   // per process; the attribute is per function
     if (!done) {
         cudaError_t e = cudaFuncSetAttribute(k_p2p_refine<F64, PW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)p2p_smem_bytes<F64, NW>());
+                                             (int)sizeof(P2PSmem) * NW);
         if (e != cudaSuccess) return e;
         done = true;
     }
@@ -794,7 +776,7 @@ template <bool F64, bool PW, int NW>
 static cudaError_t p2p_launch(const RefineArgs &a, int blocks, cudaStream_t s) {
     cudaError_t e = p2p_prepare<F64, PW, NW>();
     if (e != cudaSuccess) return e;
-    k_p2p_refine<F64, PW, NW><<<blocks, NW * 32, p2p_smem_bytes<F64, NW>(), s>>>(a);
+    k_p2p_refine<F64, PW, NW><<<blocks, NW * 32, sizeof(P2PSmem) * NW, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -826,11 +808,11 @@ int p2p_blocks_per_sm(int form) {
     if (form == SJ_FP32X) {
         if (p2p_prepare<false, false, P2P_WARPS>() != cudaSuccess) return 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_p2p_refine<false, false, P2P_WARPS>, P2P_WARPS * 32,
-                                                      p2p_smem_bytes<false, P2P_WARPS>());
+                                                      sizeof(P2PSmem) * P2P_WARPS);
     } else {
         if (p2p_prepare<true, false, P2P_WARPS>() != cudaSuccess) return 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_p2p_refine<true, false, P2P_WARPS>, P2P_WARPS * 32,
-                                                      p2p_smem_bytes<true, P2P_WARPS>());
+                                                      sizeof(P2PSmem) * P2P_WARPS);
     }
     return n > 0 ? n : 1;
 }
