@@ -817,6 +817,38 @@ static void carve(Scratch &s, JoinBufs &b, int64_t N, int G, int ch, bool to_inp
 }
 static_assert(sizeof(P2PRec) == sizeof(int2), "");
 
+// CUDA events around the launches of a span (SJ_FLAG_TIME_REFINE), kept with the
+// layer once recorded; an error sets e.
+struct TimedSpan {
+    const sj_layer *L;
+    cudaStream_t s;
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    TimedSpan(const sj_layer *layer, bool on, cudaStream_t stream, cudaError_t &e) : L(layer), s(stream) {
+        if (!on || e != cudaSuccess) return;
+        e = cudaEventCreate(&ev0);
+        if (e == cudaSuccess) e = cudaEventCreate(&ev1);
+        if (e == cudaSuccess) e = cudaEventRecord(ev0, s);
+    }
+    void stop(cudaError_t &e) {
+        if (!ev1) return;
+        if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
+        std::lock_guard<std::mutex> lk(L->ev_mu);
+        L->ev_pending.emplace_back(ev0, ev1);
+    }
+};
+
+static DirectArgs direct_args(const sj_layer *L, int32_t *out_id, double *out_d) {
+    DirectArgs g{};
+    g.cand_start = L->cand_start;
+    g.cell_algo = L->cell_algo;
+    // a point lies within its cell, the cell's FP32 frame origin within u xmax of
+    // its corner, and the coordinate's own rounding adds 2u of it
+    g.cell_mag = float_up((std::max(L->g.cw, L->g.ch) + 1.2e-7 * L->xmax) * (1.0 + 1e-6));
+    g.out_id = out_id;
+    g.out_d = out_d;
+    return g;
+}
+
 // window < 0: the layer's D; else a P2P window 0 <= window <= D for this call
 // alone (the layer's lists, built for D, hold every segment within any smaller
 // window, so the same kernels apply with the window's thresholds).
@@ -856,18 +888,36 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     if (kind == KIND_PIP) {   // one kernel over the points in input order, no scratch (sj_pip.cu)
         PipArgs pa = pip_args(L);
         if (subcells) pa.search = PIP_SEARCH_MIN;
-        cudaEvent_t ev0 = nullptr, ev1 = nullptr;
         cudaError_t e = cudaSuccess;
-        if (timed) {
-            e = cudaEventCreate(&ev0);
-            if (e == cudaSuccess) e = cudaEventCreate(&ev1);
-            if (e == cudaSuccess) e = cudaEventRecord(ev0, s);
-        }
+        TimedSpan span(L, timed, s, e);
         if (e == cudaSuccess) e = launch_pip_join(pa, (const double2 *)pts, (int)N, out_id, di->sms, s);
-        if (timed && ev1) {
-            if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
-            std::lock_guard<std::mutex> lk(L->ev_mu);
-            L->ev_pending.emplace_back(ev0, ev1);
+        span.stop(e);
+        if (e != cudaSuccess) return cuda_fail(e, "join launch");
+        return check_bounds(s);
+    }
+    RefineArgs ra{};
+    fill_refine(L, form, ra);
+    if (window >= 0.0) {
+        ra.D = window;
+        ra.Df = (float)window;
+        ra.Ddn = float_down(window * (1.0 - 1e-12));
+        ra.Dup = float_up(window * (1.0 + 1e-12) + 1e-300);
+    }
+    ra.pts = (const double2 *)pts;
+    ra.npts = (int)N;
+    // Few points: no bucketing (see k_p2p_direct).  Calls that shape their work
+    // items or order their points keep the path that has them.
+    if (N <= (form == SJ_FP32X ? P2P_DIRECT_FP32X : P2P_DIRECT_FP64) && !(o && o->pts_per_item) && budget == 0 &&
+        !subcells) {
+        cudaError_t e = cudaSuccess;
+        if (form == SJ_FP64) CUDA_TRY(dev_malloc_async((void **)&ra.rec, sizeof(P2PRec) * (size_t)N, s));
+        TimedSpan span(L, timed, s, e);
+        if (e == cudaSuccess) e = launch_p2p_direct(ra, direct_args(L, out_id, out_d), form, (int)N, di->sms, s);
+        span.stop(e);
+        if (form == SJ_FP64) {
+            if (e == cudaSuccess) e = launch_p2p_finish(ra, form, nullptr, (int)N, out_id, out_d, s);
+            cudaError_t e2 = cudaFreeAsync(ra.rec, s);
+            if (e == cudaSuccess) e = e2;
         }
         if (e != cudaSuccess) return cuda_fail(e, "join launch");
         return check_bounds(s);
@@ -919,14 +969,6 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ba.sub_start = b.sub_start;
     if (e == cudaSuccess) e = launch_bucket(ba, s);
 
-    RefineArgs ra{};
-    fill_refine(L, form, ra);
-    if (window >= 0.0) {
-        ra.D = window;
-        ra.Df = (float)window;
-        ra.Ddn = float_down(window * (1.0 - 1e-12));
-        ra.Dup = float_up(window * (1.0 + 1e-12) + 1e-300);
-    }
     ra.items = b.items;
     ra.n_items = b.totals + 1;
     ra.work_next = b.totals + 3;   // zeroed with the totals at the start of the join
@@ -939,26 +981,15 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     ra.claim = (N >= 2LL * ch * (long long)G) ? 2 : 1;
     ra.cell_start = b.cell_start;
     ra.perm = b.perm;
-    ra.pts = (const double2 *)pts;
     ra.ch = ch;
-    ra.npts = (int)N;
     ra.cell_work = ba.cell_work;
     ra.budget = ba.budget;
     ra.rec = reinterpret_cast<P2PRec *>(b.key_rank);   // every slot of a refined cell written
     ra.fb = b.fb;
     ra.n_fb = b.totals + 2;
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    if (e == cudaSuccess && timed) {
-        e = cudaEventCreate(&ev0);
-        if (e == cudaSuccess) e = cudaEventCreate(&ev1);
-        if (e == cudaSuccess) e = cudaEventRecord(ev0, s);
-    }
+    TimedSpan span(L, timed, s, e);   // the refinement launch alone
     if (e == cudaSuccess) e = launch_p2p_refine(ra, form, nw, di->sms * di->p2p_bps[form], s);
-    if (timed && ev1) {   // the refinement launch alone
-        if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
-        std::lock_guard<std::mutex> lk(L->ev_mu);
-        L->ev_pending.emplace_back(ev0, ev1);
-    }
+    span.stop(e);
     if (e == cudaSuccess) e = launch_p2p_recheck(ra, form, di->sms * 4, s);
     if (e == cudaSuccess) e = launch_p2p_finish(ra, form, b.pos, (int)N, out_id, out_d, s);   // a8
     cudaError_t e2 = cudaFreeAsync(sc.base, s);
@@ -1234,6 +1265,16 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     if (N == 0) return SJ_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const int G = L->g.G;
+    if (N <= (form == SJ_FP32X ? P2P_DIRECT_FP32X : P2P_DIRECT_FP64)) {   // as join_impl
+        RefineArgs ra{};
+        fill_refine(L, form, ra);
+        ra.pts = (const double2 *)pts;
+        ra.npts = (int)N;
+        ra.rec = reinterpret_cast<P2PRec *>(base);
+        CUDA_TRY(launch_p2p_direct(ra, direct_args(L, out_id, out_d), form, (int)N, di->sms, s));
+        if (form == SJ_FP64) CUDA_TRY(launch_p2p_finish(ra, form, nullptr, (int)N, out_id, out_d, s));
+        return check_bounds(s);
+    }
     JoinBufs b;
     size_t bytes = measure([&](Scratch &sc) { carve(sc, b, N, G, NOALLOC_CH, false); });
     if (bytes > NOALLOC_BYTES) return fail(SJ_ERR_INVALID, "sj_p2p_join_noalloc: scratch does not fit");

@@ -405,6 +405,15 @@ unsigned bounds_take_pip();
 // Host-side launchers (defined in the .cu files).
 cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block, int blocks, cudaStream_t s);
 cudaError_t launch_p2p_recheck(const RefineArgs &a, int form, int blocks, cudaStream_t s);
+// A small call without bucketing (FP32X: n <= P2P_DIRECT_FP32X; FP64 leaves a.rec by input point).
+struct DirectArgs {
+    const int *cand_start, *cell_algo;   // statistics
+    float cell_mag;    // no point of a cell has a larger |cell-relative coordinate|
+    int *out_id;       // FP32X
+    double *out_d;     //   (may be null)
+};
+constexpr int P2P_DIRECT_FP32X = 32768, P2P_DIRECT_FP64 = 131072;
+cudaError_t launch_p2p_direct(const RefineArgs &a, const DirectArgs &g, int form, int n, int sms, cudaStream_t s);
 cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int n, int *out_id, double *out_d,
                               cudaStream_t s);
 cudaError_t launch_p2p_finish_slots(const RefineArgs &a, int form, const int *in_grid, int n, int *out_id,

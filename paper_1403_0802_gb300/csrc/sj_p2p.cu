@@ -60,6 +60,8 @@
 // the join 0.50 ms instead of 3.50.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "sj_internal.cuh"
 
 namespace sj {
@@ -504,6 +506,291 @@ __global__ void __launch_bounds__(256) k_p2p_recheck(RefineArgs a) {
     }
 }
 
+// ------------------------------------------------------------------ small calls
+//
+// A call of few points spends its time on the grid, not on the points: counters
+// of every cell are cleared, counted into and scanned.  Here a warp takes each
+// point straight from the input: its cell, then the cell's segment list with the
+// lanes over the segments.  Every list entry is tested once per point and the
+// points of a cell share nothing, so the cost grows with the points, where
+// bucketing pays for the grid.  us a join, bucketed against direct, 512 x 512
+// grid, 150,000 walks, D = 100 m: FP32X 1,000 points 51 / 11, 32,000 73 / 27;
+// FP64 1,000 59 / 19, 64,000 102 / 53, 131,000 134 / 93.  The lines
+// (P2P_DIRECT_*) lie where direct still wins on every layer tried (FP64), and
+// where looking up a point's cell (below) stays a few us (FP32X).
+//
+// FP64 leaves each point's record for k_p2p_finish_fp64.  FP32X must answer
+// exactly what the bucketed refinement answers, whose certificate takes the
+// magnitude M and the tested segments from the point's work item -- the call's
+// points of its cell.  Both only grow with the item, and with them the chance
+// that the point is redone: so they are bounded from below by those of the
+// point alone and from above by those of the whole cell.  Where both agree, the
+// item does not matter; for the others (one point in 10^4) the block looks up
+// the cell's other points in the input.
+
+// Decision for a point's fold under a certificate: 0 outside the window, 1
+// final, 2 to be redone in FP64.
+__device__ __forceinline__ int fp32x_decide(const RefineArgs &a, const Best<false> &st, float mag) {
+    const float d = sqrtf(st.b1), d2 = sqrtf(st.b2);
+    const float e = fmaf(64.0f * U32, mag, 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
+    if (st.i1 < 0 || (d - e) * (1.0f - 4.0f * U32) > a.Dup) return 0;
+    const bool in_window = (d + e) * (1.0f + 4.0f * U32) < a.Ddn;
+    const bool separated = (d2 - d) * (1.0f - 4.0f * U32) > 2.0f * e * (1.0f + 4.0f * U32);
+    return in_window && separated ? 1 : 2;
+}
+
+// Squared FP32 distance to a list entry: the arithmetic of the staged loop.
+__device__ __forceinline__ float rec_d2(float2 p, const float4 r0, float inv) {
+    const float dx = __fsub_rn(p.x, r0.x), dy = __fsub_rn(p.y, r0.y);
+    const float t = __saturatef(__fmul_rn(__fmaf_rn(r0.z, dx, __fmul_rn(r0.w, dy)), inv));
+    const float qx = __fmaf_rn(-t, r0.z, dx), qy = __fmaf_rn(-t, r0.w, dy);
+    return __fmaf_rn(qx, qx, __fmul_rn(qy, qy));
+}
+
+// The staged loop's prune: whether the entry's box comes within D of the box.
+__device__ __forceinline__ bool rec_near(const RefineArgs &a, const float4 r0, float smag, float4 box, float pmag) {
+    const float bx = r0.x + r0.z, by = r0.y + r0.w;
+    const float gx = fmaxf(0.0f, fmaxf(fminf(r0.x, bx) - box.y, box.x - fmaxf(r0.x, bx)));
+    const float gy = fmaxf(0.0f, fmaxf(fminf(r0.y, by) - box.w, box.z - fmaxf(r0.y, by)));
+    const float lim = a.Df * (1.0f + 1e-6f) + 8.0f * U32 * (smag + pmag) + 8.0f * a.eps_abs;
+    return gx * gx + gy * gy <= lim * lim * (1.0f + 8.0f * U32);
+}
+
+// Smallest of the lanes' non-negative floats (their bits order as integers).
+__device__ __forceinline__ float warp_min_pos(float v) {
+    return __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(v)));
+}
+
+// FP32X fold of the lanes' folds: the best polyline, and the best distance of
+// any other (a lane's own runner-up where its best is that polyline).  Equal
+// best distances of two polylines give b2 = b1, which is never final.
+__device__ __forceinline__ Best<false> warp_best(const Best<false> &s) {
+    Best<false> r;
+    r.b1 = warp_min_pos(s.b1);
+    r.i1 = __shfl_sync(FULL, s.i1, __ffs(__ballot_sync(FULL, s.b1 == r.b1)) - 1);
+    r.b2 = warp_min_pos(s.i1 == r.i1 ? s.b2 : s.b1);
+    return r;
+}
+
+// The smallest FP64 (squared distance, id) over a cell's list, by a warp.
+__device__ __forceinline__ Best64 list_best64(const RefineArgs &a, int g0, int g1, double2 p, int lane) {
+    Best64 st{__longlong_as_double(0x7ff0000000000000LL), 0x7fffffff, -1};
+    for (int g = g0 + lane; g < g1; g += 32) {
+        const int i = a.cseg_ids[g];
+        consider64(st, seg_d2(a.seg, p, i), seg_owner(a.seg, i), i);
+    }
+    for (int o = 16; o > 0; o >>= 1)
+        consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
+                   __shfl_xor_sync(FULL, st.seg, o));
+    return st;
+}
+
+constexpr int DIRECT_WARPS = 8;
+constexpr int DIRECT_OPEN = 64;   // points of a block whose work item matters
+
+template <bool F64>
+__global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, DirectArgs g, int n) {
+    __shared__ int open[DIRECT_OPEN], open_n, box[4];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const double INF = __longlong_as_double(0x7ff0000000000000LL);
+    const float FINF = __int_as_float(0x7f800000);
+    unsigned long long c_tests = 0, c_pairs = 0, c_algo = 0;
+    unsigned c_items = 0, c_fb = 0, c_hits = 0;
+    if (!F64) {
+        if (threadIdx.x == 0) open_n = 0;
+        __syncthreads();
+    }
+    auto put = [&](int i, int id, double d) {   // one lane
+        g.out_id[i] = id;
+        if (g.out_d) g.out_d[i] = d;
+        c_hits += id >= 0;
+    };
+    auto redo = [&](int i, int g0, int g1, double2 p) {
+        const Best64 st = list_best64(a, g0, g1, p, lane);
+        const double d = sqrt(st.d2);
+        const bool hit = st.seg >= 0 && d <= a.D;
+        if (lane == 0) {
+            ++c_fb;
+            if (F64) a.rec[i] = hit ? P2PRec{st.seg, -1} : P2PRec{-1, -1};
+            else put(i, hit ? st.id : -1, hit ? d : INF);
+        }
+    };
+    for (int i = blockIdx.x * DIRECT_WARPS + w; i < n; i += gridDim.x * DIRECT_WARPS) {
+        const double2 p = a.pts[i];
+        int ix, iy, g0 = 0, g1 = 0;
+        const bool sx = axis_estimate(p.x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, ix);
+        const bool sy = axis_estimate(p.y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, iy);
+        const int c = sx && sy ? iy * a.g.nx + ix : point_cell_xy(a.g, p.x, p.y, ix, iy);
+        if (c < a.g.G) {
+            g0 = a.cseg_start[c];
+            g1 = a.cseg_start[c + 1];
+            if (lane == 0) {
+                const int nc = g.cand_start[c + 1] - g.cand_start[c];
+                c_items += nc > 0;
+                c_pairs += nc;
+                c_algo += nc > 0 ? g.cell_algo[c] : 0;
+            }
+        }
+        if (g0 == g1) {
+            if (lane == 0) {
+                if (F64) a.rec[i] = P2PRec{-1, -1};
+                else put(i, -1, INF);
+            }
+            continue;
+        }
+        float hx, lx, hy, ly;
+        split_double(p.x, hx, lx);
+        split_double(p.y, hy, ly);
+        const float2 pt = make_float2(rel_coord(hx, lx, a.frame_x[ix]), rel_coord(hy, ly, a.frame_y[iy]));
+        const float pmag = fmaxf(fabsf(pt.x), fabsf(pt.y));
+        const float4 own = make_float4(pt.x, pt.x, pt.y, pt.y);
+        Best<F64> all = best_none((Best<F64> *)nullptr), kept = all;
+        float mag_all = F64 ? pmag : g.cell_mag, mag = pmag;
+        int tests = 0;
+        for (int b = g0; b < g1; b += 32) {
+            const int k = b + lane;
+            bool keep = false;
+            if (k < g1 && SJ_IN_BOUNDS(k < a.cseg_start[a.g.G], BND_P2P_REC)) {
+                const float4 r0 = __ldg(a.cseg_rec + 2 * (size_t)k), r1 = __ldg(a.cseg_rec + 2 * (size_t)k + 1);
+                const float d = rec_d2(pt, r0, r1.x);
+                const int tag = __float_as_int(F64 ? r1.w : r1.y);
+                keep = rec_near(a, r0, r1.z, own, pmag);
+                consider(all, d, tag);
+                mag_all = fmaxf(mag_all, r1.z);
+                if (!F64 && keep) {
+                    consider(kept, d, tag);
+                    mag = fmaxf(mag, r1.z);
+                }
+            }
+            tests += __popc(__ballot_sync(FULL, keep));
+        }
+        c_tests += lane == 0 ? tests : 0;
+        mag_all = warp_max(mag_all);
+        if constexpr (F64) {
+            // segments within 2E of the best: a record for one or two of them
+            const float e = fmaf(64.0f * U32, mag_all, 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
+            const float d = sqrtf(warp_min_pos(all.b1)), sep = 2.0f * e * (1.0f + 4.0f * U32);
+            const bool n1 = !((sqrtf(all.b1) - d) * (1.0f - 4.0f * U32) > sep);
+            const bool n2 = !((sqrtf(all.b2) - d) * (1.0f - 4.0f * U32) > sep);
+            const bool n3 = !((sqrtf(all.b3) - d) * (1.0f - 4.0f * U32) > sep);
+            const unsigned m1 = __ballot_sync(FULL, n1), m2 = __ballot_sync(FULL, n2);
+            const bool three = __any_sync(FULL, n3) || __popc(m1) + __popc(m2) > 2;
+            const int l1 = __ffs(m1) - 1, l2 = m2 ? l1 : 31 - __clz(m1);
+            P2PRec r;
+            r.id = __shfl_sync(FULL, all.i1, max(l1, 0));
+            r.aux = __shfl_sync(FULL, m2 ? all.i2 : all.i1, max(l2, 0));
+            if (__popc(m1) + __popc(m2) < 2) r.aux = -1;
+            const bool out = (d - e) * (1.0f - 4.0f * U32) > a.Dup;
+            if (!(e < FINF) || (!out && three)) redo(i, g0, g1, p);
+            else if (lane == 0) a.rec[i] = out ? P2PRec{-1, -1} : r;
+        } else {
+            all = warp_best(all);
+            kept = warp_best(kept);
+            mag = warp_max(mag);
+            const int low = fp32x_decide(a, kept, mag);   // outside: nothing nearer was left out
+            if (low == 2) {
+                redo(i, g0, g1, p);
+            } else if (low == 0) {
+                if (lane == 0) put(i, -1, INF);
+            } else if (fp32x_decide(a, all, mag_all) == 1) {
+                if (lane == 0) put(i, kept.i1, widen(sqrtf(kept.b1)));
+            } else if (lane == 0) {
+                const int o = atomicAdd(&open_n, 1);
+                if (SJ_IN_BOUNDS(o < DIRECT_OPEN, BND_P2P_RES)) open[o] = i;
+            }
+        }
+    }
+    if (!F64) {
+        __syncthreads();
+        const int m = min(open_n, DIRECT_OPEN);
+        for (int k = 0; k < m; ++k) {
+            const int i = open[k];
+            const double2 p = a.pts[i];
+            int ix, iy;
+            const int c = point_cell_xy(a.g, p.x, p.y, ix, iy);
+            const float2 fo = make_float2(a.frame_x[ix], a.frame_y[iy]);
+            __syncthreads();
+            if (threadIdx.x < 4) box[threadIdx.x] = float_key((threadIdx.x & 1) ? -FINF : FINF);
+            __syncthreads();
+            for (int j0 = threadIdx.x; j0 < n; j0 += 8 * DIRECT_WARPS * 32) {
+                double2 r[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int j = j0 + u * DIRECT_WARPS * 32;
+                    r[u] = j < n ? a.pts[j] : make_double2(INF, INF);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    int x, y;
+                    // within one column and row by the estimate, then exactly
+                    axis_estimate(r[u].x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, x);
+                    axis_estimate(r[u].y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, y);
+                    if (a.g.tolx < 0.5f && a.g.toly < 0.5f && (abs(x - ix) > 1 || abs(y - iy) > 1)) continue;
+                    if (point_cell(a.g, r[u].x, r[u].y) != c) continue;
+                    float ax, bx, ay, by;
+                    split_double(r[u].x, ax, bx);
+                    split_double(r[u].y, ay, by);
+                    const int kx = float_key(rel_coord(ax, bx, fo.x)), ky = float_key(rel_coord(ay, by, fo.y));
+                    atomicMin(&box[0], kx);
+                    atomicMax(&box[1], kx);
+                    atomicMin(&box[2], ky);
+                    atomicMax(&box[3], ky);
+                }
+            }
+            __syncthreads();
+            if (w == 0) {
+                const int g0 = a.cseg_start[c], g1 = a.cseg_start[c + 1];
+                const float4 item = make_float4(key_float(box[0]), key_float(box[1]), key_float(box[2]), key_float(box[3]));
+                const float pmag = fmaxf(fmaxf(fabsf(item.x), fabsf(item.y)), fmaxf(fabsf(item.z), fabsf(item.w)));
+                float hx, lx, hy, ly;
+                split_double(p.x, hx, lx);
+                split_double(p.y, hy, ly);
+                const float2 pt = make_float2(rel_coord(hx, lx, fo.x), rel_coord(hy, ly, fo.y));
+                Best<false> st = best_none((Best<false> *)nullptr);
+                float mag = pmag;
+                for (int q = g0 + lane; q < g1; q += 32) {
+                    const float4 r0 = a.cseg_rec[2 * (size_t)q], r1 = a.cseg_rec[2 * (size_t)q + 1];
+                    if (!rec_near(a, r0, r1.z, item, pmag)) continue;
+                    consider(st, rec_d2(pt, r0, r1.x), __float_as_int(r1.y));
+                    mag = fmaxf(mag, r1.z);
+                }
+                __syncwarp();
+                st = warp_best(st);
+                mag = warp_max(mag);
+                if (fp32x_decide(a, st, mag) == 1) {
+                    if (lane == 0) put(i, st.i1, widen(sqrtf(st.b1)));
+                } else {
+                    redo(i, g0, g1, p);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (a.stats) {
+        unsigned long long v[ST_N] = {};
+        v[ST_ITEMS] = __shfl_sync(FULL, c_items, 0);
+        v[ST_PAIRS] = c_pairs;
+        v[ST_TESTS] = c_tests;
+        v[ST_ALGO] = c_algo;
+        v[ST_FALLBACK] = c_fb;
+        v[ST_HITS] = c_hits;
+        flush_stats(a.stats, v);   // lane 0's
+    }
+}
+
+// Points of a call per warp of the grid (every resident warp once, then more
+// each); DIRECT_OPEN bounds the points of a block.
+cudaError_t launch_p2p_direct(const RefineArgs &a, const DirectArgs &g, int form, int n, int sms, cudaStream_t s) {
+    const int blocks = std::max(1, std::min((n + DIRECT_WARPS - 1) / DIRECT_WARPS, sms * 8));
+    if (form == SJ_FP32X) {
+        if ((long long)n > (long long)blocks * DIRECT_OPEN) return cudaErrorInvalidValue;
+        k_p2p_direct<false><<<blocks, DIRECT_WARPS * 32, 0, s>>>(a, g, n);
+    } else {
+        k_p2p_direct<true><<<blocks, DIRECT_WARPS * 32, 0, s>>>(a, g, n);
+    }
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ outputs in input order
 
 // FP32X: out[i] from the record of i's slot (pos[i], -1: no slot): the id and
@@ -577,7 +864,7 @@ struct FinOne {
     int n;
     double window;
     __device__ __forceinline__ int count() const { return n; }
-    __device__ __forceinline__ int slot(int i) const { return pos[i]; }
+    __device__ __forceinline__ int slot(int i) const { return pos ? pos[i] : i; }   // no pos: records by point
     __device__ __forceinline__ double2 point(int i) const { return pts[i]; }
     __device__ __forceinline__ double win(int) const { return window; }
     __device__ __forceinline__ void put(int i, int id, double d) const {
@@ -736,10 +1023,11 @@ static void finish(const RefineArgs &a, int form, const Src &src, long long n_ma
             a.seg, a.rec, src, a.stats);
 }
 
-// a8: outputs in input order from the slots' records (pos: slot of each input point or -1).
+// a8: outputs in input order from the slots' records (pos: slot of each input
+// point or -1; null: the records are by input point).
 cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int n, int *out_id, double *out_d,
                               cudaStream_t s) {
-    if (form == SJ_FP32X && ((uintptr_t)out_id & 7) == 0 && ((uintptr_t)out_d & 15) == 0)
+    if (form == SJ_FP32X && pos && ((uintptr_t)out_id & 7) == 0 && ((uintptr_t)out_d & 15) == 0)
         k_p2p_finish_pairs<<<fin_blocks(((n + 1LL) / 2 + FIN_U - 1) / FIN_U, 256, 152 * 16), 256, 0, s>>>(
             a.seg, pos, a.rec, a.pts, n, out_id, out_d);
     else
