@@ -133,12 +133,20 @@ __device__ __forceinline__ int2 point_cell_exact(const GridDev &g, double x, dou
 }
 
 // Cell id of a point (Sec. III.A), G when it lies outside the half-open grid
-// box or has a NaN or infinite coordinate; (ix, iy) its column and row.
+// box or has a NaN or infinite coordinate; (ix, iy) its column and row.  The
+// estimate settles all but the points near a cell boundary (0.1 % at 512 cells
+// per axis); the tables' four 8-byte loads per axis at random places were most
+// of the cell-id pass's L1 traffic (170 M points: the join 12.39 -> 12.21 ms, the
+// pass's atomics bound it now).
 __device__ __forceinline__ int point_cell_xy(const GridDev &g, double x, double y, int &ix, int &iy) {
-    const int2 e = point_cell_exact(g, x, y);
-    ix = e.x;
-    iy = e.y;
-    if (ix < 0 || iy < 0) return g.G;
+    const bool sx = axis_estimate(x, g.x0f, g.icwf, g.tolx, g.nx, ix);
+    const bool sy = axis_estimate(y, g.y0f, g.ichf, g.toly, g.ny, iy);
+    if (!(sx && sy)) {
+        const int2 e = point_cell_exact(g, x, y);
+        ix = e.x;
+        iy = e.y;
+        if (ix < 0 || iy < 0) return g.G;
+    }
     return iy * g.nx + ix;
 }
 __device__ __forceinline__ int point_cell(const GridDev &g, double x, double y) {

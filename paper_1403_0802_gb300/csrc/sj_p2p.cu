@@ -618,9 +618,7 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
     for (int i = blockIdx.x * DIRECT_WARPS + w; i < n; i += gridDim.x * DIRECT_WARPS) {
         const double2 p = a.pts[i];
         int ix, iy, g0 = 0, g1 = 0;
-        const bool sx = axis_estimate(p.x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, ix);
-        const bool sy = axis_estimate(p.y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, iy);
-        const int c = sx && sy ? iy * a.g.nx + ix : point_cell_xy(a.g, p.x, p.y, ix, iy);
+        const int c = point_cell_xy(a.g, p.x, p.y, ix, iy);
         if (c < a.g.G) {
             g0 = a.cseg_start[c];
             g1 = a.cseg_start[c + 1];
