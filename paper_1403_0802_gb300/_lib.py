@@ -132,6 +132,8 @@ def use(path: str):
 
 def lib():
     global _lib
+    if _lib is not None:   # set once, under the lock
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(SO):

@@ -12,6 +12,7 @@ sizes of the C ABI in include/sj.h.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 
 import numpy as np
 import torch
@@ -27,8 +28,8 @@ def _grid(g) -> L.sj_grid:
 
 
 def _stream(stream) -> int | None:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:   # the current stream's handle, without building a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
 
 
@@ -38,6 +39,18 @@ def _opts(form="fp64", launch="per_request", pts_per_item=0, time_refine=False, 
     if subcell is not None:
         flags |= L.SJ_FLAG_SUBCELL_ON if subcell else L.SJ_FLAG_SUBCELL_OFF
     return L.sj_opts(FORMS[form], LAUNCHES[launch], int(block), int(pts_per_item), int(edges_per_chunk), flags)
+
+
+@functools.lru_cache(maxsize=256)
+def _opts_kept(*settings):
+    return C.pointer(_opts(*settings))   # the library only reads it
+
+
+def _opts_ref(form="fp64", launch="per_request", pts_per_item=0, time_refine=False, subcell=None, block=0,
+              edges_per_chunk=0):
+    """Pointer to the sj_opts of these settings, kept between calls by their plain values."""
+    return _opts_kept(form, launch, int(pts_per_item), bool(time_refine), None if subcell is None else bool(subcell),
+                      int(block), int(edges_per_chunk))
 
 
 def _dev(a, dtype, device="cuda") -> torch.Tensor:
@@ -145,8 +158,8 @@ def pip_join(layer: Layer, pts, out: torch.Tensor | None = None, form: str = "fp
     edges_per_chunk shape the polyline join's work items and do nothing here."""
     p = _points(pts)
     out = torch.empty(p.shape[0], dtype=torch.int32, device=p.device) if out is None else out
-    o = _opts(form, launch, pts_per_item, time_refine, subcell, block, edges_per_chunk)
-    L.check(L.lib().sj_pip_join(layer.handle, _ptr(p), p.shape[0], _ptr(out), C.byref(o), _stream(stream)),
+    o = _opts_ref(form, launch, pts_per_item, time_refine, subcell, block, edges_per_chunk)
+    L.check(L.lib().sj_pip_join(layer.handle, _ptr(p), p.shape[0], _ptr(out), o, _stream(stream)),
             "sj_pip_join")
     return out
 
@@ -163,13 +176,13 @@ def p2p_join(layer: Layer, pts, out_id: torch.Tensor | None = None, out_d: torch
     n = p.shape[0]
     out_id = torch.empty(n, dtype=torch.int32, device=p.device) if out_id is None else out_id
     out_d = torch.empty(n, dtype=torch.float64, device=p.device) if out_d is None else out_d
-    o = _opts(form, launch, pts_per_item, time_refine, subcell, block, edges_per_chunk)
+    o = _opts_ref(form, launch, pts_per_item, time_refine, subcell, block, edges_per_chunk)
     if window is None:
-        L.check(L.lib().sj_p2p_join(layer.handle, _ptr(p), n, _ptr(out_id), _ptr(out_d), C.byref(o),
+        L.check(L.lib().sj_p2p_join(layer.handle, _ptr(p), n, _ptr(out_id), _ptr(out_d), o,
                                     _stream(stream)), "sj_p2p_join")
     else:
         L.check(L.lib().sj_p2p_join_window(layer.handle, _ptr(p), n, float(window), _ptr(out_id), _ptr(out_d),
-                                           C.byref(o), _stream(stream)), "sj_p2p_join_window")
+                                           o, _stream(stream)), "sj_p2p_join_window")
     return out_id, out_d
 
 
@@ -182,8 +195,8 @@ def p2p_join_noalloc(layer: Layer, pts, out_id: torch.Tensor, out_d: torch.Tenso
     the points must already be a float64 [N, 2] CUDA tensor."""
     if not (isinstance(pts, torch.Tensor) and pts.is_cuda and pts.dtype == torch.float64 and pts.is_contiguous()):
         raise ValueError("points must be a contiguous float64 [N, 2] CUDA tensor")
-    o = _opts(form)
-    L.check(L.lib().sj_p2p_join_noalloc(layer.handle, _ptr(pts), pts.shape[0], _ptr(out_id), _ptr(out_d), C.byref(o),
+    o = _opts_ref(form)
+    L.check(L.lib().sj_p2p_join_noalloc(layer.handle, _ptr(pts), pts.shape[0], _ptr(out_id), _ptr(out_d), o,
                                         _stream(stream)), "sj_p2p_join_noalloc")
     return out_id, out_d
 
@@ -203,10 +216,10 @@ def pip_join_host(layer: Layer, pts: np.ndarray, out: np.ndarray | None = None, 
     p = np.ascontiguousarray(pts, dtype=np.float64) if not isinstance(pts, torch.Tensor) else pts
     n = p.shape[0]
     out = np.empty(n, np.int32) if out is None else out
-    o = _opts(form, pts_per_item=pts_per_item, block=block, edges_per_chunk=edges_per_chunk)
+    o = _opts_ref(form, pts_per_item=pts_per_item, block=block, edges_per_chunk=edges_per_chunk)
     pp = p.data_ptr() if isinstance(p, torch.Tensor) else p.ctypes.data
     op = out.data_ptr() if isinstance(out, torch.Tensor) else out.ctypes.data
-    L.check(L.lib().sj_pip_join_host(layer.handle, pp, n, op, C.byref(o), _stream(stream)), "sj_pip_join_host")
+    L.check(L.lib().sj_pip_join_host(layer.handle, pp, n, op, o, _stream(stream)), "sj_pip_join_host")
     return out
 
 
@@ -217,14 +230,14 @@ def p2p_join_host(layer: Layer, pts, out_id=None, out_d=None, form: str = "fp64"
     n = p.shape[0]
     out_id = np.empty(n, np.int32) if out_id is None else out_id
     out_d = np.empty(n, np.float64) if out_d is None else out_d
-    o = _opts(form, pts_per_item=pts_per_item, block=block, edges_per_chunk=edges_per_chunk)
+    o = _opts_ref(form, pts_per_item=pts_per_item, block=block, edges_per_chunk=edges_per_chunk)
     ptr = lambda a: a.data_ptr() if isinstance(a, torch.Tensor) else a.ctypes.data
     if window is None:
-        L.check(L.lib().sj_p2p_join_host(layer.handle, ptr(p), n, ptr(out_id), ptr(out_d), C.byref(o),
+        L.check(L.lib().sj_p2p_join_host(layer.handle, ptr(p), n, ptr(out_id), ptr(out_d), o,
                                          _stream(stream)), "sj_p2p_join_host")
     else:
         L.check(L.lib().sj_p2p_join_window_host(layer.handle, ptr(p), n, float(window), ptr(out_id), ptr(out_d),
-                                                C.byref(o), _stream(stream)), "sj_p2p_join_window_host")
+                                                o, _stream(stream)), "sj_p2p_join_window_host")
     return out_id, out_d
 
 

@@ -1020,9 +1020,13 @@ extern "C" sj_status sj_p2p_join_window(const sj_layer *L, const double *pts, in
 // its chunk's join), so that copies in, joins and copies out of different
 // chunks overlap (both copy directions and the SMs work at once).  Each chunk
 // is an independent join (a point's result does not depend on the other
-// points), so the outputs equal those of one join over all N points.  At most
+// points), so the outputs equal those of one join over all N points.  P2P: at most
 // three chunks: every chunk is a full join with fixed costs (scans over every
-// cell, sparser work items), so four quarter joins were measured slower.
+// cell, sparser work items), so four quarter joins were measured slower.  PIP:
+// a join costs its points and a launch, so chunks of about HOST_PIP_CHUNK points
+// keep the first join's wait and the last copy out short (5 M points: 585 us with
+// two chunks, 535 / 517 / 526 with chunks of 0.5 / 1 / 2 M).
+constexpr int64_t HOST_PIP_CHUNK = 1 << 20, HOST_MAX_CHUNKS = 16;
 static sj_status join_host(const sj_layer *L, int kind, const double *pts, int64_t N, int32_t *out_id, double *out_d,
                            const sj_opts *o, void *stream, double window = -1.0) {
     if (N < 0 || N > MAX_COUNT) return fail(SJ_ERR_INVALID, "N out of range (at most 2^31 - 2^22)");
@@ -1036,12 +1040,18 @@ static sj_status join_host(const sj_layer *L, int kind, const double *pts, int64
     sj_status st = device_info(dev, &di);
     if (st != SJ_OK) return st;
     cudaStream_t t_in = di->hstream[0], t_cmp = di->hstream[1], t_out = di->hstream[2];
-    // chunk bounds: one chunk up to 2 M points, halves up to 8 M, else quarter /
+    // chunk bounds, P2P: one chunk up to 2 M points, halves up to 8 M, else quarter /
     // half / quarter (a short first chunk starts the joins early, a short last
     // one keeps the final copy out short)
-    int64_t bound[4] = {0, N, N, N};
+    int64_t bound[HOST_MAX_CHUNKS + 1] = {0, N, N, N};
     int nchunks = 1;
-    if (N > (int64_t)8 << 20) {
+    if (kind == KIND_PIP) {
+        nchunks = (int)std::min<int64_t>(HOST_MAX_CHUNKS, (N + HOST_PIP_CHUNK - 1) / HOST_PIP_CHUNK);
+        // equal chunks of an even number of points (the device results of each
+        // start aligned)
+        const int64_t size = ((N + nchunks - 1) / nchunks + 63) & ~(int64_t)63;
+        for (int c = 1; c <= nchunks; ++c) bound[c] = std::min(N, size * c);
+    } else if (N > (int64_t)8 << 20) {
         bound[1] = N / 4;
         bound[2] = N - N / 4;
         nchunks = 3;
@@ -1067,6 +1077,7 @@ static sj_status join_host(const sj_layer *L, int kind, const double *pts, int64
     for (int c = 0; c < nchunks && e == cudaSuccess && st == SJ_OK; ++c) {
         cudaEvent_t copied = evs[2 + 2 * c], joined = evs[3 + 2 * c];
         const int64_t off = bound[c], n = bound[c + 1] - off;
+        if (n == 0) continue;
         e = cudaMemcpyAsync(dp + 2 * off, pts + 2 * off, (size_t)n * 16, cudaMemcpyHostToDevice, t_in);
         if (e == cudaSuccess) e = cudaEventRecord(copied, t_in);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(t_cmp, copied, 0);
