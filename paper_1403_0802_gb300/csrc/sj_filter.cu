@@ -330,16 +330,10 @@ struct BucketApply {
     unsigned long long *stats;
     __device__ void done(const Acc &acc) const {
         if (!stats) return;
-        unsigned long long p = acc.pairs, q = acc.algo;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            p += __shfl_xor_sync(FULL, p, o);
-            q += __shfl_xor_sync(FULL, q, o);
-        }
         unsigned long long v[ST_N] = {};
-        v[ST_PAIRS] = p;
-        v[ST_ALGO] = q;
-        flush_stats(stats, v);
+        v[ST_PAIRS] = warp_sum(acc.pairs);
+        v[ST_ALGO] = warp_sum(acc.algo);
+        flush_stats<SCAN_T / 32>(stats, v);
     }
     __device__ void operator()(int c, int2 ex, int2 v, int n, Acc &acc) const {
         if (stats && v.y > 0) {

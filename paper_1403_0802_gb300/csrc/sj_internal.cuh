@@ -232,19 +232,33 @@ enum { KIND_PIP = 0, KIND_P2P = 1 };
 enum { ST_POINTS = 0, ST_ITEMS, ST_PAIRS, ST_TESTS, ST_FALLBACK, ST_HITS, ST_ALGO, ST_RESOLVED, ST_N };
 
 // Adds counters to the layer's statistics with one global atomic per counter
-// and block: every lane 0 of the block's warps passes its warp's values
-// (others pass zeros), the block sums them in shared memory first.  Every
-// thread of the block must call it (it synchronises the block).  Thousands of
-// warps adding to the same few addresses would otherwise queue at the L2.
+// and block: every lane 0 of the block's NW warps passes its warp's values
+// (others pass anything), which are summed over the block's shared memory.
+// Every thread of the block must call it (it synchronises the block).
+// Thousands of warps adding to the same few addresses would otherwise queue at
+// the L2; a shared 64-bit atomic per counter and warp instead of the plain
+// stores cost a small call 1 us.
+template <int NW>
 __device__ __forceinline__ void flush_stats(unsigned long long *stats, const unsigned long long *v) {
-    __shared__ unsigned long long blk[ST_N];
-    if (threadIdx.x < ST_N) blk[threadIdx.x] = 0;
-    __syncthreads();
+    __shared__ unsigned long long blk[NW][ST_N];
     if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < ST_N; ++k)
-            if (v[k]) atomicAdd(&blk[k], v[k]);
+#pragma unroll
+        for (int k = 0; k < ST_N; ++k) blk[threadIdx.x >> 5][k] = v[k];
     __syncthreads();
-    if (threadIdx.x < ST_N && blk[threadIdx.x]) atomicAdd(&stats[threadIdx.x], blk[threadIdx.x]);
+    if (threadIdx.x < ST_N) {
+        unsigned long long t = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) t += blk[w][threadIdx.x];
+        if (t) atomicAdd(&stats[threadIdx.x], t);
+    }
+}
+
+// Sum of the lanes' counters: in 32 bits while they are small.
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+    if (!__any_sync(FULL, (v >> 26) != 0)) return __reduce_add_sync(FULL, (unsigned)v);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
 }
 
 // What the P2P refinement leaves in a slot, for the finishing kernels.

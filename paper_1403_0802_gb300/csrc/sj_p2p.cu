@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
         v[ST_TESTS] = c_tests;
         v[ST_FALLBACK] = __reduce_add_sync(FULL, c_fb);
         v[ST_HITS] = __reduce_add_sync(FULL, c_hits);
-        flush_stats(a.stats, v);
+        flush_stats<NW>(a.stats, v);
     }
 }
 
@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
         v[ST_ALGO] = c_algo;
         v[ST_FALLBACK] = c_fb;
         v[ST_HITS] = c_hits;
-        flush_stats(a.stats, v);   // lane 0's
+        flush_stats<DIRECT_WARPS>(a.stats, v);   // lane 0's
     }
 }
 
@@ -1003,7 +1003,7 @@ __global__ void __launch_bounds__(FIN_WARPS * 32) k_p2p_finish_fp64(SegArgs a, c
     if (stats) {
         unsigned long long v[ST_N] = {};
         v[ST_HITS] = __reduce_add_sync(FULL, hits);
-        flush_stats(stats, v);
+        flush_stats<FIN_WARPS>(stats, v);
     }
 }
 

@@ -460,21 +460,15 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
     }
     if (a.stats) {
         unsigned long long v[ST_N] = {};
-        PipSums s = sums[threadIdx.x];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s.tests += __shfl_xor_sync(FULL, s.tests, o);
-            s.pairs += __shfl_xor_sync(FULL, s.pairs, o);
-            s.algo += __shfl_xor_sync(FULL, s.algo, o);
-        }
+        const PipSums s = sums[threadIdx.x];
         v[ST_ITEMS] = items;
-        v[ST_PAIRS] = s.pairs;
-        v[ST_TESTS] = s.tests;
-        v[ST_ALGO] = s.algo;
+        v[ST_PAIRS] = warp_sum(s.pairs);
+        v[ST_TESTS] = warp_sum(s.tests);
+        v[ST_ALGO] = warp_sum(s.algo);
         v[ST_RESOLVED] = __reduce_add_sync(FULL, resolved);
         v[ST_FALLBACK] = __reduce_add_sync(FULL, fb);
         v[ST_HITS] = __reduce_add_sync(FULL, hits);
-        flush_stats(a.stats, v);
+        flush_stats<PIP_WARPS>(a.stats, v);
     }
 }
 
