@@ -21,8 +21,8 @@ cudaError_t launch_check_finite(const double2 *v, int n, int *bad, cudaStream_t 
 cudaError_t launch_pip_topology(const int *ring_off, int R, const int *poly_ring_off, int P, int V, int *poly_voff,
                                 int *nxt, int *prv, int *owner, cudaStream_t s);
 cudaError_t launch_split(const double2 *v, int n, float4 *vs, cudaStream_t s);
-cudaError_t launch_seg_table(const double2 *v, const int *line_off, int L, double2 *e64, double *inv64, float4 *seg32,
-                             cudaStream_t s);
+cudaError_t launch_seg_table(const double2 *v, const int *line_off, int L, int V, double2 *e64, double *inv64,
+                             float4 *seg32, cudaStream_t s);
 cudaError_t launch_mbb(const LayerBuildArgs &a, cudaStream_t s);
 cudaError_t launch_raster_count(const LayerBuildArgs &a, unsigned long long *total, cudaStream_t s);
 cudaError_t launch_raster_emit(const LayerBuildArgs &a, int2 *pairs, int M, int *cand_ids, cudaStream_t s);
@@ -293,6 +293,26 @@ static sj_status read_flag(int *dflag, cudaStream_t s, int *out) {
     return SJ_OK;
 }
 
+// Build scratch: stream-ordered allocations, freed with the object.
+struct BuildTmp {
+    cudaStream_t s;
+    std::vector<void *> ptrs;
+    explicit BuildTmp(cudaStream_t st) : s(st) {}
+    ~BuildTmp() {
+        for (void *p : ptrs) cudaFreeAsync(p, s);
+    }
+    template <class T>
+    cudaError_t take(T **p, size_t n) {
+        void *q = nullptr;
+        cudaError_t e = dev_malloc_async(&q, (n ? n : 1) * sizeof(T), s);
+        if (e == cudaSuccess) {
+            ptrs.push_back(q);
+            *p = (T *)q;
+        }
+        return e;
+    }
+};
+
 // Shared tail of both layer builders: MBB, cover check, rasterisation, CSR.
 static sj_status build_candidates(sj_layer *L, int *dbad, cudaStream_t s) {
     LayerBuildArgs a{};
@@ -313,19 +333,13 @@ static sj_status build_candidates(sj_layer *L, int *dbad, cudaStream_t s) {
     int2 *block_sums = nullptr, *pairs = nullptr;
     unsigned long long *total = nullptr;
     size_t nbs = bucket_scan_blocks(std::max(L->g.G, L->nobj));
-    struct Tmp {
-        void *p[7] = {};
-        ~Tmp() {
-            for (void *q : p)
-                if (q) cudaFree(q);
-        }
-    } tmp;
-    CUDA_TRY(dalloc(&cell_cnt, (size_t)L->g.G + 1)); tmp.p[0] = cell_cnt;
-    CUDA_TRY(dalloc(&cursor, (size_t)L->g.G)); tmp.p[1] = cursor;
-    CUDA_TRY(dalloc(&obj_cells, (size_t)L->nobj + 1)); tmp.p[2] = obj_cells;
-    CUDA_TRY(dalloc(&block_sums, nbs)); tmp.p[3] = block_sums;
-    CUDA_TRY(dalloc(&totals, 4)); tmp.p[4] = totals;
-    CUDA_TRY(dalloc(&total, 1)); tmp.p[5] = total;
+    BuildTmp tmp(s);
+    CUDA_TRY(tmp.take(&cell_cnt, (size_t)L->g.G + 1));
+    CUDA_TRY(tmp.take(&cursor, (size_t)L->g.G));
+    CUDA_TRY(tmp.take(&obj_cells, (size_t)L->nobj + 1));
+    CUDA_TRY(tmp.take(&block_sums, nbs));
+    CUDA_TRY(tmp.take(&totals, 4));
+    CUDA_TRY(tmp.take(&total, 1));
     CUDA_TRY(cudaMemsetAsync(cell_cnt, 0, sizeof(int) * ((size_t)L->g.G + 1), s));
     CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * (size_t)L->g.G, s));
     CUDA_TRY(cudaMemsetAsync(total, 0, sizeof(unsigned long long), s));
@@ -351,7 +365,7 @@ static sj_status build_candidates(sj_layer *L, int *dbad, cudaStream_t s) {
     L->M = (int64_t)M;
     CUDA_TRY(dalloc(&L->cand_ids, (size_t)M));
     if (L->nobj > 0) {
-        CUDA_TRY(dalloc(&pairs, (size_t)M)); tmp.p[6] = pairs;
+        CUDA_TRY(tmp.take(&pairs, (size_t)M));
         CUDA_TRY(launch_raster_emit(a, pairs, (int)M, L->cand_ids, s));
     } else {
         CUDA_TRY(cudaMemsetAsync(L->cand_start, 0, sizeof(int) * ((size_t)L->g.G + 1), s));
@@ -395,24 +409,18 @@ static sj_status build_seg_lists(sj_layer *L, cudaStream_t s) {
     a.verts = L->verts;
     a.obj_voff = L->obj_voff;
     a.cand_start = L->cand_start;
-    struct Tmp {
-        void *p[7] = {};
-        ~Tmp() {
-            for (void *q : p)
-                if (q) cudaFree(q);
-        }
-    } tmp;
+    BuildTmp tmp(s);
     int *seg_off = nullptr;
     int2 *pairs = nullptr;
     unsigned long long *total = nullptr;
     const size_t nbs = bucket_scan_blocks(std::max(G, V));
-    CUDA_TRY(dalloc(&a.cell_cnt, (size_t)G + 1)); tmp.p[0] = a.cell_cnt;
-    CUDA_TRY(dalloc(&a.cursor, (size_t)G)); tmp.p[1] = a.cursor;
-    CUDA_TRY(dalloc(&seg_off, (size_t)V + 1)); tmp.p[2] = seg_off;
-    CUDA_TRY(dalloc(&a.block_sums, nbs)); tmp.p[3] = a.block_sums;
+    CUDA_TRY(tmp.take(&a.cell_cnt, (size_t)G + 1));
+    CUDA_TRY(tmp.take(&a.cursor, (size_t)G));
+    CUDA_TRY(tmp.take(&seg_off, (size_t)V + 1));
+    CUDA_TRY(tmp.take(&a.block_sums, nbs));
     a.bs_cap = nbs;
-    CUDA_TRY(dalloc(&a.totals, 4)); tmp.p[4] = a.totals;
-    CUDA_TRY(dalloc(&total, 1)); tmp.p[5] = total;
+    CUDA_TRY(tmp.take(&a.totals, 4));
+    CUDA_TRY(tmp.take(&total, 1));
     CUDA_TRY(cudaMemsetAsync(a.cell_cnt, 0, sizeof(int) * ((size_t)G + 1), s));
     CUDA_TRY(cudaMemsetAsync(a.cursor, 0, sizeof(int) * (size_t)G, s));
     CUDA_TRY(cudaMemsetAsync(total, 0, sizeof(unsigned long long), s));
@@ -423,7 +431,7 @@ static sj_status build_seg_lists(sj_layer *L, cudaStream_t s) {
     if (MS > (unsigned long long)MAX_COUNT) return fail(SJ_ERR_INVALID, "more than 2^31 - 2^22 (cell, segment) pairs");
     L->MS = (int64_t)MS;
     CUDA_TRY(dalloc(&L->cseg_ids, (size_t)MS));
-    CUDA_TRY(dalloc(&pairs, (size_t)MS)); tmp.p[6] = pairs;
+    CUDA_TRY(tmp.take(&pairs, (size_t)MS));
     CUDA_TRY(launch_segcell_emit(a, L->seg32, L->seg_e64, seg_off, pairs, (int)MS, L->cand_ids, L->cseg_start,
                                  L->cseg_ids, L->cell_algo, s));
     CUDA_TRY(dalloc(&L->cseg_rec, 2 * (size_t)MS));
@@ -434,26 +442,6 @@ static sj_status build_seg_lists(sj_layer *L, cudaStream_t s) {
     CUDA_TRY(cudaStreamSynchronize(s));
     return SJ_OK;
 }
-
-// Build scratch: stream-ordered allocations, freed with the object.
-struct BuildTmp {
-    cudaStream_t s;
-    std::vector<void *> ptrs;
-    explicit BuildTmp(cudaStream_t st) : s(st) {}
-    ~BuildTmp() {
-        for (void *p : ptrs) cudaFreeAsync(p, s);
-    }
-    template <class T>
-    cudaError_t take(T **p, size_t n) {
-        void *q = nullptr;
-        cudaError_t e = dev_malloc_async(&q, (n ? n : 1) * sizeof(T), s);
-        if (e == cudaSuccess) {
-            ptrs.push_back(q);
-            *p = (T *)q;
-        }
-        return e;
-    }
-};
 
 // 64-bit counters on the device, read back.
 static sj_status read_totals(const unsigned long long *d, unsigned long long *h, int n, cudaStream_t s) {
@@ -532,7 +520,7 @@ static sj_status build_pip_records(sj_layer *L, const int *prv, const int *owner
     CUDA_TRY(tmp.take(&bs, slots_cap));
     CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)L->MR, s));
     CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * (size_t)L->MR, s));
-    CUDA_TRY(launch_prow_edges(b, cnt, total + 1, nullptr, nullptr, s));
+    CUDA_TRY(launch_prow_edges(b, cnt, total + 1, nullptr, nullptr, nullptr, s));
     // pairs of equal edges, while the list sizes travel
     {
         size_t slots = 64;
@@ -549,9 +537,11 @@ static sj_status build_pip_records(sj_layer *L, const int *prv, const int *owner
     CUDA_TRY(dalloc(&L->prow_start, (size_t)L->MR + 1));
     CUDA_TRY(dalloc(&L->pedge_ids, (size_t)L->ME));
     CUDA_TRY(launch_offsets(cnt, (int)L->MR, L->prow_start, bs, slots_cap, totals, s));
-    CUDA_TRY(launch_prow_edges(b, cursor, nullptr, L->prow_start, L->pedge_ids, s));
+    PipRow *rows = nullptr;
+    CUDA_TRY(tmp.take(&rows, (size_t)L->ME));
+    CUDA_TRY(launch_prow_edges(b, cursor, nullptr, L->prow_start, L->pedge_ids, rows, s));
     b.prow_start = L->prow_start;
-    b.pedge = L->pedge_ids;
+    b.rows = rows;
 
     // what each entry and cell holds; delta = 1e-7 of the largest grid coordinate
     // (0.01 m at 1e5 m) is far above FP64 rounding and far below a cell
@@ -714,7 +704,7 @@ extern "C" sj_status sj_p2p_layer_create(const double *verts, int64_t V, const i
     CUDA_TRY(dalloc(&L->seg32, (size_t)V));
     if (V > 0) {
         CUDA_TRY(launch_split(L->verts, (int)V, L->vsplit, s));
-        CUDA_TRY(launch_seg_table(L->verts, L->obj_voff, Lc, L->seg_e64, L->seg_inv64, L->seg32, s));
+        CUDA_TRY(launch_seg_table(L->verts, L->obj_voff, Lc, (int)V, L->seg_e64, L->seg_inv64, L->seg32, s));
     }
     CUDA_TRY(dalloc(&L->stats, ST_N));
     CUDA_TRY(cudaMemsetAsync(L->stats, 0, sizeof(unsigned long long) * ST_N, s));

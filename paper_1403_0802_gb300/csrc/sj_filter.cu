@@ -189,23 +189,49 @@ struct OffsetApply {
 // ------------------------------------------------------------------ cell threshold tables
 
 // keys[k] = order key of the smallest double v with floor(fl(fl(v - lo) / w)) >= k,
-// k = 0..n, by binary search over the order keys of [-inf, +inf] (the rule is
-// monotone in v, false at -inf and true at +inf).  64 steps per threshold.
-__global__ void k_axis_thresholds(double lo, double w, int n, unsigned long long *keys) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > n) return;
+// k = 0..n (the rule is monotone in v, false at -inf and true at +inf): the
+// bracket grows by doubling from lo + k w, which is a few ulps off (a bisection
+// of all doubles takes 64 FP64 divisions in a row: 64 us an axis, 9 us now),
+// then halves.  Both axes in one launch.
+__device__ unsigned long long axis_threshold(double lo, double w, int k) {
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
-    unsigned long long a = order_key(-INF), b = order_key(INF);
+    const unsigned long long kmin = order_key(-INF), kmax = order_key(INF);
+    auto reached = [&](unsigned long long m) { return axis_floor(key_value(m), lo, w) >= (double)k; };
+    const unsigned long long near = order_key(__dadd_rn(lo, __dmul_rn((double)k, w)));
+    const unsigned long long g = near > kmin && near < kmax ? near : kmin + (kmax - kmin) / 2;   // NaN, infinities
+    unsigned long long a = kmin, b = kmax;   // rule false at a, true at b
+    if (reached(g)) {
+        b = g;
+        for (int s = 0; s < 63; ++s) {   // at most 63 steps: then a is -inf
+            const unsigned long long step = 1ULL << s;
+            if (g - kmin <= step) break;
+            if (!reached(g - step)) { a = g - step; break; }
+            b = g - step;
+        }
+    } else {
+        a = g;
+        for (int s = 0; s < 63; ++s) {
+            const unsigned long long step = 1ULL << s;
+            if (kmax - g <= step) break;
+            if (reached(g + step)) { b = g + step; break; }
+            a = g + step;
+        }
+    }
     while (b - a > 1) {
         const unsigned long long m = a + (b - a) / 2;
-        if (axis_floor(key_value(m), lo, w) >= (double)k) b = m; else a = m;
+        if (reached(m)) b = m; else a = m;
     }
-    keys[k] = b;
+    return b;
+}
+
+__global__ void k_axis_thresholds(GridDev g, unsigned long long *kx, unsigned long long *ky) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k <= g.nx) kx[k] = axis_threshold(g.x0, g.cw, k);
+    else if (k - g.nx - 1 <= g.ny) ky[k - g.nx - 1] = axis_threshold(g.y0, g.ch, k - g.nx - 1);
 }
 
 cudaError_t launch_thresholds(const GridDev &g, unsigned long long *kx, unsigned long long *ky, cudaStream_t s) {
-    k_axis_thresholds<<<(g.nx + 1 + 127) / 128, 128, 0, s>>>(g.x0, g.cw, g.nx, kx);
-    k_axis_thresholds<<<(g.ny + 1 + 127) / 128, 128, 0, s>>>(g.y0, g.ch, g.ny, ky);
+    k_axis_thresholds<<<(g.nx + g.ny + 2 + 63) / 64, 64, 0, s>>>(g, kx, ky);
     return cudaGetLastError();
 }
 
@@ -531,52 +557,62 @@ cudaError_t launch_frames(const GridDev &g, float *fx, float *fy, cudaStream_t s
 // e = v[i+1] - v[i] and 1 / |e|^2 (0 for a zero-length segment, and for the
 // single vertex of a one-vertex polyline, which then acts as a point); the
 // fourth component holds l as int bits, or -1 for the last vertex of a
-// polyline of two or more vertices (which starts no segment).
-__global__ void k_seg_table(const double2 *v, const int *line_off, int L, double2 *e64, double *inv64,
+// polyline of two or more vertices (which starts no segment).  One thread per
+// vertex, which finds its polyline by binary search.
+__global__ void k_seg_table(const double2 *v, const int *line_off, int L, int V, double2 *e64, double *inv64,
                             float4 *seg32) {
-    for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < L; l += gridDim.x * blockDim.x) {
-        int b = line_off[l], e = line_off[l + 1];
-        for (int i = b; i < e; ++i) {
-            double ex = 0.0, ey = 0.0, inv = 0.0;
-            if (i + 1 < e) {
-                ex = __dsub_rn(v[i + 1].x, v[i].x);
-                ey = __dsub_rn(v[i + 1].y, v[i].y);
-                double L2 = __dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey));
-                inv = L2 > 0.0 ? __ddiv_rn(1.0, L2) : 0.0;
-            }
-            e64[i] = make_double2(ex, ey);
-            inv64[i] = inv;
-            const int owner = (i + 1 < e || e - b == 1) ? l : -1;
-            seg32[i] = make_float4(__double2float_rn(ex), __double2float_rn(ey), __double2float_rn(inv),
-                                   __int_as_float(owner));
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        const int l = run_of(line_off, L, i), b = line_off[l], e = line_off[l + 1];
+        double ex = 0.0, ey = 0.0, inv = 0.0;
+        if (i + 1 < e) {
+            ex = __dsub_rn(v[i + 1].x, v[i].x);
+            ey = __dsub_rn(v[i + 1].y, v[i].y);
+            double L2 = __dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey));
+            inv = L2 > 0.0 ? __ddiv_rn(1.0, L2) : 0.0;
         }
+        e64[i] = make_double2(ex, ey);
+        inv64[i] = inv;
+        const int owner = (i + 1 < e || e - b == 1) ? l : -1;
+        seg32[i] = make_float4(__double2float_rn(ex), __double2float_rn(ey), __double2float_rn(inv),
+                               __int_as_float(owner));
     }
 }
 
 // a3: MBB per object, one warp per object; flags an MBB outside the closed
-// grid box (bit 2 of *bad).
+// grid box (bit 2 of *bad).  The minima are taken over order keys, off the FP64
+// pipe, four vertices per lane in flight.
 __global__ void k_mbb(LayerBuildArgs a) {
+    typedef unsigned long long u64;
     int lane = lane_id();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int o = warp; o < a.nobj; o += nwarps) {
         int b = a.obj_voff[o], e = a.obj_voff[o + 1];
-        double xmin = INFINITY, ymin = INFINITY, xmax = -INFINITY, ymax = -INFINITY;
-        for (int i = b + lane; i < e; i += 32) {
-            double2 p = a.verts[i];
-            xmin = fmin(xmin, p.x); xmax = fmax(xmax, p.x);
-            ymin = fmin(ymin, p.y); ymax = fmax(ymax, p.y);
+        u64 xmin = ~0ULL, ymin = ~0ULL, xmax = 0, ymax = 0;
+        for (int i0 = b + lane; i0 < e; i0 += 4 * 32) {
+            double2 p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i0 + 32 * u < e) p[u] = a.verts[i0 + 32 * u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (i0 + 32 * u >= e) break;
+                const u64 x = order_key(p[u].x), y = order_key(p[u].y);
+                xmin = min(xmin, x); xmax = max(xmax, x);
+                ymin = min(ymin, y); ymax = max(ymax, y);
+            }
         }
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) {
-            xmin = fmin(xmin, __shfl_xor_sync(FULL, xmin, s));
-            ymin = fmin(ymin, __shfl_xor_sync(FULL, ymin, s));
-            xmax = fmax(xmax, __shfl_xor_sync(FULL, xmax, s));
-            ymax = fmax(ymax, __shfl_xor_sync(FULL, ymax, s));
+            xmin = min(xmin, __shfl_xor_sync(FULL, xmin, s));
+            ymin = min(ymin, __shfl_xor_sync(FULL, ymin, s));
+            xmax = max(xmax, __shfl_xor_sync(FULL, xmax, s));
+            ymax = max(ymax, __shfl_xor_sync(FULL, ymax, s));
         }
         if (lane == 0) {
-            a.mbb[o] = Box{xmin, ymin, xmax, ymax};
-            if (!(xmin >= a.g.x0 && xmax <= a.g.x1 && ymin >= a.g.y0 && ymax <= a.g.y1)) atomicOr(a.bad, 2);
+            const Box m{key_value(xmin), key_value(ymin), key_value(xmax), key_value(ymax)};
+            a.mbb[o] = m;
+            if (!(m.xmin >= a.g.x0 && m.xmax <= a.g.x1 && m.ymin >= a.g.y0 && m.ymax <= a.g.y1)) atomicOr(a.bad, 2);
         }
     }
 }
@@ -599,8 +635,7 @@ __device__ __forceinline__ int4 mbb_cell_box(const LayerBuildArgs &a, Box m) {
         xhi = next_up(__dadd_rn(xhi, a.D));
         yhi = next_up(__dadd_rn(yhi, a.D));
     }
-    return make_int4(clamped_axis(xlo, a.g.x0, a.g.cw, a.g.nx), clamped_axis(ylo, a.g.y0, a.g.ch, a.g.ny),
-                     clamped_axis(xhi, a.g.x0, a.g.cw, a.g.nx), clamped_axis(yhi, a.g.y0, a.g.ch, a.g.ny));
+    return make_int4(clamped_col(a.g, xlo), clamped_row(a.g, ylo), clamped_col(a.g, xhi), clamped_row(a.g, yhi));
 }
 
 __global__ void k_raster_count(LayerBuildArgs a, unsigned long long *total) {
@@ -634,30 +669,56 @@ __global__ void k_pair_scatter(const int2 *pairs, int M, const int *start, int *
     }
 }
 
-// Sort each cell's ids ascending: Shell sort with Ciura's gap sequence
-// (1, 4, 10, 23, 57, 132, 301, 701, then x 2.25), one thread per cell.  Lists
-// are short in the common case (one or two gap passes), and a long
-// one (a large D makes every object a candidate of every cell) stays near
-// n^1.3 instead of the n^2 of plain insertion.
-__global__ void k_cand_sort(const int *cand_start, int G, int *cand_ids) {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < G; c += gridDim.x * blockDim.x) {
+// Sort each cell's ids (distinct within a cell) ascending, one warp per cell.
+// Lists of up to 128 ids: every id's place is the number of smaller ones, counted
+// by its lane over the list (L1) and written once all are counted.  Longer lists
+// (a large D makes every object a candidate of every cell): Shell sort with
+// Ciura's gap sequence (1, 4, 10, 23, 57, 132, 301, 701, then x 2.25), near n^1.3,
+// the lanes taking the interleaved sublists of a gap.
+__global__ void __launch_bounds__(256) k_cand_sort(const int *cand_start, int G, int *cand_ids) {
+    const int lane = lane_id();
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int c = warp; c < G; c += nwarps) {
         const int b = cand_start[c], n = cand_start[c + 1] - b;
         int *v = cand_ids + b;
-        const int ciura[8] = {1, 4, 10, 23, 57, 132, 301, 701};
-        int gaps[32];
-        int ng = 0;
-        while (ng < 8 && ciura[ng] < n) { gaps[ng] = ciura[ng]; ++ng; }
-        if (ng == 8) {
-            long long g = 701;
-            while (ng < 32 && (g = g * 9 / 4) < n) gaps[ng++] = (int)g;
-        }
-        for (int t = ng - 1; t >= 0; --t) {
-            const int h = gaps[t];
-            for (int i = h; i < n; ++i) {
-                const int x = v[i];
-                int j = i;
-                while (j >= h && v[j - h] > x) { v[j] = v[j - h]; j -= h; }
-                v[j] = x;
+        if (n <= 1) continue;
+        if (n <= 32) {
+            const int x = lane < n ? v[lane] : 0;
+            int r = 0;
+            for (int j = 0; j < n; ++j) r += __shfl_sync(FULL, x, j) < x;
+            if (lane < n) v[r] = x;
+        } else if (n <= 128) {
+            int x[4], r[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = lane + 32 * u < n ? v[lane + 32 * u] : 0;
+            for (int j = 0; j < n; ++j) {
+                const int y = v[j];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] += y < x[u];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (lane + 32 * u < n) v[r[u]] = x[u];
+        } else {
+            const int ciura[8] = {1, 4, 10, 23, 57, 132, 301, 701};
+            int gaps[32];
+            int ng = 0;
+            while (ng < 8 && ciura[ng] < n) { gaps[ng] = ciura[ng]; ++ng; }
+            if (ng == 8) {
+                long long g = 701;
+                while (ng < 32 && (g = g * 9 / 4) < n) gaps[ng++] = (int)g;
+            }
+            for (int t = ng - 1; t >= 0; --t) {
+                const int h = gaps[t];
+                for (int q = lane; q < h; q += 32)   // sublist q, q + h, q + 2h, ...
+                    for (int i = q + h; i < n; i += h) {
+                        const int x = v[i];
+                        int j = i;
+                        while (j >= h && v[j - h] > x) { v[j] = v[j - h]; j -= h; }
+                        v[j] = x;
+                    }
+                __syncwarp();
             }
         }
     }
@@ -727,16 +788,20 @@ __global__ void k_segcell_emit(LayerBuildArgs a, const float4 *seg32, const doub
 //                  max(|ax|, |ay|, |ax + ex|, |ay + ey|), segment index bits).
 __global__ void k_cseg_records(const int *cseg_start, const int *cseg_ids, int G, int nx, const float *frame_x,
                                const float *frame_y, const float4 *vsplit, const float4 *seg32, float4 *rec) {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < G; c += gridDim.x * blockDim.x) {
+    const int lane = lane_id();
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int c = warp; c < G; c += nwarps) {   // a warp per cell
+        const int b = cseg_start[c], e = cseg_start[c + 1];
+        if (b == e) continue;
         const float2 fo = cell_frame(frame_x, frame_y, nx, c);
-        for (int g = cseg_start[c]; g < cseg_start[c + 1]; ++g) {
+        for (int g = b + lane; g < e; g += 32) {
             const int i = cseg_ids[g];
-            const float4 v = vsplit[i], e = seg32[i];
+            const float4 v = vsplit[i], s = seg32[i];
             const float ax = rel_coord(v.x, v.z, fo.x), ay = rel_coord(v.y, v.w, fo.y);
-            const float bx = ax + e.x, by = ay + e.y;
+            const float bx = ax + s.x, by = ay + s.y;
             const float mag = fmaxf(fmaxf(fabsf(ax), fabsf(ay)), fmaxf(fabsf(bx), fabsf(by)));
-            rec[2 * (size_t)g] = make_float4(ax, ay, e.x, e.y);
-            rec[2 * (size_t)g + 1] = make_float4(e.z, e.w, mag, __int_as_float(i));
+            rec[2 * (size_t)g] = make_float4(ax, ay, s.x, s.y);
+            rec[2 * (size_t)g + 1] = make_float4(s.z, s.w, mag, __int_as_float(i));
         }
     }
 }
@@ -782,8 +847,7 @@ __global__ void k_prow_count(LayerBuildArgs a, int *prow_n, int *prow_r0, unsign
         unsigned long long n = 0;
         if (P < a.nobj) {
             const Box m = a.mbb[P];
-            const int r0 = clamped_axis(m.ymin, a.g.y0, a.g.ch, a.g.ny);
-            const int r1 = clamped_axis(m.ymax, a.g.y0, a.g.ch, a.g.ny);
+            const int r0 = clamped_row(a.g, m.ymin), r1 = clamped_row(a.g, m.ymax);
             prow_r0[P] = r0;
             prow_n[P] = r1 - r0 + 1;
             n = (unsigned long long)(r1 - r0 + 1);
@@ -814,9 +878,9 @@ cudaError_t launch_split(const double2 *v, int n, float4 *vs, cudaStream_t s) {
     k_split<<<stream_blocks(n, 256, 4096), 256, 0, s>>>(v, n, vs);
     return cudaGetLastError();
 }
-cudaError_t launch_seg_table(const double2 *v, const int *line_off, int L, double2 *e64, double *inv64, float4 *seg32,
-                             cudaStream_t s) {
-    k_seg_table<<<stream_blocks(L, 128, 4096), 128, 0, s>>>(v, line_off, L, e64, inv64, seg32);
+cudaError_t launch_seg_table(const double2 *v, const int *line_off, int L, int V, double2 *e64, double *inv64,
+                             float4 *seg32, cudaStream_t s) {
+    k_seg_table<<<stream_blocks(V, 256, 8192), 256, 0, s>>>(v, line_off, L, V, e64, inv64, seg32);
     return cudaGetLastError();
 }
 cudaError_t launch_mbb(const LayerBuildArgs &a, cudaStream_t s) {
@@ -836,7 +900,7 @@ cudaError_t launch_raster_emit(const LayerBuildArgs &a, int2 *pairs, int M, int 
     cudaError_t e = run_scan(IntLoad{a.cell_cnt}, OffsetApply{a.cand_start}, a.g.G, a.block_sums, a.bs_cap, a.totals, s);
     if (e != cudaSuccess) return e;
     k_pair_scatter<<<stream_blocks(M, 256, 4096), 256, 0, s>>>(pairs, M, a.cand_start, a.cursor, cand_ids);
-    k_cand_sort<<<stream_blocks(a.g.G, 128, 8192), 128, 0, s>>>(a.cand_start, a.g.G, cand_ids);
+    k_cand_sort<<<stream_blocks(32LL * a.g.G, 256, 16384), 256, 0, s>>>(a.cand_start, a.g.G, cand_ids);
     return cudaGetLastError();
 }
 
@@ -860,7 +924,7 @@ cudaError_t launch_segcell_emit(const LayerBuildArgs &a, const float4 *seg32, co
     cudaError_t e = run_scan(IntLoad{a.cell_cnt}, OffsetApply{cseg_start}, a.g.G, a.block_sums, a.bs_cap, a.totals, s);
     if (e != cudaSuccess) return e;
     k_pair_scatter<<<stream_blocks(MS, 256, 4096), 256, 0, s>>>(pairs, MS, cseg_start, a.cursor, cseg_ids);
-    k_cand_sort<<<stream_blocks(a.g.G, 128, 8192), 128, 0, s>>>(cseg_start, a.g.G, cseg_ids);
+    k_cand_sort<<<stream_blocks(32LL * a.g.G, 256, 16384), 256, 0, s>>>(cseg_start, a.g.G, cseg_ids);
     k_cell_algo<<<stream_blocks(a.g.G, 128, 8192), 128, 0, s>>>(a.cand_start, cand_ids, a.obj_voff, a.g.G, cell_algo);
     return cudaGetLastError();
 }
@@ -878,7 +942,7 @@ cudaError_t launch_prow_count(const LayerBuildArgs &a, int *prow_base, int *prow
 cudaError_t launch_cseg_records(const int *cseg_start, const int *cseg_ids, const GridDev &g, const float *frame_x,
                                 const float *frame_y, const float4 *vsplit, const float4 *seg32, float4 *rec,
                                 cudaStream_t s) {
-    k_cseg_records<<<stream_blocks(g.G, 128, 8192), 128, 0, s>>>(cseg_start, cseg_ids, g.G, g.nx, frame_x, frame_y,
+    k_cseg_records<<<stream_blocks(32LL * g.G, 256, 16384), 256, 0, s>>>(cseg_start, cseg_ids, g.G, g.nx, frame_x, frame_y,
                                                                 vsplit, seg32, rec);
     return cudaGetLastError();
 }

@@ -220,6 +220,22 @@ __host__ __device__ __forceinline__ int cell_chunk(int ch, int work, int budget)
     return c < lo ? lo : (c > ch ? ch : (int)c);
 }
 
+// clamped_axis without FP64 for all but the values near a cell boundary or the
+// grid's ends: the FP32 estimate with four times its error bound (the values of
+// interest reach one cell beyond the grid, where the bound's max |v| may treble).
+__device__ __forceinline__ int clamped_cell(double v, double lo, double w, int n, float lof, float iwf, float tol) {
+    const float t = __fmul_rn(__fsub_rn(approx_float(v), lof), iwf);
+    const float f = floorf(t), r = t - f, e = 4.0f * tol;
+    if (r > e && r < 1.0f - e && t > -1.0f && t < (float)n + 1.0f) return min(max((int)f, 0), n - 1);
+    return clamped_axis(v, lo, w, n);
+}
+__device__ __forceinline__ int clamped_col(const GridDev &g, double x) {
+    return clamped_cell(x, g.x0, g.cw, g.nx, g.x0f, g.icwf, g.tolx);
+}
+__device__ __forceinline__ int clamped_row(const GridDev &g, double y) {
+    return clamped_cell(y, g.y0, g.ch, g.ny, g.y0f, g.ichf, g.toly);
+}
+
 // Minimum bounding box of an object.
 struct Box {
     double xmin, ymin, xmax, ymax;
@@ -372,6 +388,15 @@ struct PipEdges {
     float2 *xr;
     unsigned char *kind;
 };
+// A row list's entry, with what the cells' entries need to know of its edge.
+struct alignas(32) PipRow {
+    int edge;         // first vertex
+    float x0, x1;     // x-range, rounded outward
+    int lo, hi;       // rows of the lower and the upper end
+    int kind;         // as PipEdges::kind
+    int twin;         // polygon of the edge with the same end points, or -1
+    int pad;
+};
 struct alignas(16) PipFlipTmp {
     unsigned long long key;
     unsigned mask;
@@ -385,7 +410,8 @@ struct PipBuildArgs {
     PipEdges e;
     int *twin;                                  // [V] edge with the same end points in another place, or -1
     const int *cand_start, *cand_ids;
-    const int *prow_base, *prow_r0, *prow_start, *pedge;
+    const int *prow_base, *prow_r0, *prow_start;
+    const PipRow *rows;                         // [ME] the row lists' records
     float2 *col;                                // [nx] column limits widened by delta
     int *entry_cell, *ord, *edge_at, *flip_at;  // [M]
     int2 *ent;                                  // [M] near edges, (flips << 2 | base parity << 1 | any)
@@ -403,7 +429,7 @@ struct PipBuildArgs {
 cudaError_t launch_pip_edges(const PipBuildArgs &b, cudaStream_t s);
 cudaError_t launch_pip_twins(const PipBuildArgs &b, int *table, unsigned slots, cudaStream_t s);
 cudaError_t launch_prow_edges(const PipBuildArgs &b, int *cnt, unsigned long long *total, const int *start, int *ids,
-                              cudaStream_t s);
+                              PipRow *rows, cudaStream_t s);
 cudaError_t launch_pip_count(const PipBuildArgs &b, double delta, cudaStream_t s);
 cudaError_t launch_pip_records(const PipBuildArgs &b, cudaStream_t s);
 constexpr int PIP_LONG_MIN = 256;   // records of more elements may be listed in long_list

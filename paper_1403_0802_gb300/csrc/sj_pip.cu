@@ -498,13 +498,13 @@ cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *
 // ------------------------------------------------------------------ layer build
 
 // Where a layer's edges lie (PipEdges), one thread per edge (vertex i -> nxt[i]):
-// its grid rows under the cell rule (FP64 divisions, done once here), its
-// x-range rounded outward to FP32, and which end is the lower one.
+// its grid rows under the cell rule, its x-range rounded outward to FP32, and
+// which end is the lower one.
 __global__ void k_pip_edges(GridDev g, const double2 *verts, const int *nxt, int V, PipEdges e) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
         const double2 A = verts[i], B = verts[nxt[i]];
         const bool up = A.y <= B.y;
-        e.rows[i] = make_int2(clamped_axis(up ? A.y : B.y, g.y0, g.ch, g.ny), clamped_axis(up ? B.y : A.y, g.y0, g.ch, g.ny));
+        e.rows[i] = make_int2(clamped_row(g, up ? A.y : B.y), clamped_row(g, up ? B.y : A.y));
         e.xr[i] = make_float2(__double2float_rd(fmin(A.x, B.x)), __double2float_ru(fmax(A.x, B.x)));
         e.kind[i] = (up ? 1 : 0) | (A.y == B.y ? 2 : 0);
     }
@@ -545,16 +545,26 @@ __global__ void k_pip_twins(const double2 *verts, const int *nxt, const unsigned
 }
 
 // Row lists: for each (polygon, row of its MBB) the edges whose rows include
-// it.  One thread per edge.  Count (ids == nullptr), then emit.
-__global__ void k_prow_edges(const int2 *rows, const int *owner, int V, const int *prow_base, const int *prow_r0,
-                             int *cnt, unsigned long long *total, const int *start, int *ids) {
+// it.  One thread per edge.  Count (ids == nullptr), then emit, with the records
+// that k_pip_entries reads in list order.
+__global__ void k_prow_edges(PipBuildArgs b, int *cnt, unsigned long long *total, const int *start, int *ids,
+                             PipRow *out) {
     unsigned long long n = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
-        const int P = owner[i], base = prow_base[P] - prow_r0[P];
-        const int2 r = rows[i];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < b.V; i += gridDim.x * blockDim.x) {
+        const int P = b.owner[i], base = b.prow_base[P] - b.prow_r0[P];
+        const int2 r = b.e.rows[i];
+        PipRow q{};
+        if (ids) {
+            const float2 x = b.e.xr[i];
+            const int t = b.twin[i];
+            q = PipRow{i, x.x, x.y, r.x, r.y, b.e.kind[i], t >= 0 ? b.owner[t] : -1, 0};
+        }
         for (int y = r.x; y <= r.y; ++y) {
             const int k = atomicAdd(&cnt[base + y], 1);
-            if (ids) ids[start[base + y] + k] = i;
+            if (ids) {
+                ids[start[base + y] + k] = i;
+                out[start[base + y] + k] = q;
+            }
         }
         n += (unsigned long long)(r.y - r.x + 1);
     }
@@ -612,29 +622,25 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
         bool any = false;
         for (int base = e0; base < e1; base += 8) {
             const int t = base + sub;
-            bool is_near = false, mine = false, fl = false, fh = false;
+            bool is_near = false, mine = false, fl = false, fh = false, up = false;
             int i = 0, tk = -1;
             if (t < e1) {
-                i = b.pedge[t];
-                const float2 xr = b.e.xr[i];
-                const unsigned char kd = b.e.kind[i];
-                if (xr.x > col.y) {   // far
-                    const int2 r = b.e.rows[i];
-                    par ^= r.x < iy;
-                    if (r.x == iy || r.y == iy) {
+                const PipRow q = b.rows[t];
+                i = q.edge;
+                up = q.kind & 1;
+                if (q.x0 > col.y) {   // far
+                    par ^= q.lo < iy;
+                    if (q.lo == iy || q.hi == iy) {
                         // the ends inside the row, unless shared with another far edge
                         const bool a_far = b.e.xr[b.prv[i]].x > col.y, b_far = b.e.xr[b.nxt[i]].x > col.y;
-                        const bool up = kd & 1;
-                        fl = r.x == iy && !(up ? a_far : b_far);
-                        fh = r.y == iy && !(up ? b_far : a_far);
+                        fl = q.lo == iy && !(up ? a_far : b_far);
+                        fh = q.hi == iy && !(up ? b_far : a_far);
                     }
-                } else if (!(xr.y < col.x) && !(kd & 2)) {   // near
+                } else if (!(q.x1 < col.x) && !(q.kind & 2)) {   // near
                     is_near = mine = true;
-                    const int tw = b.twin[i];
-                    if (tw >= 0) {
-                        const int Q = b.owner[tw];
-                        if (Q != P) tk = entry_of(b, k0, k1, Q);
-                        if (tk >= 0 && Q < P) mine = false;
+                    if (q.twin >= 0 && q.twin != P) {
+                        tk = entry_of(b, k0, k1, q.twin);
+                        if (tk >= 0 && q.twin < P) mine = false;
                     }
                 }
             }
@@ -648,7 +654,6 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
                     b.tmp_edge[b.edge_at[k] + n + __popc(bn & lt & gm)] = make_int2(i, (int)m);
                 }
                 if (fl || fh) {
-                    const bool up = b.e.kind[i] & 1;
                     const int j = b.nxt[i];
                     PipFlipTmp *f = b.tmp_flip + b.flip_at[k] + nf + __popc(bl & lt & gm) + __popc(bh & lt & gm);
                     if (fl) *f++ = PipFlipTmp{y_key(b.verts[up ? i : j].y), own, 0};
@@ -937,9 +942,8 @@ cudaError_t launch_pip_twins(const PipBuildArgs &b, int *table, unsigned slots, 
     return cudaGetLastError();
 }
 cudaError_t launch_prow_edges(const PipBuildArgs &b, int *cnt, unsigned long long *total, const int *start, int *ids,
-                              cudaStream_t s) {
-    k_prow_edges<<<grid_for(b.V, 256, 8192), 256, 0, s>>>(b.e.rows, b.owner, b.V, b.prow_base, b.prow_r0, cnt, total,
-                                                         start, ids);
+                              PipRow *rows, cudaStream_t s) {
+    k_prow_edges<<<grid_for(b.V, 256, 8192), 256, 0, s>>>(b, cnt, total, start, ids, rows);
     return cudaGetLastError();
 }
 // Step 1: what each candidate entry and cell holds.
