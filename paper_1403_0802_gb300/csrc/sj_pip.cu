@@ -595,18 +595,22 @@ __device__ __forceinline__ int entry_of(const PipBuildArgs &b, int k0, int k1, i
     return -1;
 }
 
-// Candidate entries, eight lanes each.  Count pass: near edges (a shared edge
+// Candidate entries, a warp each.  Count pass: near edges (a shared edge
 // counted with its polygon of smaller id), flips, base parity and whether the
 // entry has any near edge or flip (ent[k] = near, flips << 2 | base << 1 | any).
 // Emit pass: the near edges (vid, mask) and flips (key, bit) of the relevant
 // entries, unordered, at edge_at[k] / flip_at[k] in the temporary units.
-// Eight lanes: a (polygon, row) list holds 5 - 60 edges on average.
+// A whole warp although a (polygon, row) list holds 5 - 60 edges on average: the
+// lists of thousands of a few large polygons set the time (the two passes on the
+// 40,000 tiles at 768 x 768: 286 + 507 us with eight lanes an entry, 240 + 234 with
+// 32; the layer build of the heavy-tail tiling 17.2 ms with 8, 9.7 with 16, 7.5
+// with 32).
 template <bool EMIT>
 __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
-    const int lane = lane_id(), sub = lane & 7, gsh = lane & 24;
-    const unsigned gm = 0xffu << gsh, lt = (1u << lane) - 1u;
+    const int lane = lane_id();
+    const unsigned lt = (1u << lane) - 1u;
     const long long T = (long long)gridDim.x * blockDim.x;
-    for (long long kk = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3; kk < b.M; kk += T >> 3) {
+    for (long long kk = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; kk < b.M; kk += T >> 5) {
         const int k = (int)kk;
         const int bit = EMIT ? b.ord[k] : 0;
         if (EMIT && bit < 0) continue;
@@ -620,8 +624,8 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
         const unsigned own = EMIT ? 1u << (bit & 31) : 0u;
         int n = 0, nf = 0, par = 0;
         bool any = false;
-        for (int base = e0; base < e1; base += 8) {
-            const int t = base + sub;
+        for (int base = e0; base < e1; base += 32) {
+            const int t = base + lane;
             bool is_near = false, mine = false, fl = false, fh = false, up = false;
             int i = 0, tk = -1;
             if (t < e1) {
@@ -644,18 +648,18 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
                     }
                 }
             }
-            const unsigned bn = __ballot_sync(gm, mine);
-            const unsigned bl = __ballot_sync(gm, fl), bh = __ballot_sync(gm, fh);
-            any |= __any_sync(gm, is_near) || bl || bh;
+            const unsigned bn = __ballot_sync(FULL, mine);
+            const unsigned bl = __ballot_sync(FULL, fl), bh = __ballot_sync(FULL, fh);
+            any |= __any_sync(FULL, is_near) || bl || bh;
             if (EMIT) {
                 if (mine) {
                     unsigned m = own;
                     if (tk >= 0 && b.ord[tk] >= 0) m |= 1u << (b.ord[tk] & 31);
-                    b.tmp_edge[b.edge_at[k] + n + __popc(bn & lt & gm)] = make_int2(i, (int)m);
+                    b.tmp_edge[b.edge_at[k] + n + __popc(bn & lt)] = make_int2(i, (int)m);
                 }
                 if (fl || fh) {
                     const int j = b.nxt[i];
-                    PipFlipTmp *f = b.tmp_flip + b.flip_at[k] + nf + __popc(bl & lt & gm) + __popc(bh & lt & gm);
+                    PipFlipTmp *f = b.tmp_flip + b.flip_at[k] + nf + __popc(bl & lt) + __popc(bh & lt);
                     if (fl) *f++ = PipFlipTmp{y_key(b.verts[up ? i : j].y), own, 0};
                     if (fh) *f = PipFlipTmp{y_key(b.verts[up ? j : i].y), own, 0};
                 }
@@ -664,8 +668,8 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
             nf += __popc(bl) + __popc(bh);
         }
         if (!EMIT) {
-            par = (int)__popc(__ballot_sync(gm, par & 1)) & 1;
-            if (sub == 0) b.ent[k] = make_int2(n, (nf << 2) | (par << 1) | (any ? 1 : 0));
+            par = (int)__popc(__ballot_sync(FULL, par & 1)) & 1;
+            if (lane == 0) b.ent[k] = make_int2(n, (nf << 2) | (par << 1) | (any ? 1 : 0));
         }
     }
 }
@@ -799,12 +803,11 @@ __device__ __forceinline__ float key_rel(unsigned long long key, float fo) {
 constexpr int PIP_LONG = PIP_LONG_MIN;
 
 // The records' edges (ordered by lower y) and flips (ordered by key, masks
-// accumulated), eight lanes per cell: each element's place is its rank.
+// accumulated), a warp per cell: each element's place is its rank.
 __global__ void __launch_bounds__(256) k_pip_order(PipBuildArgs b) {
-    const int lane = lane_id(), sub = lane & 7;
-    const unsigned gm = 0xffu << (lane & 24);
+    const int lane = lane_id();
     const long long T = (long long)gridDim.x * blockDim.x;
-    for (long long cc = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3; cc < b.g.G; cc += T >> 3) {
+    for (long long cc = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; cc < b.g.G; cc += T >> 5) {
         const int c = (int)cc, code = b.cell_code[c];
         if (code >= -1) continue;
         const float2 fo = cell_frame(b.frame_x, b.frame_y, b.g.nx, c);
@@ -814,34 +817,55 @@ __global__ void __launch_bounds__(256) k_pip_order(PipBuildArgs b) {
             const int4 u0 = u[0];
             const int n = u0.x, nf = u0.y;
             if (n > PIP_LONG || nf > PIP_LONG) {
-                if (sub == 0) b.long_list[atomicAdd(b.long_n, 1)] = make_int4(off, c, te, tf);
+                if (lane == 0) b.long_list[atomicAdd(b.long_n, 1)] = make_int4(off, c, te, tf);
             } else {
                 PipEdge *E = reinterpret_cast<PipEdge *>(u + 2);
                 float hmax = 0.0f;
-                for (int i = sub; i < n; i += 8) {
-                    const float4 r = edge_rel(b, b.tmp_edge[te + i].x, fo);
-                    b.tmp_rel[te + i] = r;
-                    hmax = fmaxf(hmax, edge_height(r));
-                }
-                __syncwarp(gm);
-                for (int i = sub; i < n; i += 8) {
-                    const float4 r = b.tmp_rel[te + i];
-                    const int2 v = b.tmp_edge[te + i];
+                if (n <= 32) {   // in registers
+                    int2 v = make_int2(0, 0);
+                    float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (lane < n) {
+                        v = b.tmp_edge[te + lane];
+                        r = edge_rel(b, v.x, fo);
+                        hmax = edge_height(r);
+                    }
                     const float key = list_key(r.y);
                     int rank = 0;
                     for (int j = 0; j < n; ++j) {
-                        const float kj = list_key(b.tmp_rel[te + j].y);
-                        rank += kj < key || (kj == key && j < i);
+                        const float kj = __shfl_sync(FULL, key, j);
+                        rank += kj < key || (kj == key && j < lane);
                     }
-                    reinterpret_cast<float4 *>(E + rank)[0] = r;
-                    reinterpret_cast<int4 *>(E + rank)[1] = make_int4(v.x, v.y, 0, 0);
+                    if (lane < n) {
+                        reinterpret_cast<float4 *>(E + rank)[0] = r;
+                        reinterpret_cast<int4 *>(E + rank)[1] = make_int4(v.x, v.y, 0, 0);
+                    }
+                } else {
+                    for (int i = lane; i < n; i += 32) {
+                        const float4 r = edge_rel(b, b.tmp_edge[te + i].x, fo);
+                        b.tmp_rel[te + i] = r;
+                        hmax = fmaxf(hmax, edge_height(r));
+                    }
+                    __syncwarp();
+                    for (int i = lane; i < n; i += 32) {
+                        const float4 r = b.tmp_rel[te + i];
+                        const int2 v = b.tmp_edge[te + i];
+                        const float key = list_key(r.y);
+                        int rank = 0;
+#pragma unroll 4
+                        for (int j = 0; j < n; ++j) {
+                            const float kj = list_key(b.tmp_rel[te + j].y);
+                            rank += kj < key || (kj == key && j < i);
+                        }
+                        reinterpret_cast<float4 *>(E + rank)[0] = r;
+                        reinterpret_cast<int4 *>(E + rank)[1] = make_int4(v.x, v.y, 0, 0);
+                    }
                 }
                 if (u0.w & PIP_EXT) {
-                    for (int o = 4; o > 0; o >>= 1) hmax = fmaxf(hmax, __shfl_xor_sync(gm, hmax, o));
-                    if (sub == 0) reinterpret_cast<int *>(u)[5] = __float_as_int(hmax);
+                    for (int o = 16; o > 0; o >>= 1) hmax = fmaxf(hmax, __shfl_xor_sync(FULL, hmax, o));
+                    if (lane == 0) reinterpret_cast<int *>(u)[5] = __float_as_int(hmax);
                 }
                 PipFlip *F = reinterpret_cast<PipFlip *>(E + n);
-                for (int i = sub; i < nf; i += 8) {
+                for (int i = lane; i < nf; i += 32) {
                     const PipFlipTmp v = b.tmp_flip[tf + i];
                     int rank = 0;
                     unsigned m = (unsigned)u0.z;
@@ -950,15 +974,15 @@ cudaError_t launch_prow_edges(const PipBuildArgs &b, int *cnt, unsigned long lon
 cudaError_t launch_pip_count(const PipBuildArgs &b, double delta, cudaStream_t s) {
     k_pip_columns<<<grid_for(b.g.nx, 256, 4096), 256, 0, s>>>(b.g, delta, b.col);
     k_pip_entry_cells<<<grid_for(b.g.G, 256, 8192), 256, 0, s>>>(b.cand_start, b.g.G, b.entry_cell);
-    k_pip_entries<false><<<grid_for(8LL * b.M, 256, 16384), 256, 0, s>>>(b);
+    k_pip_entries<false><<<grid_for(32LL * b.M, 256, 32768), 256, 0, s>>>(b);
     k_pip_cells<<<grid_for(b.g.G, 256, 8192), 256, 0, s>>>(b);
     return cudaGetLastError();
 }
 // Step 2: the records (units, temporary lists and offsets allocated).
 cudaError_t launch_pip_records(const PipBuildArgs &b, cudaStream_t s) {
     k_pip_heads<<<grid_for(b.g.G, 256, 8192), 256, 0, s>>>(b);
-    k_pip_entries<true><<<grid_for(8LL * b.M, 256, 16384), 256, 0, s>>>(b);
-    k_pip_order<<<grid_for(8LL * b.g.G, 256, 16384), 256, 0, s>>>(b);
+    k_pip_entries<true><<<grid_for(32LL * b.M, 256, 32768), 256, 0, s>>>(b);
+    k_pip_order<<<grid_for(32LL * b.g.G, 256, 32768), 256, 0, s>>>(b);
     k_pip_order_long<<<152 * 2, 512, 0, s>>>(b);
     return cudaGetLastError();
 }
