@@ -234,7 +234,7 @@ void sj::fill_refine(const sj_layer *L, int form, RefineArgs &ra) {
 PipArgs sj::pip_args(const sj_layer *L) {
     PipArgs a{};
     a.g = L->g;
-    a.cell_code = L->cell_code;
+    a.cells = L->cells;
     a.units = L->units;
     a.units_n = (int)L->units_n;
     a.verts = L->verts;
@@ -269,7 +269,7 @@ static void layer_free(sj_layer *L) {
     void *ptrs[] = {L->verts, L->vsplit, L->obj_voff, L->nxt, L->ring_off, L->poly_ring_off, L->seg_e64,
                     L->seg_inv64, L->seg32, L->mbb, L->cand_start, L->cand_ids, L->stats, L->cell_keys,
                     L->frames, L->cseg_start, L->cseg_ids, L->cell_algo, L->cseg_rec, L->prow_base, L->prow_r0,
-                    L->prow_start, L->pedge_ids, L->cell_work, L->cell_code, L->units};
+                    L->prow_start, L->pedge_ids, L->cell_work, L->cells, L->units};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete L;
@@ -457,13 +457,13 @@ static sj_status build_pip_records(sj_layer *L, const int *prv, const int *owner
     const int P = L->nobj, G = L->g.G, V = L->V, M = (int)L->M;
     CUDA_TRY(dalloc(&L->prow_base, (size_t)P + 1));
     CUDA_TRY(dalloc(&L->prow_r0, (size_t)P));
-    CUDA_TRY(dalloc(&L->cell_code, (size_t)G));
+    CUDA_TRY(dalloc(&L->cells, (size_t)G));
     if (P == 0) {
         L->MR = L->ME = L->units_n = 0;
         CUDA_TRY(dalloc(&L->prow_start, 1));
         CUDA_TRY(dalloc(&L->pedge_ids, 0));
         CUDA_TRY(dalloc(&L->units, 0));
-        CUDA_TRY(cudaMemsetAsync(L->cell_code, 0xff, sizeof(int) * (size_t)G, s));   // -1: no candidates
+        CUDA_TRY(cudaMemsetAsync(L->cells, 0xff, sizeof(int4) * (size_t)G, s));   // -1: no candidates
         CUDA_TRY(cudaMemsetAsync(L->prow_base, 0, sizeof(int), s));
         CUDA_TRY(cudaMemsetAsync(L->prow_start, 0, sizeof(int), s));
         CUDA_TRY(cudaStreamSynchronize(s));
@@ -558,7 +558,19 @@ static sj_status build_pip_records(sj_layer *L, const int *prv, const int *owner
         CUDA_TRY(tmp.take(of[q], (size_t)G));
         CUDA_TRY(tmp.take(&at[q], (size_t)G + 1));
     }
-    b.cell_code = L->cell_code;
+    b.cells = L->cells;
+    // sub-cell classes: margin for delta, for twice the error of a point's place in
+    // its cell (the place and the cell's edge), and for the frame origin's rounding
+    // and the box's own; none where it would fill the sub-cell
+    b.cwf = (float)L->g.cw;
+    b.chf = (float)L->g.ch;
+    b.eps = pip_args(L).eps;
+    const double u = 5.9604644775390625e-08, rest = delta + 4.0 * u * L->xmax;
+    const double mx = 1.01 * (rest + (2.0 * L->g.tolx + 8.0 * u) * L->g.cw);
+    const double my = 1.01 * (rest + (2.0 * L->g.toly + 8.0 * u) * L->g.ch);
+    const bool subs = mx < L->g.cw / 32 && my < L->g.ch / 32 && L->xmax <= 1e15 && L->xmax >= 1e-6;
+    b.sub_mx = subs ? float_up(mx) : -1.0f;
+    b.sub_my = subs ? float_up(my) : -1.0f;
     CUDA_TRY(launch_pip_count(b, delta, s));
     int2 *bs2 = nullptr;
     const size_t cells_cap = bucket_scan_blocks(G);

@@ -54,7 +54,7 @@ struct sj_layer {
     int *prow_start = nullptr;   // [MR + 1] list ranges in pedge_ids
     int *pedge_ids = nullptr;    // [ME] edge (= first vertex) indices
     // PIP: per cell the result of its points or its record (sj_pip.cu)
-    int *cell_code = nullptr;    // [G]
+    int4 *cells = nullptr;       // [G] PipArgs::cells
     int4 *units = nullptr;       // [2 units_n] the records, 32-byte units
     int64_t units_n = 0;
     int *cell_work = nullptr;    // P2P: [G] per-point segment work of each cell (item sizes)

@@ -109,14 +109,20 @@ __device__ __forceinline__ int axis_cell(double v, const unsigned long long *key
 
 // Cell index along one axis from FP32 alone: true when the estimate lies
 // farther than its error bound tol from every cell boundary and inside the
-// grid, so that i is certain.  The bound (make_grid) covers the truncation of v
+// grid, so that i is certain; r is then the place within the cell, 0 to 1, off
+// by at most tol.  The bound (make_grid) covers the truncation of v
 // to FP32, the rounding of lo and 1 / w, and the two operations; NaN, infinite
 // and far outside values are never certain.
-__device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i) {
+__device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i, float &r) {
     const float t = __fmul_rn(__fsub_rn(approx_float(v), lof), iwf);
-    const float f = floorf(t), r = t - f;
+    const float f = floorf(t);
+    r = t - f;
     i = (int)f;
     return r > tol && r < 1.0f - tol && t > 0.0f && t < (float)n;
+}
+__device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i) {
+    float r;
+    return axis_estimate(v, lof, iwf, tol, n, i, r);
 }
 
 // Column and row of a point, (-1 in an axis) outside the half-open grid box or
@@ -367,7 +373,8 @@ constexpr int PIP_SEARCH = 32, PIP_SEARCH_MIN = 16;
 // Arguments of the PIP join (the records are described in sj_pip.cu).
 struct PipArgs {
     GridDev g;
-    const int *cell_code;    // [G] result of a classified cell, else -2 - first unit of its record
+    const int4 *cells;       // [G] code (result of a classified cell, else -2 - first unit of its
+                             //     record), sub-cell classes, the ids of classes 1 and 2
     const int4 *units;       // [2 per 32-byte unit]
     int units_n;
     const double2 *verts;
@@ -414,8 +421,11 @@ struct PipBuildArgs {
     const PipRow *rows;                         // [ME] the row lists' records
     float2 *col;                                // [nx] column limits widened by delta
     int *entry_cell, *ord, *edge_at, *flip_at;  // [M]
-    int2 *ent;                                  // [M] near edges, (flips << 2 | base parity << 1 | any)
-    int *cell_code;                             // [G]
+    int2 *ent;                                  // [M] near edges, (flips << 3 | horizontal << 2 | base parity << 1 | any)
+    int4 *cells;                                // [G] as PipArgs
+    float cwf, chf;                             // cell size
+    float sub_mx, sub_my;                       // margins of the sub-cell classes (< 0: none)
+    float eps;                                  // as PipArgs
     int *units_of, *edges_of, *flips_of;        // [G]
     const int *units_at, *edges_at, *flips_at;  // [G + 1] their exclusive sums
     int4 *units;

@@ -8,10 +8,16 @@
 // input order: no bucketing, no scratch, one coalesced read of the points and
 // one coalesced write of the ids.
 //
-// Per cell (cell_code):
+// Per cell (PipArgs::cells), a code:
 //   >= -1   the result of every point of the cell (no candidate's edge comes
 //           near the cell, so each candidate holds all of it or none of it);
-//   <= -2   -2 - (first 32-byte unit of the cell's record).
+//   <= -2   -2 - (first 32-byte unit of the cell's record),
+// and for the latter the class of each of 4 x 4 sub-cells, two bits: 1 or 2 -- no
+// near edge meets the sub-cell widened by a margin, and its points' result is
+// the cell's first or second id --, 3 -- the same with no polygon --, or 0: the
+// record decides.  One 16-byte read answers four of five points of the cells
+// that edges pass (the tiles: 36 % of the points are in such cells, 8 % in a
+// sub-cell that an edge meets).
 // A record is a chain of groups of up to 32 relevant candidates in id order (a
 // candidate that holds none of the cell is left out, and so is every candidate
 // after one that holds all of it): a header, the near edges, the flips.  For a
@@ -168,7 +174,13 @@ struct RoundSource {
 // code, record), the join is fastest at the most warps whose 64 registers hold
 // the loop without spills: 100 M points on the 40,000 tiles 1.87 / 1.70 / 1.61 ms
 // with 6 / 7 / 8 blocks, 2.8 ms with 10 (48 registers, spilled).
-constexpr int PIP_WARPS = 4, PIP_BLOCKS = 8;
+#ifndef VB
+#define VB 8
+#endif
+#ifndef VU
+#define VU 2
+#endif
+constexpr int PIP_WARPS = 4, PIP_BLOCKS = VB;
 // Code of a queued point whose cell the FP32 estimate leaves open (no record
 // starts there: units are fewer than 2^31 - 2^22).
 constexpr int PIP_UNSURE = -2147483647 - 1;
@@ -376,11 +388,18 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
             for (int u = 0; u < U; ++u) {
                 code[u] = -1;
                 if (i0 + 32u * u < n) {
-                    const bool sx = axis_estimate(p[u].x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, ix[u]);
-                    const bool sy = axis_estimate(p[u].y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, iy[u]);
+                    float rx, ry;
+                    const bool sx = axis_estimate(p[u].x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, ix[u], rx);
+                    const bool sy = axis_estimate(p[u].y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, iy[u], ry);
                     code[u] = PIP_UNSURE;
                     if (sx && sy) {
-                        code[u] = __ldg(a.cell_code + iy[u] * a.g.nx + ix[u]);
+                        const int4 c = __ldg(a.cells + iy[u] * a.g.nx + ix[u]);
+                        code[u] = c.x;
+                        if (c.x < -1) {
+                            const int k = (int)(ry * 4.0f) * 4 + (int)(rx * 4.0f);
+                            const unsigned cls = ((unsigned)c.y >> (2 * k)) & 3u;
+                            if (cls) code[u] = cls == 1 ? c.z : (cls == 2 ? c.w : -1);
+                        }
                         resolved += code[u] >= -1;
                     }
                 }
@@ -426,7 +445,7 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
             head = src.get((unsigned)q.i);
             q.p = src.point((unsigned)q.i);
             const int2 e = point_cell_exact(a.g, q.p.x, q.p.y);
-            const int code = e.x >= 0 && e.y >= 0 ? a.cell_code[e.y * a.g.nx + e.x] : -1;
+            const int code = e.x >= 0 && e.y >= 0 ? a.cells[e.y * a.g.nx + e.x].x : -1;
             const bool unsure = !(axis_estimate(q.p.x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, q.ix) &&
                                   axis_estimate(q.p.y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, q.iy));
             q.ix = e.x;
@@ -475,7 +494,7 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
 // Points per lane and tile: two once that still gives every SM all its warps
 // twice over (100 M points: 1.69 / 1.55 / 1.90 ms with 1 / 2 / 4); smaller calls
 // spread over more warps, one point per lane.
-constexpr int PIP_U = 2;
+constexpr int PIP_U = VU;
 
 static int pip_blocks(int U, long long n, int sms) {
     const long long tiles = (n + 32LL * U - 1) / (32LL * U);
@@ -597,7 +616,8 @@ __device__ __forceinline__ int entry_of(const PipBuildArgs &b, int k0, int k1, i
 
 // Candidate entries, a warp each.  Count pass: near edges (a shared edge
 // counted with its polygon of smaller id), flips, base parity and whether the
-// entry has any near edge or flip (ent[k] = near, flips << 2 | base << 1 | any).
+// entry has any near edge or flip, and whether a horizontal edge is near (ent[k]
+// = near, flips << 3 | horizontal << 2 | base << 1 | any).
 // Emit pass: the near edges (vid, mask) and flips (key, bit) of the relevant
 // entries, unordered, at edge_at[k] / flip_at[k] in the temporary units.
 // A whole warp although a (polygon, row) list holds 5 - 60 edges on average: the
@@ -623,7 +643,7 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
         const int k0 = b.cand_start[c], k1 = b.cand_start[c + 1];
         const unsigned own = EMIT ? 1u << (bit & 31) : 0u;
         int n = 0, nf = 0, par = 0;
-        bool any = false;
+        bool any = false, level = false;
         for (int base = e0; base < e1; base += 32) {
             const int t = base + lane;
             bool is_near = false, mine = false, fl = false, fh = false, up = false;
@@ -640,7 +660,9 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
                         fl = q.lo == iy && !(up ? a_far : b_far);
                         fh = q.hi == iy && !(up ? b_far : a_far);
                     }
-                } else if (!(q.x1 < col.x) && !(q.kind & 2)) {   // near
+                } else if (!(q.x1 < col.x) && (q.kind & 2)) {    // near, horizontal
+                    level = true;
+                } else if (!(q.x1 < col.x)) {   // near
                     is_near = mine = true;
                     if (q.twin >= 0 && q.twin != P) {
                         tk = entry_of(b, k0, k1, q.twin);
@@ -669,7 +691,8 @@ __global__ void __launch_bounds__(256) k_pip_entries(PipBuildArgs b) {
         }
         if (!EMIT) {
             par = (int)__popc(__ballot_sync(FULL, par & 1)) & 1;
-            if (lane == 0) b.ent[k] = make_int2(n, (nf << 2) | (par << 1) | (any ? 1 : 0));
+            level = __any_sync(FULL, level);
+            if (lane == 0) b.ent[k] = make_int2(n, (nf << 3) | (level ? 4 : 0) | (par << 1) | (any ? 1 : 0));
         }
     }
 }
@@ -681,7 +704,7 @@ __global__ void k_pip_cells(PipBuildArgs b) {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < b.g.G; c += gridDim.x * blockDim.x) {
         const int k0 = b.cand_start[c], k1 = b.cand_start[c + 1];
         int rel = 0, code = -1;
-        bool done = false, any = false;
+        bool done = false, any = false, level = false;
         long long units = 0, tn = 0, tf = 0;
         int n = 0, nf = 0, ng = 0;
         for (int k = k0; k < k1; ++k) {
@@ -696,9 +719,10 @@ __global__ void k_pip_cells(PipBuildArgs b) {
                 done = true;
             }
             any |= bd;
+            level |= (e.y & 4) != 0;
             b.ord[k] = rel++;
             n += e.x;
-            nf += e.y >> 2;
+            nf += e.y >> 3;
             if (++ng == 32) {
                 units += group_units(n, nf, ng);
                 tn += n;
@@ -715,7 +739,7 @@ __global__ void k_pip_cells(PipBuildArgs b) {
         } else {
             code = -2;
         }
-        b.cell_code[c] = code;
+        b.cells[c] = make_int4(code, level ? -1 : 0, -1, -1);   // -1: no sub-cell classes (k_pip_order)
         b.units_of[c] = (int)min(units, 2147483647LL);
         b.edges_of[c] = (int)min(tn, 2147483647LL);
         b.flips_of[c] = (int)min(tf, 2147483647LL);
@@ -725,10 +749,10 @@ __global__ void k_pip_cells(PipBuildArgs b) {
 // Headers, ids and the entries' places in the temporary lists, one thread per cell.
 __global__ void k_pip_heads(PipBuildArgs b) {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < b.g.G; c += gridDim.x * blockDim.x) {
-        if (b.cell_code[c] != -2) continue;
+        if (b.cells[c].x != -2) continue;
         const int k0 = b.cand_start[c], k1 = b.cand_start[c + 1];
         int off = b.units_at[c], te = b.edges_at[c], tf = b.flips_at[c];
-        b.cell_code[c] = -2 - off;
+        b.cells[c].x = -2 - off;
         long long algo = 0;
         int last = k0;   // last relevant entry
         for (int k = k0; k < k1; ++k) {
@@ -749,7 +773,7 @@ __global__ void k_pip_heads(PipBuildArgs b) {
                 if (e.y & 2) h.base |= 1u << ng;
                 if (ng < PIP_INLINE_IDS) h.id[ng] = b.cand_ids[q];
                 h.n += e.x;
-                h.nf += e.y >> 2;
+                h.nf += e.y >> 3;
                 ++ng;
             }
             int4 *u = b.units + 2 * (size_t)off;
@@ -799,6 +823,70 @@ __device__ __forceinline__ float key_rel(unsigned long long key, float fo) {
     return rel_coord(a, c, fo);
 }
 
+// Classes of a cell's 4 x 4 sub-cells (see the top of the file), by a warp: lane
+// l takes sub-cell l & 15 with every second edge.  The sub-cell's box in cell-
+// relative coordinates is widened by the margins (the classes' delta, the error
+// of a point's estimated place, that of the frame origin); where an edge may
+// meet it (separating axes, rounding included) or the parity at its centre is
+// not certain in FP32, the class is 0.  Elsewhere every point of the sub-cell
+// has the centre's result, by the argument for whole cells -- which needs every
+// edge near the cell: a cell with a near horizontal edge (not in its record) has
+// no classes, nor has one whose record has several groups or a long list.
+template <class EdgeAt>
+__device__ __forceinline__ void pip_sub_classes(const PipBuildArgs &b, int c, const int4 u0, const int4 *u, EdgeAt edge_at,
+                                                float eps, int lane) {
+    const int n = u0.x, nf = u0.y, sub = lane & 15;
+    const float qx = 0.25f * b.cwf, qy = 0.25f * b.chf;
+    const float cx = ((float)(sub & 3) + 0.5f) * qx, cy = ((float)(sub >> 2) + 0.5f) * qy;
+    unsigned m = lane < 16 ? (unsigned)u0.z : 0u;
+    bool bad = false;
+    if (lane < 16) {   // flips at or below the centre
+        const PipFlip *F = reinterpret_cast<const PipFlip *>(reinterpret_cast<const PipEdge *>(u + 2) + n);
+        for (int f = 0; f < nf; ++f) {
+            const float d = __fsub_rn(cy, F[f].y);
+            bad |= !(fabsf(d) > diff_bound(cy, F[f].y, eps));
+            if (!(d > 0.0f)) break;
+            m = F[f].mask;
+        }
+    }
+    for (int j = 0; j < n; j += 2) {
+        unsigned mask;
+        const float4 e = edge_at(min(j + (lane >> 4), n - 1), mask);
+        if (j + (lane >> 4) >= n) continue;
+        const float mag = fmaxf(fmaxf(fabsf(e.x), fabsf(e.z)), fmaxf(fabsf(e.y), fabsf(e.w)));
+        const float hx = 0.5f * qx + b.sub_mx + fmaf(8.0f * U32, mag, 2.0f * eps);
+        const float hy = 0.5f * qy + b.sub_my + fmaf(8.0f * U32, mag, 2.0f * eps);
+        const bool box = !(fminf(e.x, e.z) > cx + hx || fmaxf(e.x, e.z) < cx - hx || e.y > cy + hy || e.w < cy - hy);
+        const float dx = e.z - e.x, dy = e.w - e.y;
+        const float p1 = dx * (cy - e.y), p2 = dy * (cx - e.x);
+        bad |= box && !(fabsf(p1 - p2) > (fabsf(dx) * hy + fabsf(dy) * hx) + 16.0f * U32 * (fabsf(p1) + fabsf(p2)));
+        const int x = bad ? 0 : edge_cross(cx, cy, e, eps);
+        bad |= x < 0;
+        if (x > 0) m ^= mask;
+    }
+    m ^= __shfl_xor_sync(FULL, m, 16);
+    bad = ((__ballot_sync(FULL, bad) >> sub) & 0x10001u) != 0;
+    // ids of the lowest set bits; the first two that occur get classes 1 and 2
+    int id = -1;
+    if (!bad && m) {
+        const int k = __ffs(m) - 1;
+        const int4 u1 = u[1];
+        if (u0.w & PIP_EXT) id = reinterpret_cast<const int *>(u + 2 + 2 * (size_t)n + nf)[k];
+        else id = k == 0 ? u1.x : (k == 1 ? u1.y : u1.z);
+    }
+    const unsigned some = __ballot_sync(FULL, !bad && id >= 0);
+    const int id1 = some ? __shfl_sync(FULL, id, __ffs(some) - 1) : -1;
+    const unsigned more = __ballot_sync(FULL, !bad && id >= 0 && id != id1);
+    const int id2 = more ? __shfl_sync(FULL, id, __ffs(more) - 1) : -1;
+    const unsigned cls = bad ? 0u : (id < 0 ? 3u : (id == id1 ? 1u : (id == id2 ? 2u : 0u)));
+    const unsigned all = __reduce_or_sync(FULL, lane < 16 ? cls << (2 * sub) : 0u);
+    if (lane == 0) {
+        b.cells[c].y = (int)all;
+        b.cells[c].z = id1;
+        b.cells[c].w = id2;
+    }
+}
+
 // Record groups larger than this are ordered by a whole block (k_pip_order_long).
 constexpr int PIP_LONG = PIP_LONG_MIN;
 
@@ -808,10 +896,14 @@ __global__ void __launch_bounds__(256) k_pip_order(PipBuildArgs b) {
     const int lane = lane_id();
     const long long T = (long long)gridDim.x * blockDim.x;
     for (long long cc = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; cc < b.g.G; cc += T >> 5) {
-        const int c = (int)cc, code = b.cell_code[c];
+        const int c = (int)cc;
+        const int2 cell = *reinterpret_cast<const int2 *>(&b.cells[c]);   // code, -1: a horizontal edge
+        const int code = cell.x;
         if (code >= -1) continue;
         const float2 fo = cell_frame(b.frame_x, b.frame_y, b.g.nx, c);
         int off = -2 - code, te = b.edges_at[c], tf = b.flips_at[c];
+        __syncwarp();
+        if (cell.y && lane == 0) b.cells[c].y = 0;
         while (true) {
             int4 *u = b.units + 2 * (size_t)off;
             const int4 u0 = u[0];
@@ -821,9 +913,9 @@ __global__ void __launch_bounds__(256) k_pip_order(PipBuildArgs b) {
             } else {
                 PipEdge *E = reinterpret_cast<PipEdge *>(u + 2);
                 float hmax = 0.0f;
+                int2 v = make_int2(0, 0);
+                float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 if (n <= 32) {   // in registers
-                    int2 v = make_int2(0, 0);
-                    float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                     if (lane < n) {
                         v = b.tmp_edge[te + lane];
                         r = edge_rel(b, v.x, fo);
@@ -876,6 +968,21 @@ __global__ void __launch_bounds__(256) k_pip_order(PipBuildArgs b) {
                         if (before) m ^= w.mask;
                     }
                     F[rank - 1] = PipFlip{key_rel(v.key, fo.y), m, v.key};
+                }
+                if (b.sub_mx >= 0.0f && cell.y == 0 && !(u0.w & PIP_MORE) && off == -2 - code) {   // one group
+                    __syncwarp();
+                    if (n <= 32) {
+                        pip_sub_classes(b, c, u0, u, [&](int j, unsigned &mask) {
+                            mask = (unsigned)__shfl_sync(FULL, v.y, j);
+                            return make_float4(__shfl_sync(FULL, r.x, j), __shfl_sync(FULL, r.y, j),
+                                               __shfl_sync(FULL, r.z, j), __shfl_sync(FULL, r.w, j));
+                        }, b.eps, lane);
+                    } else {
+                        pip_sub_classes(b, c, u0, u, [&](int j, unsigned &mask) {
+                            mask = (unsigned)b.tmp_edge[te + j].y;
+                            return b.tmp_rel[te + j];
+                        }, b.eps, lane);
+                    }
                 }
             }
             if (!(u0.w & PIP_MORE)) break;

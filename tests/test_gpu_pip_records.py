@@ -127,3 +127,39 @@ def test_point_counts(api, oracle, n):
         out = torch.full((n + 1,), 7, dtype=torch.int32, device="cuda")[1:]   # any 4-byte alignment
         got = api.pip_join(layer, torch.as_tensor(pts, device="cuda"), out, form="fp32x").cpu().numpy()
     np.testing.assert_array_equal(got, ref)
+
+
+def test_sub_cells(api, oracle):
+    """Cells cut by few edges, whose sub-cells without an edge answer from the
+    cell table: stars, a rectangle and a comb with horizontal and vertical sides
+    on and off the cell and sub-cell lines, a polygon with a hole, dense points
+    around the sub-cell lines."""
+    rng = np.random.default_rng(3)
+    g = dict(x0=0.0, y0=0.0, x1=64.0, y1=64.0, nx=8, ny=8)
+    rings = [star(rng, 14, 14, 5, 12, 7), star(rng, 46, 14, 5, 12, 11),
+             np.array([[3.0, 34.0], [27.0, 34.0], [27.0, 49.5], [3.0, 49.5]]),
+             np.array([[33.0, 33.3], [61.0, 33.3], [61.0, 60.0], [54.0, 60.0], [54.0, 41.0], [47.0, 41.0],
+                       [47.0, 60.0], [33.0, 60.0]])]
+    hole = star(rng, 14, 14, 1, 3, 5)
+    verts = np.concatenate([rings[0], hole] + rings[1:])
+    off = np.concatenate([[0], np.cumsum([len(rings[0]), len(hole)] + [len(r) for r in rings[1:]])]).astype(np.int64)
+    poly = np.array([0, 2, 3, 4, 5], np.int64)
+    line = np.repeat(np.arange(0, 64, 2.0), 200)
+    jit = rng.normal(0, 1e-4, line.size)
+    pts = np.concatenate([rng.uniform(0, 64, (200_000, 2)), np.stack([line + jit, rng.uniform(0, 64, line.size)], 1),
+                          np.stack([rng.uniform(0, 64, line.size), line + jit], 1), points_of(rng, verts, g)])
+    ref = oracle.pip_join(g, pts, verts, off, poly)
+    with api.pip_layer(verts, off, poly, g) as layer:
+        got = api.pip_join(layer, torch.as_tensor(pts, device="cuda"), form="fp32x").cpu().numpy()
+        st = layer.stats()
+    np.testing.assert_array_equal(got, ref)
+    # more points are answered without an edge test than those of the cells that no edge's box meets
+    nxt = np.arange(1, len(verts) + 1)
+    nxt[off[1:] - 1] = off[:-1]
+    lo, hi = np.minimum(verts, verts[nxt]), np.maximum(verts, verts[nxt])
+    free = np.ones((8, 8), bool)
+    for (ax, ay), (bx, by) in zip((lo / 8).astype(int), (hi / 8).astype(int)):
+        free[ay:by + 1, ax:bx + 1] = False
+    inside = np.isfinite(pts).all(1) & (pts >= 0).all(1) & (pts < 64).all(1)
+    cell = (pts[inside] / 8).astype(int)
+    assert st["resolved"] > free[cell[:, 1], cell[:, 0]].sum()
