@@ -170,17 +170,11 @@ struct RoundSource {
     }
 };
 
-// Warps per block and blocks per SM: bound by the latency of its gathers (cell
-// code, record), the join is fastest at the most warps whose 64 registers hold
-// the loop without spills: 100 M points on the 40,000 tiles 1.87 / 1.70 / 1.61 ms
-// with 6 / 7 / 8 blocks, 2.8 ms with 10 (48 registers, spilled).
-#ifndef VB
-#define VB 8
-#endif
-#ifndef VU
-#define VU 2
-#endif
-constexpr int PIP_WARPS = 4, PIP_BLOCKS = VB;
+// Warps per block and blocks per SM: bound by the latency of its gathers, the
+// join is fastest at the most warps whose 64 registers hold the loop without
+// spills: 10 M points on the heavy-tail tiles 458 / 430 / 445 us with 7 / 8 / 10
+// blocks (48 registers, spilled), 100 M on the 40,000 tiles 1.12 / 1.14 / 1.32 ms.
+constexpr int PIP_WARPS = 4, PIP_BLOCKS = 8;
 // Code of a queued point whose cell the FP32 estimate leaves open (no record
 // starts there: units are fewer than 2^31 - 2^22).
 constexpr int PIP_UNSURE = -2147483647 - 1;
@@ -267,9 +261,12 @@ __device__ __forceinline__ bool pip_fast(const PipArgs &a, const PipQueued &q, P
     return true;
 }
 
-// The general case, one point by the whole warp: any number of groups, long
-// lists searched by y, tests that FP32 leaves open redone with the FP64 rule.
-__device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, PipSums &sum, int lane, unsigned &fb) {
+// The general case, one point by HARD lanes (lane: 0 .. HARD - 1, mask gm): any
+// number of groups, long lists searched by y, tests that FP32 leaves open redone
+// with the FP64 rule.
+constexpr int HARD = 16;   // 4 / 8 / 16 / 32: 506 / 420 / 401 / 425 us on the heavy-tail tiles (lists of 30 to 3,000 edges)
+__device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, PipSums &sum, int lane, unsigned gm,
+                                        unsigned &fb) {
     const double2 p = q.p;
     const float2 r = point_rel(a, q);
     const unsigned long long ky = y_key(p.y);
@@ -316,25 +313,25 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
             }
         }
         unsigned mm = 0;
-        for (int t = lo + lane; t < hi; t += 4 * 32) {   // four loads in flight per lane
+        for (int t = lo + lane; t < hi; t += 4 * HARD) {   // four loads in flight per lane
             float4 e[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (t + 32 * k < hi) e[k] = __ldg(reinterpret_cast<const float4 *>(E + t + 32 * k));
+                if (t + HARD * k < hi) e[k] = __ldg(reinterpret_cast<const float4 *>(E + t + HARD * k));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                if (t + 32 * k >= hi) break;
+                if (t + HARD * k >= hi) break;
                 int x = edge_cross(r.x, r.y, e[k], a.eps);
                 if (x < 0) {
-                    const int i = E[t + 32 * k].vid;
+                    const int i = E[t + HARD * k].vid;
                     const double2 A = a.verts[i], B = a.verts[a.nxt[i]];
                     x = cross64(p.x, p.y, A.x, A.y, B.x, B.y);
                     ++fb;
                 }
-                if (x) mm ^= E[t + 32 * k].mask;
+                if (x) mm ^= E[t + HARD * k].mask;
             }
         }
-        m ^= __reduce_xor_sync(FULL, mm);
+        m ^= __reduce_xor_sync(gm, mm);
         tests += (unsigned)(hi - lo);
         if (m) {
             const int k = __ffs(m) - 1;
@@ -359,12 +356,13 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 // then their general, register-hungry code costs the loop nothing (with a call
 // to it inside the loop the 100 M point join took 2.3 - 4.5 ms instead of 1.6).
 //
-// Bound by the latency and the L1 wavefronts of the random reads of cell codes
-// and records, both L2-resident (ncu at 20 M points on the tiles: issue slots
-// 53 % busy, long-scoreboard the top stall, DRAM 13 % of peak).  Measured, us a
-// join, against bucketing the points and refining (cell, point-chunk) items:
-// 1,003 points 53 -> 12, 1 M points on the stars (FP64 form) 119 -> 30, 10 M on
-// the heavy-tail tiles 2,450 -> 531, 100 M on the 40,000 tiles 4,486 -> 1,548.
+// Bound by the latency and the L1 wavefronts of the random reads of the cell
+// table and the records, both L2-resident (ncu at 20 M points on the tiles: issue
+// slots half busy, long-scoreboard the top stall, DRAM 14 % of peak).  Measured, us
+// a join, against bucketing the points and refining (cell, point-chunk) items,
+// then without and with the sub-cell classes: 1,003 points 53 -> 11 -> 11, 1 M on
+// the stars (FP64 form) 119 -> 29 -> 21, 10 M on the heavy-tail tiles 2,450 -> 536
+// -> 426 (401 with HARD = 16), 100 M on the 40,000 tiles 4,486 -> 1,590 -> 1,130.
 template <int U, class Src>
 __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src) {
     __shared__ PipQueued queue[PIP_WARPS][32 * (U + 1)];
@@ -461,19 +459,30 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
                 act = false;
             }
         }
-        for (unsigned left = __ballot_sync(FULL, act); left; left &= left - 1) {
-            const int j = __ffs(left) - 1;
-            PipQueued r;
-            r.p = make_double2(__shfl_sync(FULL, q.p.x, j), __shfl_sync(FULL, q.p.y, j));
-            r.i = __shfl_sync(FULL, q.i, j);
-            r.code = __shfl_sync(FULL, q.code, j);
-            r.ix = __shfl_sync(FULL, q.ix, j);
-            r.iy = __shfl_sync(FULL, q.iy, j);
-            const int id = pip_hard(a, r, sums[threadIdx.x], lane, fb);
-            if (lane == 0) {
-                src.put((unsigned)r.i, id);
-                hits += id >= 0;
+        const int sub = lane & (HARD - 1), grp = lane / HARD;
+        const unsigned gm = (HARD == 32 ? FULL : (1u << (HARD & 31)) - 1u) << (lane & ~(HARD - 1));
+        for (unsigned left = __ballot_sync(FULL, act); left;) {   // a point for each group of lanes
+            int j = -1;
+#pragma unroll
+            for (int k = 0; k < 32 / HARD; ++k) {
+                if (grp == k && left) j = __ffs(left) - 1;
+                left &= left - 1;
             }
+            const int from = j < 0 ? lane : j;
+            PipQueued r;
+            r.p = make_double2(__shfl_sync(FULL, q.p.x, from), __shfl_sync(FULL, q.p.y, from));
+            r.i = __shfl_sync(FULL, q.i, from);
+            r.code = __shfl_sync(FULL, q.code, from);
+            r.ix = __shfl_sync(FULL, q.ix, from);
+            r.iy = __shfl_sync(FULL, q.iy, from);
+            if (j >= 0) {
+                const int id = pip_hard(a, r, sums[threadIdx.x], sub, gm, fb);
+                if (sub == 0) {
+                    src.put((unsigned)r.i, id);
+                    hits += id >= 0;
+                }
+            }
+            __syncwarp();
         }
         if (__any_sync(FULL, act)) ++items;
     }
@@ -492,9 +501,9 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
 }
 
 // Points per lane and tile: two once that still gives every SM all its warps
-// twice over (100 M points: 1.69 / 1.55 / 1.90 ms with 1 / 2 / 4); smaller calls
-// spread over more warps, one point per lane.
-constexpr int PIP_U = VU;
+// twice over (100 M points: 1.32 / 1.14 / 1.13 / 1.38 ms with 1 / 2 / 3 / 4); smaller
+// calls spread over more warps, one point per lane.
+constexpr int PIP_U = 2;
 
 static int pip_blocks(int U, long long n, int sms) {
     const long long tiles = (n + 32LL * U - 1) / (32LL * U);
