@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
     const unsigned n = (unsigned)src.count(), tiles = (n + 32u * U - 1u) / (32u * U);
     unsigned items = 0, resolved = 0, hits = 0, fb = 0;
     sums[threadIdx.x] = PipSums{0, 0, 0};
-    int qn = 0, head = -1;
+    int qn = 0, head = -1, waiting = 0;
     for (unsigned t = blockIdx.x * PIP_WARPS + w;; t += gridDim.x * PIP_WARPS) {
         const bool more = t < tiles;   // else: the points left in the queues
         if (more) {
@@ -425,7 +425,10 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
                 const bool done = pip_fast(a, q, sums[threadIdx.x], res);
                 if (SJ_IN_BOUNDS((unsigned)q.i < n, BND_PIP_RES)) {
                     src.put((unsigned)q.i, done ? res : head);
-                    if (!done) head = q.i;
+                    if (!done) {
+                        head = q.i;
+                        ++waiting;
+                    }
                     hits += done && res >= 0;
                 }
             }
@@ -434,10 +437,13 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
         if (!more) break;
         __syncwarp();
     }
-    while (__any_sync(FULL, head >= 0)) {   // the lists, one point of each lane at a time
+    // The lists, one point of each lane at a time; counted, and their links
+    // checked, so that a caller's overlapping outputs cannot lead them astray.
+    while (__any_sync(FULL, waiting > 0)) {
         PipQueued q;
         q.i = head;
-        bool act = head >= 0;
+        bool act = waiting > 0 && (unsigned)head < n;
+        waiting = act ? waiting - 1 : 0;
         int res = -1;
         if (act) {
             head = src.get((unsigned)q.i);
