@@ -803,21 +803,27 @@ __device__ __forceinline__ void fp32x_output(const SegArgs &a, const P2PRec r, d
     }
 }
 
+// Points (pairs of points) per thread in the finishing kernels: four in flight
+// once the call fills the GPU that way, else one, over four times the blocks
+// (whole FP64 calls, four against one: 60,007 points 63.0 and 58.4 us, 131,000
+// points 92.0 and 90.0, 400,000 points 194.8 and 197.3).
 constexpr int FIN_U = 4;
+constexpr long long FIN_MANY = 152LL * 2048;
 
 // One request, two consecutive points per thread and step (one 8-byte load of
 // their slots, 8- and 16-byte stores): half the memory instructions of one
 // point at a time, whose load / store queue fills first.  out_id 8-byte and
 // out_d 16-byte aligned, n even or odd.
+template <int U>
 __global__ void k_p2p_finish_pairs(SegArgs a, const int *pos, const P2PRec *rec, const double2 *pts, int n, int *out_id,
                                    double *out_d) {
     const unsigned T = gridDim.x * blockDim.x;
     const unsigned pairs = ((unsigned)n + 1u) / 2u;
-    for (unsigned p0 = blockIdx.x * blockDim.x + threadIdx.x; p0 < pairs; p0 += FIN_U * T) {
-        int2 j[FIN_U];
-        P2PRec r0[FIN_U], r1[FIN_U];
+    for (unsigned p0 = blockIdx.x * blockDim.x + threadIdx.x; p0 < pairs; p0 += U * T) {
+        int2 j[U];
+        P2PRec r0[U], r1[U];
 #pragma unroll
-        for (int u = 0; u < FIN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
             const unsigned p = p0 + u * T, i = 2u * p;
             j[u] = make_int2(-1, -1);
             if (p < pairs) {
@@ -826,14 +832,14 @@ __global__ void k_p2p_finish_pairs(SegArgs a, const int *pos, const P2PRec *rec,
             }
         }
 #pragma unroll
-        for (int u = 0; u < FIN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
             if (j[u].x >= 0 && !SJ_IN_BOUNDS(j[u].x < n, BND_UNSORT)) j[u].x = -1;
             if (j[u].y >= 0 && !SJ_IN_BOUNDS(j[u].y < n, BND_UNSORT)) j[u].y = -1;
             r0[u] = j[u].x >= 0 ? rec[j[u].x] : P2PRec{-1, -1};
             r1[u] = j[u].y >= 0 ? rec[j[u].y] : P2PRec{-1, -1};
         }
 #pragma unroll
-        for (int u = 0; u < FIN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
             const unsigned p = p0 + u * T, i = 2u * p;
             if (p >= pairs) continue;
             const bool two = i + 1u < (unsigned)n;
@@ -918,7 +924,7 @@ __global__ void k_p2p_finish_fp32x(SegArgs a, const P2PRec *rec, Src src) {
 }
 
 // FP64: the FP64 distances to the one or two segments of each point's record.
-// A warp takes FIN_U x 32 points; the second segments, which about a third of
+// A warp takes U x 32 points; the second segments, which about a third of
 // the points have, are gathered in shared memory and evaluated with full warps,
 // since the FP64 pipe takes as long for one lane as for 32.  The compares of
 // the (non-negative, finite) distances and of t are made on their bit patterns,
@@ -937,29 +943,29 @@ __device__ __forceinline__ double seg_d2_finite(const SegArgs &a, double2 p, int
 
 constexpr int FIN_WARPS = 8;
 
-template <class Src>
+template <int U, class Src>
 __global__ void __launch_bounds__(FIN_WARPS * 32) k_p2p_finish_fp64(SegArgs a, const P2PRec *rec, Src src,
                                                                     unsigned long long *stats) {
-    __shared__ int2 q[FIN_WARPS][32 * FIN_U];        // (point of the tile, second segment)
-    __shared__ double d2s[FIN_WARPS][32 * FIN_U];
+    __shared__ int2 q[FIN_WARPS][32 * U];        // (point of the tile, second segment)
+    __shared__ double d2s[FIN_WARPS][32 * U];
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const long long n = src.count();
     unsigned hits = 0;
-    for (long long base = (blockIdx.x * (long long)FIN_WARPS + w) * (32 * FIN_U); base < n;
-         base += (long long)gridDim.x * FIN_WARPS * (32 * FIN_U)) {
-        P2PRec r[FIN_U];
-        double d2[FIN_U];
+    for (long long base = (blockIdx.x * (long long)FIN_WARPS + w) * (32 * U); base < n;
+         base += (long long)gridDim.x * FIN_WARPS * (32 * U)) {
+        P2PRec r[U];
+        double d2[U];
         int nq = 0;
 #pragma unroll
-        for (int u = 0; u < FIN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
             const long long i = base + 32 * u + lane;
             const int j = i < n ? src.slot((int)i) : -1;
             r[u] = j >= 0 ? rec[j] : P2PRec{-1, -1};
         }
 #pragma unroll
-        for (int u = 0; u < FIN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
             const bool two = r[u].id >= 0 && r[u].aux >= 0;
             const unsigned bal = __ballot_sync(FULL, two);
             if (two) q[w][nq + __popc(bal & lt)] = make_int2(32 * u + lane, r[u].aux);
@@ -973,7 +979,7 @@ __global__ void __launch_bounds__(FIN_WARPS * 32) k_p2p_finish_fp64(SegArgs a, c
         }
         __syncwarp();
 #pragma unroll
-        for (int u = 0; u < FIN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
             const long long i = base + 32 * u + lane;
             if (i >= n) continue;
             int id = -1;
@@ -1017,7 +1023,8 @@ static void finish(const RefineArgs &a, int form, const Src &src, long long n_ma
     if (form == SJ_FP32X)
         k_p2p_finish_fp32x<Src><<<fin_blocks(n_max, 256, 152 * 16), 256, 0, s>>>(a.seg, a.rec, src);
     else
-        k_p2p_finish_fp64<Src><<<fin_blocks(n_max, 32 * FIN_U * FIN_WARPS, 152 * 16), FIN_WARPS * 32, 0, s>>>(
+        (n_max >= FIN_MANY ? k_p2p_finish_fp64<FIN_U, Src> : k_p2p_finish_fp64<1, Src>)<<<
+            fin_blocks(n_max, 32 * FIN_WARPS * (n_max >= FIN_MANY ? FIN_U : 1), 152 * 16), FIN_WARPS * 32, 0, s>>>(
             a.seg, a.rec, src, a.stats);
 }
 
@@ -1026,8 +1033,9 @@ static void finish(const RefineArgs &a, int form, const Src &src, long long n_ma
 cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int n, int *out_id, double *out_d,
                               cudaStream_t s) {
     if (form == SJ_FP32X && pos && ((uintptr_t)out_id & 7) == 0 && ((uintptr_t)out_d & 15) == 0)
-        k_p2p_finish_pairs<<<fin_blocks(((n + 1LL) / 2 + FIN_U - 1) / FIN_U, 256, 152 * 16), 256, 0, s>>>(
-            a.seg, pos, a.rec, a.pts, n, out_id, out_d);
+        (n >= FIN_MANY ? k_p2p_finish_pairs<FIN_U> : k_p2p_finish_pairs<1>)<<<
+            fin_blocks((n + 1LL) / 2, 256 * (n >= FIN_MANY ? FIN_U : 1), 152 * 16), 256, 0, s>>>(a.seg, pos, a.rec, a.pts, n,
+                                                                                            out_id, out_d);
     else
         finish(a, form, FinOne{pos, a.pts, out_id, out_d, n, a.D}, n, s);
     return cudaGetLastError();
