@@ -393,7 +393,6 @@ __global__ void k_scatter(BucketArgs a) {
     for (unsigned q0 = blockIdx.x * blockDim.x + threadIdx.x; q0 < pairs; q0 += (UNR / 2) * T) {
         auto elem = [&](int u) { return 2u * (q0 + (unsigned)(u >> 1) * T) + (unsigned)(u & 1); };
         int2 k[UNR];
-        double2 p[UNR];
 #pragma unroll
         for (int u = 0; u < UNR; u += 2) {
             const unsigned i = elem(u);
@@ -404,13 +403,6 @@ __global__ void k_scatter(BucketArgs a) {
                 k[u + 1] = make_int2(kk.z, kk.w);
             } else if (i < (unsigned)a.n) {
                 k[u] = a.key_rank[i];
-            }
-        }
-        if (a.spts) {
-#pragma unroll
-            for (int u = 0; u < UNR; ++u) {
-                const unsigned i = elem(u);
-                if (i < (unsigned)a.n) p[u] = a.pts[i];
             }
         }
         // With a.pos (cell_base set): only points of cells that yield work
@@ -431,10 +423,7 @@ __global__ void k_scatter(BucketArgs a) {
         }
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
-            if (pos[u] >= 0 && SJ_IN_BOUNDS(pos[u] < a.n, BND_SCATTER)) {
-                a.perm[pos[u]] = (int)elem(u);
-                if (a.spts) a.spts[pos[u]] = p[u];
-            }
+            if (pos[u] >= 0 && SJ_IN_BOUNDS(pos[u] < a.n, BND_SCATTER)) a.perm[pos[u]] = (int)elem(u);
         }
         if (a.pos) {
 #pragma unroll

@@ -489,7 +489,6 @@ struct BucketArgs {
     int2 *key_rank;      // [n] (cell, rank within cell)
     int *cell_start;     // [G + 1]
     int *perm;           // [n]
-    double2 *spts;       // [n] cell-ordered copy of the points, or null (not written)
     const int *cand_start;  // layer candidates (null: no work items)
     int ch;
     const int *cell_work;   // with budget > 0: work items of cell_chunk(ch, cell_work[c], budget) points
