@@ -454,11 +454,18 @@ cudaError_t launch_bucket_scan(const BucketArgs &a, cudaStream_t s) {
 }
 
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t s) {
-    int nb = stream_blocks(a.n, 256, 152 * 32);
+    constexpr int NB_MAX = 152 * 32;
+    int nb = stream_blocks(a.n, 256, NB_MAX);
+    // The largest grid runs in eight whole waves of four blocks per SM, which
+    // the shared memory that a block asks for holds it to (five fit by
+    // registers): the atomics bound it either way (170 M points, the join 12.81
+    // and 12.82 ms), and the ranks of a cell's points, which decide the points
+    // that share a work item, then vary least from run to run.
+    const size_t waves = nb == NB_MAX ? 46 * 1024 : 0;
     if (a.sub_lx < 0 || a.sub_ly < 0 || a.sub_lx > 3 || a.sub_ly > 3 || ((a.sub_lx + a.sub_ly) && !a.sub_start) ||
         (a.budget > 0 && !a.cell_work))
         return cudaErrorInvalidValue;
-    k_cell_hist<<<nb, 256, 0, s>>>(a);
+    k_cell_hist<<<nb, 256, waves, s>>>(a);
     cudaError_t e = launch_bucket_scan(a, s);
     if (e != cudaSuccess) return e;
     k_scatter<<<nb, 256, 0, s>>>(a);
