@@ -644,10 +644,10 @@ def run_ours(args):
     stream = torch.cuda.current_stream(dev)
     baselines = rank == 0 and world == 1 and not args.no_baselines
     head = join_leg(api, args, w, dev, stream, world, args.steps, args.warmup, peaks, baselines=baselines)
-    # PIP: one kernel.  P2P: cell_hist, the scan (2 phases up to 256 tiles of 1,024 cells, else 3), scatter;
-    # refine; FP32X recheck; unsort
+    # PIP: one kernel.  P2P: cell_hist, scatter, refine, recheck and the finishing kernel, and the scan (2 phases
+    # up to 256 tiles of 1,024 cells, else 3)
     scan_tiles = (int(w.grid["nx"]) * int(w.grid["ny"]) + 1023) // 1024
-    kernels_per_join = 1 if w.kind == "pip" else 5 + (1 if scan_tiles <= 256 else 2) - 1 + (args.form == "fp32x")
+    kernels_per_join = 1 if w.kind == "pip" else 5 + (2 if scan_tiles <= 256 else 3)
     extra = {}
     if rank == 0 and world == 1 and args.workload == "p2p" and not args.no_extra and not args.points:
         import copy

@@ -1,11 +1,12 @@
 """Autotuner for the join's launch knobs.
 
-Knobs (none changes a result):
+Knobs (none changes a result; the first three shape polyline joins only, a
+polygon join is one kernel without work items):
   * points per work item -- how many points of a cell one warp refines
     against the cell's staged candidates;
   * edges per chunk -- the edge budget of a work item: a cell whose points
-    each test more edges is cut into smaller items, so heavy cells (complex
-    polygons, Sec. IV.C; dense polyline cells) spread over more warps;
+    each test more segments is cut into smaller items, so dense cells spread
+    over more warps;
   * block -- warps per refinement block (2, 4 or 8);
   * the filter grid resolution (Sec. III.A: a finer grid gives fewer false
     candidates but more cells and smaller items -- the paper's own

@@ -15,7 +15,7 @@ constexpr int MAX_CH = 128;        // largest point chunk per work item
 // (points, vertices, candidate and list entries): every grid-stride loop with
 // a 32-bit index advances by at most 2^22 (grids are capped below that), so an
 // index i < MAX_COUNT never passes 2^31 - 1 when it advances; loops with a
-// larger step (the unrolled bucketing and unsort kernels) count in 64 bits.
+// larger step (the unrolled bucketing and finishing kernels) count in unsigned 32 or 64 bits.
 constexpr long long MAX_COUNT = (1LL << 31) - (1LL << 22);
 constexpr float U32 = 5.9604644775390625e-08f;   // 2^-24, unit roundoff of FP32
 
