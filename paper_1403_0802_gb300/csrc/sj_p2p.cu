@@ -809,6 +809,11 @@ __device__ __forceinline__ void fp32x_output(const SegArgs &a, const P2PRec r, d
 // points 92.0 and 90.0, 400,000 points 194.8 and 197.3).
 constexpr int FIN_U = 4;
 constexpr long long FIN_MANY = 152LL * 2048;
+// Blocks of k_p2p_finish_pairs at most: one tile each, in input order, for all
+// but the largest calls.  Blocks that each walk the whole input (16 per SM)
+// gather their records from all over the array at once: whole calls, 16 and 512
+// blocks per SM, 170 M points 12.23 and 12.12 ms, 10 M points 746 and 741 us.
+constexpr int PAIRS_MAX = 152 * 512;
 
 // One request, two consecutive points per thread and step (one 8-byte load of
 // their slots, 8- and 16-byte stores): half the memory instructions of one
@@ -1034,7 +1039,7 @@ cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int
                               cudaStream_t s) {
     if (form == SJ_FP32X && pos && ((uintptr_t)out_id & 7) == 0 && ((uintptr_t)out_d & 15) == 0)
         (n >= FIN_MANY ? k_p2p_finish_pairs<FIN_U> : k_p2p_finish_pairs<1>)<<<
-            fin_blocks((n + 1LL) / 2, 256 * (n >= FIN_MANY ? FIN_U : 1), 152 * 16), 256, 0, s>>>(a.seg, pos, a.rec, a.pts, n,
+            fin_blocks((n + 1LL) / 2, 256 * (n >= FIN_MANY ? FIN_U : 1), PAIRS_MAX), 256, 0, s>>>(a.seg, pos, a.rec, a.pts, n,
                                                                                             out_id, out_d);
     else
         finish(a, form, FinOne{pos, a.pts, out_id, out_d, n, a.D}, n, s);
