@@ -163,6 +163,17 @@ static bool grid_ok(const sj_grid *g) {
     return g->x1 > g->x0 && g->y1 > g->y0;
 }
 
+// Bound of axis_estimate's error, in cells: |v - fl(v)| < 2u |v| (truncation) or
+// 2^-126 (flushed to zero), |x0f - x0| <= u |x0|, the difference's rounding u per
+// cell index, 1 / w rounded (2u) and the product (u): at most (3u max|x| + 2^-126)
+// / w + 4u n cells, times 1.5.  Beyond 1e37 the estimate is never certain (2 cells):
+// from 3.4e38 on approx_float clamps, and 1 / w leaves the FP32 normal range at
+// 8.5e37.  Below, a clamped value maps past the grid's end.
+static float estimate_tol(double lo, double hi, double w, int n) {
+    const double u = 5.9604644775390625e-08, m = std::max(std::fabs(lo), std::fabs(hi));
+    return m <= 1e37 ? (float)(1.5 * ((3.0 * u * m + 1.1754943508222875e-38) / w + 4.0 * u * n)) : 2.0f;
+}
+
 static GridDev make_grid(const sj_grid *g) {
     GridDev d;
     d.x0 = g->x0; d.y0 = g->y0; d.x1 = g->x1; d.y1 = g->y1;
@@ -173,12 +184,8 @@ static GridDev make_grid(const sj_grid *g) {
     d.cw = cw; d.ch = ch;
     d.x0f = (float)g->x0; d.y0f = (float)g->y0;
     d.icwf = (float)(1.0 / cw); d.ichf = (float)(1.0 / ch);
-    // axis_estimate: |v - fl(v)| < 2u |v| (truncation), |x0f - x0| <= u |x0|, the
-    // difference's rounding u per cell index, 1 / cw rounded (2u) and the product
-    // (u): at most 3u max|x| / cw + 4u nx cells, times 1.5
-    const double u = 5.9604644775390625e-08;
-    d.tolx = (float)(1.5 * u * (3.0 * std::max(std::fabs(g->x0), std::fabs(g->x1)) / cw + 4.0 * g->nx));
-    d.toly = (float)(1.5 * u * (3.0 * std::max(std::fabs(g->y0), std::fabs(g->y1)) / ch + 4.0 * g->ny));
+    d.tolx = estimate_tol(g->x0, g->x1, cw, g->nx);
+    d.toly = estimate_tol(g->y0, g->y1, ch, g->ny);
     d.kx = d.ky = nullptr;
     return d;
 }

@@ -110,9 +110,10 @@ __device__ __forceinline__ int axis_cell(double v, const unsigned long long *key
 // Cell index along one axis from FP32 alone: true when the estimate lies
 // farther than its error bound tol from every cell boundary and inside the
 // grid, so that i is certain; r is then the place within the cell, 0 to 1, off
-// by at most tol.  The bound (make_grid) covers the truncation of v
-// to FP32, the rounding of lo and 1 / w, and the two operations; NaN, infinite
-// and far outside values are never certain.
+// by at most tol.  The bound (estimate_tol) covers the truncation of v to FP32
+// (subnormals to zero), the rounding of lo and 1 / w, and the two operations; it
+// is above 1 for grids that leave the FP32 range.  NaN, infinite and far outside
+// values are never certain.
 __device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i, float &r) {
     const float t = __fmul_rn(__fsub_rn(approx_float(v), lof), iwf);
     const float f = floorf(t);
