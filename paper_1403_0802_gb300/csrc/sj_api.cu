@@ -215,7 +215,7 @@ static float float_up(double x) {
 }
 
 // Layer-dependent fields of the P2P refinement arguments.
-void sj::fill_refine(const sj_layer *L, int form, RefineArgs &ra) {
+void sj::fill_refine(const sj_layer *L, RefineArgs &ra) {
     ra.g = L->g;
     ra.seg = SegArgs{L->verts, L->seg_e64, L->seg_inv64, L->seg32};
     ra.cseg_start = L->cseg_start;
@@ -226,10 +226,9 @@ void sj::fill_refine(const sj_layer *L, int form, RefineArgs &ra) {
     ra.Ddn = L->Ddn;
     ra.Dup = L->Dup;
     ra.eps_abs = L->eps_abs;
-    // FP64 form: where the squares of coordinates or the FP32 inverse lengths
-    // could leave the FP32 range, an infinite bound sends every point to the
-    // FP64 recheck
-    if (form == SJ_FP64 && !(L->xmax <= 1e15 && L->xmax >= 1e-6)) ra.eps_abs = INFINITY;
+    // where the squares of coordinates or the FP32 inverse lengths could leave
+    // the FP32 range, an infinite bound sends every point to the FP64 recheck
+    if (!(L->xmax <= 1e15 && L->xmax >= 1e-6)) ra.eps_abs = INFINITY;
     ra.frame_x = L->frames;
     ra.frame_y = L->frames + L->g.nx;
     ra.stats = L->stats;
@@ -905,7 +904,7 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
         return check_bounds(s);
     }
     RefineArgs ra{};
-    fill_refine(L, form, ra);
+    fill_refine(L, ra);
     if (window >= 0.0) {
         ra.D = window;
         ra.Df = (float)window;
@@ -1287,7 +1286,7 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     const int G = L->g.G;
     if (N <= (form == SJ_FP32X ? P2P_DIRECT_FP32X : P2P_DIRECT_FP64)) {   // as join_impl
         RefineArgs ra{};
-        fill_refine(L, form, ra);
+        fill_refine(L, ra);
         ra.pts = (const double2 *)pts;
         ra.npts = (int)N;
         ra.rec = reinterpret_cast<P2PRec *>(base);
@@ -1327,7 +1326,7 @@ extern "C" sj_status sj_p2p_join_noalloc(const sj_layer *L, const double *pts, i
     CUDA_TRY(cudaMemsetAsync(b.key_rank, 0xff, sizeof(int2) * (size_t)N, s));
 
     RefineArgs ra{};
-    fill_refine(L, form, ra);
+    fill_refine(L, ra);
     ra.items = b.items;
     ra.n_items = b.totals + 1;
     ra.cell_start = b.cell_start;

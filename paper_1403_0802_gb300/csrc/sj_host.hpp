@@ -96,7 +96,7 @@ bool fault_fires(int kind);
 cudaError_t dev_malloc(void **p, size_t bytes);
 cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s);
 sj_status device_info(int dev, DevInfo **out);
-void fill_refine(const sj_layer *L, int form, RefineArgs &ra);
+void fill_refine(const sj_layer *L, RefineArgs &ra);
 PipArgs pip_args(const sj_layer *L);
 
 inline bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }

@@ -220,8 +220,8 @@ __device__ __forceinline__ void p2p_result(const RefineArgs &a, const P2PItem &i
     if (PW && pw) window_f32(a.win[j], Ddn, Dup);
     P2PRec r{-1, -1};
     bool redo = false;
-    // F64, e infinite: coordinates beyond the range of the bound (every point is redone)
-    if (F64 && !(e < __int_as_float(0x7f800000))) {
+    // e infinite: coordinates beyond the range of the bound (every point is redone)
+    if (!(e < __int_as_float(0x7f800000))) {
         redo = true;
     } else if (st.i1 >= 0 && !((d - e) * (1.0f - 4.0f * U32) > Dup)) {   // not certainly outside the window
         const bool alone = (d2 - d) * (1.0f - 4.0f * U32) > sep;         // no other one within 2E
@@ -533,6 +533,7 @@ __global__ void __launch_bounds__(256) k_p2p_recheck(RefineArgs a) {
 __device__ __forceinline__ int fp32x_decide(const RefineArgs &a, const Best<false> &st, float mag) {
     const float d = sqrtf(st.b1), d2 = sqrtf(st.b2);
     const float e = fmaf(64.0f * U32, mag, 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
+    if (!(e < __int_as_float(0x7f800000))) return 2;   // as in p2p_result
     if (st.i1 < 0 || (d - e) * (1.0f - 4.0f * U32) > a.Dup) return 0;
     const bool in_window = (d + e) * (1.0f + 4.0f * U32) < a.Ddn;
     const bool separated = (d2 - d) * (1.0f - 4.0f * U32) > 2.0f * e * (1.0f + 4.0f * U32);

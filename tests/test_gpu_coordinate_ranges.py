@@ -103,3 +103,39 @@ def test_polylines(api, oracle, x0, cell):
             # and to the coordinates that it is taken from
             tol = 1e-12 * np.maximum(rd[hit], cell) + 4e-16 * abs(x0)
             assert np.all(np.abs(gd[hit] - rd[hit]) <= tol)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-9, 1.0, 1e17, 1e27])
+def test_fp32x_squares_out_of_range(api, oracle, scale):
+    """FP32X where the squares of distances overflow or underflow FP32: every
+    point within D of a polyline is found, none beyond it is."""
+    rng = np.random.default_rng(2)
+    verts = rng.uniform(20, 230, (90, 2)) * scale
+    off = np.arange(0, 91, 3, dtype=np.int64)
+    g = dict(x0=0.0, y0=0.0, x1=256.0 * scale, y1=256.0 * scale, nx=32, ny=32)
+    pts = rng.uniform(-5, 260, (3_000, 2)) * scale
+    dev = torch.as_tensor(pts, device="cuda")
+    far = 256 * 2 ** 0.5 * scale
+    for D in (12.0 * scale, 150.0 * scale):
+        rid, rd, d1, d2 = oracle.p2p_join(g, pts, verts, off, D)
+        # the distance bound of FP32X (E = 64 u M, u = 2^-24, M at most twice the extent) is below 1e-5 of the extent
+        with np.errstate(invalid="ignore"):
+            clear = ~((np.abs(d2 - d1) <= 1e-5 * far) | (np.abs(d1 - D) <= 1e-5 * far))
+        with api.p2p_layer(verts, off, D, g) as layer:
+            got = [api.p2p_join(layer, dev, form="fp32x", pts_per_item=ppi) for ppi in (0, 128)]
+            got.append(api.p2p_join(layer, dev, form="fp32x", window=D))
+            oid, od = torch.empty_like(got[0][0]), torch.empty_like(got[0][1])
+            got.append(api.p2p_join_noalloc(layer, dev, oid, od, form="fp32x"))
+            out = (torch.empty_like(oid), torch.empty_like(od))
+            with api.Engine(max_points=len(pts), max_requests=1, form="fp32x") as eng:
+                s = torch.cuda.Stream()
+                eng.round([(layer, dev, *out)], s)
+                s.synchronize()
+            got.append(out)
+            torch.cuda.synchronize()
+        for gid, gd in got:
+            gid, gd = gid.cpu().numpy(), gd.cpu().numpy()
+            np.testing.assert_array_equal(gid[clear], rid[clear])
+            hit = (gid >= 0) & (rid >= 0)
+            assert hit.sum() > 100
+            assert np.all(np.abs(gd[hit] - rd[hit]) <= 1e-5 * far)
