@@ -472,6 +472,16 @@ struct DirectArgs {
     double *out_d;     //   (may be null)
 };
 constexpr int P2P_DIRECT_FP32X = 32768, P2P_DIRECT_FP64 = 131072;
+constexpr int DIRECT_WARPS = 8;   // of a block
+constexpr int DIRECT_OPEN = 64;   // FP32X: points of a block whose work item matters, at most
+// Blocks of a direct call: a warp per point up to eight blocks an SM, then
+// several points a warp, but (a part of a GPU with few SMs) no block more points
+// than it can leave open.
+constexpr int p2p_direct_blocks(int n, int sms) {
+    const int most = (n + DIRECT_WARPS - 1) / DIRECT_WARPS, least = (n + DIRECT_OPEN - 1) / DIRECT_OPEN;
+    const int blocks = most < sms * 8 ? most : (least > sms * 8 ? least : sms * 8);
+    return blocks > 1 ? blocks : 1;
+}
 cudaError_t launch_p2p_direct(const RefineArgs &a, const DirectArgs &g, int form, int n, int sms, cudaStream_t s);
 cudaError_t launch_p2p_finish(const RefineArgs &a, int form, const int *pos, int n, int *out_id, double *out_d,
                               cudaStream_t s);

@@ -586,9 +586,6 @@ __device__ __forceinline__ Best64 list_best64(const RefineArgs &a, int g0, int g
     return st;
 }
 
-constexpr int DIRECT_WARPS = 8;
-constexpr int DIRECT_OPEN = 64;   // points of a block whose work item matters
-
 template <bool F64>
 __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, DirectArgs g, int n) {
     __shared__ int open[DIRECT_OPEN], open_n, box[4];
@@ -777,16 +774,10 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
     }
 }
 
-// Points of a call per warp of the grid (every resident warp once, then more
-// each); DIRECT_OPEN bounds the points of a block.
 cudaError_t launch_p2p_direct(const RefineArgs &a, const DirectArgs &g, int form, int n, int sms, cudaStream_t s) {
-    const int blocks = std::max(1, std::min((n + DIRECT_WARPS - 1) / DIRECT_WARPS, sms * 8));
-    if (form == SJ_FP32X) {
-        if ((long long)n > (long long)blocks * DIRECT_OPEN) return cudaErrorInvalidValue;
-        k_p2p_direct<false><<<blocks, DIRECT_WARPS * 32, 0, s>>>(a, g, n);
-    } else {
-        k_p2p_direct<true><<<blocks, DIRECT_WARPS * 32, 0, s>>>(a, g, n);
-    }
+    const int blocks = p2p_direct_blocks(n, sms);
+    if (form == SJ_FP32X) k_p2p_direct<false><<<blocks, DIRECT_WARPS * 32, 0, s>>>(a, g, n);
+    else k_p2p_direct<true><<<blocks, DIRECT_WARPS * 32, 0, s>>>(a, g, n);
     return cudaGetLastError();
 }
 
