@@ -304,8 +304,8 @@ typedef struct {
  * requests per layer.  opts selects form and points per work item (as for the
  * joins; NULL = defaults).  The engine allocates one workspace per layer on
  * the first round that uses the layer (for a polyline layer about 60 bytes per
- * point and 8 bytes per grid cell; for a polygon layer the request table alone) and captures that layer's graph then; later rounds allocate
- * nothing.  Layers must outlive the engine.  Errors: SJ_ERR_INVALID. */
+ * point and 8 bytes per grid cell, for a polygon layer up to 4 bytes per point) and
+ * captures that layer's graph then; later rounds allocate nothing.  Layers must outlive the engine.  Errors: SJ_ERR_INVALID. */
 sj_status sj_engine_create(int64_t max_points, int32_t max_requests, const sj_opts *opts, sj_engine **out);
 
 /* One round over reqs[0..n): asynchronous on stream (a non-NULL stream is

@@ -893,13 +893,20 @@ static sj_status join_impl(const sj_layer *L, int kind, const double *pts, int64
     cudaStream_t s = (cudaStream_t)stream;
     const bool timed = o && (o->flags & SJ_FLAG_TIME_REFINE);
     const bool subcells = o && (o->flags & SJ_FLAG_SUBCELL_ON) && !(o->flags & SJ_FLAG_SUBCELL_OFF);
-    if (kind == KIND_PIP) {   // one kernel over the points in input order, no scratch (sj_pip.cu)
+    if (kind == KIND_PIP) {   // one kernel over the points in input order (sj_pip.cu)
         PipArgs pa = pip_args(L);
         if (subcells) pa.search = PIP_SEARCH_MIN;
         cudaError_t e = cudaSuccess;
+        unsigned *lists = nullptr;
+        const size_t nl = (size_t)pip_list_ints(N, di->sms);
+        if (nl) CUDA_TRY(dev_malloc_async((void **)&lists, sizeof(unsigned) * nl, s));
         TimedSpan span(L, timed, s, e);
-        if (e == cudaSuccess) e = launch_pip_join(pa, (const double2 *)pts, (int)N, out_id, di->sms, s);
+        if (e == cudaSuccess) e = launch_pip_join(pa, (const double2 *)pts, (int)N, out_id, lists, di->sms, s);
         span.stop(e);
+        if (lists) {
+            cudaError_t e2 = cudaFreeAsync(lists, s);
+            if (e == cudaSuccess) e = e2;
+        }
         if (e != cudaSuccess) return cuda_fail(e, "join launch");
         return check_bounds(s);
     }

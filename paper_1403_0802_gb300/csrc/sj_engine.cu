@@ -82,6 +82,7 @@ struct LayerWork {
     RefineArgs ra{};
     MultiArgs ma{};
     PipArgs pa{};
+    unsigned *lists = nullptr;   // PIP
     // pinned request tables (two, so the host can fill one while the other's
     // copy may still be pending) and the events that mark their copies done
     RoundReq *h_reqs[2] = {nullptr, nullptr};
@@ -120,7 +121,7 @@ static void work_free(LayerWork *w) {
 }
 
 // Workspace of one layer, carved like the per-request join's scratch.
-static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
+static sj_status work_create(sj_engine *E, const sj_layer *L, const DevInfo *di, LayerWork **out) {
     LayerWork *w = new LayerWork();
     struct Guard {
         LayerWork *w;
@@ -138,7 +139,11 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
     auto lay = [&](Scratch &x) {
         w->d_reqs = x.take<RoundReq>((size_t)E->max_requests);
         w->d_meta = x.take<int>(4);
-        if (!p2p) return;   // the PIP join needs no scratch
+        if (!p2p) {
+            const int64_t n = pip_round_list_ints(N, di->sms);
+            w->lists = n ? x.take<unsigned>((size_t)n) : nullptr;
+            return;
+        }
         cnt = x.take<int>((size_t)G + 1);
         cell_start = x.take<int>((size_t)G + 1);
         totals = x.take<int>(4);
@@ -219,7 +224,7 @@ static sj_status work_create(sj_engine *E, const sj_layer *L, LayerWork **out) {
 static cudaError_t enqueue_round(const sj_engine *E, const LayerWork *w, const DevInfo *di, cudaStream_t s) {
     const sj_layer *L = w->L;
     const int blocks = di->sms * 8;
-    if (L->kind == KIND_PIP) return launch_pip_round(w->pa, w->d_reqs, w->d_meta, E->max_points, di->sms, s);
+    if (L->kind == KIND_PIP) return launch_pip_round(w->pa, w->d_reqs, w->d_meta, E->max_points, w->lists, di->sms, s);
     cudaError_t e = cudaMemsetAsync(w->ba.cnt, 0, sizeof(int) * ((size_t)L->g.G + 1), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w->ba.totals, 0, sizeof(int) * 4, s);
     if (e != cudaSuccess) return e;
@@ -303,7 +308,7 @@ extern "C" sj_status sj_engine_round(sj_engine *E, const sj_request *reqs, int32
         for (LayerWork *x : E->work)
             if (x->L == L) w = x;
         if (!w) {
-            st = work_create(E, L, &w);
+            st = work_create(E, L, di, &w);
             if (st != SJ_OK) return st;
             E->work.push_back(w);
         }

@@ -385,9 +385,14 @@ struct PipArgs {
     int search;              // lists longer than this are searched by y
     unsigned long long *stats;
 };
-cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, int sms, cudaStream_t s);
-cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points, int sms,
-                             cudaStream_t s);
+// Scratch of the lists of a join's or a round's points, in 4-byte integers (0 for
+// small calls: lists null).
+long long pip_list_ints(long long n, int sms);
+long long pip_round_list_ints(long long max_points, int sms);
+cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, unsigned *lists, int sms,
+                            cudaStream_t s);
+cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points,
+                             unsigned *lists, int sms, cudaStream_t s);
 
 // PIP layer build: per edge its rows (of the lower and the upper end), x-range
 // and kind (bit 0: the first end is the lower one; bit 1: horizontal).

@@ -138,20 +138,22 @@ __host__ __device__ __forceinline__ long long group_units(int n, int nf, int ng)
 
 // ------------------------------------------------------------------ the join
 
-// Where a join's points come from and its ids go.
+// Where a join's points come from and its ids go, and the scratch of the lists of
+// points that wait (pip_list_ints; null: in shared memory).
 struct OneSource {
     const double2 *pts;
     int *out;
+    unsigned *lists;
     int n;
     __device__ __forceinline__ int count() const { return n; }
     __device__ __forceinline__ double2 point(unsigned i) const { return __ldcs(pts + i); }
     __device__ __forceinline__ void put(unsigned i, int id) const { out[i] = id; }
-    __device__ __forceinline__ int get(unsigned i) const { return out[i]; }
 };
 // Many requests as one point set (batched rounds).
 struct RoundSource {
     const RoundReq *reqs;
     const int *meta;   // requests, points
+    unsigned *lists;
     __device__ __forceinline__ int count() const { return meta[1]; }
     __device__ __forceinline__ const RoundReq &find(unsigned i) const {
         return reqs[find_request(reqs, meta[0], (int)i)];
@@ -163,10 +165,6 @@ struct RoundSource {
     __device__ __forceinline__ void put(unsigned i, int id) const {
         const RoundReq &r = find(i);
         r.out_id[i - r.off] = id;
-    }
-    __device__ __forceinline__ int get(unsigned i) const {
-        const RoundReq &r = find(i);
-        return r.out_id[i - r.off];
     }
 };
 
@@ -350,11 +348,14 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 // certain and classified is answered at once.  The others are queued in shared
 // memory and refined 32 at a time, so that the refinement runs with full warps
 // although only some of a tile's points (6 - 54 %) need it.  The few that this
-// cannot finish wait until the warp has seen its last tile, in one list per
-// lane threaded through their own places in the output (out[i] = the index
-// before i in the lane's list), which needs no scratch and has no limit; by
-// then their general, register-hungry code costs the loop nothing (with a call
-// to it inside the loop the 100 M point join took 2.3 - 4.5 ms instead of 1.6).
+// cannot finish wait until the warp has seen its last tile, in the warp's list
+// (in scratch, or while it is short in shared memory); by then their general, register-hungry code costs the loop
+// nothing (with a call to it inside the loop the 100 M point join took 2.3 - 4.5 ms
+// instead of 1.6; with lists of up to 64 points in shared memory, refined whenever
+// 32 wait, 1.31 instead of 1.22 ms, and 10 M points on the heavy-tail tiles 433
+// instead of 396 us).  Not in the output, threaded through the points' own places:
+// requests and streams may share an output, and a list lost there takes other
+// requests' points with it.
 //
 // Bound by the latency and the L1 wavefronts of the random reads of the cell
 // table and the records, both L2-resident (ncu at 20 M points on the tiles: issue
@@ -366,13 +367,20 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 template <int U, class Src>
 __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src) {
     __shared__ PipQueued queue[PIP_WARPS][32 * (U + 1)];
+    __shared__ unsigned *lists[PIP_WARPS];
+    extern __shared__ unsigned short_lists[];
     __shared__ PipSums sums[PIP_WARPS * 32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const unsigned n = (unsigned)src.count(), tiles = (n + 32u * U - 1u) / (32u * U);
     unsigned items = 0, resolved = 0, hits = 0, fb = 0;
     sums[threadIdx.x] = PipSums{0, 0, 0};
-    int qn = 0, head = -1, waiting = 0;
+    int qn = 0, wn = 0;   // points queued, points that wait
+    if (lane == 0) {   // the warp's list: room for every point of its tiles
+        const unsigned warps = gridDim.x * PIP_WARPS, room = (tiles + warps - 1u) / warps * (32u * U);
+        lists[w] = src.lists ? src.lists + (size_t)(blockIdx.x * PIP_WARPS + w) * room : short_lists + w * room;
+    }
+    __syncwarp();
     for (unsigned t = blockIdx.x * PIP_WARPS + w;; t += gridDim.x * PIP_WARPS) {
         const bool more = t < tiles;   // else: the points left in the queues
         if (more) {
@@ -419,34 +427,34 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
         while (more ? qn >= 32 : qn > 0) {
             const int cnt = min(qn, 32);
             qn -= cnt;
+            bool wait = false;
+            unsigned i = 0;
             if (lane < cnt) {
                 const PipQueued q = queue[w][qn + lane];
+                i = (unsigned)q.i;
                 int res;
                 const bool done = pip_fast(a, q, sums[threadIdx.x], res);
-                if (SJ_IN_BOUNDS((unsigned)q.i < n, BND_PIP_RES)) {
-                    src.put((unsigned)q.i, done ? res : head);
-                    if (!done) {
-                        head = q.i;
-                        ++waiting;
-                    }
+                if (SJ_IN_BOUNDS(i < n, BND_PIP_RES)) {
+                    if (done) src.put(i, res);
                     hits += done && res >= 0;
+                    wait = !done;
                 }
             }
+            const unsigned bal = __ballot_sync(FULL, wait);
+            if (wait) lists[w][wn + __popc(bal & lt)] = i;
+            wn += __popc(bal);
             ++items;
         }
         if (!more) break;
         __syncwarp();
     }
-    // The lists, one point of each lane at a time; counted, and their links
-    // checked, so that a caller's overlapping outputs cannot lead them astray.
-    while (__any_sync(FULL, waiting > 0)) {
+    __syncwarp();
+    for (int k0 = 0; k0 < wn; k0 += 32) {   // the points that wait, one per lane
         PipQueued q;
-        q.i = head;
-        bool act = waiting > 0 && (unsigned)head < n;
-        waiting = act ? waiting - 1 : 0;
+        bool act = k0 + lane < wn;
         int res = -1;
         if (act) {
-            head = src.get((unsigned)q.i);
+            q.i = (int)lists[w][k0 + lane];
             q.p = src.point((unsigned)q.i);
             const int2 e = point_cell_exact(a.g, q.p.x, q.p.y);
             const int code = e.x >= 0 && e.y >= 0 ? a.cells[e.y * a.g.nx + e.x].x : -1;
@@ -516,17 +524,42 @@ static int pip_blocks(int U, long long n, int sms) {
     return (int)std::max(1LL, std::min((tiles + PIP_WARPS - 1) / PIP_WARPS, (long long)sms * PIP_BLOCKS));
 }
 
-cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, int sms, cudaStream_t s) {
-    const OneSource src{pts, out, n};
-    if (n >= sms * PIP_WARPS * PIP_BLOCKS * 32 * 2 * PIP_U) k_pip_join<PIP_U><<<pip_blocks(PIP_U, n, sms), PIP_WARPS * 32, 0, s>>>(a, src);
-    else k_pip_join<1><<<pip_blocks(1, n, sms), PIP_WARPS * 32, 0, s>>>(a, src);
+// Points of a call's warps at most (a call of fewer points on the same grid: no more).
+static long long pip_room(int U, long long n, int sms) {
+    const long long tiles = (n + 32LL * U - 1) / (32LL * U), warps = (long long)pip_blocks(U, n, sms) * PIP_WARPS;
+    return (tiles + warps - 1) / warps * (32LL * U);
+}
+
+// Lists of up to this many points are held in shared memory (calls of up to 1.2 M
+// points: the stream-ordered allocation of scratch takes 2 us of a call).
+constexpr int PIP_SHORT = 256;
+
+static int pip_unroll(long long n, int sms) { return n >= sms * PIP_WARPS * PIP_BLOCKS * 32LL * 2 * PIP_U ? PIP_U : 1; }
+
+static long long list_ints(int U, long long n, int sms) {
+    const long long room = pip_room(U, n, sms);
+    return room <= PIP_SHORT ? 0 : room * pip_blocks(U, n, sms) * PIP_WARPS;
+}
+long long pip_list_ints(long long n, int sms) { return list_ints(pip_unroll(n, sms), n, sms); }
+long long pip_round_list_ints(long long max_points, int sms) { return list_ints(1, max_points, sms); }
+
+template <int U, class Src>
+static cudaError_t pip_launch(const PipArgs &a, const Src &src, long long n, int sms, cudaStream_t s) {
+    if (!src.lists && list_ints(U, n, sms) > 0) return cudaErrorInvalidValue;
+    const size_t smem = src.lists ? 0 : sizeof(unsigned) * PIP_WARPS * (size_t)pip_room(U, n, sms);
+    k_pip_join<U><<<pip_blocks(U, n, sms), PIP_WARPS * 32, smem, s>>>(a, src);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points, int sms,
-                             cudaStream_t s) {
-    k_pip_join<1><<<pip_blocks(1, max_points, sms), PIP_WARPS * 32, 0, s>>>(a, RoundSource{reqs, meta});
-    return cudaGetLastError();
+cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, unsigned *lists, int sms,
+                            cudaStream_t s) {
+    const OneSource src{pts, out, lists, n};
+    return pip_unroll(n, sms) == PIP_U ? pip_launch<PIP_U>(a, src, n, sms, s) : pip_launch<1>(a, src, n, sms, s);
+}
+
+cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points,
+                             unsigned *lists, int sms, cudaStream_t s) {
+    return pip_launch<1>(a, RoundSource{reqs, meta, lists}, max_points, sms, s);
 }
 
 // ------------------------------------------------------------------ layer build
