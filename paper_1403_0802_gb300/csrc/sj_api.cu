@@ -166,12 +166,12 @@ static bool grid_ok(const sj_grid *g) {
 // Bound of axis_estimate's error, in cells: |v - fl(v)| < 2u |v| (truncation) or
 // 2^-126 (flushed to zero), |x0f - x0| <= u |x0|, the difference's rounding u per
 // cell index, 1 / w rounded (2u) and the product (u): at most (3u max|x| + 2^-126)
-// / w + 4u n cells, times 1.5.  Beyond 1e37 the estimate is never certain (2 cells):
-// from 3.4e38 on approx_float clamps, and 1 / w leaves the FP32 normal range at
-// 8.5e37.  Below, a clamped value maps past the grid's end.
+// / w + 4u n cells, times 1.5.  Beyond 1e37 the estimate is never certain: from
+// 3.4e38 on approx_float clamps, and 1 / w leaves the FP32 normal range at 8.5e37.
+// Below, a clamped value maps past the grid's end.
 static float estimate_tol(double lo, double hi, double w, int n) {
     const double u = 5.9604644775390625e-08, m = std::max(std::fabs(lo), std::fabs(hi));
-    return m <= 1e37 ? (float)(1.5 * ((3.0 * u * m + 1.1754943508222875e-38) / w + 4.0 * u * n)) : 2.0f;
+    return m <= 1e37 ? (float)(1.5 * ((3.0 * u * m + 1.1754943508222875e-38) / w + 4.0 * u * n)) : INFINITY;
 }
 
 static GridDev make_grid(const sj_grid *g) {

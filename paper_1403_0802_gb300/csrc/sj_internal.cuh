@@ -112,7 +112,7 @@ __device__ __forceinline__ int axis_cell(double v, const unsigned long long *key
 // grid, so that i is certain; r is then the place within the cell, 0 to 1, off
 // by at most tol.  The bound (estimate_tol) covers the truncation of v to FP32
 // (subnormals to zero), the rounding of lo and 1 / w, and the two operations; it
-// is above 1 for grids that leave the FP32 range.  NaN, infinite and far outside
+// is infinite for grids that leave the FP32 range.  NaN, infinite and far outside
 // values are never certain.
 __device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i, float &r) {
     const float t = __fmul_rn(__fsub_rn(approx_float(v), lof), iwf);
@@ -124,6 +124,21 @@ __device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, fl
 __device__ __forceinline__ bool axis_estimate(double v, float lof, float iwf, float tol, int n, int &i) {
     float r;
     return axis_estimate(v, lof, iwf, tol, n, i, r);
+}
+
+// Whether a point certainly lies outside the grid box (NaN and infinite
+// coordinates among them, which approx_float clamps): the estimate is monotone in
+// v, so where it is farther than twice its bound from the grid's range, v is
+// farther than the bound from it, hence no rounding of the exact rule puts it in.
+// (Left to the exact rule such points wait in the PIP join's lists: 5 M points,
+// 15 of 16 outside the stars' 64 x 64 grid, 160 us against 49; the 100 M points
+// of the tilings, of which a few are outside, 1,211 against 1,138 us.)
+__device__ __forceinline__ bool axis_outside(double v, float lof, float iwf, float tol, int n) {
+    const float t = __fmul_rn(__fsub_rn(approx_float(v), lof), iwf);
+    return t < -2.0f * tol || t > (float)n + 2.0f * tol;
+}
+__device__ __forceinline__ bool point_outside(const GridDev &g, double x, double y) {
+    return axis_outside(x, g.x0f, g.icwf, g.tolx, g.nx) || axis_outside(y, g.y0f, g.ichf, g.toly, g.ny);
 }
 
 // Column and row of a point, (-1 in an axis) outside the half-open grid box or

@@ -407,6 +407,8 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
                             if (cls) code[u] = cls == 1 ? c.z : (cls == 2 ? c.w : -1);
                         }
                         resolved += code[u] >= -1;
+                    } else if (point_outside(a.g, p[u].x, p[u].y)) {
+                        code[u] = -1;
                     }
                 }
             }

@@ -139,3 +139,26 @@ def test_fp32x_squares_out_of_range(api, oracle, scale):
             hit = (gid >= 0) & (rid >= 0)
             assert hit.sum() > 100
             assert np.all(np.abs(gd[hit] - rd[hit]) <= 1e-5 * far)
+
+
+@pytest.mark.parametrize("x0,cell,n", [(0.0, 1.0, 64), (4.5e6, 0.37, 64), (-8e6, 250.0, 2048), (-1e5, 1e-3, 1024),
+                                       (0.0, 1e40, 64), (-37.995e-36, 1e-36, 64)])
+def test_points_outside(api, oracle, x0, cell, n):
+    """Points on, next to and far from the grid's ends: a polygon that covers the grid holds those inside alone."""
+    g = grid(x0, cell, n)
+    rng = np.random.default_rng(11)
+    verts = np.array([[g["x0"], g["y0"]], [g["x1"], g["y0"]], [g["x1"], g["y1"]], [g["x0"], g["y1"]]])
+    off, poly = np.array([0, 4], np.int64), np.array([0, 1], np.int64)
+    end = np.repeat([g["x0"], g["x1"]], 400)
+    near = [end, np.nextafter(end, np.inf), np.nextafter(end, -np.inf),
+            end + rng.uniform(-1, 1, end.size) * 10.0 ** rng.uniform(-9, 2, end.size) * cell,
+            end * (1 + rng.uniform(-1, 1, end.size) * 10.0 ** rng.uniform(-16, -5, end.size)),
+            rng.uniform(-1, 1, end.size) * 10.0 ** rng.uniform(-40, 300, end.size)]
+    edge = np.concatenate(near + [np.array([np.inf, -np.inf, np.nan, 0.0, -0.0])])
+    mid = rng.uniform(g["x0"], g["x1"], edge.size)
+    pts = np.concatenate([np.stack([edge, mid], 1), np.stack([mid, edge], 1), np.stack([edge, edge[::-1]], 1)])
+    ref = oracle.pip_join(g, pts, verts, off, poly)
+    assert (ref >= 0).any() and (ref < 0).any()
+    with api.pip_layer(verts, off, poly, g) as layer:
+        got = api.pip_join(layer, torch.as_tensor(pts, device="cuda"), form="fp64").cpu().numpy()
+    np.testing.assert_array_equal(got, ref)
