@@ -364,10 +364,10 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 // then without and with the sub-cell classes: 1,003 points 53 -> 11 -> 11, 1 M on
 // the stars (FP64 form) 119 -> 29 -> 21, 10 M on the heavy-tail tiles 2,450 -> 536
 // -> 426 (401 with HARD = 16), 100 M on the 40,000 tiles 4,486 -> 1,590 -> 1,130.
+// room: points of a warp's list at most.
 template <int U, class Src>
-__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src) {
+__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src, unsigned room) {
     __shared__ PipQueued queue[PIP_WARPS][32 * (U + 1)];
-    __shared__ unsigned *lists[PIP_WARPS];
     extern __shared__ unsigned short_lists[];
     __shared__ PipSums sums[PIP_WARPS * 32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
@@ -376,11 +376,6 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
     unsigned items = 0, resolved = 0, hits = 0, fb = 0;
     sums[threadIdx.x] = PipSums{0, 0, 0};
     int qn = 0, wn = 0;   // points queued, points that wait
-    if (lane == 0) {   // the warp's list: room for every point of its tiles
-        const unsigned warps = gridDim.x * PIP_WARPS, room = (tiles + warps - 1u) / warps * (32u * U);
-        lists[w] = src.lists ? src.lists + (size_t)(blockIdx.x * PIP_WARPS + w) * room : short_lists + w * room;
-    }
-    __syncwarp();
     for (unsigned t = blockIdx.x * PIP_WARPS + w;; t += gridDim.x * PIP_WARPS) {
         const bool more = t < tiles;   // else: the points left in the queues
         if (more) {
@@ -443,7 +438,11 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
                 }
             }
             const unsigned bal = __ballot_sync(FULL, wait);
-            if (wait) lists[w][wn + __popc(bal & lt)] = i;
+            if (wait) {   // (a pointer to the list kept through the loop would cost it two registers)
+                const unsigned k = (unsigned)(wn + __popc(bal & lt));
+                if (src.lists) src.lists[(size_t)(blockIdx.x * PIP_WARPS + w) * room + k] = i;
+                else short_lists[w * room + k] = i;
+            }
             wn += __popc(bal);
             ++items;
         }
@@ -456,7 +455,8 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
         bool act = k0 + lane < wn;
         int res = -1;
         if (act) {
-            q.i = (int)lists[w][k0 + lane];
+            const unsigned k = (unsigned)(k0 + lane);
+            q.i = (int)(src.lists ? src.lists[(size_t)(blockIdx.x * PIP_WARPS + w) * room + k] : short_lists[w * room + k]);
             q.p = src.point((unsigned)q.i);
             const int2 e = point_cell_exact(a.g, q.p.x, q.p.y);
             const int code = e.x >= 0 && e.y >= 0 ? a.cells[e.y * a.g.nx + e.x].x : -1;
@@ -548,8 +548,9 @@ long long pip_round_list_ints(long long max_points, int sms) { return list_ints(
 template <int U, class Src>
 static cudaError_t pip_launch(const PipArgs &a, const Src &src, long long n, int sms, cudaStream_t s) {
     if (!src.lists && list_ints(U, n, sms) > 0) return cudaErrorInvalidValue;
-    const size_t smem = src.lists ? 0 : sizeof(unsigned) * PIP_WARPS * (size_t)pip_room(U, n, sms);
-    k_pip_join<U><<<pip_blocks(U, n, sms), PIP_WARPS * 32, smem, s>>>(a, src);
+    const unsigned room = (unsigned)pip_room(U, n, sms);
+    const size_t smem = src.lists ? 0 : sizeof(unsigned) * PIP_WARPS * room;
+    k_pip_join<U><<<pip_blocks(U, n, sms), PIP_WARPS * 32, smem, s>>>(a, src, room);
     return cudaGetLastError();
 }
 
