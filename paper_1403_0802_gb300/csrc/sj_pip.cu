@@ -364,31 +364,32 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 // then without and with the sub-cell classes: 1,003 points 53 -> 11 -> 11, 1 M on
 // the stars (FP64 form) 119 -> 29 -> 21, 10 M on the heavy-tail tiles 2,450 -> 536
 // -> 426 (401 with HARD = 16), 100 M on the 40,000 tiles 4,486 -> 1,590 -> 1,130.
-// room: points of a warp's list at most.
+// per: points of a tile (32 U, fewer in small calls); room: points of a warp's list
+// at most.
 template <int U, class Src>
-__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src, unsigned room) {
+__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src, unsigned per, unsigned room) {
     __shared__ PipQueued queue[PIP_WARPS][32 * (U + 1)];
     extern __shared__ unsigned short_lists[];
     __shared__ PipSums sums[PIP_WARPS * 32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const unsigned n = (unsigned)src.count(), tiles = (n + 32u * U - 1u) / (32u * U);
+    const unsigned n = (unsigned)src.count(), step = U == 1 ? per : 32u * U, tiles = (n + step - 1u) / step;
     unsigned items = 0, resolved = 0, hits = 0, fb = 0;
     sums[threadIdx.x] = PipSums{0, 0, 0};
     int qn = 0, wn = 0;   // points queued, points that wait
     for (unsigned t = blockIdx.x * PIP_WARPS + w;; t += gridDim.x * PIP_WARPS) {
         const bool more = t < tiles;   // else: the points left in the queues
         if (more) {
-            const unsigned i0 = t * (32u * U) + lane;
+            const unsigned i0 = t * step + lane, end = U == 1 && (unsigned)lane >= per ? 0u : n;
             double2 p[U];
             int code[U], ix[U], iy[U];
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (i0 + 32u * u < n) p[u] = src.point(i0 + 32u * u);
+                if (i0 + 32u * u < end) p[u] = src.point(i0 + 32u * u);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 code[u] = -1;
-                if (i0 + 32u * u < n) {
+                if (i0 + 32u * u < end) {
                     float rx, ry;
                     const bool sx = axis_estimate(p[u].x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, ix[u], rx);
                     const bool sy = axis_estimate(p[u].y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, iy[u], ry);
@@ -410,8 +411,8 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const unsigned i = i0 + 32u * u;
-                const bool q = i < n && code[u] < -1;
-                if (i < n && !q) {
+                const bool q = i < end && code[u] < -1;
+                if (i < end && !q) {
                     src.put(i, code[u]);
                     hits += code[u] >= 0;
                 }
@@ -521,48 +522,61 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
 // calls spread over more warps, one point per lane.
 constexpr int PIP_U = 2;
 
-static int pip_blocks(int U, long long n, int sms) {
-    const long long tiles = (n + 32LL * U - 1) / (32LL * U);
+// Points per lane of a call's tiles.
+static int pip_unroll(long long n, int sms) { return n >= sms * PIP_WARPS * PIP_BLOCKS * 32LL * 2 * PIP_U ? PIP_U : 1; }
+
+// Points per tile: 32 U, but calls of fewer tiles than the GPU holds warps take
+// tiles of 16, 8 or 4 points, since a warp refines two of the points that wait at
+// a time (1,003 points in cells of some 500 edges, stars on a 16 x 16 grid: 70 / 39 /
+// 23 / 14 / 10 us with 32 / 16 / 8 / 4 / 1; on the 40,000 tiles 8.2 / 6.9 / 6.2 / 6.2 / 6.2).
+static int pip_per(int U, long long n, int sms) {
+    const long long warps = (long long)sms * PIP_BLOCKS * PIP_WARPS;
+    int per = 32 * U;
+    while (U == 1 && per > 4 && (n + per / 2 - 1) / (per / 2) <= warps) per /= 2;
+    return per;
+}
+
+static int pip_blocks(int per, long long n, int sms) {
+    const long long tiles = (n + per - 1) / per;
     return (int)std::max(1LL, std::min((tiles + PIP_WARPS - 1) / PIP_WARPS, (long long)sms * PIP_BLOCKS));
 }
 
 // Points of a call's warps at most (a call of fewer points on the same grid: no more).
-static long long pip_room(int U, long long n, int sms) {
-    const long long tiles = (n + 32LL * U - 1) / (32LL * U), warps = (long long)pip_blocks(U, n, sms) * PIP_WARPS;
-    return (tiles + warps - 1) / warps * (32LL * U);
+static long long pip_room(int per, long long n, int sms) {
+    const long long tiles = (n + per - 1) / per, warps = (long long)pip_blocks(per, n, sms) * PIP_WARPS;
+    return (tiles + warps - 1) / warps * per;
 }
 
 // Lists of up to this many points are held in shared memory (calls of up to 1.2 M
 // points: the stream-ordered allocation of scratch takes 2 us of a call).
 constexpr int PIP_SHORT = 256;
 
-static int pip_unroll(long long n, int sms) { return n >= sms * PIP_WARPS * PIP_BLOCKS * 32LL * 2 * PIP_U ? PIP_U : 1; }
-
-static long long list_ints(int U, long long n, int sms) {
-    const long long room = pip_room(U, n, sms);
-    return room <= PIP_SHORT ? 0 : room * pip_blocks(U, n, sms) * PIP_WARPS;
+static long long list_ints(int per, long long n, int sms) {
+    const long long room = pip_room(per, n, sms);
+    return room <= PIP_SHORT ? 0 : room * pip_blocks(per, n, sms) * PIP_WARPS;
 }
-long long pip_list_ints(long long n, int sms) { return list_ints(pip_unroll(n, sms), n, sms); }
-long long pip_round_list_ints(long long max_points, int sms) { return list_ints(1, max_points, sms); }
+long long pip_list_ints(long long n, int sms) { return list_ints(pip_per(pip_unroll(n, sms), n, sms), n, sms); }
+long long pip_round_list_ints(long long max_points, int sms) { return list_ints(32, max_points, sms); }
 
 template <int U, class Src>
-static cudaError_t pip_launch(const PipArgs &a, const Src &src, long long n, int sms, cudaStream_t s) {
-    if (!src.lists && list_ints(U, n, sms) > 0) return cudaErrorInvalidValue;
-    const unsigned room = (unsigned)pip_room(U, n, sms);
+static cudaError_t pip_launch(const PipArgs &a, const Src &src, int per, long long n, int sms, cudaStream_t s) {
+    if (!src.lists && list_ints(per, n, sms) > 0) return cudaErrorInvalidValue;
+    const unsigned room = (unsigned)pip_room(per, n, sms);
     const size_t smem = src.lists ? 0 : sizeof(unsigned) * PIP_WARPS * room;
-    k_pip_join<U><<<pip_blocks(U, n, sms), PIP_WARPS * 32, smem, s>>>(a, src, room);
+    k_pip_join<U><<<pip_blocks(per, n, sms), PIP_WARPS * 32, smem, s>>>(a, src, (unsigned)per, room);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *out, unsigned *lists, int sms,
                             cudaStream_t s) {
     const OneSource src{pts, out, lists, n};
-    return pip_unroll(n, sms) == PIP_U ? pip_launch<PIP_U>(a, src, n, sms, s) : pip_launch<1>(a, src, n, sms, s);
+    const int U = pip_unroll(n, sms), per = pip_per(U, n, sms);
+    return U == PIP_U ? pip_launch<PIP_U>(a, src, per, n, sms, s) : pip_launch<1>(a, src, per, n, sms, s);
 }
 
 cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points,
                              unsigned *lists, int sms, cudaStream_t s) {
-    return pip_launch<1>(a, RoundSource{reqs, meta, lists}, max_points, sms, s);
+    return pip_launch<1>(a, RoundSource{reqs, meta, lists}, 32, max_points, sms, s);
 }
 
 // ------------------------------------------------------------------ layer build

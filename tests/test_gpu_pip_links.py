@@ -73,3 +73,18 @@ def test_scratch_refused(lib, rough, oracle, n):
             L.lib().sj_fault_inject(0, 0, 0)
         A.pip_join(layer, p, out)
         np.testing.assert_array_equal(out.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 1_003, 19_456, 19_457, 38_912, 38_913, 77_824, 77_825, 155_648])
+def test_small_tiles(lib, rough, oracle, n):
+    """Small calls take tiles of 4, 8, 16 or 32 points (the sizes where they change on 152 SMs); every point waits."""
+    A, _ = lib
+    pts = np.random.default_rng(n).uniform(-1, 65, (n, 2))
+    out = torch.full((n + 1,), 7, dtype=torch.int32, device="cuda")
+    with A.pip_layer(*rough, GRID) as layer:
+        A.pip_join(layer, torch.as_tensor(pts, device="cuda"), out[:n], form="fp32x")
+        st = layer.stats()
+    got = out.cpu().numpy()
+    want = oracle.pip_join(GRID, pts, *rough)
+    np.testing.assert_array_equal(got[:n], want)
+    assert got[n] == 7 and st["hits"] == (want >= 0).sum()
