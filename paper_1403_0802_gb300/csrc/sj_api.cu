@@ -168,10 +168,12 @@ static bool grid_ok(const sj_grid *g) {
 // cell index, 1 / w rounded (2u) and the product (u): at most (3u max|x| + 2^-126)
 // / w + 4u n cells, times 1.5.  Beyond 1e37 the estimate is never certain: from
 // 3.4e38 on approx_float clamps, and 1 / w leaves the FP32 normal range at 8.5e37.
-// Below, a clamped value maps past the grid's end.
+// Below, a clamped value maps past the grid's end.  Nor is it with cells below
+// 1e-37: from 2.9e-39 on 1 / w is infinite, and every point seems far outside.
 static float estimate_tol(double lo, double hi, double w, int n) {
     const double u = 5.9604644775390625e-08, m = std::max(std::fabs(lo), std::fabs(hi));
-    return m <= 1e37 ? (float)(1.5 * ((3.0 * u * m + 1.1754943508222875e-38) / w + 4.0 * u * n)) : INFINITY;
+    if (!(m <= 1e37 && w >= 1e-37)) return INFINITY;
+    return (float)(1.5 * ((3.0 * u * m + 1.1754943508222875e-38) / w + 4.0 * u * n));
 }
 
 static GridDev make_grid(const sj_grid *g) {

@@ -142,7 +142,7 @@ def test_fp32x_squares_out_of_range(api, oracle, scale):
 
 
 @pytest.mark.parametrize("x0,cell,n", [(0.0, 1.0, 64), (4.5e6, 0.37, 64), (-8e6, 250.0, 2048), (-1e5, 1e-3, 1024),
-                                       (0.0, 1e40, 64), (-37.995e-36, 1e-36, 64)])
+                                       (0.0, 1e40, 64), (-37.995e-36, 1e-36, 64), (0.0, 1e-38, 64), (1e-38, 1e-39, 64)])
 def test_points_outside(api, oracle, x0, cell, n):
     """Points on, next to and far from the grid's ends: a polygon that covers the grid holds those inside alone."""
     g = grid(x0, cell, n)
