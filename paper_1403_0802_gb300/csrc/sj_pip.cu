@@ -184,6 +184,17 @@ struct PipSums {
     unsigned long long tests, pairs, algo;
 };
 
+// Points of a tile with one point per lane: 32, but calls and rounds of fewer tiles
+// than there are warps take tiles of 16, 8 or 4 points, since a warp refines two of
+// the points that wait at a time (1,003 points in cells of some 500 edges, stars on
+// a 16 x 16 grid: 70 / 39 / 23 / 14 / 10 us with 32 / 16 / 8 / 4 / 1; on the 40,000
+// tiles 8.2 / 6.9 / 6.2 / 6.2 / 6.2).
+__host__ __device__ __forceinline__ unsigned tile_points(unsigned n, unsigned warps) {
+    unsigned per = 32;
+    while (per > 4 && (n + per / 2 - 1) / (per / 2) <= warps) per /= 2;
+    return per;
+}
+
 // A point that waits for its refinement.
 struct PipQueued {
     double2 p;
@@ -364,23 +375,23 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 // then without and with the sub-cell classes: 1,003 points 53 -> 11 -> 11, 1 M on
 // the stars (FP64 form) 119 -> 29 -> 21, 10 M on the heavy-tail tiles 2,450 -> 536
 // -> 426 (401 with HARD = 16), 100 M on the 40,000 tiles 4,486 -> 1,590 -> 1,130.
-// per: points of a tile (32 U, fewer in small calls); room: points of a warp's list
-// at most.
+// room: points of a warp's list at most.
 template <int U, class Src>
-__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src, unsigned per, unsigned room) {
+__global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs a, Src src, unsigned room) {
     __shared__ PipQueued queue[PIP_WARPS][32 * (U + 1)];
     extern __shared__ unsigned short_lists[];
     __shared__ PipSums sums[PIP_WARPS * 32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const unsigned n = (unsigned)src.count(), step = U == 1 ? per : 32u * U, tiles = (n + step - 1u) / step;
+    const unsigned n = (unsigned)src.count(), step = U == 1 ? tile_points(n, gridDim.x * PIP_WARPS) : 32u * U;
+    const unsigned tiles = (n + step - 1u) / step;
     unsigned items = 0, resolved = 0, hits = 0, fb = 0;
     sums[threadIdx.x] = PipSums{0, 0, 0};
     int qn = 0, wn = 0;   // points queued, points that wait
     for (unsigned t = blockIdx.x * PIP_WARPS + w;; t += gridDim.x * PIP_WARPS) {
         const bool more = t < tiles;   // else: the points left in the queues
         if (more) {
-            const unsigned i0 = t * step + lane, end = U == 1 && (unsigned)lane >= per ? 0u : n;
+            const unsigned i0 = t * step + lane, end = U == 1 && (unsigned)lane >= step ? 0u : n;
             double2 p[U];
             int code[U], ix[U], iy[U];
 #pragma unroll
@@ -525,15 +536,8 @@ constexpr int PIP_U = 2;
 // Points per lane of a call's tiles.
 static int pip_unroll(long long n, int sms) { return n >= sms * PIP_WARPS * PIP_BLOCKS * 32LL * 2 * PIP_U ? PIP_U : 1; }
 
-// Points per tile: 32 U, but calls of fewer tiles than the GPU holds warps take
-// tiles of 16, 8 or 4 points, since a warp refines two of the points that wait at
-// a time (1,003 points in cells of some 500 edges, stars on a 16 x 16 grid: 70 / 39 /
-// 23 / 14 / 10 us with 32 / 16 / 8 / 4 / 1; on the 40,000 tiles 8.2 / 6.9 / 6.2 / 6.2 / 6.2).
 static int pip_per(int U, long long n, int sms) {
-    const long long warps = (long long)sms * PIP_BLOCKS * PIP_WARPS;
-    int per = 32 * U;
-    while (U == 1 && per > 4 && (n + per / 2 - 1) / (per / 2) <= warps) per /= 2;
-    return per;
+    return U == 1 ? (int)tile_points((unsigned)n, (unsigned)(sms * PIP_BLOCKS * PIP_WARPS)) : 32 * U;
 }
 
 static int pip_blocks(int per, long long n, int sms) {
@@ -556,14 +560,14 @@ static long long list_ints(int per, long long n, int sms) {
     return room <= PIP_SHORT ? 0 : room * pip_blocks(per, n, sms) * PIP_WARPS;
 }
 long long pip_list_ints(long long n, int sms) { return list_ints(pip_per(pip_unroll(n, sms), n, sms), n, sms); }
-long long pip_round_list_ints(long long max_points, int sms) { return list_ints(32, max_points, sms); }
+long long pip_round_list_ints(long long max_points, int sms) { return list_ints(pip_per(1, max_points, sms), max_points, sms); }
 
 template <int U, class Src>
 static cudaError_t pip_launch(const PipArgs &a, const Src &src, int per, long long n, int sms, cudaStream_t s) {
     if (!src.lists && list_ints(per, n, sms) > 0) return cudaErrorInvalidValue;
     const unsigned room = (unsigned)pip_room(per, n, sms);
     const size_t smem = src.lists ? 0 : sizeof(unsigned) * PIP_WARPS * room;
-    k_pip_join<U><<<pip_blocks(per, n, sms), PIP_WARPS * 32, smem, s>>>(a, src, (unsigned)per, room);
+    k_pip_join<U><<<pip_blocks(per, n, sms), PIP_WARPS * 32, smem, s>>>(a, src, room);
     return cudaGetLastError();
 }
 
@@ -576,7 +580,7 @@ cudaError_t launch_pip_join(const PipArgs &a, const double2 *pts, int n, int *ou
 
 cudaError_t launch_pip_round(const PipArgs &a, const RoundReq *reqs, const int *meta, long long max_points,
                              unsigned *lists, int sms, cudaStream_t s) {
-    return pip_launch<1>(a, RoundSource{reqs, meta, lists}, 32, max_points, sms, s);
+    return pip_launch<1>(a, RoundSource{reqs, meta, lists}, pip_per(1, max_points, sms), max_points, sms, s);
 }
 
 // ------------------------------------------------------------------ layer build

@@ -88,3 +88,25 @@ def test_small_tiles(lib, rough, oracle, n):
     want = oracle.pip_join(GRID, pts, *rough)
     np.testing.assert_array_equal(got[:n], want)
     assert got[n] == 7 and st["hits"] == (want >= 0).sum()
+
+
+@pytest.mark.parametrize("most", [1, 1_003, 19_457, 155_649, 1_300_000])
+def test_small_rounds(lib, rough, oracle, most):
+    """Rounds of an engine for at most `most` points, from one point to all of them, in two requests: tiles of 4 to
+    32 points on one grid (every point waits; the largest engine has its lists in scratch)."""
+    A, _ = lib
+    pts = np.random.default_rng(most).uniform(-1, 65, (most, 2))
+    want = oracle.pip_join(GRID, pts, *rough)
+    p = torch.as_tensor(pts, device="cuda")
+    with A.pip_layer(*rough, GRID) as layer, A.Engine(max_points=most, max_requests=2, form="fp32x") as eng:
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        for n in sorted({1, min(most, 2), min(most, 129), (most + 3) // 4, (most + 1) // 2, most}):
+            out = torch.full((n + 1,), 7, dtype=torch.int32, device="cuda")
+            s.wait_stream(torch.cuda.current_stream())
+            k = n // 3
+            eng.round([(layer, p[:k], out[:k], None), (layer, p[k:n], out[k:n], None)], s)
+            s.synchronize()
+            got = out.cpu().numpy()
+            np.testing.assert_array_equal(got[:n], want[:n])
+            assert got[n] == 7
