@@ -176,7 +176,7 @@ constexpr int PIP_WARPS = 4, PIP_BLOCKS = 8;
 // Code of a queued point whose cell the FP32 estimate leaves open (no record
 // starts there: units are fewer than 2^31 - 2^22).
 constexpr int PIP_UNSURE = -2147483647 - 1;
-constexpr int PIP_SCAN_FLIPS = 8;   // flips scanned one by one by pip_fast
+constexpr int PIP_SCAN_FLIPS = 8;   // flips scanned one by one by pip_short
 
 // A lane's counters of the points refined.  In shared memory: the refinement
 // has no registers for three 64-bit sums.
@@ -213,6 +213,12 @@ __device__ __forceinline__ int edge_cross(float px, float py, const float4 r, fl
     return sure ? (int)pos : -1;
 }
 
+// The same for edge i by the FP64 rule on the original vertices.
+__device__ __forceinline__ int edge_cross64(const PipArgs &a, double2 p, int i) {
+    const double2 A = a.verts[i], B = a.verts[a.nxt[i]];
+    return cross64(p.x, p.y, A.x, A.y, B.x, B.y);
+}
+
 __device__ __forceinline__ float2 point_rel(const PipArgs &a, const PipQueued &q) {
     float hx, lx, hy, ly;
     split_double(q.p.x, hx, lx);
@@ -220,12 +226,14 @@ __device__ __forceinline__ float2 point_rel(const PipArgs &a, const PipQueued &q
     return make_float2(rel_coord(hx, lx, a.frame_x[q.ix]), rel_coord(hy, ly, a.frame_y[q.iy]));
 }
 
-// Results of up to 32 queued points, one per lane (act), in the common case: a
-// short record whose tests are all certain in FP32.  Returns false for a point
-// that needs pip_hard instead, otherwise its id in res.
-__device__ __forceinline__ bool pip_fast(const PipArgs &a, const PipQueued &q, PipSums &sum, int &res) {
+// Results of up to 32 points, one per lane, whose records are short: n <= a.search
+// near edges, the id in the first group.  Returns false for a point that needs
+// pip_hard, otherwise its id in res.  EXACT: tests that FP32 leaves open are redone
+// with the FP64 rule (fb counts them); else such a point returns false too.
+template <bool EXACT>
+__device__ __forceinline__ bool pip_short(const PipArgs &a, const PipQueued &q, PipSums &sum, int &res, unsigned &fb) {
     res = -1;
-    if (q.code == PIP_UNSURE) return false;
+    if (!EXACT && q.code == PIP_UNSURE) return false;
     const int off = -2 - q.code;
     if (!SJ_IN_BOUNDS(off < a.units_n, BND_PIP_REC)) return true;
     const int4 *u = a.units + 2 * (size_t)off;
@@ -239,8 +247,12 @@ __device__ __forceinline__ bool pip_fast(const PipArgs &a, const PipQueued &q, P
     const PipFlip *F = reinterpret_cast<const PipFlip *>(E + n);
     const float2 r = point_rel(a, q);
     bool unsure = false;
-    unsigned m = (unsigned)h0.z;
-    for (int f = 0; f < nf; ++f) {   // flips at or below y
+    unsigned m = (unsigned)h0.z, redone = 0;
+    if (EXACT) {
+        const unsigned long long ky = y_key(q.p.y);
+        for (int f = 0; f < nf && F[f].key <= ky; ++f) m = F[f].mask;
+    }
+    for (int f = 0; !EXACT && f < nf; ++f) {   // flips at or below y
         const float4 v = __ldg(reinterpret_cast<const float4 *>(F + f));
         const float d = __fsub_rn(r.y, v.x);
         unsure |= !(fabsf(d) > diff_bound(r.y, v.x, a.eps));
@@ -254,7 +266,11 @@ __device__ __forceinline__ bool pip_fast(const PipArgs &a, const PipQueued &q, P
         if (t + 2 < n) e1 = __ldg(reinterpret_cast<const float4 *>(E + t + 2));
         // lower ends ascend: from the first edge wholly above y on, none straddles
         if (__fsub_rn(e.y, r.y) > diff_bound(r.y, e.y, a.eps)) break;
-        const int x = edge_cross(r.x, r.y, e, a.eps);
+        int x = edge_cross(r.x, r.y, e, a.eps);
+        if (EXACT && x < 0) {
+            x = edge_cross64(a, q.p, E[t].vid);
+            ++redone;
+        }
         unsure |= x < 0;
         if (x > 0) m ^= __ldg(&E[t].mask);
     }
@@ -262,6 +278,7 @@ __device__ __forceinline__ bool pip_fast(const PipArgs &a, const PipQueued &q, P
     sum.tests += (unsigned)t;
     sum.pairs += (unsigned)(h0.w & (PIP_EXT - 1));
     sum.algo += (unsigned)h1.w;
+    fb += redone;
     if (m) {
         const int k = __ffs(m) - 1;
         if (h0.w & PIP_EXT) res = __ldg(reinterpret_cast<const int *>(F + nf) + k);
@@ -332,9 +349,7 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
                 if (t + HARD * k >= hi) break;
                 int x = edge_cross(r.x, r.y, e[k], a.eps);
                 if (x < 0) {
-                    const int i = E[t + HARD * k].vid;
-                    const double2 A = a.verts[i], B = a.verts[a.nxt[i]];
-                    x = cross64(p.x, p.y, A.x, A.y, B.x, B.y);
+                    x = edge_cross64(a, p, E[t + HARD * k].vid);
                     ++fb;
                 }
                 if (x) mm ^= E[t + HARD * k].mask;
@@ -442,7 +457,7 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
                 const PipQueued q = queue[w][qn + lane];
                 i = (unsigned)q.i;
                 int res;
-                const bool done = pip_fast(a, q, sums[threadIdx.x], res);
+                const bool done = pip_short<false>(a, q, sums[threadIdx.x], res, fb);
                 if (SJ_IN_BOUNDS(i < n, BND_PIP_RES)) {
                     if (done) src.put(i, res);
                     hits += done && res >= 0;
@@ -462,7 +477,10 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
         __syncwarp();
     }
     __syncwarp();
-    for (int k0 = 0; k0 < wn; k0 += 32) {   // the points that wait, one per lane
+    // The points that wait, one per lane: those of short records end here (5 M points
+    // on the sides of 500 m squares, all of whose tests FP64 decides: 2,100 us with
+    // all of them by pip_hard, 310 - 390 so).
+    for (int k0 = 0; k0 < wn; k0 += 32) {
         PipQueued q;
         bool act = k0 + lane < wn;
         int res = -1;
@@ -472,15 +490,13 @@ __global__ void __launch_bounds__(PIP_WARPS * 32, PIP_BLOCKS) k_pip_join(PipArgs
             q.p = src.point((unsigned)q.i);
             const int2 e = point_cell_exact(a.g, q.p.x, q.p.y);
             const int code = e.x >= 0 && e.y >= 0 ? a.cells[e.y * a.g.nx + e.x].x : -1;
-            const bool unsure = !(axis_estimate(q.p.x, a.g.x0f, a.g.icwf, a.g.tolx, a.g.nx, q.ix) &&
-                                  axis_estimate(q.p.y, a.g.y0f, a.g.ichf, a.g.toly, a.g.ny, q.iy));
             q.ix = e.x;
             q.iy = e.y;
             q.code = code;
             bool done = code >= -1;
             res = code;
             if (done) resolved += e.x >= 0 && e.y >= 0;
-            else if (unsure) done = pip_fast(a, q, sums[threadIdx.x], res);   // only its cell was open
+            else done = pip_short<true>(a, q, sums[threadIdx.x], res, fb);
             if (done) {
                 src.put((unsigned)q.i, res);
                 hits += res >= 0;
