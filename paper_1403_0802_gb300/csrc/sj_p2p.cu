@@ -469,35 +469,132 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) k_p2p_refine(RefineArgs a) {
     }
 }
 
-// FP64 recomputation of the points the FP32 pass did not settle: one warp
-// per point, lanes over the cell's segment list, each lane keeping the
-// smallest (squared distance, polyline id), then a warp fold.  The record is
-// left as the segment found, for the finishing kernel.
+// Squared FP32 distance to a list entry: the arithmetic of the staged loop.
+__device__ __forceinline__ float rec_d2(float2 p, const float4 r0, float inv) {
+    const float dx = __fsub_rn(p.x, r0.x), dy = __fsub_rn(p.y, r0.y);
+    const float t = __saturatef(__fmul_rn(__fmaf_rn(r0.z, dx, __fmul_rn(r0.w, dy)), inv));
+    const float qx = __fmaf_rn(-t, r0.z, dx), qy = __fmaf_rn(-t, r0.w, dy);
+    return __fmaf_rn(qx, qx, __fmul_rn(qy, qy));
+}
+
+// Smallest of the lanes' non-negative floats (their bits order as integers).
+__device__ __forceinline__ float warp_min_pos(float v) {
+    return __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(v)));
+}
+
+// The smallest FP64 (squared distance, id) over a cell's list, by a warp.
+__device__ __forceinline__ Best64 list_best64(const RefineArgs &a, int g0, int g1, double2 p, int lane) {
+    Best64 st{__longlong_as_double(0x7ff0000000000000LL), 0x7fffffff, -1};
+    for (int g = g0 + lane; g < g1; g += 32) {
+        const int i = a.cseg_ids[g];
+        consider64(st, seg_d2(a.seg, p, i), seg_owner(a.seg, i), i);
+    }
+    for (int o = 16; o > 0; o >>= 1)
+        consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
+                   __shfl_xor_sync(FULL, st.seg, o));
+    return st;
+}
+
+// FP64 recomputation of the points that the FP32 pass did not settle, a warp per
+// point: the lanes test the cell's list in FP32, the segments within 2E of the
+// nearest (E as above, M over the whole list) are queued, and FP64 distances are
+// taken for a queue of several points with full warps, lane k keeping the smallest
+// (squared distance, polyline id) of the queue's k-th point.  What is more than 2E
+// behind cannot be the nearest in FP64 arithmetic.  A point with more such segments
+// than a warp has lanes (all of them, where E is infinite) takes its whole list in
+// FP64.  The record is left as the segment found, for the finishing kernel.
+// Bound by the FP32 tests and the latency of the records; with every list entry
+// in FP64 it was bound by that pipe (the join of 3 M points with 50,000 walks given
+// three times each, FP64 form: 4,852 us then, 1,220 now).
+constexpr int RECHECK_WARPS = 8, RECHECK_QUEUE = 64;
+
 template <bool F64>
-__global__ void __launch_bounds__(256) k_p2p_recheck(RefineArgs a) {
-    const int lane = lane_id();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+__global__ void __launch_bounds__(RECHECK_WARPS * 32) k_p2p_recheck(RefineArgs a) {
+    __shared__ int2 queue[RECHECK_WARPS][RECHECK_QUEUE];   // (segment, place of its point)
+    __shared__ int owner[RECHECK_WARPS][RECHECK_QUEUE];
+    __shared__ double dist[RECHECK_WARPS][RECHECK_QUEUE];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int nwarps = gridDim.x * RECHECK_WARPS;
+    const unsigned lt = (1u << lane) - 1u;
     const int n = *a.n_fb;
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     const bool pw = a.win_on && *a.win_on;
     unsigned c_hits = 0;
-    for (int f = warp; f < n; f += nwarps) {
-        const int2 e = a.fb[f];
-        const int j = e.x, c = e.y;
-        const double2 p = slot_point(a, j);
-        Best64 st{INF, 0x7fffffff, -1};
-        for (int g = a.cseg_start[c] + lane; g < a.cseg_start[c + 1]; g += 32) {
-            const int i = a.cseg_ids[g];
-            consider64(st, seg_d2(a.seg, p, i), seg_owner(a.seg, i), i);
+    int np = 0, nq = 0;                  // points and segments in the queue
+    int slot = -1, q0 = 0, q1 = 0;       // of the queue's lane-th point, its segments
+    double2 mine = make_double2(0.0, 0.0);
+    auto put = [&](int j, int seg, double d2) {   // one lane
+        const bool hit = seg >= 0 && sqrt(d2) <= (pw ? a.win[j] : a.D);
+        a.rec[j] = !hit ? P2PRec{-1, -1} : (F64 ? P2PRec{seg, -1} : P2PRec{-2 - seg, 0});
+        c_hits += hit;
+    };
+    for (int f = blockIdx.x * RECHECK_WARPS + w;; f += nwarps) {
+        if (np > 0 && (f >= n || np == 32 || nq > RECHECK_QUEUE - 32)) {
+            __syncwarp();
+            for (int k = 0; k < nq; k += 32) {
+                const int2 q = k + lane < nq ? queue[w][k + lane] : make_int2(-1, 0);
+                const double2 p = make_double2(__shfl_sync(FULL, mine.x, q.y), __shfl_sync(FULL, mine.y, q.y));
+                if (q.x >= 0) dist[w][k + lane] = seg_d2(a.seg, p, q.x);
+            }
+            __syncwarp();
+            if (lane < np) {
+                Best64 st{INF, 0x7fffffff, -1};
+                for (int k = q0; k < q1; ++k)
+                    consider64(st, dist[w][k], owner[w][k], queue[w][k].x);
+                put(slot, st.seg, st.d2);
+            }
+            __syncwarp();
+            np = nq = 0;
         }
-        for (int o = 16; o > 0; o >>= 1)
-            consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
-                       __shfl_xor_sync(FULL, st.seg, o));
-        const bool hit = st.seg >= 0 && sqrt(st.d2) <= (pw ? a.win[j] : a.D);
-        if (lane == 0) {
-            a.rec[j] = !hit ? P2PRec{-1, -1} : (F64 ? P2PRec{st.seg, -1} : P2PRec{-2 - st.seg, 0});
-            if (hit) ++c_hits;
+        if (f >= n) break;
+        const int2 e = a.fb[f];
+        const int j = e.x, c = e.y, g0 = a.cseg_start[c], g1 = a.cseg_start[c + 1];
+        const double2 p = slot_point(a, j);
+        const float2 fo = cell_frame(a.frame_x, a.frame_y, a.g.nx, c);
+        float hx, lx, hy, ly;
+        split_double(p.x, hx, lx);
+        split_double(p.y, hy, ly);
+        const float2 pt = make_float2(rel_coord(hx, lx, fo.x), rel_coord(hy, ly, fo.y));
+        float mag = fmaxf(fabsf(pt.x), fabsf(pt.y)), d = __int_as_float(0x7f800000);
+        for (int g = g0 + lane; g < g1; g += 32) {
+            const float4 r0 = __ldg(a.cseg_rec + 2 * (size_t)g), r1 = __ldg(a.cseg_rec + 2 * (size_t)g + 1);
+            d = fminf(d, rec_d2(pt, r0, r1.x));
+            mag = fmaxf(mag, r1.z);
+        }
+        d = sqrtf(warp_min_pos(d));
+        const float bound = fmaf(64.0f * U32, warp_max(mag), 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
+        const float sep = 2.0f * bound * (1.0f + 4.0f * U32);
+        int cnt = 0;
+        for (int b = g0; b < g1 && cnt <= 32; b += 32) {
+            const int g = b + lane;
+            bool near = false;
+            int seg = 0, own = 0;
+            if (g < g1) {
+                const float4 r0 = __ldg(a.cseg_rec + 2 * (size_t)g), r1 = __ldg(a.cseg_rec + 2 * (size_t)g + 1);
+                near = !((sqrtf(rec_d2(pt, r0, r1.x)) - d) * (1.0f - 4.0f * U32) > sep);
+                seg = __float_as_int(r1.w);
+                own = __float_as_int(r1.y);
+            }
+            const unsigned bal = __ballot_sync(FULL, near);
+            const int at = cnt + __popc(bal & lt);
+            if (near && at < 32) {
+                queue[w][nq + at] = make_int2(seg, np);
+                owner[w][nq + at] = own;
+            }
+            cnt += __popc(bal);
+        }
+        if (cnt > 32) {
+            const Best64 st = list_best64(a, g0, g1, p, lane);
+            if (lane == 0) put(j, st.seg, st.d2);
+        } else {   // at least the nearest
+            if (lane == np) {
+                slot = j;
+                q0 = nq;
+                q1 = nq + cnt;
+                mine = p;
+            }
+            ++np;
+            nq += cnt;
         }
     }
     if (!F64 && a.stats) {   // F64: the finishing kernel counts the hits
@@ -540,14 +637,6 @@ __device__ __forceinline__ int fp32x_decide(const RefineArgs &a, const Best<fals
     return in_window && separated ? 1 : 2;
 }
 
-// Squared FP32 distance to a list entry: the arithmetic of the staged loop.
-__device__ __forceinline__ float rec_d2(float2 p, const float4 r0, float inv) {
-    const float dx = __fsub_rn(p.x, r0.x), dy = __fsub_rn(p.y, r0.y);
-    const float t = __saturatef(__fmul_rn(__fmaf_rn(r0.z, dx, __fmul_rn(r0.w, dy)), inv));
-    const float qx = __fmaf_rn(-t, r0.z, dx), qy = __fmaf_rn(-t, r0.w, dy);
-    return __fmaf_rn(qx, qx, __fmul_rn(qy, qy));
-}
-
 // The staged loop's prune: whether the entry's box comes within D of the box.
 __device__ __forceinline__ bool rec_near(const RefineArgs &a, const float4 r0, float smag, float4 box, float pmag) {
     const float bx = r0.x + r0.z, by = r0.y + r0.w;
@@ -555,11 +644,6 @@ __device__ __forceinline__ bool rec_near(const RefineArgs &a, const float4 r0, f
     const float gy = fmaxf(0.0f, fmaxf(fminf(r0.y, by) - box.w, box.z - fmaxf(r0.y, by)));
     const float lim = a.Df * (1.0f + 1e-6f) + 8.0f * U32 * (smag + pmag) + 8.0f * a.eps_abs;
     return gx * gx + gy * gy <= lim * lim * (1.0f + 8.0f * U32);
-}
-
-// Smallest of the lanes' non-negative floats (their bits order as integers).
-__device__ __forceinline__ float warp_min_pos(float v) {
-    return __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(v)));
 }
 
 // FP32X fold of the lanes' folds: the best polyline, and the best distance of
@@ -571,19 +655,6 @@ __device__ __forceinline__ Best<false> warp_best(const Best<false> &s) {
     r.i1 = __shfl_sync(FULL, s.i1, __ffs(__ballot_sync(FULL, s.b1 == r.b1)) - 1);
     r.b2 = warp_min_pos(s.i1 == r.i1 ? s.b2 : s.b1);
     return r;
-}
-
-// The smallest FP64 (squared distance, id) over a cell's list, by a warp.
-__device__ __forceinline__ Best64 list_best64(const RefineArgs &a, int g0, int g1, double2 p, int lane) {
-    Best64 st{__longlong_as_double(0x7ff0000000000000LL), 0x7fffffff, -1};
-    for (int g = g0 + lane; g < g1; g += 32) {
-        const int i = a.cseg_ids[g];
-        consider64(st, seg_d2(a.seg, p, i), seg_owner(a.seg, i), i);
-    }
-    for (int o = 16; o > 0; o >>= 1)
-        consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
-                   __shfl_xor_sync(FULL, st.seg, o));
-    return st;
 }
 
 template <bool F64>
@@ -1089,8 +1160,8 @@ cudaError_t launch_p2p_refine(const RefineArgs &a, int form, int warps_per_block
 }
 
 cudaError_t launch_p2p_recheck(const RefineArgs &a, int form, int blocks, cudaStream_t s) {
-    if (form == SJ_FP32X) k_p2p_recheck<false><<<blocks, 256, 0, s>>>(a);
-    else k_p2p_recheck<true><<<blocks, 256, 0, s>>>(a);
+    if (form == SJ_FP32X) k_p2p_recheck<false><<<blocks, RECHECK_WARPS * 32, 0, s>>>(a);
+    else k_p2p_recheck<true><<<blocks, RECHECK_WARPS * 32, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -133,3 +133,22 @@ def test_fp64_coordinate_ranges(api, oracle, scale, x0):
     hit = (gid >= 0) & (rid >= 0)
     assert hit.any()
     assert np.all(np.abs(gd[hit] - rd[hit]) <= 1e-12 * np.maximum(rd[hit], scale) + 4e-16 * abs(x0))
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("copies", [2, 3, 15, 16, 17, 31, 32, 33, 70])
+def test_coincident_lines(api, oracle, form, copies):
+    """Routes that share their streets: every line given `copies` times, so that no point has a single nearest one.
+    The points of a warp's FP64 queue hold 2 to 32 segments each, more than 32 leave it; one point and many."""
+    rng = np.random.default_rng(copies)
+    one = rng.uniform(5, 251, (12, 3, 2))
+    verts = np.concatenate([one] * copies).reshape(-1, 2)
+    off = np.arange(0, 3 * 12 * copies + 1, 3, dtype=np.int64)
+    g = dict(x0=0.0, y0=0.0, x1=256.0, y1=256.0, nx=4, ny=4)
+    ref = P2PRef(oracle, g, verts, off, 90.0)
+    with api.p2p_layer(verts, off, 90.0, g) as layer:
+        for n in (1, 33, 40_000):
+            pts = rng.uniform(-5, 261, (n, 2))
+            gid, gd = both_paths(api, layer, pts, form)
+            ref.check(pts, gid, gd, form)
+            assert (gid < 12).all()          # of equal distances the smallest id
