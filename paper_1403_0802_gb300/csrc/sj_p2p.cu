@@ -482,6 +482,13 @@ __device__ __forceinline__ float warp_min_pos(float v) {
     return __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(v)));
 }
 
+__device__ __forceinline__ Best64 warp_fold64(Best64 st) {
+    for (int o = 16; o > 0; o >>= 1)
+        consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
+                   __shfl_xor_sync(FULL, st.seg, o));
+    return st;
+}
+
 // The smallest FP64 (squared distance, id) over a cell's list, by a warp.
 __device__ __forceinline__ Best64 list_best64(const RefineArgs &a, int g0, int g1, double2 p, int lane) {
     Best64 st{__longlong_as_double(0x7ff0000000000000LL), 0x7fffffff, -1};
@@ -489,10 +496,53 @@ __device__ __forceinline__ Best64 list_best64(const RefineArgs &a, int g0, int g
         const int i = a.cseg_ids[g];
         consider64(st, seg_d2(a.seg, p, i), seg_owner(a.seg, i), i);
     }
-    for (int o = 16; o > 0; o >>= 1)
-        consider64(st, __shfl_xor_sync(FULL, st.d2, o), __shfl_xor_sync(FULL, st.id, o),
-                   __shfl_xor_sync(FULL, st.seg, o));
-    return st;
+    return warp_fold64(st);
+}
+
+// The segments of a cell's list [g0, g1) that can be the nearest to point p (pt
+// cell-relative) in FP64, by a warp: those that FP32 finds within 2E of its nearest.
+// The first 32 and their polylines go to seg and own (shared memory); the result is
+// their number, or more than 32.  The caller synchronises the warp.
+__device__ __forceinline__ int near_segments(const RefineArgs &a, int g0, int g1, float2 pt, int *seg, int *own, int lane) {
+    float mag = fmaxf(fabsf(pt.x), fabsf(pt.y)), d = __int_as_float(0x7f800000);
+    for (int g = g0 + lane; g < g1; g += 32) {
+        const float4 r0 = __ldg(a.cseg_rec + 2 * (size_t)g), r1 = __ldg(a.cseg_rec + 2 * (size_t)g + 1);
+        d = fminf(d, rec_d2(pt, r0, r1.x));
+        mag = fmaxf(mag, r1.z);
+    }
+    d = sqrtf(warp_min_pos(d));
+    const float bound = fmaf(64.0f * U32, warp_max(mag), 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
+    const float sep = 2.0f * bound * (1.0f + 4.0f * U32);
+    int cnt = 0;
+    for (int b = g0; b < g1 && cnt <= 32; b += 32) {
+        const int g = b + lane;
+        bool near = false;
+        float4 r1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (g < g1) {
+            r1 = __ldg(a.cseg_rec + 2 * (size_t)g + 1);
+            near = !((sqrtf(rec_d2(pt, __ldg(a.cseg_rec + 2 * (size_t)g), r1.x)) - d) * (1.0f - 4.0f * U32) > sep);
+        }
+        const unsigned bal = __ballot_sync(FULL, near);
+        const int at = cnt + __popc(bal & ((1u << lane) - 1u));
+        if (near && at < 32) {
+            seg[at] = __float_as_int(r1.w);
+            own[at] = __float_as_int(r1.y);
+        }
+        cnt += __popc(bal);
+    }
+    return cnt;
+}
+
+// FP64 result of one point, by a warp (seg and own as near_segments).
+__device__ __forceinline__ Best64 point_best64(const RefineArgs &a, int g0, int g1, double2 p, float2 pt, int *seg, int *own,
+                                               int lane) {
+    const int cnt = near_segments(a, g0, g1, pt, seg, own, lane);
+    if (cnt > 32) return list_best64(a, g0, g1, p, lane);
+    Best64 st{__longlong_as_double(0x7ff0000000000000LL), 0x7fffffff, -1};
+    __syncwarp();
+    if (lane < cnt) consider64(st, seg_d2(a.seg, p, seg[lane]), own[lane], seg[lane]);
+    __syncwarp();
+    return warp_fold64(st);
 }
 
 // FP64 recomputation of the points that the FP32 pass did not settle, a warp per
@@ -510,12 +560,11 @@ constexpr int RECHECK_WARPS = 8, RECHECK_QUEUE = 64;
 
 template <bool F64>
 __global__ void __launch_bounds__(RECHECK_WARPS * 32) k_p2p_recheck(RefineArgs a) {
-    __shared__ int2 queue[RECHECK_WARPS][RECHECK_QUEUE];   // (segment, place of its point)
-    __shared__ int owner[RECHECK_WARPS][RECHECK_QUEUE];
+    __shared__ int seg[RECHECK_WARPS][RECHECK_QUEUE], owner[RECHECK_WARPS][RECHECK_QUEUE];
+    __shared__ unsigned char place[RECHECK_WARPS][RECHECK_QUEUE];   // of the segment's point
     __shared__ double dist[RECHECK_WARPS][RECHECK_QUEUE];
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const int nwarps = gridDim.x * RECHECK_WARPS;
-    const unsigned lt = (1u << lane) - 1u;
     const int n = *a.n_fb;
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     const bool pw = a.win_on && *a.win_on;
@@ -523,25 +572,25 @@ __global__ void __launch_bounds__(RECHECK_WARPS * 32) k_p2p_recheck(RefineArgs a
     int np = 0, nq = 0;                  // points and segments in the queue
     int slot = -1, q0 = 0, q1 = 0;       // of the queue's lane-th point, its segments
     double2 mine = make_double2(0.0, 0.0);
-    auto put = [&](int j, int seg, double d2) {   // one lane
-        const bool hit = seg >= 0 && sqrt(d2) <= (pw ? a.win[j] : a.D);
-        a.rec[j] = !hit ? P2PRec{-1, -1} : (F64 ? P2PRec{seg, -1} : P2PRec{-2 - seg, 0});
+    auto put = [&](int j, const Best64 &st) {   // one lane
+        const bool hit = st.seg >= 0 && sqrt(st.d2) <= (pw ? a.win[j] : a.D);
+        a.rec[j] = !hit ? P2PRec{-1, -1} : (F64 ? P2PRec{st.seg, -1} : P2PRec{-2 - st.seg, 0});
         c_hits += hit;
     };
     for (int f = blockIdx.x * RECHECK_WARPS + w;; f += nwarps) {
         if (np > 0 && (f >= n || np == 32 || nq > RECHECK_QUEUE - 32)) {
             __syncwarp();
             for (int k = 0; k < nq; k += 32) {
-                const int2 q = k + lane < nq ? queue[w][k + lane] : make_int2(-1, 0);
-                const double2 p = make_double2(__shfl_sync(FULL, mine.x, q.y), __shfl_sync(FULL, mine.y, q.y));
-                if (q.x >= 0) dist[w][k + lane] = seg_d2(a.seg, p, q.x);
+                const bool one = k + lane < nq;
+                const int from = one ? place[w][k + lane] : 0;
+                const double2 p = make_double2(__shfl_sync(FULL, mine.x, from), __shfl_sync(FULL, mine.y, from));
+                if (one) dist[w][k + lane] = seg_d2(a.seg, p, seg[w][k + lane]);
             }
             __syncwarp();
             if (lane < np) {
                 Best64 st{INF, 0x7fffffff, -1};
-                for (int k = q0; k < q1; ++k)
-                    consider64(st, dist[w][k], owner[w][k], queue[w][k].x);
-                put(slot, st.seg, st.d2);
+                for (int k = q0; k < q1; ++k) consider64(st, dist[w][k], owner[w][k], seg[w][k]);
+                put(slot, st);
             }
             __syncwarp();
             np = nq = 0;
@@ -555,37 +604,10 @@ __global__ void __launch_bounds__(RECHECK_WARPS * 32) k_p2p_recheck(RefineArgs a
         split_double(p.x, hx, lx);
         split_double(p.y, hy, ly);
         const float2 pt = make_float2(rel_coord(hx, lx, fo.x), rel_coord(hy, ly, fo.y));
-        float mag = fmaxf(fabsf(pt.x), fabsf(pt.y)), d = __int_as_float(0x7f800000);
-        for (int g = g0 + lane; g < g1; g += 32) {
-            const float4 r0 = __ldg(a.cseg_rec + 2 * (size_t)g), r1 = __ldg(a.cseg_rec + 2 * (size_t)g + 1);
-            d = fminf(d, rec_d2(pt, r0, r1.x));
-            mag = fmaxf(mag, r1.z);
-        }
-        d = sqrtf(warp_min_pos(d));
-        const float bound = fmaf(64.0f * U32, warp_max(mag), 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
-        const float sep = 2.0f * bound * (1.0f + 4.0f * U32);
-        int cnt = 0;
-        for (int b = g0; b < g1 && cnt <= 32; b += 32) {
-            const int g = b + lane;
-            bool near = false;
-            int seg = 0, own = 0;
-            if (g < g1) {
-                const float4 r0 = __ldg(a.cseg_rec + 2 * (size_t)g), r1 = __ldg(a.cseg_rec + 2 * (size_t)g + 1);
-                near = !((sqrtf(rec_d2(pt, r0, r1.x)) - d) * (1.0f - 4.0f * U32) > sep);
-                seg = __float_as_int(r1.w);
-                own = __float_as_int(r1.y);
-            }
-            const unsigned bal = __ballot_sync(FULL, near);
-            const int at = cnt + __popc(bal & lt);
-            if (near && at < 32) {
-                queue[w][nq + at] = make_int2(seg, np);
-                owner[w][nq + at] = own;
-            }
-            cnt += __popc(bal);
-        }
+        const int cnt = near_segments(a, g0, g1, pt, &seg[w][nq], &owner[w][nq], lane);
         if (cnt > 32) {
             const Best64 st = list_best64(a, g0, g1, p, lane);
-            if (lane == 0) put(j, st.seg, st.d2);
+            if (lane == 0) put(j, st);
         } else {   // at least the nearest
             if (lane == np) {
                 slot = j;
@@ -593,6 +615,7 @@ __global__ void __launch_bounds__(RECHECK_WARPS * 32) k_p2p_recheck(RefineArgs a
                 q1 = nq + cnt;
                 mine = p;
             }
+            if (lane < cnt) place[w][nq + lane] = (unsigned char)np;
             ++np;
             nq += cnt;
         }
@@ -657,9 +680,11 @@ __device__ __forceinline__ Best<false> warp_best(const Best<false> &s) {
     return r;
 }
 
+// Registers for 5 blocks per SM (FP64: 61 registers without the bound, 60,007 points
+// 61.6 us a call instead of 59.6) and 4 (FP32X).
 template <bool F64>
-__global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, DirectArgs g, int n) {
-    __shared__ int open[DIRECT_OPEN], open_n, box[4];
+__global__ void __launch_bounds__(DIRECT_WARPS * 32, F64 ? 5 : 4) k_p2p_direct(RefineArgs a, DirectArgs g, int n) {
+    __shared__ int open[DIRECT_OPEN], open_n, box[4], near_seg[DIRECT_WARPS][32], near_own[DIRECT_WARPS][32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     const float FINF = __int_as_float(0x7f800000);
@@ -674,8 +699,10 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
         if (g.out_d) g.out_d[i] = d;
         c_hits += id >= 0;
     };
-    auto redo = [&](int i, int g0, int g1, double2 p) {
-        const Best64 st = list_best64(a, g0, g1, p, lane);
+    auto redo = [&](int i, int g0, int g1, double2 p, float2 pt) {
+        Best64 st;
+        if constexpr (F64) st = point_best64(a, g0, g1, p, pt, near_seg[w], near_own[w], lane);
+        else st = list_best64(a, g0, g1, p, lane);   // few points, and no registers for more
         const double d = sqrt(st.d2);
         const bool hit = st.seg >= 0 && d <= a.D;
         if (lane == 0) {
@@ -748,7 +775,7 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
             r.aux = __shfl_sync(FULL, m2 ? all.i2 : all.i1, max(l2, 0));
             if (__popc(m1) + __popc(m2) < 2) r.aux = -1;
             const bool out = (d - e) * (1.0f - 4.0f * U32) > a.Dup;
-            if (!(e < FINF) || (!out && three)) redo(i, g0, g1, p);
+            if (!(e < FINF) || (!out && three)) redo(i, g0, g1, p, pt);
             else if (lane == 0) a.rec[i] = out ? P2PRec{-1, -1} : r;
         } else {
             all = warp_best(all);
@@ -756,7 +783,7 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
             mag = warp_max(mag);
             const int low = fp32x_decide(a, kept, mag);   // outside: nothing nearer was left out
             if (low == 2) {
-                redo(i, g0, g1, p);
+                redo(i, g0, g1, p, pt);
             } else if (low == 0) {
                 if (lane == 0) put(i, -1, INF);
             } else if (fp32x_decide(a, all, mag_all) == 1) {
@@ -827,7 +854,7 @@ __global__ void __launch_bounds__(DIRECT_WARPS * 32) k_p2p_direct(RefineArgs a, 
                 if (fp32x_decide(a, st, mag) == 1) {
                     if (lane == 0) put(i, st.i1, widen(sqrtf(st.b1)));
                 } else {
-                    redo(i, g0, g1, p);
+                    redo(i, g0, g1, p, pt);
                 }
             }
         }
