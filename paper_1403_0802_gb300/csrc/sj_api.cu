@@ -301,6 +301,30 @@ static sj_status read_flag(int *dflag, cudaStream_t s, int *out) {
     return SJ_OK;
 }
 
+// What a layer's build leaves reserved in the stream-ordered pool: what was
+// reserved before, or BUILD_KEEP; the rest goes back to the device when this object,
+// declared before the scratch, ends.  Kept for the next build, which would map it
+// again: with nothing kept the 40,000 tiles take 2.65 instead of 2.19 ms to build,
+// the heavy-tail tiling (850 MB of scratch) 10.1 instead of 7.8.  1 GB of the
+// device's 280, so that what is sized from the free memory hardly shrinks.
+constexpr uint64_t BUILD_KEEP = 1u << 30;
+struct BuildPool {
+    cudaStream_t s;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = BUILD_KEEP;
+    BuildPool(int dev, cudaStream_t st) : s(st) {
+        uint64_t r = 0;
+        if (cudaDeviceGetDefaultMemPool(&pool, dev) != cudaSuccess) pool = nullptr;
+        else if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &r) == cudaSuccess && r > keep) keep = r;
+    }
+    ~BuildPool() {
+        uint64_t r = 0;
+        if (!pool || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &r) != cudaSuccess || r <= keep) return;
+        cudaStreamSynchronize(s);   // the scratch has been given back by then
+        cudaMemPoolTrimTo(pool, keep);
+    }
+};
+
 // Build scratch: stream-ordered allocations, freed with the object.
 struct BuildTmp {
     cudaStream_t s;
@@ -636,6 +660,7 @@ extern "C" sj_status sj_pip_layer_create(const double *verts, int64_t V, const i
     sj_layer *L = guard.L;
     L->kind = KIND_PIP;
     CUDA_TRY(cudaGetDevice(&L->device));
+    BuildPool bounded(L->device, s);
     L->grid = *g;
     L->g = make_grid(g);
     {
@@ -693,6 +718,7 @@ extern "C" sj_status sj_p2p_layer_create(const double *verts, int64_t V, const i
     sj_layer *L = guard.L;
     L->kind = KIND_P2P;
     CUDA_TRY(cudaGetDevice(&L->device));
+    BuildPool bounded(L->device, s);
     L->grid = *g;
     L->g = make_grid(g);
     {
