@@ -18,15 +18,17 @@ work items (a5), refinement (a6 / a7) with the scatter of results (a8).  The
 layer's MBBs and candidate lists (a3, a4) are built once before the timed
 region, as in serving; that build time is reported as config.layer_build_ms.
 
-The default run (the P2P workload at one GPU) prints ONE JSON line: the P2P
-headline, plus the other halves of the metric as extra keys, each timed the
-same way (CUDA events on the join's stream, its own clock record, roofline,
-CPU baseline with the GPU's measured error against the oracle, and plain FP64
-comparison): "pip_stars" (the PIP workload), "pip_at_scale_layer1" and
-"pip_at_scale_layer2" (100 M points against the 40,000-tile and the
-heavy-tail tilings), "p2p_at_scale_D50" / "_D100" / "_D200" (170 M points,
-150,000 walks) and "serve" (the serving workload); --no-extra leaves them
-out.
+The default run (the P2P workload at one GPU) prints ONE JSON line on stdout:
+the P2P headline, plus the other halves of the metric in short under "legs",
+each timed the same way (CUDA events on the join's stream, its own clock record,
+roofline, CPU baseline with the GPU's measured error against the oracle, and a
+comparison with the FP64 form): "pip_stars" (the PIP workload),
+"pip_at_scale_layer1" and "pip_at_scale_layer2" (100 M points against the
+40,000-tile and the heavy-tail tilings), "p2p_at_scale_D50" / "_D100" / "_D200"
+(170 M points, 150,000 walks) and "serve" (the serving workload); --no-extra
+leaves them out.  The full record of every leg goes to stderr, a JSON line
+each: with all of them on it the one line was too long for a reader that keeps
+some kilobytes of the output.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--workload ...] [--form fp32x|fp64]
@@ -42,7 +44,7 @@ is the algorithmic test count the candidate lists imply -- P2P: every
 (point, edge of a candidate polygon) pair, 2 compares each plus 7 flops for
 the fraction of edges that straddle the point's y (counted by sj_pip_census)
 -- divided by the refinement launch time (CUDA events on the join's stream)
-and by the FP32 (or FP64) peak measured by sj_peaks_measure.  The HBM side is
+and by the FP32 peak measured by sj_peaks_measure (both forms test in FP32).  The HBM side is
 the algorithmic bytes of the join (points in, results out, the layer once)
 over the whole join time against MEASURED_PEAKS' copy bandwidth.
 """
@@ -524,7 +526,7 @@ def roofline_of(w, form, st, ms_per_join, peaks, census=None):
         fpt = FLOPS_PER_COMPARE + FLOPS_PER_STRADDLE * frac_s
         work_note = (f"unpruned (point, candidate-polygon edge) tests x (2 + 7 x {frac_s:.4f}: the straddling "
                      f"fraction counted by sj_pip_census)")
-    peak = peaks["fp32"] if form == "fp32x" else peaks["fp64"]
+    peak = peaks["fp32"]   # both forms test in FP32; FP64 decides what that leaves open
     refine_s = refine_ms / 1e3
     achieved = algo * fpt / refine_s / 1e12 if refine_ms > 0 else None
     n = len(w.points)
@@ -535,8 +537,8 @@ def roofline_of(w, form, st, ms_per_join, peaks, census=None):
     r = {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
          "frac": achieved / peak if achieved else None,
          "traffic": measured_traffic(kernel, w.name, w.kind),
-         "peak_source": peaks["source"] + ("; FP32" if form == "fp32x" else "; FP64"),
-         "peak_derived_cross_check": peaks["derived"]["fp32" if form == "fp32x" else "fp64"],
+         "peak_source": peaks["source"] + "; FP32",
+         "peak_derived_cross_check": peaks["derived"]["fp32"],
          "work": work_note, "flops_per_test": fpt,
          "refine_ms_per_launch": refine_ms, "algorithmic_tests_per_launch": algo,
          "executed_tests_per_launch": executed,
@@ -555,7 +557,7 @@ def gpu_index(local):
 
 
 def join_leg(api, args, w, dev, stream, world, steps, warmup, peaks, baselines=True, clocks_own=True):
-    """Time `steps` joins of workload w (and, with baselines, the plain FP64
+    """Time `steps` joins of workload w (and, with baselines, the FP64
     form, the host-buffer form and the oracle on the host cores)."""
     import torch
     layer, layer_ms = build_layer(api, w, dev, stream)
@@ -587,10 +589,10 @@ def join_leg(api, args, w, dev, stream, world, steps, warmup, peaks, baselines=T
         k64 = max(3, min(steps, 20))
         with ClockSampler(gpu_index(dist_env()[2])) as clk64:
             ms64, st64, _ = time_joins(api, layer, w, pts, "fp64", k64, 2, 1, stream, ppi=ppi, clk=clk64, knobs=kn)
-        res["fp64_plain"] = {"value": n * k64 / (ms64 / 1000.0), "unit": "points/s", "ms_per_step": ms64 / k64,
-                             "steps": k64, "roofline": roofline_of(w, "fp64", st64, ms64 / k64, peaks, census),
-                             "clocks": clk64.summary()}
-        res["speedup_vs_fp64_plain"] = res["value"] / res["fp64_plain"]["value"]
+        res["fp64_form"] = {"value": n * k64 / (ms64 / 1000.0), "unit": "points/s", "ms_per_step": ms64 / k64,
+                            "steps": k64, "roofline": roofline_of(w, "fp64", st64, ms64 / k64, peaks, census),
+                            "clocks": clk64.summary()}
+        res["speedup_vs_fp64_form"] = res["value"] / res["fp64_form"]["value"]
     if baselines:
         hp = torch.empty((n, 2), dtype=torch.float64, pin_memory=True)
         hp.copy_(torch.from_numpy(w.points))
@@ -620,6 +622,31 @@ def join_leg(api, args, w, dev, stream, world, steps, warmup, peaks, baselines=T
     del pts, outs
     torch.cuda.empty_cache()
     return res
+
+
+def in_short(leg):
+    """What a leg measured, for the one line on stdout (four digits)."""
+    r = {k: leg[k] for k in ("error", "value", "unit", "ms_per_step", "p50_ms", "speedup_vs_fp64_form") if k in leg}
+    if leg.get("e2e"):
+        r["e2e"] = leg["e2e"]["value"]
+    if leg.get("roofline"):
+        r["frac"] = leg["roofline"]["frac"]
+    return {k: float(f"{v:.4g}") if isinstance(v, float) else v for k, v in r.items()}
+
+
+def one_line(args, kind, world, head, extra, launches):
+    """The record on stdout: the headline leg, the others in short."""
+    return {
+        "metric": metric_name(kind), "value": head["value"], "unit": "points/s", "n_gpus": world,
+        "steps": args.steps, "warmup": args.warmup, "ms_per_step": head["ms_per_step"],
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+        "dtype": head["dtype"], "data": "synthetic", "config": head["config"],
+        "roofline": {k: v for k, v in head["roofline"].items() if k not in ("work", "peak_derived_cross_check", "census")},
+        "cpu_baseline": head.get("cpu_baseline"), "e2e": head.get("e2e"),
+        "clocks": head["clocks"], "gpu_launches": launches,
+        **{k: head[k] for k in ("fallbacks_per_join", "speedup_vs_fp64_form") if k in head},
+        "legs": {name: in_short(leg) for name, leg in extra.items()},
+    }
 
 
 def sub_steps(ms_hint: float, steps: int) -> int:
@@ -679,19 +706,9 @@ def run_ours(args):
                                                         peaks, baselines=not args.no_baselines)
         del w4
     if rank == 0:
-        line = {
-            "metric": metric_name(w.kind), "value": head["value"], "unit": "points/s", "n_gpus": world,
-            "steps": args.steps, "warmup": args.warmup, "ms_per_step": head["ms_per_step"],
-            "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": head["dtype"], "data": "synthetic", "config": head["config"],
-            "roofline": head["roofline"], "cpu_baseline": head.get("cpu_baseline"), "e2e": head.get("e2e"),
-            "clocks": head["clocks"], "gpu_launches": kernels_per_join * args.steps,
-            "alu_peaks_tflops": {k: peaks[k] for k in ("fp32", "fp64", "source")},
-            **{k: head[k] for k in ("fallbacks_per_join", "edge_tests_per_s_algorithmic", "fp64_plain",
-                                    "speedup_vs_fp64_plain") if k in head},
-            **extra,
-        }
-        print(json.dumps(line))
+        for name, leg in {"head": head, **extra}.items():
+            print(json.dumps({"leg": name, **leg}), file=sys.stderr)
+        print(json.dumps(one_line(args, w.kind, world, head, extra, kernels_per_join * args.steps)))
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
@@ -715,7 +732,7 @@ def serve_leg_child(args):
 def serve_leg(args):
     """Continuous batching (native server, batched engine rounds) against one
     join call per request in the same native loop -- in the same form and in
-    the plain FP64 form -- on one Poisson stream of requests."""
+    the FP64 form -- on one Poisson stream of requests."""
     import torch
     world, rank, local = dist_env()
     from paper_1403_0802_gb300 import api, build, serve, synth
@@ -751,7 +768,7 @@ def serve_leg(args):
         sat = {f"{m}_{f}": timed(serve.make_stream(min(args.requests, 300), 0.0, pool_p, pool_l, seed=3), m, f)
                for m, f in arms}
         mean_pts = sat[f"batched_{args.form}"]["points"] / sat[f"batched_{args.form}"]["requests"]
-        base = sat["per_request_fp64"]["points_per_s"]          # the plain FP64 one-launch-per-request form
+        base = sat["per_request_fp64"]["points_per_s"]          # the FP64 one-launch-per-request form
         res = {}
         for rho in (0.5, 0.8):
             rate = rho * base / mean_pts
@@ -771,14 +788,14 @@ def serve_leg(args):
             "config": {"workload": f"serve_{args.requests}req_pip40k_p2p150k", "requests": args.requests,
                        "grids": f"PIP {args.serve_grid_pip}^2, P2P {args.serve_grid_p2p}^2",
                        "sizes": "log-uniform 1e3..5e6 points", "mix": "70% PIP / 30% P2P (D=100 m)",
-                       "arrivals": "Poisson, rate = rho x capacity of the plain FP64 one-join-per-request form",
+                       "arrivals": "Poisson, rate = rho x capacity of the FP64 one-join-per-request form",
                        "form": args.form, "server": "native (sj_server_*), batched engine rounds",
                        "bounded": "nothing: 10,000 requests per stream as stated; point pools of 20 M points "
                                   "per kind (requests are slices of them)"},
             "p50_ms": b["p50_ms"], "p99_ms": b["p99_ms"], "points_per_s": b["points_per_s"],
             "per_request_p50_ms": pr["p50_ms"], "per_request_p99_ms": pr["p99_ms"],
-            "plain_fp64_per_request_p50_ms": p64["p50_ms"], "plain_fp64_per_request_p99_ms": p64["p99_ms"],
-            "plain_fp64_per_request_points_per_s": p64["points_per_s"],
+            "fp64_per_request_p50_ms": p64["p50_ms"], "fp64_per_request_p99_ms": p64["p99_ms"],
+            "fp64_per_request_points_per_s": p64["points_per_s"],
             "capacity_points_per_s": {k: v["points_per_s"] for k, v in sat.items()},
             "clocks": clk.summary(), "capacity": sat, "runs": res}
     srv.close()
