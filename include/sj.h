@@ -70,7 +70,9 @@ typedef enum {
 
 /* Refinement arithmetic. */
 enum {
-    SJ_FP64 = 0,  /* plain FP64 refinement                                        */
+    SJ_FP64 = 0,  /* the results of FP64 arithmetic, bit for bit: FP32 tests rule
+                     out, with an error bound, what cannot be the answer, and
+                     FP64 decides the rest                                        */
     SJ_FP32X = 1  /* cell-relative FP32 with FP64 fallback: P2P ids are exact
                      (ties aside) and the distance error is bounded per point.
                      PIP: both forms run the same code (FP32 decides only what its
@@ -140,12 +142,13 @@ typedef struct {
 typedef struct {
     int64_t joins;
     int64_t points;        /* points submitted                                  */
-    int64_t items;         /* P2P: (cell, point-chunk) work items; PIP: batches of up
-                              to 32 points refined together                     */
+    int64_t items;         /* P2P: (cell, point-chunk) work items, or in small calls,
+                              which have none, points of cells with candidates;
+                              PIP: batches of up to 32 points refined together  */
     int64_t pairs;         /* (point, candidate object) pairs refined            */
     int64_t edge_tests;    /* PIP: point x edge tests; P2P: point x segment tests */
-    int64_t fallbacks;     /* PIP: edges redone in FP64; P2P: points refined again
-                              in FP64 over their cell's whole list              */
+    int64_t fallbacks;     /* PIP: edges redone in FP64; P2P: points that the FP32
+                              tests did not settle, refined again in FP64       */
     int64_t hits;          /* points given an id                                 */
     int64_t refine_launches; /* refinement launches timed (SJ_FLAG_TIME_REFINE)  */
     double refine_ms;        /* their summed device time, milliseconds           */
@@ -156,10 +159,10 @@ typedef struct {
     int64_t census_tests;     /* sj_pip_census totals since the last reset: the  */
     int64_t census_straddles; /* edges of the points' candidate polygons, and how
                                  many of them straddle the point's y              */
-    int64_t resolved;         /* PIP: points whose cell's candidates are all
-                                 classified inside / outside, answered without
-                                 refinement (counted in hits, not in items,
-                                 pairs or algo_tests)                             */
+    int64_t resolved;         /* PIP: points of the grid answered without refinement:
+                                 all candidates of their cell, or of their 4 x 4
+                                 sub-cell, are classified inside / outside (counted
+                                 in hits, not in items, pairs or algo_tests)      */
 } sj_run_stats;
 
 /* Build a resident polygon layer and its candidate lists (Sec. III.A: MBB of
@@ -230,8 +233,9 @@ sj_status sj_p2p_join_window(const sj_layer *layer, const double *pts, int64_t N
 
 /* Same joins from HOST buffers: the library copies the points to the device,
  * joins, copies the results back, and synchronises `stream` before returning
- * (the work starts after what is already queued on `stream`).  Inputs of more
- * than 2 M points are split into two or three chunks, pipelined on three
+ * (the work starts after what is already queued on `stream`).  Larger inputs are
+ * split into chunks (polyline joins of more than 2 M points two, of more than 8 M
+ * three; polygon joins about 1 M points each, at most 16), pipelined on three
  * library-owned streams (copy in, join, copy out), so that copies and joins of
  * different chunks overlap; every point's result is the one sj_*_join gives.  pts / out_id /
  * out_d are host pointers (pinned memory gives asynchronous full-bandwidth
@@ -273,14 +277,17 @@ sj_status sj_layer_reset_stats(sj_layer *layer);
 /* ------------------------------------------------------------------ batched rounds
  *
  * Continuous batching: an engine joins many requests per call ("round").
- * Requests against the same layer are joined as one point set -- one cell-id
- * pass, one scan, one scatter, ONE refinement launch over their merged work
- * items and one pass that writes each request's outputs -- so a round costs
- * a fixed number of launches per layer whatever the number of requests.  The
- * per-layer kernel sequence has a fixed shape (sizes live in device memory),
- * is captured into a CUDA graph on its first round and replayed afterwards.
- * Results are exactly those of joining each request alone (Sec. III.B-C:
- * a point's result depends only on the point and the layer). */
+ * Requests against the same layer are joined as one point set -- polygon
+ * layers: one launch; polyline layers: one cell-id pass, one scan, one scatter,
+ * ONE refinement launch over their merged work items and one pass that writes
+ * each request's outputs -- so a round costs a fixed number of launches per
+ * layer whatever the number of requests.  The per-layer kernel sequence has a
+ * fixed shape (sizes live in device memory), is captured into a CUDA graph on
+ * its first round and replayed afterwards.  Ids are exactly those of joining
+ * each request alone, FP64 distances too; an FP32X distance keeps its bound
+ * (Sec. III.B-C: a point's result depends only on the point and the layer;
+ * which of its FP32 and FP64 distances is given, also on the points that share
+ * its work item). */
 
 typedef struct sj_engine sj_engine;
 

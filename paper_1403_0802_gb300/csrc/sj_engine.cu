@@ -1,12 +1,12 @@
 // sj_engine.cu -- batched rounds for continuous batching (sj_engine_*).
 //
 // A round joins many requests at once.  Requests against the same layer are
-// treated as one point set: one cell-id pass over all of them (a request
-// table maps the global point index to its request), one scan over the grid,
-// one scatter, ONE refinement launch over the merged work items (results in
-// cell order), and one coalesced pass that writes every request's outputs.
-// The results are those of joining each request alone: a point's result
-// depends only on the point and the layer.
+// treated as one point set: a request table maps the global point index to its
+// request.  A polygon layer's round is one launch of the join over all of its
+// points.  A polyline layer's is one cell-id pass, one scan over the grid, one
+// scatter, ONE refinement launch over the merged work items (results in cell
+// order) and one coalesced pass that writes every request's outputs.  Ids are
+// those of joining each request alone, distances too up to the form's bound.
 //
 // All sizes a round needs are read from device memory (the request table and
 // the counters the scan writes) and every grid is sized for the engine's

@@ -636,13 +636,20 @@ __global__ void __launch_bounds__(RECHECK_WARPS * 32) k_p2p_recheck(RefineArgs a
 // bucketing pays for the grid.  us a join, bucketed against direct, 512 x 512
 // grid, 150,000 walks, D = 100 m: FP32X 1,000 points 51 / 11, 32,000 73 / 27;
 // FP64 1,000 59 / 19, 64,000 102 / 53, 131,000 134 / 93.  The lines
-// (P2P_DIRECT_*) lie where direct still wins on every layer tried (FP64), and
-// where looking up a point's cell (below) stays a few us (FP32X).
+// (P2P_DIRECT_*) lie where direct wins on every layer tried but two, by 6 % (FP64), and
+// where looking up a point's cell (below) stays a few us (FP32X).  Longer lists do
+// not move them: bucketed work items test their lists once per point as well.
+// 150,000 walks on coarser grids, bucketed / direct: FP32X 32,000 points 77 / 44
+// (128 x 128 cells), 107 / 99 (64 x 64), 303 / 214 (32 x 32); FP64 131,000 points
+// 118 / 126, 220 / 233, 786 / 627, and 5,000 walks on 4 x 4 cells 2,599 / 934.
 //
-// FP64 leaves each point's record for k_p2p_finish_fp64.  FP32X must answer
-// exactly what the bucketed refinement answers, whose certificate takes the
-// magnitude M and the tested segments from the point's work item -- the call's
-// points of its cell.  Both only grow with the item, and with them the chance
+// FP64 leaves each point's record for k_p2p_finish_fp64.  FP32X answers as the
+// bucketed refinement would with all of the call's points of a cell in one work
+// item (which it is up to 128 of them; beyond, ids still agree, and a point at the
+// edge of the certificate can have its FP32 distance on one path and its FP64
+// distance on the other).  The refinement's certificate takes the
+// magnitude M and the tested segments from the point's work item.  Both only
+// grow with the item, and with them the chance
 // that the point is redone: so they are bounded from below by those of the
 // point alone and from above by those of the whole cell.  Where both agree, the
 // item does not matter; for the others (one point in 10^4) the block looks up

@@ -5,8 +5,8 @@
 // The paper refines (cell, points) pairs against whole candidate polygons; here
 // all that a point of a cell needs is laid out once with the layer, in one
 // contiguous record per grid cell, so the join is one kernel over the points in
-// input order: no bucketing, no scratch, one coalesced read of the points and
-// one coalesced write of the ids.
+// input order: no bucketing, one coalesced read of the points and one coalesced
+// write of the ids.
 //
 // Per cell (PipArgs::cells), a code:
 //   >= -1   the result of every point of the cell (no candidate's edge comes

@@ -14,7 +14,7 @@ arrival) and throughput.
 
 mode="per_request" runs the same native loop with one join call per request
 in arrival order -- the baseline the batched form is measured against -- in
-the server's form or another one (form="fp64" gives the plain FP64 form).
+the server's form or another one (form="fp64" gives the FP64 form).
 """
 from __future__ import annotations
 
