@@ -514,6 +514,7 @@ __device__ __forceinline__ int near_segments(const RefineArgs &a, int g0, int g1
     const float bound = fmaf(64.0f * U32, warp_max(mag), 4.0f * a.eps_abs) * (1.0f + 8.0f * U32);
     const float sep = 2.0f * bound * (1.0f + 4.0f * U32);
     int cnt = 0;
+    __syncwarp();   // a point of more than 32 leaves seg and own as it filled them: orders the writes
     for (int b = g0; b < g1 && cnt <= 32; b += 32) {
         const int g = b + lane;
         bool near = false;

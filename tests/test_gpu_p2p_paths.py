@@ -152,3 +152,23 @@ def test_coincident_lines(api, oracle, form, copies):
             gid, gd = both_paths(api, layer, pts, form)
             ref.check(pts, gid, gd, form)
             assert (gid < 12).all()          # of equal distances the smallest id
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_few_and_many_coincident_lines(api, oracle, form):
+    """Lines given 3 times beside lines given 40 times: a warp takes points that fit its FP64 queue and points that
+    leave it in turn, in the same places of shared memory."""
+    rng = np.random.default_rng(6)
+    one = rng.uniform(5, 251, (24, 3, 2))
+    times = np.where(np.arange(24) % 2, 3, 40)
+    verts = np.repeat(one, times, axis=0).reshape(-1, 2)
+    off = np.arange(0, 3 * times.sum() + 1, 3, dtype=np.int64)
+    g = dict(x0=0.0, y0=0.0, x1=256.0, y1=256.0, nx=4, ny=4)
+    ref = P2PRef(oracle, g, verts, off, 90.0)
+    first = np.concatenate([[0], np.cumsum(times)[:-1]])
+    with api.p2p_layer(verts, off, 90.0, g) as layer:
+        for n in (40, 40_000, 140_000):
+            pts = rng.uniform(-5, 261, (n, 2))
+            gid, gd = both_paths(api, layer, pts, form)
+            ref.check(pts, gid, gd, form)
+            assert np.isin(gid[gid >= 0], first).all()   # of equal distances the smallest id
