@@ -172,3 +172,23 @@ def test_few_and_many_coincident_lines(api, oracle, form):
             gid, gd = both_paths(api, layer, pts, form)
             ref.check(pts, gid, gd, form)
             assert np.isin(gid[gid >= 0], first).all()   # of equal distances the smallest id
+
+
+def test_dense_cells_fp32x(api, oracle):
+    """A cell with more points than a work item holds: the direct path certifies each point with all of the call's
+    points of its cell, bucketing with those of its item.  Ids are the same; where the distances are not, one is the
+    FP32 and the other the FP64 distance, each within the oracle's bound."""
+    rng = np.random.default_rng(13)
+    segs = rng.uniform(10, 246, (60, 2, 2))
+    segs[1::2] = segs[::2] + rng.uniform(1e-3, 3e-3, (30, 1, 1))   # near-ties, which the item can decide
+    verts, off = segs.reshape(-1, 2), np.arange(0, 121, 2, dtype=np.int64)
+    g = dict(x0=0.0, y0=0.0, x1=256.0, y1=256.0, nx=4, ny=4)
+    pts = rng.uniform(0, 256, (32_768, 2))
+    ref = P2PRef(oracle, g, verts, off, 400.0)
+    r = ref.join(pts)
+    with api.p2p_layer(verts, off, 400.0, g) as layer:
+        p = torch.as_tensor(pts, device="cuda")
+        a, b = api.p2p_join(layer, p, form="fp32x"), api.p2p_join(layer, p, form="fp32x", pts_per_item=128)
+        torch.testing.assert_close(a[0], b[0], rtol=0, atol=0)
+        for gid, gd in (a, b):
+            ref.check(pts, gid.cpu().numpy(), gd.cpu().numpy(), "fp32x", ref=r)
