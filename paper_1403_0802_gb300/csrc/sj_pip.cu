@@ -374,14 +374,14 @@ __device__ __forceinline__ int pip_hard(const PipArgs &a, const PipQueued &q, Pi
 // certain and classified is answered at once.  The others are queued in shared
 // memory and refined 32 at a time, so that the refinement runs with full warps
 // although only some of a tile's points (6 - 54 %) need it.  The few that this
-// cannot finish wait until the warp has seen its last tile, in the warp's list
-// (in scratch, or while it is short in shared memory); by then their general, register-hungry code costs the loop
-// nothing (with a call to it inside the loop the 100 M point join took 2.3 - 4.5 ms
-// instead of 1.6; with lists of up to 64 points in shared memory, refined whenever
-// 32 wait, 1.31 instead of 1.22 ms, and 10 M points on the heavy-tail tiles 433
-// instead of 396 us).  Not in the output, threaded through the points' own places:
-// requests and streams may share an output, and a list lost there takes other
-// requests' points with it.
+// cannot finish wait until the warp has seen its last tile, in the warp's list (in
+// scratch, or while it is short in shared memory); by then their general,
+// register-hungry code costs the loop nothing (with a call to it inside the loop the
+// 100 M point join took 2.3 - 4.5 ms instead of 1.6; with lists of up to 64 points in
+// shared memory, refined whenever 32 wait, 1.31 instead of 1.22 ms, and 10 M points on
+// the heavy-tail tiles 433 instead of 396 us).  Not in the output, threaded through
+// the points' own places: requests and streams may share an output, and a list lost
+// there takes other requests' points with it.
 //
 // Bound by the latency and the L1 wavefronts of the random reads of the cell
 // table and the records, both L2-resident (ncu at 20 M points on the tiles: issue
